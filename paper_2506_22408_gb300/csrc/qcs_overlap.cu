@@ -18,13 +18,11 @@
 //  3. pf(B + w_k D) at the node plan's evaluation points w_k (a Gauss rule on the
 //     unit circle by default, roots of unity on request), D = C_0^(s): the node
 //     matrices differ only in their empty x empty block, so the occupied block is
-//     eliminated once (schur_occupied, pivots inside that block) and each node's
-//     2d x 2d complement is eliminated by Parlett-Reid with partial pivoting, the
-//     nodes in lockstep.  The matrices (packed upper triangles) stay in shared
-//     memory; the elimination keeps the original index order (no physical swaps)
-//     and tracks the sign of each pivot's position; every rank-2 update step
-//     spreads (node, entry) items over the lanes.  Pivot magnitudes are compared
-//     as integer keys (no FP64 work).
+//     eliminated once (pivots inside that block) and each node's 2d x 2d complement
+//     is eliminated by Parlett-Reid with partial pivoting, the nodes in lockstep;
+//     up to 16 modes in 64-bit fixed point on the integer pipe (qcs_fixed.cuh: the
+//     n = 12, 201 x 3001 per-pair case went from 29.5 to 23.5 ms), above in FP64 by
+//     two warps (qcs_group.cuh).
 //  4. S_p = sum_k gamma_k pf_k, where gamma_k folds the node plan's weights, the
 //     inverse-channel weights C(2n,2x)/C(n,x) and the palindromic symmetry
 //     c_{n-x} = c_x of parity +1 snapshots (parity -1 snapshots are exactly zero
@@ -35,6 +33,7 @@
 // snapshot of the tile in turn and writes one partial sum per warp slot, reduced
 // in a fixed order afterwards, so the result does not depend on scheduling.
 #include "qcs_internal.h"
+#include "qcs_fixed.cuh"
 #include "qcs_group.cuh"
 
 namespace {
@@ -81,15 +80,14 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
     cd *Rg = reinterpret_cast<cd *>(wbase);
     cd *Qs = Rg;  // staged snapshot rows (shared-memory path only)
     cd *Ts = reinterpret_cast<cd *>(wbase + A.off_T);
-    cd *Ns = Rg;  // node matrices, once T is consumed
+    fx2 *Ns = reinterpret_cast<fx2 *>(wbase);  // node matrices, once T is consumed
     double *Uss = reinterpret_cast<double *>(Uts + n * ld_ut(n));  // re + im of Ut
     cd *Bs = reinterpret_cast<cd *>(wbase + A.off_B);
-    cd *Uv = reinterpret_cast<cd *>(wbase + A.off_U);
-    cd *Vv = reinterpret_cast<cd *>(wbase + A.off_V);
-    cd *pf = reinterpret_cast<cd *>(wbase + A.off_pf);
-    uint8_t *act0 = reinterpret_cast<uint8_t *>(wbase + A.off_act);
-    uint8_t *act1 = act0 + A.vm;
-    cd *pv = reinterpret_cast<cd *>(wbase + A.off_pv);
+    const FxWarp tm = {lane, lane, 0, 0, nullptr};
+    const int npv = pv_records(A.vm, A.NB);
+    fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
+    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
+                       reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
     const int span = A.chunk * wpb;  // snapshots per tile; warp w takes every wpb-th
     // chunk-major tile order: consecutive tiles share one snapshot chunk and run over
     // the walkers (whose rows all fit in L2), so each snapshot is fetched from HBM once
@@ -237,20 +235,7 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
             __syncwarp();
             build_B(A.n, A.ne, Ts, Bs, tab, lane);
             __syncwarp();
-            // occupied block eliminated once for all nodes when that is stable
-            cd *pvo = pv + pv_records(A.vm, A.NB, A.ne);  // the occupied pivots
-            const bool shared = schur_occupied(A.m, A.ne, Bs, Ns, Uv, Vv, act0, act1, tab, pvo, lane);
-            const int mm = shared ? A.m - A.ne : A.m, nee = shared ? 0 : A.ne;
-            const int NBr = shared ? A.NB : 1;  // the rare full eliminations run one node per round
-            cd S = cmk(0.0, 0.0);
-            for (int k0 = 0; k0 < A.nev; k0 += NBr) {
-                int nb = A.nev - k0 < NBr ? A.nev - k0 : NBr;
-                node_pfaffians(mm, nee, A.wnode + k0, A.gamma + k0, nb, Bs, Ns, Uv, Vv, pf, act0, act1, tab, pv,
-                               shared ? A.ne / 2 : 0, pvo, lane);
-                if (lane == 0)
-                    for (int v = 0; v < nb; ++v) S = cadd(S, pf[v]);  // pf[v] carries gamma
-                __syncwarp();
-            }
+            const cd S = fx_pair_sum(tm, A.m, A.ne, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, Ns, tab);
             if (lane == 0) {
                 if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
                 acc = cadd(acc, S);
@@ -349,12 +334,8 @@ size_t pair_warp_layout(PairArgs &A, int NB) {
     o = align16(o + (size_t)A.vm * sizeof(cd));
     A.off_V = (int)o;
     o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNB * sizeof(cd));
-    A.off_act = (int)o;
-    o = align16(o + (size_t)2 * A.vm);
-    A.off_pv = (int)o;  // node products (gamma and the occupied pivots included), then those pivots
-    o = align16(o + (size_t)(pv_records(A.vm, NB, A.ne) + A.ne / 2) * sizeof(cd));
+    A.off_pv = (int)o;  // records of the node products, then of the occupied pivots
+    o = align16(o + pv_bytes(A.vm, NB, A.ne));
     return o;
 }
 

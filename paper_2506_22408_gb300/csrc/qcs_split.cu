@@ -21,6 +21,7 @@
 // accumulated in FP32, B^(s) an FP32 rounding of its 2n-term sums; the Pfaffian
 // elimination, its pivoting and the node sums stay FP64.
 #include "qcs_internal.h"
+#include "qcs_fixed.cuh"
 #include "qcs_group.cuh"
 #include "qcs_tc.cuh"
 
@@ -171,7 +172,7 @@ __device__ void build_B_f32(int n, int ne, const float2 *__restrict__ Ts, int ld
     }
 }
 
-__global__ void __launch_bounds__(128) split_pair_kernel(const __grid_constant__ SplitArgs A) {
+__global__ void __launch_bounds__(128, 3) split_pair_kernel(const __grid_constant__ SplitArgs A) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t mbar_load, mbar_mma;
@@ -196,13 +197,12 @@ __global__ void __launch_bounds__(128) split_pair_kernel(const __grid_constant__
     unsigned char *wbase = region + (size_t)warp * A.warp_bytes;
     float2 *Ts = reinterpret_cast<float2 *>(wbase + A.off_T);
     cd *Bs = reinterpret_cast<cd *>(wbase + A.off_B);
-    cd *Ns = reinterpret_cast<cd *>(wbase);  // node matrices start the warp region (T is consumed first)
-    cd *Uv = reinterpret_cast<cd *>(wbase + A.off_U);
-    cd *Vv = reinterpret_cast<cd *>(wbase + A.off_V);
-    cd *pf = reinterpret_cast<cd *>(wbase + A.off_pf);
-    uint8_t *act0 = wbase + A.off_act;
-    uint8_t *act1 = act0 + A.vm;
-    cd *pv = reinterpret_cast<cd *>(wbase + A.off_pv);
+    fx2 *Ns = reinterpret_cast<fx2 *>(wbase);  // node matrices start the warp region (T is consumed first)
+    const FxWarp tm = {lane, lane, 0, 0, nullptr};
+    const int npv = pv_records(A.vm, A.NB);
+    fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
+    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
+                       reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
     const int ldT = 2 * n + 1;
 
     if (warp == 0) {
@@ -313,20 +313,7 @@ __global__ void __launch_bounds__(128) split_pair_kernel(const __grid_constant__
                 if (w >= A.W) continue;
                 build_B_f32(n, A.ne, Ts, ldT, Bs, tab, lane);
                 __syncwarp();
-                // occupied block eliminated once for all nodes when that is stable
-                cd *pvo = pv + pv_records(A.vm, A.NB, A.ne);  // the occupied pivots
-                const bool shared = schur_occupied(A.m, A.ne, Bs, Ns, Uv, Vv, act0, act1, tab, pvo, lane);
-                const int mm = shared ? A.m - A.ne : A.m, nee = shared ? 0 : A.ne;
-                const int NBr = shared ? A.NB : 1;  // the rare full eliminations run one node per round
-                cd S = cmk(0.0, 0.0);
-                for (int k0 = 0; k0 < A.nev; k0 += NBr) {
-                    const int nb = A.nev - k0 < NBr ? A.nev - k0 : NBr;
-                    node_pfaffians(mm, nee, A.wnode + k0, A.gamma + k0, nb, Bs, Ns, Uv, Vv, pf, act0, act1, tab, pv,
-                                   shared ? A.ne / 2 : 0, pvo, lane);
-                    if (lane == 0)
-                        for (int vv = 0; vv < nb; ++vv) S = cadd(S, pf[vv]);  // pf[vv] carries gamma
-                    __syncwarp();
-                }
+                const cd S = fx_pair_sum(tm, A.m, A.ne, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, Ns, tab);
                 if (lane == 0) {
                     if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
                     acc = cadd(acc, S);
@@ -628,12 +615,8 @@ size_t split_warp_layout(SplitArgs &A, int NB) {
     o = align16(o + (size_t)A.vm * sizeof(cd));
     A.off_V = (int)o;
     o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNB * sizeof(cd));
-    A.off_act = (int)o;
-    o = align16(o + (size_t)2 * A.vm);
-    A.off_pv = (int)o;  // node products (gamma and the occupied pivots included), then those pivots
-    o = align16(o + (size_t)(pv_records(A.vm, NB, A.ne) + A.ne / 2) * sizeof(cd));
+    A.off_pv = (int)o;  // records of the node products, then of the occupied pivots
+    o = align16(o + pv_bytes(A.vm, NB, A.ne));
     return o;
 }
 

@@ -36,13 +36,14 @@
 //     writes the seven slices straight from the lanes as the next A operand, laid out
 //     MN-major (lane k owns column k of Z_i^T);
 //  4. 14 more MMAs form P_i = M Z_i (lane b of warp i, column a: P_i[a][b]); each warp
-//     converts its lanes to FP64, keeps the upper triangle of P_i, assembles B^(s) and
-//     runs the node Pfaffians of the FP64 path (qcs_pair.cuh).
+//     shifts its lanes to the pair's common scale, keeps the upper triangle of P_i,
+//     assembles B^(s) and runs the node Pfaffians, all in fixed point (qcs_fixed.cuh;
+//     1024 x 20000 at n = 16, ne = 8: 377 ms with FP64 eliminations, 263 ms).
 // Every wait is bounded: a time-out raises QCS_ERR_TIMEOUT, drains and frees the
 // tensor memory.
 #include "qcs_internal.h"
 #include "qcs_ozaki.cuh"
-#include "qcs_pair.cuh"
+#include "qcs_fixed.cuh"
 #include "qcs_tc.cuh"
 
 using namespace qcs_tc;
@@ -174,7 +175,7 @@ struct TcArgs {
     int teams;        // four-warp teams in the block
     int team_bytes;   // shared bytes per team: records (and workspaces if not in them)
     int tslots;       // tensor-memory accumulators of 256 columns
-    int off_P, off_N, off_U, off_V, off_pf, off_act, off_pv;  // B^(s) at offset 0
+    int off_P, off_N, off_U, off_V, off_pv;  // B^(s) at offset 0
     int vm;
     int smem_tab;     // byte offset of the pair table (after the teams' regions)
     const unsigned char *snap_rec;
@@ -229,48 +230,53 @@ __device__ __forceinline__ void read_levels8(uint32_t taddr, int cb, long long (
     }
 }
 
-// P[a][b] (a != b) from the upper triangle Pu (P is skew-symmetric): the sign of the
-// lower triangle flipped on the bit pattern, without a branch or an FP64 instruction.
-__device__ __forceinline__ double pget(const double *__restrict__ Pu, int a, int b) {
+// P[a][b] (a != b) from the upper triangle Pu (P is skew-symmetric), fixed point.
+__device__ __forceinline__ long long pget(const long long *__restrict__ Pu, int a, int b) {
     const bool sw = a > b;
-    const long long v = __double_as_longlong(Pu[tri_index(sw ? b : a, sw ? a : b)]);
-    return __longlong_as_double(sw ? v ^ (long long)0x8000000000000000ull : v);
+    const long long v = Pu[tri_index(sw ? b : a, sw ? a : b)];
+    return sw ? -v : v;
 }
 
-// B^(s) (packed upper, m x m) from P = R J R^T, R = [Re T; Im T]: selected row x < ne is
-// T_x (= R[x] + i R[n+x]); x >= ne is Re T_j (even offset) or -Im T_j (odd offset) for
-// the empty mode j = ne + (x - ne)/2.  One loop per block (occupied x occupied, occupied
-// x empty, empty x empty), so that no pass of the warp diverges across the three forms.
-__device__ void build_B_from_P(int n, int ne, int m, const double *__restrict__ Pu, cd *__restrict__ Bs,
-                               const uint16_t *__restrict__ tab, int lane) {
-    // occupied x occupied: (R_x + i R_nx) J (R_y + i R_ny)^T, the first tri(ne) entries
-    for (int t = lane; t < tri_count(ne); t += 32) {
-        int x, y;
-        pair_of(tab, t, x, y);  // x < y
-        const double prr = pget(Pu, x, y), pii = pget(Pu, n + x, n + y);
-        const double pri = pget(Pu, x, n + y), pir = pget(Pu, n + x, y);
-        Bs[t] = cmk(prr - pii, pri + pir);
-    }
-    // occupied x empty: (R_x + i R_nx) J (+-R_ry)^T, column y = ne + c, row x < ne
+// B^(s) (packed upper, m x m, fixed point, the empty modes' rows first) from P = R J R^T,
+// R = [Re T; Im T]: an empty row c is Re T_j (c even) or -Im T_j (c odd) of mode
+// j = ne + c/2; the occupied row x is T_x (= R[x] + i R[n+x]).  One loop per block (empty x
+// empty, empty x occupied, occupied x occupied), so that no pass of the warp diverges
+// across the three forms.  Returns this lane's OR of the entries' upper words.
+__device__ unsigned build_B_from_P(int n, int ne, int m, const long long *__restrict__ Pu, fx2 *__restrict__ Bs,
+                                   const uint16_t *__restrict__ tab, int lane) {
+    unsigned top = 0u;
     const int d2 = m - ne;
-    for (int e = lane; e < d2 * ne; e += 32) {
-        const int c = e / ne, x = e - c * ne;
-        const int jy = ne + (c >> 1);
-        const bool yim = c & 1;
-        const int ry = yim ? n + jy : jy;
-        cd v = cmk(pget(Pu, x, ry), pget(Pu, n + x, ry));
-        Bs[tri_index(x, ne + c)] = flip_if(v, yim);
-    }
     // empty x empty: (+-R_rx) J (+-R_ry)^T, real
     for (int t = lane; t < tri_count(d2); t += 32) {
         int cx, cy;
         pair_of(tab, t, cx, cy);  // cx < cy
         const int jx = ne + (cx >> 1), jy = ne + (cy >> 1);
         const bool xim = cx & 1, yim = cy & 1;
-        const long long re = __double_as_longlong(pget(Pu, xim ? n + jx : jx, yim ? n + jy : jy));
-        Bs[tri_index(ne + cx, ne + cy)] =
-            cmk(__longlong_as_double(xim != yim ? re ^ (long long)0x8000000000000000ull : re), 0.0);
+        const long long re = pget(Pu, xim ? n + jx : jx, yim ? n + jy : jy);
+        const fx2 v = make_longlong2(xim != yim ? -re : re, 0ll);
+        top |= fx_top(v);
+        Bs[t] = v;
     }
+    // empty x occupied: (+-R_rc) J (R_x + i R_nx)^T
+    for (int e = lane; e < d2 * ne; e += 32) {
+        const int x = e / d2, c = e - x * d2;
+        const int jc = ne + (c >> 1);
+        const bool cim = c & 1;
+        const int rc = cim ? n + jc : jc;
+        const long long re = pget(Pu, rc, x), im = pget(Pu, rc, n + x);
+        const fx2 v = make_longlong2(cim ? -re : re, cim ? -im : im);
+        top |= fx_top(v);
+        Bs[tri_index(c, d2 + x)] = v;
+    }
+    // occupied x occupied: (R_x + i R_nx) J (R_y + i R_ny)^T
+    for (int t = lane; t < tri_count(ne); t += 32) {
+        int x, y;
+        pair_of(tab, t, x, y);  // x < y
+        const fx2 v = make_longlong2(pget(Pu, x, y) - pget(Pu, n + x, n + y), pget(Pu, x, n + y) + pget(Pu, n + x, y));
+        top |= fx_top(v);
+        Bs[tri_index(d2 + x, d2 + y)] = v;
+    }
+    return __reduce_or_sync(QCS_FULL, top);
 }
 
 // Byte offset of element (row, k) of a 16-bit MN-major operand of 128 rows x 32 (K) with
@@ -367,15 +373,14 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem_tc + A.smem_tab);
     build_pair_table(tab, tri_count(A.m));
     unsigned char *wbase = (A.ws_in_operands ? X : X + kSnapRecBytes + kWalkRecBytes) + (size_t)wt * A.ws_bytes;
-    cd *Bs = reinterpret_cast<cd *>(wbase);
-    double *Pu = reinterpret_cast<double *>(wbase + A.off_P);
-    cd *Ns = reinterpret_cast<cd *>(wbase + A.off_N);  // aliases Pu: written once B^(s) is assembled
-    cd *Uv = reinterpret_cast<cd *>(wbase + A.off_U);
-    cd *Vv = reinterpret_cast<cd *>(wbase + A.off_V);
-    cd *pf = reinterpret_cast<cd *>(wbase + A.off_pf);
-    uint8_t *act0 = wbase + A.off_act;
-    uint8_t *act1 = act0 + A.vm;
-    cd *pv = reinterpret_cast<cd *>(wbase + A.off_pv);
+    fx2 *Bs = reinterpret_cast<fx2 *>(wbase);
+    long long *Pu = reinterpret_cast<long long *>(wbase + A.off_P);
+    fx2 *Ns = reinterpret_cast<fx2 *>(wbase + A.off_N);  // aliases Pu: written once the occupied block is eliminated
+    const FxWarp tm = {lane, lane, 0, 0, nullptr};
+    const int npv = pv_records(A.vm, A.NB);
+    fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
+    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
+                       reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
 
     if (warp == 0) {
         tmem_alloc(&tmem_base, (uint32_t)A.tslots * kTmemCols);
@@ -484,54 +489,45 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
             // ---- Z_i = H_i M^T: lane k holds row k; sliced by rows of Z^T (MN-major)
             if (!(ok = product(false, tbase))) break;
             // the operand region held H_i, which the completed MMAs no longer read
-            const int Fb = slice_zt(tlane, g_exp[wt * kRowsPer + lane], e_exp[lane], X, wt * kRowsPer, lane);
+            const int g_exp_lane = g_exp[wt * kRowsPer + lane];
+            const int Fb = slice_zt(tlane, g_exp_lane, e_exp[lane], X, wt * kRowsPer, lane);
             fence_proxy_async_smem();
             fence_before_sync();
             team_sync(team);  // every warp's tensor-memory reads and operand writes are done
             // ---- P_i = M Z_i: lane b, column a holds P_i[a][b] = z 2^{e_a + F_b - 56}
             if (!(ok = product(true, tbase))) break;
+            // the snapshot's largest row exponent G bounds |H| < 2^G: an orthogonal H (norm one)
+            // and walker rows of norm at most one give |P| <= 1 < 2^{G+2}, any H of that size
+            // |P| <= 32 2^G; P is held as X 2^-fP, fP = 57 - G (below 2^59 and 2^62)
+            const int G = __reduce_max_sync(QCS_FULL, g_exp_lane);
+            const int fP = 57 - (G == kNoRow ? 0 : G);
+            const int shb = Fb == kNoRow ? kNoRow : Fb - 56 + fP;
 #pragma unroll 1
             for (int cb = 0; cb < 4; ++cb) {
                 long long z[8];
                 read_levels8(tlane, cb, z);
-                // every lane converts all eight entries (no divergence); the upper
-                // triangle of P_i (a < lane) is stored into the free operand region
-                bool in_range = true;
+                // the upper triangle of P_i (a < lane) goes into the free operand region
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const int a = 8 * cb + c;
-                    const int ea = e_exp[a];
-                    const bool zero = Fb == kNoRow || ea == kNoRow;
-                    const double val = fixed_to_f64(zero ? 0ll : z[c], ea + Fb - 56, in_range);
-                    if (a < lane) Pu[tri_index(a, lane)] = val;
-                }
-                if (!__all_sync(QCS_FULL, in_range)) {  // an exponent outside the normal range
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const int a = 8 * cb + c;
-                        const int ea = e_exp[a];
-                        if (a < lane && Fb != kNoRow && ea != kNoRow)
-                            Pu[tri_index(a, lane)] = fixed_to_f64_exact(z[c], ea + Fb - 56);
-                    }
+                    const int sh = e_exp[a] + shb;  // far below -64 for a zero row
+                    if (a < lane) Pu[tri_index(a, lane)] = fx_shift_any(z[c], sh);
                 }
             }
             release();  // this team's tensor-memory reads are done; another team may use the slot
             const int64_t slot = pb + wt;
             if (slot < L && QCS_IN_BOUNDS(A.idx[slot] >= 0 && A.idx[slot] < A.P, A.status)) {
-                build_B_from_P(n, A.ne, A.m, Pu, Bs, tab, lane);
+                int f = fP, mb = fx_top_bits(build_B_from_P(n, A.ne, A.m, Pu, Bs, tab, lane));
                 __syncwarp();
-                cd *pvo = pv + pv_records(A.vm, A.NB, A.ne);  // the occupied pivots
-                const bool shared = schur_occupied(A.m, A.ne, Bs, Ns, Uv, Vv, act0, act1, tab, pvo, lane);
-                const int mm = shared ? A.m - A.ne : A.m, nee = shared ? 0 : A.ne;
-                const int NBr = shared ? A.NB : 1;  // the rare full eliminations run one node per round
-                cd S = cmk(0.0, 0.0);
-                for (int k0 = 0; k0 < A.nev; k0 += NBr) {
-                    const int nb = A.nev - k0 < NBr ? A.nev - k0 : NBr;
-                    node_pfaffians(mm, nee, A.wnode + k0, A.gamma + k0, nb, Bs, Ns, Uv, Vv, pf, act0, act1, tab, pv,
-                                   shared ? A.ne / 2 : 0, pvo, lane);
-                    if (lane == 0)
-                        for (int v = 0; v < nb; ++v) S = cadd(S, pf[v]);  // pf[v] carries gamma
+                cd S;
+                if (fx_schur_occupied(tm, A.m, A.ne, Bs, wk.Gv, wk.Vv, tab, wk.pv + npv, wk.pe + npv, f, mb)) {
+                    S = fx_node_sum(tm, A.m, A.ne, true, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, f, mb, Ns, tab);
+                } else {  // rare: B^(s) again, every node matrix in full
                     __syncwarp();
+                    f = fP;
+                    mb = fx_top_bits(build_B_from_P(n, A.ne, A.m, Pu, Bs, tab, lane));
+                    __syncwarp();
+                    S = fx_node_sum(tm, A.m, A.ne, false, A.nev, 1, A.wnode, A.gamma, wk, Bs, f, mb, Ns, tab);
                 }
                 if (lane == 0) {
                     if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
@@ -579,12 +575,8 @@ size_t tc_warp_layout(TcArgs &A, int NB) {
     o = align16(o + (size_t)A.vm * sizeof(cd));
     A.off_V = (int)o;
     o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNB * sizeof(cd));
-    A.off_act = (int)o;
-    o = align16(o + (size_t)2 * A.vm);
-    A.off_pv = (int)o;  // node products (gamma and the occupied pivots included), then those pivots
-    o = align16(o + (size_t)(pv_records(A.vm, NB, A.ne) + A.ne / 2) * sizeof(cd));
+    A.off_pv = (int)o;  // records of the node products, then of the occupied pivots
+    o = align16(o + pv_bytes(A.vm, NB, A.ne));
     return o;
 }
 

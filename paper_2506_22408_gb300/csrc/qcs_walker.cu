@@ -190,7 +190,8 @@ __global__ void walker_prep_kernel(int n, int ne, int64_t W, const cd *__restric
                 default: ip = cmk(0, -1); break;
             }
             double sc = 2.0 * ldexp(1.0, -(n - ne / 2));
-            pref[w] = cscale(cmul(detR, ip), sc);
+            // a non-finite walker: NaN from here on (the fixed-point eliminations hold none)
+            pref[w] = bad ? cmk(nan(""), nan("")) : cscale(cmul(detR, ip), sc);
             if (bad || !cfinite(detR)) raise_status(status, QCS_ERR_NONFINITE);
         }
         __syncwarp();
