@@ -401,12 +401,17 @@ extern "C" int qcs_snapshots_modes(const qcs_snapshots *s) { return s ? s->n : -
 namespace {
 
 const int kChunk = 4;  // snapshots per warp in an overlap tile
+const size_t kBatchBytes = (size_t)512 << 20;  // pair records of one tensor-core batch
 
 struct OverlapWork {
     cd *Ut, *pref, *partial;
     unsigned long long *counter;
     float *Mhi, *Mlo;          // split precision: walker operand slabs
     unsigned char *walk_rec;   // tensor-core congruence: walker slice records
+    unsigned char *rec;        // ... pair records of a batch of wblock walkers x span list positions
+    cd *sum;                   // ... and their Pfaffian sums
+    int64_t wblock;
+    int span;
     int *mode;                 // FP64 ALU path: per-walker form of the occupied rows (walker prep)
     int nchunks, nparts;
     int config, chunk;         // resolved kernel configuration, ALU snapshots per warp in a tile
@@ -471,9 +476,20 @@ qcs_status overlap_common(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t 
     wk->tc = tc;
     wk->chunk = cfg.chunk > 0 ? cfg.chunk : kChunk;
     // partial sums: FP64 ALU path one per (walker, tile, warp); split path one per
-    // (walker, tile of snapshots); tensor-core path one per (walker, tile)
-    const int span = split ? qcs_split_snaps_per_tile(n, cfg.subs) : tc ? qcs_tc_snaps_per_tile(cfg.subs)
-                                                             : wk->chunk * qcs_pair_warps_per_block();
+    // (walker, tile of snapshots); tensor-core path one per (walker, batch)
+    wk->wblock = W > 0 ? W : 1;
+    int span = split ? qcs_split_snaps_per_tile(n, cfg.subs) : wk->chunk * qcs_pair_warps_per_block();
+    if (tc) {
+        // a batch's pair records take at most kBatchBytes: all walkers and as many list
+        // positions as fit, walkers in blocks when 32 positions of all of them do not
+        const int64_t fit = (int64_t)(kBatchBytes / (size_t)qcs_pf_rec_bytes(n, ne));
+        if (wk->wblock > fit / 32) wk->wblock = fit / 32;
+        const int64_t all = (s->P + 31) / 32 * 32;
+        int64_t sp = fit / wk->wblock / 32 * 32;
+        if (sp > all) sp = all > 0 ? all : 32;
+        span = (int)sp;
+    }
+    wk->span = span;
     wk->nchunks = (int)((s->P + span - 1) / span);
     if (wk->nchunks < 1) wk->nchunks = 1;
     wk->nparts = (split || tc) ? wk->nchunks : wk->nchunks * qcs_pair_warps_per_block();
@@ -486,11 +502,17 @@ qcs_status overlap_common(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t 
     size_t b_slab = split ? align16(qcs_split_walker_bytes(n, W)) : 0;
     size_t b_rec = tc ? align16(qcs_tc_walker_bytes(W)) : 0;
     size_t b_mode = (split || tc) ? 0 : align16(sizeof(int) * (size_t)(W > 0 ? W : 1));
+    const size_t batch = tc ? (size_t)wk->wblock * wk->span : 0;
+    size_t b_pair = tc ? align16(batch * qcs_pf_rec_bytes(n, ne)) : 0, b_sum = align16(batch * sizeof(cd));
+    size_t b_cnt = tc ? align16(sizeof(unsigned long long) * (size_t)qcs_tc_counters(W > 0 ? W : 1, wk->wblock, wk->nchunks)) : 0;
+    const size_t b_all = 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec + b_mode;
     void *base = nullptr;
-    qcs_status ws = qcs_workspace(ctx, 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec + b_mode, &base, st);
+    qcs_status ws = qcs_workspace(ctx, b_all + b_cnt + b_sum + b_pair, &base, st);
     if (ws != QCS_OK) return ws;
     char *pb = (char *)base;
-    wk->counter = (unsigned long long *)pb;
+    wk->counter = (unsigned long long *)(tc ? pb + b_all : pb);
+    wk->sum = (cd *)(pb + b_all + b_cnt);
+    wk->rec = (unsigned char *)(pb + b_all + b_cnt + b_sum);
     wk->Ut = (cd *)(pb + 16);
     wk->pref = (cd *)(pb + 16 + b_ut);
     wk->partial = (cd *)(pb + 16 + b_ut + b_pref);
@@ -538,6 +560,10 @@ extern "C" qcs_status qcs_overlap(qcs_ctx *ctx, const qcs_snapshots *s, int ne, 
     L.plan = plan;
     L.counter = wk.counter;
     L.config = wk.config;
+    L.rec = wk.rec;
+    L.sum = wk.sum;
+    L.wblock = wk.wblock;
+    L.span = wk.span;
     if (wk.split) {
         r = qcs_split_prepare_snapshots(ctx, const_cast<qcs_snapshots *>(s), st);
         if (r != QCS_OK) return r;

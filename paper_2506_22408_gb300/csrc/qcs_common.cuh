@@ -128,8 +128,9 @@ __device__ __forceinline__ cd warp_csum(cd v) {
 }
 
 // Packed strict upper triangle: entry (i, j), i < j, at j(j-1)/2 + i.
-__host__ __device__ __forceinline__ int tri_index(int i, int j) { return (j * (j - 1)) / 2 + i; }
-__host__ __device__ __forceinline__ int tri_count(int m) { return (m * (m - 1)) / 2; }
+// (m (m - 1) is never negative: an unsigned shift spares the rounding of a signed division.)
+__host__ __device__ __forceinline__ int tri_count(int m) { return (int)((unsigned)(m * (m - 1)) >> 1); }
+__host__ __device__ __forceinline__ int tri_index(int i, int j) { return tri_count(j) + i; }
 
 __device__ __forceinline__ void raise_status(unsigned *status, unsigned bits) {
     if (status) atomicOr(status, bits);

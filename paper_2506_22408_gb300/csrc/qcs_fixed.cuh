@@ -20,6 +20,9 @@
 // prefix of the packed triangle, updated in place without index lists; pivots are compared
 // on upper words; products of pivots are taken in normalised fixed point as well.
 #pragma once
+#include <cmath>
+
+#include "qcs_internal.h"
 #include "qcs_ozaki.cuh"
 #include "qcs_pair.cuh"
 
@@ -60,22 +63,61 @@ struct FxTeam {
 };
 typedef FxTeam<1> FxWarp;
 
+// A node plan in fixed point: w_k (modulus one) worth X 2^-58, gamma_k worth X 2^ge.
+struct FxPlan {
+    int nev;
+    fx2 w[QCS_MAX_NODES];
+    fx2 g[QCS_MAX_NODES];
+    int ge[QCS_MAX_NODES];
+};
+
+inline void fx_make_plan(const qcs_node_plan &p, FxPlan &q) {
+    q.nev = p.nev;
+    for (int k = 0; k < p.nev; ++k) {
+        q.w[k] = make_longlong2(std::llround(std::ldexp(p.wnode[k].x, 58)), std::llround(std::ldexp(p.wnode[k].y, 58)));
+        int e = 0;
+        std::frexp(std::fmax(std::fabs(p.gamma[k].x), std::fabs(p.gamma[k].y)), &e);
+        q.g[k] = make_longlong2(std::llround(std::ldexp(p.gamma[k].x, 60 - e)),
+                                std::llround(std::ldexp(p.gamma[k].y, 60 - e)));
+        q.ge[k] = e - 60;
+    }
+}
+
 struct fxl {  // a fixed-point number as limbs h 2^31 + l
     int h, l;
 };
 __device__ __forceinline__ fxl fx_split(long long X) {
-    const int h = (int)((X + (1ll << 30)) >> 31);
-    return fxl{h, (int)((unsigned)X - ((unsigned)h << 31))};
+    const unsigned long long y = (unsigned long long)X + (1ull << 30);
+    return fxl{(int)__funnelshift_l((unsigned)y, (unsigned)(y >> 32), 1), (int)((unsigned)X << 1) >> 1};
 }
 __device__ __forceinline__ fxl fx_neg(fxl a) { return fxl{-a.h, -a.l}; }
+
+// a b and s + a b in 64 bits, one instruction each: written out because the compiler, when
+// it sees a limb's sign extension, multiplies 64-bit numbers with three.
+__device__ __forceinline__ long long mul_wide(int a, int b) {
+    long long r;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ long long mad_wide(int a, int b, long long s) {
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(s));
+    return r;
+}
 
 struct fxacc {  // hh 2^62 + cr 2^31
     long long hh, cr;
 };
+// The sum starts at half a unit of its fx_value: a mean over many pairs must not collect the
+// half unit that a plain shift loses each time.
+__device__ __forceinline__ fxacc fx_mul(fxl a, fxl b, long long half) {
+    return fxacc{mul_wide(a.h, b.h), mad_wide(a.l, b.h, mad_wide(a.h, b.l, half))};
+}
+__device__ __forceinline__ long long fx_half(int up) { return 1ll << (30 - up); }
 __device__ __forceinline__ void fx_mac(fxacc &s, fxl a, fxl b) {
-    s.hh += (long long)a.h * b.h;
-    s.cr += (long long)a.h * b.l;
-    s.cr += (long long)a.l * b.h;
+    s.hh = mad_wide(a.h, b.h, s.hh);
+    s.cr = mad_wide(a.h, b.l, s.cr);
+    s.cr = mad_wide(a.l, b.h, s.cr);
 }
 // (hh 2^62 + cr 2^31) 2^{-62 + up}, 0 <= up < 31
 __device__ __forceinline__ long long fx_value(const fxacc &s, int up) { return (s.hh << up) + (s.cr >> (31 - up)); }
@@ -136,78 +178,57 @@ __device__ __forceinline__ long long fx_of1(double x, int f) {
 __device__ __forceinline__ fx2 fx_of(cd x, int f) { return make_longlong2(fx_of1(x.x, f), fx_of1(x.y, f)); }
 
 // X 2^E as an FP64.
-__device__ __forceinline__ double fx_f64(long long X, int E) {
+static __device__ __noinline__ double fx_f64(long long X, int E) {
     bool ok = true;
     const double v = qcs_oz::fixed_to_f64(X, E, ok);
     return ok ? v : qcs_oz::fixed_to_f64_exact(X, E);
 }
 
-// Entry (i, j), i != j, of a packed skew-symmetric matrix.
-__device__ __forceinline__ fx2 fx_skew(const fx2 *__restrict__ N, int i, int j) {
-    const bool lo = i > j;
-    const fx2 v = N[lo ? tri_index(j, i) : tri_index(i, j)];
-    const long long m = lo ? -1ll : 0ll;
-    return make_longlong2((v.x ^ m) - m, (v.y ^ m) - m);
-}
-
-// A(i, j) = x, A(j, i) = -x.
-__device__ __forceinline__ void fx_put(fx2 *__restrict__ N, int i, int j, fx2 x) {
-    const long long m = i > j ? -1ll : 0ll;
-    N[i > j ? tri_index(j, i) : tri_index(i, j)] = make_longlong2((x.x ^ m) - m, (x.y ^ m) - m);
-}
-
-// 1 / (q.x + i q.y) 2^119 as limbs, for max(|q.x|, |q.y|) in [2^60, 2^61): conj(q) / |q|^2,
+// 1 / (q.x + i q.y) 2^119 as packed limbs, for max(|q.x|, |q.y|) in [2^60, 2^61): conj(q) / |q|^2,
 // the reciprocal R = 2^118 / (|q|^2 2^-62) by one third-order step from the FP32 seed R0
 // (relative error e < 2^-22: R = R0 (1 + e + e^2), e^3 < 2^-66) in integers.
-__device__ __forceinline__ void fx_inverse(fx2 q, fxl &ir, fxl &ii) {
+__device__ __forceinline__ int4 fx_inverse(fx2 q) {
     const fxl a = fx_split(q.x), b = fx_split(q.y);
-    fxacc s = {0, 0};
-    fx_mac(s, a, a);
+    fxacc s = fx_mul(a, a, 0);
     fx_mac(s, b, b);
     const long long D = s.hh + (s.cr >> 31);  // |q|^2 2^-62 in [2^58, 2^61]
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(int)(D >> 31)));
     const int R0 = (int)(y * 18014398509481984.0f);  // 2^54 y in [2^24, 2^27]
-    const long long e = -(long long)((unsigned long long)D * (unsigned long long)(long long)R0);  // 2^85 (1 - D R0 2^-85)
+    const long long e = -(long long)((unsigned long long)(unsigned)D * (unsigned)R0 +
+                                    ((unsigned long long)((unsigned)(D >> 32) * (unsigned)R0) << 32));  // 2^85 (1 - D R0 2^-85)
     const int eh = (int)(e >> 32);
     const int e2 = __mulhi(eh, eh);
-    const long long R = ((long long)R0 << 33) + (((long long)R0 * eh) >> 20) +
-                        (long long)(((unsigned long long)(unsigned)R0 * (unsigned)e) >> 52) + (((long long)R0 * e2) >> 41);
+    const long long R = ((long long)R0 << 33) + (mul_wide(R0, eh) >> 20) +
+                        (long long)(__umulhi((unsigned)R0, (unsigned)e) >> 20) + (mul_wide(R0, e2) >> 41);
     const fxl r = fx_split(R);
-    fxacc u = {0, 0}, v = {0, 0};
-    fx_mac(u, a, r);
-    fx_mac(v, b, r);
-    ir = fx_split(fx_value(u, 1));
-    ii = fx_neg(fx_split(fx_value(v, 1)));
+    const fxacc u = fx_mul(a, r, fx_half(1)), v = fx_mul(b, r, fx_half(1));
+    return fx_pack(fx_split(fx_value(u, 1)), fx_neg(fx_split(fx_value(v, 1))));
 }
 
 // z I 2^-60 for I = 2^119 / q as limbs: 2^59 z / q, as packed limbs.
 __device__ __forceinline__ int4 fx_times_inverse(fx2 z, fxl ir, fxl ii) {
     const fxl a = fx_split(z.x), b = fx_split(z.y);
-    fxacc re = {0, 0}, im = {0, 0};
-    fx_mac(re, a, ir);
-    fx_mac(re, b, fx_neg(ii));
-    fx_mac(im, a, ii);
+    fxacc re = fx_mul(a, ir, fx_half(2)), im = fx_mul(a, ii, fx_half(2));
+    fx_mac(re, fx_neg(b), ii);
     fx_mac(im, b, ir);
     return fx_pack(fx_split(fx_value(re, 2)), fx_split(fx_value(im, 2)));
 }
 
-// A complex number (x + i y) 2^e, the larger part of 60 bits unless it is zero.
+// A complex number (x + i y) 2^e, the larger part of 60 bits (61 at most) unless it is zero.
 struct fxp {
     long long x, y;
     int e;
 };
 __device__ __forceinline__ fxp fx_norm(fx2 a, int e) {
-    const int sh = 60 - fx_bits(a);
-    const fx2 z = fx_shift(a, sh < 60 ? sh : 0);
-    return fxp{z.x, z.y, e - sh};
+    const unsigned t = fx_mag32(a);
+    const int sh = (t ? __clz((int)t) : 64 - fx_bits(a) > 63 ? 4 : 64 - fx_bits(a)) - 4;
+    return sh >= 0 ? fxp{a.x << sh, a.y << sh, e - sh} : fxp{a.x >> -sh, a.y >> -sh, e - sh};
 }
-__device__ __forceinline__ fxp fx_prod(const fxp &a, const fxp &b) {
+__device__ __forceinline__ fxp fx_prod(fxp a, fxp b) {
     const fxl ar = fx_split(a.x), ai = fx_split(a.y), br = fx_split(b.x), bi = fx_split(b.y);
-    fxacc re = {0, 0}, im = {0, 0};
-    fx_mac(re, ar, br);
+    fxacc re = fx_mul(ar, br, fx_half(0)), im = fx_mul(ar, bi, fx_half(0));
     fx_mac(re, fx_neg(ai), bi);
-    fx_mac(im, ar, bi);
     fx_mac(im, ai, br);
     return fx_norm(make_longlong2(fx_value(re, 0), fx_value(im, 0)), a.e + b.e + 62);
 }
@@ -215,37 +236,45 @@ __device__ __forceinline__ fxp fx_shfl_xor(const fxp &a, int o) {
     return fxp{__shfl_xor_sync(QCS_FULL, a.x, o), __shfl_xor_sync(QCS_FULL, a.y, o), __shfl_xor_sync(QCS_FULL, a.e, o)};
 }
 
+// The Gauss vectors' entries of one index as limbs, g before v.
+struct FxGauss {
+    int4 g, v;
+};
+
 // Rank-2 update, in place, of the leading rv x rv blocks of nb packed matrices (stride T):
 //     A_ij = (A_ij + g_i v_j - v_i g_j) 2^-q,   g scaled by 2^{59-eu}.
 // Entry t of the packed triangle is read and written by one thread; (i, j) comes from the
 // pair table.  Returns this thread's OR of the new entries' upper words.
-template <class Team>
-__device__ __forceinline__ unsigned fx_rank2(const Team &tm, int nb, int T, int rv, fx2 *__restrict__ Ns,
-                                             const int4 *__restrict__ Gv, const int4 *__restrict__ Vv, int ldv, int eu,
-                                             int q, const uint16_t *__restrict__ tab) {
+template <int NT>
+__device__ __forceinline__ unsigned fx_rank2(int t0, int nb, int T, int rv, fx2 *__restrict__ Ns,
+                                             const FxGauss *__restrict__ GV, int ldv, int eu, int q,
+                                             const uint16_t *__restrict__ tab) {
     const int Tr = tri_count(rv), total = nb * Tr;
     const int up = 3 + eu - q;
+    const long long half = fx_half(up), qhalf = (1ll << q) >> 1;
     unsigned top = 0u;
-    int u = tm.t;
-    const int4 *G = Gv, *V = Vv;
-    fx2 *N = Ns;
-    for (int e = tm.t; e < total; e += Team::NT) {
-        while (u >= Tr) {
+    int u = t0;
+#pragma unroll 1
+    for (int e = t0; e < total; e += NT) {
+        if (u >= Tr) {  // the next matrix; several for the smallest blocks
             u -= Tr;
-            N += T;
-            G += ldv;
-            V += ldv;
+            Ns += T;
+            GV += ldv;
+            if (Tr < NT)
+                while (u >= Tr) {
+                    u -= Tr;
+                    Ns += T;
+                    GV += ldv;
+                }
         }
         int ia, ib;
         pair_of(tab, u, ia, ib);
-        fx2 x = N[u];
-        const int4 gi = G[ia], vi = V[ia], gj = G[ib], vj = V[ib];
+        fx2 x = Ns[u];
+        const int4 gi = GV[ia].g, vi = GV[ia].v, gj = GV[ib].g, vj = GV[ib].v;
         const fxl gir = {gi.x, gi.y}, gii = {gi.z, gi.w}, gjr = {gj.x, gj.y}, gji = {gj.z, gj.w};
         const fxl vir = {vi.x, vi.y}, vii = {vi.z, vi.w}, vjr = {vj.x, vj.y}, vji = {vj.z, vj.w};
         const fxl mgii = fx_neg(gii), mvir = fx_neg(vir), mvii = fx_neg(vii);
-        fxacc re = {0, 0}, im = {0, 0};
-        fx_mac(re, gir, vjr);
-        fx_mac(im, gir, vji);
+        fxacc re = fx_mul(gir, vjr, half), im = fx_mul(gir, vji, half);
         fx_mac(re, mgii, vji);
         fx_mac(im, gii, vjr);
         fx_mac(re, mvir, gjr);
@@ -253,21 +282,21 @@ __device__ __forceinline__ unsigned fx_rank2(const Team &tm, int nb, int T, int 
         fx_mac(re, vii, gji);
         fx_mac(im, mvii, gjr);
         if (q > 0) {
-            x.x >>= q;
-            x.y >>= q;
+            x.x = (x.x + qhalf) >> q;
+            x.y = (x.y + qhalf) >> q;
         }
         x.x += fx_value(re, up);
         x.y += fx_value(im, up);
         top |= fx_top(x);
-        N[u] = x;
-        u += Team::NT;
+        Ns[u] = x;
+        u += NT;
     }
     return top;
 }
 
 // Multiply the entries of nb packed matrices (tri(r) entries each, stride T) by 2^sh.
 template <class Team>
-__device__ __noinline__ void fx_renorm(const Team &tm, int nb, int T, int r, fx2 *Ns, int sh) {
+static __device__ __noinline__ void fx_renorm(const Team &tm, int nb, int T, int r, fx2 *Ns, int sh) {
     const int Tr = tri_count(r);
     tm.sync();
     for (int w = 0; w < nb; ++w)
@@ -286,10 +315,10 @@ __host__ __device__ inline size_t pv_bytes(int vm, int NB, int ne) {
 
 // Workspace of one pair in the team's shared memory, besides its matrices.
 struct FxWork {
-    int4 *Gv, *Vv;  // Gauss vectors as limbs: max(m, NB 2d) entries each
-    fx2 *pv;        // records
-    int *pe;        // ... and their fraction bits
-    int npv;        // index of the first occupied pivot's record
+    FxGauss *GV;  // Gauss vectors: max(m, NB 2d) entries
+    fx2 *pv;      // records
+    int *pe;      // ... and their fraction bits
+    int npv;      // index of the first occupied pivot's record
 };
 
 // Position of selected row x (occupied rows 0 .. ne-1, then the empty modes' rows) in the
@@ -305,6 +334,7 @@ __device__ inline bool fx_load(const Team &tm, int m, int ne, const cd *__restri
                                const uint16_t *__restrict__ tab) {
     const int T = tri_count(m);
     unsigned kb = 0u;
+#pragma unroll 2
     for (int e = tm.lane; e < T; e += 32) {  // every warp of the team takes the maximum itself
         const unsigned k = pivot_key(Bs[e]);
         kb = k > kb ? k : kb;
@@ -313,6 +343,7 @@ __device__ inline bool fx_load(const Team &tm, int m, int ne, const cd *__restri
     const int hx = (int)(kb >> 20);  // |x| < 2^{hx - 1022}
     f = kFxTop + 1022 - hx;
     if (hx == 0x7ff) return false;
+#pragma unroll 1
     for (int e = tm.t; e < T; e += Team::NT) {
         int a, b;
         pair_of(tab, e, a, b);
@@ -324,324 +355,338 @@ __device__ inline bool fx_load(const Team &tm, int m, int ne, const cd *__restri
     return true;
 }
 
-// Elimination of the occupied block, shared by every node matrix.  The node matrices
-// B + w D differ only in their empty x empty block (D pairs the empty modes), so
-// eliminating the ne occupied indices first is the same for all of them:
-// pf(B + w D) = pf0 pf(S + w D_ee), S the Schur complement of the occupied block.
-// In place on X (tri(m) entries, worth X 2^-f, the largest of at most mb bits).  Each step
-// takes the largest entry (p, k) of the active occupied block as pivot, moves k to the
-// last and p to the last but one position (a swap flips the sign) and updates the leading
-// block; the ne/2 signed pivots become the records pvo (their product pf0 enters each
-// node's product).  On success the leading tri(2d) entries of X hold S and f and mb are
-// S's.  Returns false when a pivot is zero, an element of a Gauss vector exceeds 2^20 or
-// the largest entry of S exceeds 2^8 times the largest entry of B (the caller then
-// eliminates each node matrix in full).
-template <class Team>
-__device__ inline bool fx_schur_occupied(const Team &tm, int m, int ne, fx2 *__restrict__ X, int4 *__restrict__ Gv,
-                                         int4 *__restrict__ Vv, const uint16_t *__restrict__ tab,
-                                         fx2 *__restrict__ pvo, int *__restrict__ peo, int &f, int &mb) {
-    const int d2 = m - ne;
-    const int bound = mb - f + 8;
-    for (int s = 0, r = m; r > d2; ++s, r -= 2) {
-        const int ro = r - d2;  // the active occupied indices are 2d .. r - 1
-        if (mb > kFxMax || mb < kFxLow) {
-            fx_renorm(tm, 1, 0, r, X, kFxTop - mb);
-            f += kFxTop - mb;
-            mb = kFxTop;
-        }
-        // the largest entry of the active occupied block (every warp finds it by itself)
-        unsigned bk = 0u;
-        for (int t = tm.lane; t < tri_count(ro); t += 32) {
-            int a, b;
-            pair_of(tab, t, a, b);
-            const unsigned c = ((fx_mag32(X[tri_index(d2 + a, d2 + b)]) >> 6) << 9) | (unsigned)(511 - t);
-            bk = c > bk ? c : bk;
-        }
-        bk = __reduce_max_sync(QCS_FULL, bk);
-        int bt = 511 - (int)(bk & 511u);
-        if ((bk >> 9) < 64u) {  // small against the matrix: compare by the whole words
-            unsigned kk = 0u, kt = 0u;
-            for (int t = tm.lane; t < tri_count(ro); t += 32) {
-                int a, b;
-                pair_of(tab, t, a, b);
-                const unsigned key = fx_key(X[tri_index(d2 + a, d2 + b)]);
-                if (key > kk) {
-                    kk = key;
-                    kt = (unsigned)t;
-                }
-            }
-            const unsigned top = __reduce_max_sync(QCS_FULL, kk);
-            if (top == 0u) return false;  // the active occupied block is zero
-            bt = (int)__reduce_min_sync(QCS_FULL, kk == top ? kt : 0xffffffffu);
-        }
-        int P, K;
-        pair_of(tab, bt, P, K);
-        P += d2;
-        K += d2;
-        // row K can hold larger entries than the pivot among the empty indices
-        unsigned rt = 0u;
-        for (int a = tm.lane; a < r; a += 32)
-            if (a != K) rt |= fx_top(X[a < K ? tri_index(a, K) : tri_index(K, a)]);
-        rt = __reduce_or_sync(QCS_FULL, rt);
-        const fx2 piv = X[tri_index(P, K)];
-        const int pb = fx_bits(piv), rb = fx_top_bits(rt);
-        const int eu = rb >= pb ? rb - pb + 1 : 0;  // |g| 2^-eu < sqrt 2
-        if (eu > 20) return false;
-        if (tm.t == 0) {
-            const bool neg = (K != r - 1) != (P != r - 2);
-            pvo[s] = neg ? make_longlong2(-piv.x, -piv.y) : piv;
-            peo[s] = f;
-        }
-        if (r == 2) break;  // no empty modes: the last pivot closes the Pfaffian
-        const int sn = 61 - pb;
-        fxl ir, ii;
-        fx_inverse(make_longlong2(piv.x << sn, piv.y << sn), ir, ii);
-        const int sP = K == r - 2 ? r - 1 : r - 2;  // what takes place P (if P stays), and r - 1 takes K
-        tm.sync();  // every warp has read the pivot and row K
-        const int rv = r - 2;
-        for (int i = tm.t; i < rv; i += Team::NT) {
-            const int o = i == K ? r - 1 : i == P ? sP : i;
-            // g = A_{i,k} / A_{p,k}, v = A_{i,p}
-            Gv[i] = fx_times_inverse(fx_shift(fx_skew(X, o, K), sn - eu), ir, ii);
-            const fx2 v = fx_skew(X, o, P);
-            Vv[i] = fx_pack(fx_split(v.x), fx_split(v.y));
-            if (i != P && i != K) {
-                if (K < rv) fx_put(X, i, K, fx_skew(X, i, r - 1));
-                if (P < rv) fx_put(X, i, P, fx_skew(X, i, sP));
-            } else if (i == K && P < rv) {
-                fx_put(X, P, K, fx_skew(X, sP, r - 1));
-            }
-        }
-        tm.sync();
-        const int q = mb + eu > kFxRoom ? mb + eu - kFxRoom : 0;
-        unsigned o = fx_rank2(tm, 1, 0, rv, X, Gv, Vv, 0, eu, q, tab);
-        o = tm.or_put(o, s & 1);
-        tm.sync();
-        mb = fx_top_bits(tm.or_get(o, s & 1));
-        f -= q;
-    }
-    return d2 == 0 || mb - f <= bound;
+// x or -x.
+__device__ __forceinline__ fx2 fx_neg_if(fx2 x, bool neg) {
+    const long long m = neg ? -1ll : 0ll;
+    return make_longlong2((x.x ^ m) - m, (x.y ^ m) - m);
 }
 
-// Pfaffians of nb node matrices S + wnode[v] D (S packed, m x m, empty modes first, worth
-// X 2^-fS, its largest entry of at most mbS bits; D pairs the d leading index pairs), each
-// times its node weight and the npo records pvo (the signed pivots of a shared occupied
-// elimination, or none); pf[v] of lane seg v is returned on the first lane of the node's
-// segment.  Each warp of the team is cut into segments of seg lanes, one per node matrix it
-// owns (node v belongs to warp v mod the team's warps); a segment finds the pivot of its
-// node's last active row (|g_i| <= sqrt 2 then), inverts it on every lane, moves its index
-// to the last but one position and forms the Gauss vectors; the rank-2 updates of all
-// nodes are spread over the whole team.  The steps run down to four active indices, whose
-// Pfaffian closes the product in three terms, a01 a23 - a02 a13 + a03 a12 (two: a01).
-// Returns sum_v gamma[v] prod(pvo) pf(S + wnode[v] D) on thread 0 of the team (NW = 1) or on
-// the first lane of each warp its own nodes' sum (NW = 2).
+// Swap of index K with the last of r active ones (K < r - 1) in a packed skew-symmetric
+// matrix: the rows' entries change places (each pair by one thread), and the entry between
+// the two changes its sign.
 template <class Team>
-__device__ inline cd fx_node_pfaffians(const Team &tm, int m, int d, const cd *__restrict__ wnode,
-                                       const cd *__restrict__ gamma, int nb, const fx2 *__restrict__ Sx, int fS,
-                                       int mbS, fx2 *__restrict__ Ns, int4 *__restrict__ Gv, int4 *__restrict__ Vv,
-                                       const uint16_t *__restrict__ tab, fx2 *__restrict__ pv, int *__restrict__ pe,
-                                       int npo, const fx2 *__restrict__ pvo, const int *__restrict__ peo) {
-    const int npw = (nb + Team::kWarps - 1) / Team::kWarps;  // nodes per warp
-    const int seg = npw <= 1 ? 32 : npw <= 2 ? 16 : npw <= 4 ? 8 : 4;
-    const int slot = tm.lane / seg, sl = tm.lane - slot * seg;
-    const int v = slot * Team::kWarps + tm.wid;
-    const bool live = slot < npw && v < nb;
-    const int vr = live ? v : 0;  // lanes past the last node read node 0 and write nothing
-    const int S0 = m == 0 ? 0 : (m >= 4 ? m / 2 - 1 : 1);  // pivots and the closing Pfaffian
-    if (m > 0) {
-        const int T = tri_count(m);
-        // scale: room for S and for wnode (of modulus one)
-        int f = fS;
-        if (f > kFxTop || mbS > kFxTop + 1 || mbS < kFxLow) {
-            f = fS + kFxTop - mbS;
-            f = f < kFxTop ? f : kFxTop;
-        }
-        if (f == fS) {
-            for (int u = tm.t; u < T; u += Team::NT) {
-                const fx2 x = Sx[u];
-                for (int w = 0; w < nb; ++w) Ns[w * T + u] = x;
-            }
+__device__ __forceinline__ void fx_swap_last(const Team &tm, fx2 *__restrict__ N, int r, int K) {
+    const int last = tri_count(r - 1), tk = tri_count(K);
+#pragma unroll 1
+    for (int i = tm.t; i < r - 1; i += Team::NT) {
+        const bool lo = i > K;
+        fx2 *a = N + (lo ? tri_count(i) + K : tk + i), *b = N + last + i;
+        if (i != K) {
+            const fx2 x = *a, y = *b;
+            *a = fx_neg_if(y, lo);
+            *b = fx_neg_if(x, lo);
         } else {
+            *b = fx_neg_if(*b, true);
+        }
+    }
+}
+
+// sum_k gamma_k pf(B + w_k D) of one pair, k over the plan's nodes; the sum's parts are on
+// the first lanes of the team's warps (each its own nodes).
+//
+// The node matrices B + w D differ only in their empty x empty block (D pairs the empty
+// modes), so eliminating the ne occupied indices first is the same for all of them:
+// pf(B + w D) = pf0 pf(S + w D_ee), S the Schur complement of the occupied block.  With
+// shared set, job -1 eliminates it in place on X (tri(m) entries worth X 2^-f, the largest of
+// at most mb bits, the empty modes first): each step takes the largest entry of the active
+// occupied block as pivot (p, k), moves k to the last and p to the last but one position (a
+// swap flips the sign) and updates the leading block; S ends as the leading tri(2d)
+// entries.  The job fails (ok = false, X overwritten; the caller repeats with a fresh X and
+// shared = false) when a pivot is zero, an element of a Gauss vector exceeds 2^20 or
+// the largest entry of S exceeds 2^8 times that of B.
+//
+// The other jobs are rounds of up to NB node matrices S + w D (one full matrix B + w D per
+// round without shared) in Ns.  Each warp of the team is cut into segments of seg lanes,
+// one per node matrix it owns (node v belongs to warp v mod the team's warps); a segment
+// finds the pivot of its node's last active row (so |g_i| <= sqrt 2), inverts it on every
+// lane, moves its index to the last but one position and forms the Gauss vectors; the
+// rank-2 updates of all nodes are spread over the whole team.  The steps run down to four
+// active indices, whose Pfaffian closes the product in three terms,
+// a01 a23 - a02 a13 + a03 a12 (two indices: a01).  Signed pivots, the closing Pfaffian, the
+// occupied pivots and gamma are records multiplied by a shuffle tree over the segment.
+//
+// Both kinds of job run the same step code: one copy keeps the loop in the instruction
+// caches (two inlined copies cost the 20-warp kernel 20 % of its issue slots in
+// instruction misses).
+template <class Team>
+__device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool shared, int NB, const FxPlan &plan,
+                                       const FxWork &wk, fx2 *X, fx2 *Ns, int f, int mb,
+                                       const uint16_t *__restrict__ tab, bool &ok) {
+    const int d2 = m - ne, nev = plan.nev;
+    const int bound = mb - f + 8;
+    const int mm = shared ? d2 : m, npo = shared ? ne / 2 : 0, NBr = shared ? NB : 1;
+    fx2 *pvo = wk.pv + wk.npv;
+    int *peo = wk.pe + wk.npv;
+    cd total = cmk(0.0, 0.0);
+    ok = true;
+#pragma unroll 1
+    for (int k0 = shared ? -1 : 0; k0 < nev; k0 = k0 < 0 ? 0 : k0 + NBr) {
+        const bool occ = k0 < 0;
+        const int nb = occ ? 1 : nev - k0 < NBr ? nev - k0 : NBr;
+        const int npw = (nb + Team::kWarps - 1) / Team::kWarps;  // nodes per warp
+        const int seg = npw <= 1 ? 32 : npw <= 2 ? 16 : npw <= 4 ? 8 : 4;
+        const int slot = tm.lane / seg, sl = tm.lane - slot * seg;
+        const int v = occ ? 0 : slot * Team::kWarps + tm.wid;
+        const bool live = occ || (slot < npw && v < nb);
+        const int vr = live ? v : 0;  // lanes past the last node read node 0 and write nothing
+        const int mc = occ ? m : mm, T = occ ? 0 : tri_count(mc), stop = occ ? d2 : 4;
+        const int S0 = mm == 0 ? 0 : (mm >= 4 ? mm / 2 - 1 : 1);  // a node's pivots and closing Pfaffian
+        fx2 *N0 = occ ? X : Ns;  // the job's matrices, stride T
+        int fc = f, mbc = mb;
+        if (!occ && mm > 0) {
+            // scale: room for S and for w_k (of modulus one)
+            if (f > kFxTop || mb > kFxTop + 1 || mb < kFxLow) {
+                fc = f + kFxTop - mb;
+                fc = fc < kFxTop ? fc : kFxTop;
+            }
+            mbc = kFxTop + 2;
+#pragma unroll 2
             for (int u = tm.t; u < T; u += Team::NT) {
-                const fx2 x = fx_shift(Sx[u], f - fS);
+                fx2 x = X[u];
+                if (fc != f) x = fx_shift(x, fc - f);
                 for (int w = 0; w < nb; ++w) Ns[w * T + u] = x;
             }
+            tm.sync();
+            const int d = d2 / 2;
+#pragma unroll 1
+            for (int e = tm.t; e < nb * d; e += Team::NT) {
+                const int w = e / d, i = e - w * d;
+                fx2 *x = Ns + w * T + tri_index(2 * i, 2 * i + 1);
+                const fx2 z = fx_shift(plan.w[k0 + w], fc - kFxTop);
+                *x = make_longlong2(x->x + z.x, x->y + z.y);
+            }
+            tm.sync();
         }
-        tm.sync();
-        for (int e = tm.t; e < nb * d; e += Team::NT) {
-            const int w = e / d, i = e - w * d;
-            fx2 *x = Ns + w * T + tri_index(2 * i, 2 * i + 1);
-            const fx2 z = fx_of(wnode[w], f);
-            *x = make_longlong2(x->x + z.x, x->y + z.y);
-        }
-        tm.sync();
-        fx2 *__restrict__ Nv = Ns + vr * T;
-        int mb = kFxTop + 2;
+        fx2 *Nv = N0 + vr * T;
         int s = 0;
-        for (int r = m; r > 4; r -= 2, ++s) {
-            if (mb > kFxMax || mb < kFxLow) {
-                fx_renorm(tm, nb, T, r, Ns, kFxTop - mb);
-                f += kFxTop - mb;
-                mb = kFxTop;
+#pragma unroll 1
+        for (int r = mc; r > stop; r -= 2, ++s) {
+            if (mbc > kFxMax || mbc < kFxLow) {
+                fx_renorm(tm, nb, T, r, N0, kFxTop - mbc);
+                fc += kFxTop - mbc;
+                mbc = kFxTop;
             }
-            // pivot: largest |A_{a,r-1}| of the last row (contiguous entries), each lane
-            // scanning every seg-th candidate, then a shuffle reduction in the segment; the
-            // key's low bits prefer the first candidate among equal magnitudes
             const fx2 *row = Nv + tri_count(r - 1);
-            unsigned bk = 0u;
-            for (int a = sl; a < r - 1; a += seg) {
-                const unsigned c = ((fx_mag32(row[a]) >> 3) << 6) | (unsigned)(63 - a);
-                bk = c > bk ? c : bk;
-            }
-            for (int o = seg >> 1; o > 0; o >>= 1) {
-                const unsigned ob = __shfl_xor_sync(QCS_FULL, bk, o);
-                bk = ob > bk ? ob : bk;
-            }
-            bool zero = false;
-            if (__any_sync(QCS_FULL, (bk >> 6) < 64u)) {  // small against the matrix: by the whole words
-                bk = 0u;
+            int P, eu = 0;
+            bool neg, zero = false;
+            if (occ) {
+                // the largest entry of the active occupied block (every warp finds it by itself)
+                const int ro = r - d2;  // its indices are 2d .. r - 1
+                unsigned bk = 0u;
+#pragma unroll 1
+                for (int t = tm.lane; t < tri_count(ro); t += 32) {
+                    int a, b;
+                    pair_of(tab, t, a, b);
+                    const unsigned c =
+                        ((fx_mag32(X[tri_index(d2 + a, d2 + b)]) >> 6) << 9) | (unsigned)(511 - t);
+                    bk = c > bk ? c : bk;
+                }
+                bk = __reduce_max_sync(QCS_FULL, bk);
+                int bt = 511 - (int)(bk & 511u);
+                if ((bk >> 9) < 64u) {  // small against the matrix: compare by the whole words
+                    unsigned kk = 0u, kt = 0u;
+#pragma unroll 1
+                    for (int t = tm.lane; t < tri_count(ro); t += 32) {
+                        int a, b;
+                        pair_of(tab, t, a, b);
+                        const unsigned key = fx_key(X[tri_index(d2 + a, d2 + b)]);
+                        if (key > kk) {
+                            kk = key;
+                            kt = (unsigned)t;
+                        }
+                    }
+                    const unsigned top = __reduce_max_sync(QCS_FULL, kk);
+                    if (top == 0u) {  // the active occupied block is zero
+                        ok = false;
+                        return total;
+                    }
+                    bt = (int)__reduce_min_sync(QCS_FULL, kk == top ? kt : 0xffffffffu);
+                }
+                int K;
+                pair_of(tab, bt, P, K);
+                P += d2;
+                K += d2;
+                neg = false;
+                if (K != r - 1) {
+                    tm.sync();  // every warp has scanned the block
+                    fx_swap_last(tm, X, r, K);
+                    neg = true;
+                    tm.sync();
+                }
+                // row k can hold larger entries than the pivot among the empty indices
+                unsigned rt = 0u;
+#pragma unroll 1
+                for (int a = tm.lane; a < r - 1; a += 32) rt |= fx_top(row[a]);
+                const int rb = fx_top_bits(__reduce_or_sync(QCS_FULL, rt)), pb = fx_bits(row[P]);
+                if (rb >= pb) eu = rb - pb + 1;  // |g| 2^-eu < sqrt 2
+                if (eu > 20) {
+                    ok = false;
+                    return total;
+                }
+            } else {
+                // the largest of the last row, each lane scanning every seg-th candidate, then a
+                // shuffle reduction in the segment; the key's low bits prefer the first
+                // candidate among equal magnitudes
+                unsigned bk = 0u;
+#pragma unroll 1
                 for (int a = sl; a < r - 1; a += seg) {
-                    const unsigned c = (fx_key(row[a]) << 6) | (unsigned)(63 - a);
+                    const unsigned c = ((fx_mag32(row[a]) >> 3) << 6) | (unsigned)(63 - a);
                     bk = c > bk ? c : bk;
                 }
                 for (int o = seg >> 1; o > 0; o >>= 1) {
                     const unsigned ob = __shfl_xor_sync(QCS_FULL, bk, o);
                     bk = ob > bk ? ob : bk;
                 }
-                zero = (bk >> 6) == 0u;
+                if (__any_sync(QCS_FULL, (bk >> 6) < 64u)) {  // small against the matrix: by the whole words
+                    bk = 0u;
+#pragma unroll 1
+                    for (int a = sl; a < r - 1; a += seg) {
+                        const unsigned c = (fx_key(row[a]) << 6) | (unsigned)(63 - a);
+                        bk = c > bk ? c : bk;
+                    }
+                    for (int o = seg >> 1; o > 0; o >>= 1) {
+                        const unsigned ob = __shfl_xor_sync(QCS_FULL, bk, o);
+                        bk = ob > bk ? ob : bk;
+                    }
+                    zero = (bk >> 6) == 0u;
+                }
+                P = 63 - (int)(bk & 63u);  // 0 .. r - 2
+                neg = false;
             }
-            const int P = 63 - (int)(bk & 63u);  // 0 .. r - 2
-            const fx2 piv = row[P];
             const int rv = r - 2;
-            if (live && sl == 0) {
-                pv[v * S0 + s] = P != rv ? make_longlong2(-piv.x, -piv.y) : piv;
-                pe[v * S0 + s] = f;
+            const fx2 piv = row[P];
+            if (live && (occ ? tm.t : sl) == 0) {
+                const int rec = occ ? wk.npv + s : v * S0 + s;
+                wk.pv[rec] = fx_neg_if(piv, neg != (P != rv));
+                wk.pe[rec] = fc;
             }
+            if (r == 2) break;  // no empty modes: the last pivot closes the Pfaffian
             const int sn = zero ? 0 : 61 - fx_bits(piv);
-            fxl ir, ii;
-            fx_inverse(zero ? make_longlong2(1ll << 60, 0ll) : make_longlong2(piv.x << sn, piv.y << sn), ir, ii);
+            int4 inv = fx_inverse(zero ? make_longlong2(1ll << 60, 0ll) : make_longlong2(piv.x << sn, piv.y << sn));
+            if (zero) inv = make_int4(0, 0, 0, 0);  // a zero row: g = 0, and the product is zero
             if (live) {
-                for (int i = sl; i < rv; i += seg) {
-                    const bool isP = i == P;
-                    const fx2 z = row[isP ? rv : i];
-                    // g = A_{i,k} / A_{p,k}, v = A_{i,p}
-                    Gv[v * m + i] = zero ? make_int4(0, 0, 0, 0)
-                                         : fx_times_inverse(make_longlong2(z.x << sn, z.y << sn), ir, ii);
-                    const int o = isP ? rv : i;
-                    const fx2 c = P == rv ? Nv[tri_index(i, rv)] : fx_skew(Nv, o, P);
-                    Vv[v * m + i] = fx_pack(fx_split(c.x), fx_split(c.y));
-                    if (P != rv && !isP) fx_put(Nv, i, P, Nv[tri_index(i, rv)]);
+                // g_i = A_{i,k} / A_{p,k} scaled by 2^{59-eu}, v_i = A_{i,p}, over the other r - 2
+                // positions once what was at the last but one has taken place P: index i reads
+                // and writes entries of its own
+                const fxl ir = {inv.x, inv.y}, ii = {inv.z, inv.w};
+                const int sh = sn - eu, tP = tri_count(P), tL = tri_count(rv);
+                const int i0 = occ ? tm.t : sl, step = occ ? Team::NT : seg;
+                FxGauss *GV = wk.GV + vr * mc;
+#pragma unroll 1
+                for (int i = i0; i < rv; i += step) {
+                    const int o = i == P ? rv : i;
+                    const bool lo = o > P;
+                    fx2 *a = Nv + (lo ? tri_count(o) + P : tP + o);
+                    fx2 z = row[o];
+                    const fx2 y = Nv[tL + i];
+                    // P = rv: o = i < P, and y is its own entry (i, P)
+                    const fx2 x = fx_neg_if(*a, lo);
+                    if (i != P) *a = fx_neg_if(y, lo);
+                    if (sh >= 0) {
+                        z.x <<= sh;
+                        z.y <<= sh;
+                    } else {
+                        z = fx_shift(z, sh);
+                    }
+                    GV[i].v = fx_pack(fx_split(x.x), fx_split(x.y));
+                    GV[i].g = fx_times_inverse(z, ir, ii);
                 }
             }
             tm.sync();
-            const int q = mb > kFxRoom ? mb - kFxRoom : 0;
-            unsigned o = fx_rank2(tm, nb, T, rv, Ns, Gv, Vv, m, 0, q, tab);
+            const int q = mbc + eu > kFxRoom ? mbc + eu - kFxRoom : 0;
+            unsigned o = fx_rank2<Team::NT>(tm.t, nb, T, rv, N0, wk.GV, mc, eu, q, tab);
             o = tm.or_put(o, s & 1);
             tm.sync();
-            mb = fx_top_bits(tm.or_get(o, s & 1));
-            f -= q;
+            mbc = fx_top_bits(tm.or_get(o, s & 1));
+            fc -= q;
+        }
+        if (occ) {
+            if (d2 > 0 && mbc - fc > bound) {
+                ok = false;
+                return total;
+            }
+            f = fc;
+            mb = mbc;
+            tm.sync();
+            continue;
         }
         // the closing Pfaffian of the last four (or two) active indices: packed entries
         // 01, 02, 12, 03, 13, 23
-        if (live && sl == 0) {
-            if (m >= 4) {
-                const int sh = kFxTop - mb;
-                fxacc re = {0, 0}, im = {0, 0};
-#pragma unroll
-                for (int t = 0; t < 3; ++t) {
-                    const fx2 x = fx_shift(Nv[t == 0 ? 0 : t == 1 ? 1 : 3], sh),
-                              y = fx_shift(Nv[t == 0 ? 5 : t == 1 ? 4 : 2], sh);
-                    fxl xr = fx_split(x.x), xi = fx_split(x.y);
-                    const fxl yr = fx_split(y.x), yi = fx_split(y.y);
-                    if (t == 1) {
-                        xr = fx_neg(xr);
-                        xi = fx_neg(xi);
-                    }
-                    fx_mac(re, xr, yr);
-                    fx_mac(re, fx_neg(xi), yi);
-                    fx_mac(im, xr, yi);
-                    fx_mac(im, xi, yr);
-                }
-                // |re|, |im| <= 6 2^{116}: kept to 2^{-58} of that
-                pv[v * S0 + s] = make_longlong2(fx_value(re, 5), fx_value(im, 5));
-                pe[v * S0 + s] = 2 * (f + sh) - 57;
-            } else {
-                pv[v * S0 + s] = Nv[0];
-                pe[v * S0 + s] = f;
+        if (mm >= 4) {  // one product on each of the segment's first three lanes
+            const int t = sl < 3 ? sl : 0, sh = kFxTop - mbc;
+            fx2 x = fx_shift(Nv[t == 2 ? 3 : t], sh);
+            const fx2 y = fx_shift(Nv[t == 0 ? 5 : t == 1 ? 4 : 2], sh);
+            x = fx_neg_if(x, t == 1);
+            const fxl xr = fx_split(x.x), xi = fx_split(x.y), yr = fx_split(y.x), yi = fx_split(y.y);
+            fxacc re = fx_mul(xr, yr, fx_half(5)), im = fx_mul(xr, yi, fx_half(5));
+            fx_mac(re, fx_neg(xi), yi);
+            fx_mac(im, xi, yr);
+            // |re|, |im| <= 2 2^{116} each: kept to 2^{-58} of that
+            const long long qx = fx_value(re, 5), qy = fx_value(im, 5);
+            const long long q1 = __shfl_down_sync(QCS_FULL, qx, 1), q2 = __shfl_down_sync(QCS_FULL, qx, 2);
+            const long long p1 = __shfl_down_sync(QCS_FULL, qy, 1), p2 = __shfl_down_sync(QCS_FULL, qy, 2);
+            if (live && sl == 0) {
+                wk.pv[v * S0 + s] = make_longlong2(qx + q1 + q2, qy + p1 + p2);
+                wk.pe[v * S0 + s] = 2 * (fc + sh) - 57;
             }
+        } else if (mm > 0 && live && sl == 0) {
+            wk.pv[v * S0 + s] = Nv[0];
+            wk.pe[v * S0 + s] = fc;
         }
-    }
-    tm.sync();
-    // gamma[v] times the records of node v and the npo common ones: each lane of the segment
-    // multiplies every seg-th of them, then a shuffle tree over the segment
-    fxp z = {1ll << 59, 0, -59};
-    bool any = false;
-    for (int i = sl; i < S0 + npo + 1; i += seg) {
-        fxp y;
-        if (i < S0) y = fx_norm(pv[vr * S0 + i], -pe[vr * S0 + i]);
-        else if (i < S0 + npo) y = fx_norm(pvo[i - S0], -peo[i - S0]);
-        else {
-            const cd g = gamma[vr];
-            const int E = 1022 - (int)(pivot_key(g) >> 20);
-            y = fx_norm(fx_of(g, 58 + E), -(58 + E));
-        }
-        z = any ? fx_prod(z, y) : y;
-        any = true;
-    }
-    const int w = S0 + npo + 1 < seg ? S0 + npo + 1 : seg;  // lanes that hold a factor
-    for (int o = seg >> 1; o > 0; o >>= 1) {
-        const fxp y = fx_shfl_xor(z, o);
-        if (w > o) z = fx_prod(z, y);  // lanes without a factor hold one
-    }
-    // sum over the warp's nodes on the segments' first lanes
-    cd S = cmk(0.0, 0.0);
-    if (live && sl == 0) S = cmk(fx_f64(z.x, z.e), fx_f64(z.y, z.e));
-    for (int o = seg; o < 32; o <<= 1) {
-        const double sx = __shfl_xor_sync(QCS_FULL, S.x, o), sy = __shfl_xor_sync(QCS_FULL, S.y, o);
-        if (o < seg * npw) S = cadd(S, cmk(sx, sy));
-    }
-    tm.sync();
-    return S;
-}
-
-// sum_k gamma_k pf(S + wnode_k D) prod(pvo) over nev nodes in rounds of at most NB, on the
-// first lane of the team's warps (each its own nodes' part): after a shared elimination
-// (shared) of the 2d x 2d complement S, otherwise of the full m x m matrix, one node per
-// round.  Ns: NB tri(2d) or tri(m) entries.
-template <class Team>
-__device__ inline cd fx_node_sum(const Team &tm, int m, int ne, bool shared, int nev, int NB,
-                                 const cd *__restrict__ wnode, const cd *__restrict__ gamma, const FxWork &wk,
-                                 const fx2 *__restrict__ Sx, int f, int mb, fx2 *__restrict__ Ns,
-                                 const uint16_t *__restrict__ tab) {
-    cd S = cmk(0.0, 0.0);
-    const int mm = shared ? m - ne : m, npo = shared ? ne / 2 : 0, NBr = shared ? NB : 1;
-    for (int k0 = 0; k0 < nev; k0 += NBr) {
-        const int nb = nev - k0 < NBr ? nev - k0 : NBr;
-        const cd s = fx_node_pfaffians(tm, mm, (m - ne) / 2, wnode + k0, gamma + k0, nb, Sx, f, mb, Ns, wk.Gv, wk.Vv,
-                                       tab, wk.pv, wk.pe, npo, wk.pv + wk.npv, wk.pe + wk.npv);
-        if (tm.lane == 0) S = cadd(S, s);
-    }
-    return S;
-}
-
-// The same from B^(s) in FP64 (packed, in the order of the selection, overwritten): the
-// occupied block is eliminated in Ns and S replaces B; a pair for which that is not stable
-// takes the full elimination of every node matrix.
-template <class Team>
-__device__ inline cd fx_pair_sum(const Team &tm, int m, int ne, int nev, int NB, const cd *__restrict__ wnode,
-                                 const cd *__restrict__ gamma, const FxWork &wk, cd *Bs, fx2 *Ns,
-                                 const uint16_t *__restrict__ tab) {
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    fx2 *Bx = reinterpret_cast<fx2 *>(Bs);
-    int f, mb = kFxTop;
-    if (!fx_load(tm, m, ne, Bs, Ns, f, tab)) return cmk(nan, nan);
-    if (fx_schur_occupied(tm, m, ne, Ns, wk.Gv, wk.Vv, tab, wk.pv + wk.npv, wk.pe + wk.npv, f, mb)) {
-        for (int t = tm.t; t < tri_count(m - ne); t += Team::NT) Bx[t] = Ns[t];
         tm.sync();
-        return fx_node_sum(tm, m, ne, true, nev, NB, wnode, gamma, wk, Bx, f, mb, Ns, tab);
+        // gamma[v] times the records of node v and the npo common ones: each lane of the segment
+        // multiplies every seg-th of them, then a shuffle tree over the segment
+        fxp z = {1ll << 59, 0, -59};
+        const int nrec = S0 + npo + 1, w = nrec < seg ? nrec : seg;  // lanes that hold a factor
+#pragma unroll 1
+        for (int i = sl, o = seg; o > 0;) {
+            fxp y;
+            bool mul;
+            if (i - sl < nrec) {  // uniform over the segment
+                mul = i < nrec;
+                const bool node = i < S0, po = i < S0 + npo;
+                const fx2 *x = !mul || node ? wk.pv + vr * S0 + (mul ? i : 0) : po ? pvo + (i - S0) : plan.g + k0 + vr;
+                const int e = !mul ? 0 : node ? -wk.pe[vr * S0 + i] : po ? -peo[i - S0] : plan.ge[k0 + vr];
+                if (mul) y = fx_norm(*x, e);
+                i += seg;
+            } else {
+                o >>= 1;
+                if (o == 0) break;
+                y = fx_shfl_xor(z, o);
+                mul = w > o;  // lanes without a factor hold one
+            }
+            if (mul) z = fx_prod(z, y);
+        }
+        // sum over the warp's nodes on the segments' first lanes
+        cd S = cmk(0.0, 0.0);
+        if (live && sl == 0) S = cmk(fx_f64(z.x, z.e), fx_f64(z.y, z.e));
+        for (int o = seg; o < 32; o <<= 1) {
+            const double sx = __shfl_xor_sync(QCS_FULL, S.x, o), sy = __shfl_xor_sync(QCS_FULL, S.y, o);
+            if (o < seg * npw) S = cadd(S, cmk(sx, sy));
+        }
+        total = cadd(total, S);
+        tm.sync();
     }
-    tm.sync();
-    mb = kFxTop;
-    fx_load(tm, m, ne, Bs, Ns, f, tab);
-    return fx_node_sum(tm, m, ne, false, nev, 1, wnode, gamma, wk, Ns, f, mb, Bx, tab);
+    return total;
+}
+
+// The same from B^(s) in FP64 (packed, in the order of the selection, overwritten by the
+// node matrices: max(tri(m), NB tri(2d)) entries); the occupied block is eliminated in X
+// (tri(m) entries).  A pair for which that is not stable takes the full elimination of
+// every node matrix.
+template <class Team>
+__device__ inline cd fx_pair_sum(const Team &tm, int m, int ne, int NB, const FxPlan &plan, const FxWork &wk, cd *Bs,
+                                 fx2 *X, const uint16_t *__restrict__ tab) {
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    bool shared = true, ok;
+    cd S;
+#pragma unroll 1
+    do {
+        int f;
+        if (!fx_load(tm, m, ne, Bs, X, f, tab)) return cmk(nan, nan);
+        S = fx_pair_eliminate(tm, m, ne, shared, NB, plan, wk, X, reinterpret_cast<fx2 *>(Bs), f, kFxTop, tab, ok);
+        shared = false;
+        tm.sync();
+    } while (!ok);
+    return S;
 }

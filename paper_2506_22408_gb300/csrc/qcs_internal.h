@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <map>
 #include <string>
@@ -175,7 +176,12 @@ struct qcs_pair_launch {
     cd *per_pair;    // W x P or null
     qcs_node_plan plan;
     int config;      // qcs_config encoding; 0 = heuristic
-    unsigned long long *counter;  // device tile counter (reset by the launcher)
+    unsigned long long *counter;  // device tile counters (reset by the launcher)
+    // tensor-core path: batches of wblock walkers x span list positions through pair records
+    unsigned char *rec = nullptr;  // wblock x span records of qcs_pf_rec_bytes
+    cd *sum = nullptr;             // wblock x span
+    int64_t wblock = 0;
+    int span = 0;
 };
 
 qcs_status qcs_launch_pairs(qcs_ctx *ctx, const qcs_pair_launch &L, cudaStream_t st);
@@ -188,13 +194,31 @@ qcs_status qcs_launch_split(qcs_ctx *ctx, const qcs_pair_launch &L, float *Mhi, 
 // FP64-accurate congruence on tensor cores (qcs_tcpair.cu)
 bool qcs_tc_supported(int n);      // n <= 16
 size_t qcs_tc_walker_bytes(int64_t W);
-int qcs_tc_snaps_per_tile(int subs);  // parity +1 snapshots per tile (subs sub-tiles; 0 = default)
+int64_t qcs_tc_counters(int64_t W, int64_t wblock, int nchunks);  // tile counters of a call
 qcs_status qcs_tc_prepare_snapshots(qcs_ctx *ctx, qcs_snapshots *s, cudaStream_t st);
 // Whether the FP64 ALU pair kernel runs (n, config) on its two-warp path, which forms
 // K = Ut [H1 | G2] from the set's rows [H1^T; G2^T] and B from K.
 bool qcs_pair_forms_K(int n, int config);
 // The rows [H1^T; G2^T] of every dense snapshot into s->Qh (allocated and formed once).
 qcs_status qcs_hform_prepare_snapshots(qcs_ctx *ctx, qcs_snapshots *s, cudaStream_t st);
+// Pfaffian sums of a batch of pair records (qcs_pfaff.cu)
+struct qcs_pf_launch {
+    int n, ne;
+    int64_t W;                 // walkers of the batch
+    const qcs_snapshots *s;
+    const qcs_node_plan *plan;
+    int config;
+    int64_t p0;                // first list position
+    int span;                  // list positions, at most
+    int nchunks;               // batches per walker
+    const unsigned char *rec;  // span x W records of qcs_pf_rec_bytes
+    const cd *pref;
+    cd *sum;                   // W x span
+    cd *partial;               // partial[w nchunks]: the batch's sum of walker w
+    cd *per_pair;              // W x P or null
+};
+int qcs_pf_rec_bytes(int n, int ne);
+qcs_status qcs_launch_pfaffians(qcs_ctx *ctx, const qcs_pf_launch &L, cudaStream_t st);
 qcs_status qcs_launch_tc_pairs(qcs_ctx *ctx, const qcs_pair_launch &L, unsigned char *walk_rec, cudaStream_t st);
 qcs_status qcs_launch_pairs_batched(qcs_ctx *ctx, int nsys, const qcs_pair_launch *Ls, unsigned long long *counter,
                                     cudaStream_t st);

@@ -66,6 +66,7 @@ struct PairArgs {
     unsigned *status;
     cd wnode[QCS_MAX_NODES];
     cd gamma[QCS_MAX_NODES];
+    FxPlan plan;  // the same in fixed point
 };
 
 // One tile of system A: walker w = tile / nchunks, the tile's snapshots spread
@@ -80,13 +81,13 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
     cd *Rg = reinterpret_cast<cd *>(wbase);
     cd *Qs = Rg;  // staged snapshot rows (shared-memory path only)
     cd *Ts = reinterpret_cast<cd *>(wbase + A.off_T);
-    fx2 *Ns = reinterpret_cast<fx2 *>(wbase);  // node matrices, once T is consumed
+    fx2 *Xs = reinterpret_cast<fx2 *>(wbase);  // B^(s) in fixed point, once T is consumed
     double *Uss = reinterpret_cast<double *>(Uts + n * ld_ut(n));  // re + im of Ut
     cd *Bs = reinterpret_cast<cd *>(wbase + A.off_B);
     const FxWarp tm = {lane, lane, 0, 0, nullptr};
     const int npv = pv_records(A.vm, A.NB);
     fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
-    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
+    const FxWork wk = {reinterpret_cast<FxGauss *>(wbase + A.off_U), pv,
                        reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
     const int span = A.chunk * wpb;  // snapshots per tile; warp w takes every wpb-th
     // chunk-major tile order: consecutive tiles share one snapshot chunk and run over
@@ -235,7 +236,7 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
             __syncwarp();
             build_B(A.n, A.ne, Ts, Bs, tab, lane);
             __syncwarp();
-            const cd S = fx_pair_sum(tm, A.m, A.ne, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, Ns, tab);
+            const cd S = fx_pair_sum(tm, A.m, A.ne, A.NB, A.plan, wk, Bs, Xs, tab);
             if (lane == 0) {
                 if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
                 acc = cadd(acc, S);
@@ -312,8 +313,8 @@ namespace {
 
 // Per-warp shared layout for nb node matrices; returns bytes per warp.  The first
 // region holds the staged snapshot rows and T (T alone on the register path), then
-// the node matrices: one full copy of B (shared elimination; the rare full
-// eliminations, one node per round) or NB complements of 2d x 2d.
+// B^(s) in fixed point, whose occupied block is eliminated there; the second B^(s) in
+// FP64, then the node matrices (NB complements of 2d x 2d, or a full matrix).
 size_t pair_group_layout(PairArgs &A, int NB);
 
 size_t pair_warp_layout(PairArgs &A, int NB) {
@@ -324,12 +325,11 @@ size_t pair_warp_layout(PairArgs &A, int NB) {
     A.off_qs = (int)align16(R);  // staged rows' re + im sums (shared-memory path)
     if (A.t3) R = (size_t)A.off_qs + (size_t)2 * n * n * sizeof(double);
     if ((size_t)T * sizeof(cd) > R) R = (size_t)T * sizeof(cd);
-    if ((size_t)NB * tri_count(d2) * sizeof(cd) > R) R = (size_t)NB * tri_count(d2) * sizeof(cd);
     A.vm = m > NB * d2 ? m : NB * d2;
     A.off_T = (int)qbytes;
     size_t o = align16(R);
-    A.off_B = (int)o;
-    o = align16(o + (size_t)T * sizeof(cd));
+    A.off_B = (int)o;  // B^(s), then the node matrices
+    o = align16(o + (size_t)(T > NB * tri_count(d2) ? T : NB * tri_count(d2)) * sizeof(cd));
     A.off_U = (int)o;
     o = align16(o + (size_t)A.vm * sizeof(cd));
     A.off_V = (int)o;
@@ -449,6 +449,7 @@ void setup_pair_args(qcs_ctx *ctx, const qcs_pair_launch &L, PairArgs &A) {
         A.wnode[k] = L.plan.wnode[k];
         A.gamma[k] = L.plan.gamma[k];
     }
+    fx_make_plan(L.plan, A.plan);
 }
 
 }  // namespace

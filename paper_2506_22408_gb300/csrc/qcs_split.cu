@@ -114,6 +114,7 @@ struct SplitArgs {
     unsigned *status;
     cd wnode[QCS_MAX_NODES];
     cd gamma[QCS_MAX_NODES];
+    FxPlan plan;  // the same in fixed point
 };
 
 // B^(s) (FP64 packed upper) from T (FP32 complex, row stride ld) in FP32 arithmetic.
@@ -197,11 +198,11 @@ __global__ void __launch_bounds__(128, 3) split_pair_kernel(const __grid_constan
     unsigned char *wbase = region + (size_t)warp * A.warp_bytes;
     float2 *Ts = reinterpret_cast<float2 *>(wbase + A.off_T);
     cd *Bs = reinterpret_cast<cd *>(wbase + A.off_B);
-    fx2 *Ns = reinterpret_cast<fx2 *>(wbase);  // node matrices start the warp region (T is consumed first)
+    fx2 *Xs = reinterpret_cast<fx2 *>(wbase);  // B^(s) in fixed point (T is consumed first)
     const FxWarp tm = {lane, lane, 0, 0, nullptr};
     const int npv = pv_records(A.vm, A.NB);
     fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
-    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
+    const FxWork wk = {reinterpret_cast<FxGauss *>(wbase + A.off_U), pv,
                        reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
     const int ldT = 2 * n + 1;
 
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(128, 3) split_pair_kernel(const __grid_constan
                 if (w >= A.W) continue;
                 build_B_f32(n, A.ne, Ts, ldT, Bs, tab, lane);
                 __syncwarp();
-                const cd S = fx_pair_sum(tm, A.m, A.ne, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, Ns, tab);
+                const cd S = fx_pair_sum(tm, A.m, A.ne, A.NB, A.plan, wk, Bs, Xs, tab);
                 if (lane == 0) {
                     if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
                     acc = cadd(acc, S);
@@ -601,16 +602,14 @@ size_t split_group_layout(SplitArgs &A, int NB) {
 // Per-warp workspace of the split kernel for nb node matrices.
 size_t split_warp_layout(SplitArgs &A, int NB) {
     const int n = A.n, m = A.m, T = tri_count(m), d2 = m - A.ne;
-    // node matrices: one full copy of B (shared elimination; the rare full eliminations,
-    // one node per round) or NB complements of 2d x 2d
-    size_t nodes = (size_t)(T > NB * tri_count(d2) ? T : NB * tri_count(d2)) * sizeof(cd);
+    const size_t nodes = (size_t)(T > NB * tri_count(d2) ? T : NB * tri_count(d2)) * sizeof(cd);
     A.vm = m > NB * d2 ? m : NB * d2;
-    size_t tbytes = (size_t)n * (2 * n + 1) * sizeof(float2);
-    // T is consumed (into B) before the node matrices are written: they may share
-    size_t o = align16(nodes > tbytes ? nodes : tbytes);
+    // T is consumed (into B) before B^(s) is converted to fixed point: they may share
+    const size_t tbytes = (size_t)n * (2 * n + 1) * sizeof(float2), xbytes = (size_t)T * sizeof(cd);
+    size_t o = align16(xbytes > tbytes ? xbytes : tbytes);
     A.off_T = 0;
-    A.off_B = (int)o;
-    o = align16(o + (size_t)T * sizeof(cd));
+    A.off_B = (int)o;  // B^(s), then the node matrices (NB complements of 2d x 2d, or a full matrix)
+    o = align16(o + nodes);
     A.off_U = (int)o;
     o = align16(o + (size_t)A.vm * sizeof(cd));
     A.off_V = (int)o;
@@ -797,6 +796,7 @@ qcs_status qcs_launch_split(qcs_ctx *ctx, const qcs_pair_launch &L, float *Mhi, 
         A.wnode[k] = L.plan.wnode[k];
         A.gamma[k] = L.plan.gamma[k];
     }
+    fx_make_plan(L.plan, A.plan);
     const size_t smem = (size_t)A.region_bytes + tab;
     if (smem + 1024 > ctx->smem_optin) return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "split kernel: shared memory");
     if (qcs_set_smem(ctx, (const void *)split_pair_kernel, smem) != QCS_OK) return QCS_ERR_CUDA;

@@ -37,8 +37,8 @@
 //     MN-major (lane k owns column k of Z_i^T);
 //  4. 14 more MMAs form P_i = M Z_i (lane b of warp i, column a: P_i[a][b]); each warp
 //     shifts its lanes to the pair's common scale, keeps the upper triangle of P_i,
-//     assembles B^(s) and runs the node Pfaffians, all in fixed point (qcs_fixed.cuh;
-//     1024 x 20000 at n = 16, ne = 8: 377 ms with FP64 eliminations, 263 ms).
+//     assembles B^(s) in fixed point (qcs_fixed.cuh) and writes it as a pair record;
+//     qcs_pfaff.cu takes the node Pfaffians from the records.
 // Every wait is bounded: a time-out raises QCS_ERR_TIMEOUT, drains and frees the
 // tensor memory.
 #include "qcs_internal.h"
@@ -91,15 +91,11 @@ __global__ void tc_walker_prep_kernel(int n, int64_t W, const cd *__restrict__ U
 #pragma unroll
         for (int kk = 0; kk < kRowsPer; ++kk)
             if (x[kk] != 0.0) e = max(e, row_exp_of(x[kk]));
-        uint64_t u[kRowsPer];
-        uint32_t neg = 0u;
+        long long u[kRowsPer];
 #pragma unroll
-        for (int kk = 0; kk < kRowsPer; ++kk) {
-            u[kk] = e == kNoRow ? 0ull : fixed_of(x[kk], e);
-            neg |= (x[kk] < 0.0 ? 1u : 0u) << kk;
-        }
+        for (int kk = 0; kk < kRowsPer; ++kk) u[kk] = e == kNoRow ? 0ll : fixed_of(x[kk], e);
         unsigned char *base = rec + (size_t)w * kWalkRecBytes;
-        store_row_slices(base, kSliceBytes, r, u, neg);
+        store_row_slices(base, kSliceBytes, r, u);
         reinterpret_cast<int *>(base + kSlices * kSliceBytes)[r] = e;
     }
 }
@@ -147,16 +143,12 @@ __global__ void tc_snapshot_prep_kernel(int n, int64_t nslots, const cd *__restr
 #pragma unroll
         for (int l = 0; l < kRowsPer; ++l)
             if (h[l] != 0.0) e = max(e, row_exp_of(h[l]));
-        uint64_t u[kRowsPer];
-        uint32_t neg = 0u;
+        long long u[kRowsPer];
 #pragma unroll
-        for (int l = 0; l < kRowsPer; ++l) {
-            u[l] = e == kNoRow ? 0ull : fixed_of(h[l], e);
-            neg |= (h[l] < 0.0 ? 1u : 0u) << l;
-        }
+        for (int l = 0; l < kRowsPer; ++l) u[l] = e == kNoRow ? 0ll : fixed_of(h[l], e);
         unsigned char *base = rec + (size_t)(p / kSnapsPerSub) * kSnapRecBytes;
         const int row = (int)(p % kSnapsPerSub) * kRowsPer + k;
-        store_row_slices(base, kSnapSlab, row, u, neg);
+        store_row_slices(base, kSnapSlab, row, u);
         reinterpret_cast<int *>(base + kSlices * kSnapSlab)[row] = e;
         __syncwarp();
     }
@@ -165,30 +157,24 @@ __global__ void tc_snapshot_prep_kernel(int n, int64_t nslots, const cd *__restr
 // ---------------------------------------------------------------- pair kernel
 
 struct TcArgs {
-    int n, ne, m, d, nev, NB;
+    int n, ne, m;
     int64_t W, P;
     int64_t nrec;     // snapshot records allocated (4 list slots each)
-    int nchunks;      // tiles per walker (chunks of 4 subs list positions)
+    int64_t p0;       // first list position of the batch (a multiple of 4)
+    int span;         // list positions of the batch, at most
+    int ntile;        // tiles per walker (4 subs list positions each)
     int subs;         // sub-tiles of kSnapsPerSub snapshots per tile
-    int ws_bytes;     // Pfaffian workspace per warp
-    int ws_in_operands;  // 1: the workspaces are quarters of the operand region
     int teams;        // four-warp teams in the block
-    int team_bytes;   // shared bytes per team: records (and workspaces if not in them)
+    int team_bytes;   // shared bytes per team: the operand records
     int tslots;       // tensor-memory accumulators of 256 columns
-    int off_P, off_N, off_U, off_V, off_pv;  // B^(s) at offset 0
-    int vm;
     int smem_tab;     // byte offset of the pair table (after the teams' regions)
+    int rec_bytes;    // bytes per pair record
     const unsigned char *snap_rec;
     const unsigned char *walk_rec;
-    const cd *pref;
-    const int *idx;
     const int *d_count;
-    cd *partial;      // W x nchunks
-    cd *per_pair;
+    unsigned char *out;  // pair records: list position p0 + p, walker w at p W + w
     unsigned long long *counter;
     unsigned *status;
-    cd wnode[QCS_MAX_NODES];
-    cd gamma[QCS_MAX_NODES];
 };
 
 // The MMAs of one sliced product, levels 2..8: per A slice i one instruction pair
@@ -289,8 +275,9 @@ __host__ __device__ __forceinline__ uint32_t mnmajor16(int row, int k) {
 
 // Slices of Z_i^T, read from tensor memory (lane k holds row k of Z_i, z_kb worth
 // z 2^{g_k + e_b - 56}): row b of Z_i^T gets the scale 2^{F_b}, F_b = e_b + G_b - 56 with
-// G_b = max_k (g_k + bitlen z_kb) (a warp max-reduction); the slices go MN-major into
-// the A operand rows row0 + b.  Returns F_b for b = lane (kNoRow for a zero row).
+// 2^{G_b} above max_k |z_kb| 2^{g_k} (1 + 2^-7) (a warp max-reduction on the upper words;
+// on the whole ones for a row that is zero there); the slices go MN-major into the A operand
+// rows row0 + b.  Returns F_b for b = lane (kNoRow for a zero row).
 __device__ __forceinline__ int slice_zt(uint32_t tlane, int gk, int eb_lane, unsigned char *Abase, int row0, int lane) {
     int Gl = kNoRow;
 #pragma unroll 1
@@ -298,22 +285,22 @@ __device__ __forceinline__ int slice_zt(uint32_t tlane, int gk, int eb_lane, uns
         long long z[8];
         read_levels8(tlane, cb, z);
         uint64_t u[8];
-        SliceSign g[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const int t = z[c] != 0 ? gk + bitlen64(z[c]) : kNoRow;
-            const int G = __reduce_max_sync(QCS_FULL, t);
+            const int zh = abs((int)(z[c] >> 32));
+            int G = __reduce_max_sync(QCS_FULL, zh != 0 ? gk + 64 - __clz(zh + (zh >> 6) + 1) : kNoRow);
+            if (G == kNoRow) G = __reduce_max_sync(QCS_FULL, z[c] != 0 ? gk + bitlen64(z[c]) + 1 : kNoRow);
             if (8 * cb + c == lane) Gl = G;
-            u[c] = (z[c] == 0 || G == kNoRow) ? 0ull : rescale_mag(z[c], 56 + gk - G);
-            g[c] = slice_sign(z[c] < 0);
+            const long long v = G == kNoRow ? 0ll : fx_shift_any(z[c], 55 + gk - G);
+            u[c] = (uint64_t)v + kDigitBias;
         }
 #pragma unroll
         for (int i = 1; i <= kSlices; ++i) {
             uint4 w;
-            w.x = bf16x2_of(slice_f32(u[0], i, g[0]), slice_f32(u[1], i, g[1]));
-            w.y = bf16x2_of(slice_f32(u[2], i, g[2]), slice_f32(u[3], i, g[3]));
-            w.z = bf16x2_of(slice_f32(u[4], i, g[4]), slice_f32(u[5], i, g[5]));
-            w.w = bf16x2_of(slice_f32(u[6], i, g[6]), slice_f32(u[7], i, g[7]));
+            w.x = bf16x2_of(slice_f32(u[0], i), slice_f32(u[1], i));
+            w.y = bf16x2_of(slice_f32(u[2], i), slice_f32(u[3], i));
+            w.z = bf16x2_of(slice_f32(u[4], i), slice_f32(u[5], i));
+            w.w = bf16x2_of(slice_f32(u[6], i), slice_f32(u[7], i));
             *reinterpret_cast<uint4 *>(Abase + (size_t)(i - 1) * kSnapSlab + mnmajor16(row0 + 8 * cb, lane)) = w;
         }
     }
@@ -351,7 +338,6 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
     __shared__ int slot_of[kMaxTeams];
     __shared__ int slot_owner[kTmemSlots];
     __shared__ int abort_flag;
-    __shared__ cd red[kMaxTeams][4];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int team = warp >> 2, wt = warp & 3, ttid = tid & (kTeamThreads - 1);
     const int n = A.n;
@@ -359,28 +345,18 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
     unsigned char *Wrec = X + kSnapRecBytes;                      // walker record
     const int *g_exp = reinterpret_cast<const int *>(X + kOperandBytes);              // snapshot row exponents
     const int *e_exp = reinterpret_cast<const int *>(Wrec + kSlices * kSliceBytes);  // walker row exponents
-    // the teams' records, their workspaces and the pair table fit the launch's shared
-    // memory, and the block is a whole number of teams (block-uniform: nothing is
-    // allocated or issued yet)
+    // the teams' records and the pair table fit the launch's shared memory, and the block is
+    // a whole number of teams (block-uniform: nothing is allocated or issued yet)
     if (!QCS_IN_BOUNDS((int)blockDim.x == kTeamThreads * A.teams && A.teams <= kMaxTeams &&
-                           A.tslots >= 1 && A.tslots <= (int)kTmemSlots &&
-                           A.teams * A.team_bytes <= A.smem_tab &&
+                           A.tslots >= 1 && A.tslots <= (int)kTmemSlots && A.teams * A.team_bytes <= A.smem_tab &&
                            A.smem_tab + tri_count(A.m) * (int)sizeof(uint16_t) <= (int)dyn_smem_bytes() &&
-                           (A.ws_in_operands ? 4 * A.ws_bytes <= kOperandBytes
-                                             : kSnapRecBytes + kWalkRecBytes + 4 * A.ws_bytes <= A.team_bytes),
+                           4 * kPuBytes <= kOperandBytes && kSnapRecBytes + kWalkRecBytes <= A.team_bytes,
                        A.status))
         return;
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem_tc + A.smem_tab);
     build_pair_table(tab, tri_count(A.m));
-    unsigned char *wbase = (A.ws_in_operands ? X : X + kSnapRecBytes + kWalkRecBytes) + (size_t)wt * A.ws_bytes;
-    fx2 *Bs = reinterpret_cast<fx2 *>(wbase);
-    long long *Pu = reinterpret_cast<long long *>(wbase + A.off_P);
-    fx2 *Ns = reinterpret_cast<fx2 *>(wbase + A.off_N);  // aliases Pu: written once the occupied block is eliminated
-    const FxWarp tm = {lane, lane, 0, 0, nullptr};
-    const int npv = pv_records(A.vm, A.NB);
-    fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
-    const FxWork wk = {reinterpret_cast<int4 *>(wbase + A.off_U), reinterpret_cast<int4 *>(wbase + A.off_V), pv,
-                       reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
+    // the upper triangle of this warp's P, in the operand region once the products are done
+    long long *Pu = reinterpret_cast<long long *>(X + (size_t)wt * kPuBytes);
 
     if (warp == 0) {
         tmem_alloc(&tmem_base, (uint32_t)A.tslots * kTmemCols);
@@ -399,7 +375,8 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
     fence_after_sync();
     const uint32_t tmem0 = tmem_base;
     const int64_t L = *A.d_count;
-    const int64_t ntiles = A.W * (int64_t)A.nchunks;
+    const int64_t Lb = L < A.p0 + A.span ? L : A.p0 + A.span;  // end of the batch's list positions
+    const int64_t ntiles = A.W * (int64_t)A.ntile;
     uint32_t ph_load = 0, ph_mma = 0;
     bool load_pending = false, mma_pending = false;
     bool ok = true;
@@ -458,17 +435,12 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
         if (t >= ntiles) break;
         const int ch = (int)(t / A.W);  // chunk-major: a chunk's records stay in L2 over the walkers
         const int64_t w = t - (int64_t)ch * A.W;
-        const int64_t p0 = (int64_t)ch * (kSnapsPerSub * A.subs);
-        if (!QCS_IN_BOUNDS(ch < A.nchunks && L >= 0 && L <= A.P, A.status)) continue;  // team-uniform
-        if (p0 >= L) {
-            if (ttid == 0) A.partial[w * A.nchunks + ch] = cmk(0.0, 0.0);
-            continue;
-        }
-        const cd prefw = A.pref[w];
-        cd acc = cmk(0.0, 0.0);
+        const int64_t p0 = A.p0 + (int64_t)ch * (kSnapsPerSub * A.subs);
+        if (!QCS_IN_BOUNDS(ch < A.ntile && L >= 0 && L <= A.P, A.status)) continue;  // team-uniform
+        if (p0 >= Lb) continue;
         for (int s = 0; s < A.subs; ++s) {
             const int64_t pb = p0 + (int64_t)s * kSnapsPerSub;
-            if (pb >= L) break;
+            if (pb >= Lb) break;
             if (!QCS_IN_BOUNDS(pb / kSnapsPerSub < A.nrec, A.status)) break;  // the record to copy exists
             if (ttid == 0) {
                 const uint32_t bytes = kSnapRecBytes + (s == 0 ? kWalkRecBytes : 0);
@@ -516,26 +488,15 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
             }
             release();  // this team's tensor-memory reads are done; another team may use the slot
             const int64_t slot = pb + wt;
-            if (slot < L && QCS_IN_BOUNDS(A.idx[slot] >= 0 && A.idx[slot] < A.P, A.status)) {
-                int f = fP, mb = fx_top_bits(build_B_from_P(n, A.ne, A.m, Pu, Bs, tab, lane));
+            if (slot < Lb) {
                 __syncwarp();
-                cd S;
-                if (fx_schur_occupied(tm, A.m, A.ne, Bs, wk.Gv, wk.Vv, tab, wk.pv + npv, wk.pe + npv, f, mb)) {
-                    S = fx_node_sum(tm, A.m, A.ne, true, A.nev, A.NB, A.wnode, A.gamma, wk, Bs, f, mb, Ns, tab);
-                } else {  // rare: B^(s) again, every node matrix in full
-                    __syncwarp();
-                    f = fP;
-                    mb = fx_top_bits(build_B_from_P(n, A.ne, A.m, Pu, Bs, tab, lane));
-                    __syncwarp();
-                    S = fx_node_sum(tm, A.m, A.ne, false, A.nev, 1, A.wnode, A.gamma, wk, Bs, f, mb, Ns, tab);
-                }
-                if (lane == 0) {
-                    if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
-                    acc = cadd(acc, S);
-                    if (A.per_pair) A.per_pair[w * A.P + A.idx[slot]] = cmul(prefw, S);
-                }
+                unsigned char *rec = A.out + (size_t)((slot - A.p0) * A.W + w) * A.rec_bytes;
+                fx2 *B = reinterpret_cast<fx2 *>(rec);
+                const unsigned top = build_B_from_P(n, A.ne, A.m, Pu, B, tab, lane);
+                if (lane == 0)
+                    *reinterpret_cast<int2 *>(rec + (size_t)tri_count(A.m) * sizeof(fx2)) = make_int2(fP, fx_top_bits(top));
             }
-            fence_proxy_async_smem();  // workspace writes precede the next sub-tile's bulk copy
+            fence_proxy_async_smem();  // writes of P precede the next sub-tile's bulk copy
             team_sync(team);
         }
         if (!ok) {
@@ -547,9 +508,6 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
             // the other teams stop at the abort flag instead of waiting for it
             continue;  // every thread of the team leaves through the abort check at the top
         }
-        if (lane == 0) red[team][wt] = acc;
-        team_sync(team);
-        if (ttid == 0) A.partial[w * A.nchunks + ch] = cadd(cadd(red[team][0], red[team][1]), cadd(red[team][2], red[team][3]));
     }
     if (ttid == 0 && (load_pending || mma_pending)) {  // a wait gave up: let a copy or MMAs in flight land first
         if (load_pending) mbar_wait_bounded(&mbar_load[team], ph_load, kWaitIter);
@@ -561,30 +519,11 @@ __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(co
     if (warp == 0) tmem_dealloc(tmem0, (uint32_t)A.tslots * kTmemCols);
 }
 
-// Pfaffian workspace of one warp for nb node matrices: B^(s), then the upper triangle
-// of P aliased by the node matrices (written once B^(s) is assembled), then the Gauss
-// vectors and the step records; returns its bytes.
-size_t tc_warp_layout(TcArgs &A, int NB) {
-    const int m = A.m, T = tri_count(m), d2 = m - A.ne;
-    const size_t nodes = (size_t)(T > NB * tri_count(d2) ? T : NB * tri_count(d2)) * sizeof(cd);
-    A.vm = m > NB * d2 ? m : NB * d2;
-    size_t o = align16((size_t)T * sizeof(cd));
-    A.off_P = A.off_N = (int)o;
-    o = align16(o + (nodes > (size_t)kPuBytes ? nodes : (size_t)kPuBytes));
-    A.off_U = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_V = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pv = (int)o;  // records of the node products, then of the occupied pivots
-    o = align16(o + pv_bytes(A.vm, NB, A.ne));
-    return o;
-}
-
 }  // namespace
 
-size_t qcs_tc_walker_bytes(int64_t W) { return (size_t)(W > 0 ? W : 1) * kWalkRecBytes; }
+int64_t qcs_tc_counters(int64_t W, int64_t wblock, int nchunks) { return (W + wblock - 1) / wblock * nchunks; }
 
-int qcs_tc_snaps_per_tile(int subs) { return kSnapsPerSub * (subs > 0 ? subs : kSubPerTile); }
+size_t qcs_tc_walker_bytes(int64_t W) { return (size_t)(W > 0 ? W : 1) * kWalkRecBytes; }
 
 bool qcs_tc_supported(int n) { return n >= 2 && 2 * n <= kRowsPer; }
 
@@ -628,39 +567,12 @@ qcs_status qcs_launch_tc_pairs(qcs_ctx *ctx, const qcs_pair_launch &L, unsigned 
     A.n = n;
     A.ne = L.ne;
     A.m = 2 * n - L.ne;
-    A.d = n - L.ne;
-    A.nev = L.plan.nev;
-    A.W = L.W;
     A.P = L.P;
     A.nrec = (L.P + kSnapsPerSub - 1) / kSnapsPerSub;
-    A.nchunks = L.nchunks;
-    // node matrices per round: the requested count, or the largest balanced count whose
-    // four workspaces fit in the operand region; when even one node per round does not
-    // fit there (large m), the workspaces get their own shared memory
-    auto fits = [&](int nb) { return 4 * tc_warp_layout(A, nb) <= (size_t)kOperandBytes; };
-    int NB = 1;
-    const qcs_config cfg = qcs_decode_config(L.config);
-    A.subs = cfg.subs > 0 ? cfg.subs : kSubPerTile;
-    if (cfg.nb > 0) {
-        NB = cfg.nb < A.nev ? cfg.nb : A.nev;
-        if (NB > kMaxNB) NB = kMaxNB;
-        while (NB > 1 && !fits(NB)) --NB;
-    } else {
-        for (int rounds = 1; rounds <= A.nev; ++rounds) {
-            const int nb = (A.nev + rounds - 1) / rounds;
-            if (nb > kMaxNB) continue;
-            if (fits(nb)) {
-                NB = nb;
-                break;
-            }
-        }
-    }
-    A.NB = NB;
-    A.ws_in_operands = fits(NB) ? 1 : 0;
-    A.ws_bytes = (int)tc_warp_layout(A, NB);
+    A.span = L.span;
     // teams per block: as many as the block's shared memory holds (about 1 KB kept for
     // the static words), at most kMaxTeams; one block per SM
-    A.team_bytes = kSnapRecBytes + kWalkRecBytes + (A.ws_in_operands ? 0 : 4 * A.ws_bytes);
+    A.team_bytes = kSnapRecBytes + kWalkRecBytes;
     const size_t tab = align16((size_t)tri_count(A.m) * sizeof(uint16_t));
     int teams = (int)((ctx->smem_optin - 1024 - tab) / (size_t)A.team_bytes);
     if (teams > kMaxTeams) teams = kMaxTeams;
@@ -669,33 +581,62 @@ qcs_status qcs_launch_tc_pairs(qcs_ctx *ctx, const qcs_pair_launch &L, unsigned 
     A.tslots = teams >= 2 ? 2 : 1;
     A.smem_tab = teams * A.team_bytes;
     const size_t smem = (size_t)A.smem_tab + tab;
+    A.rec_bytes = qcs_pf_rec_bytes(n, L.ne);
     A.snap_rec = (const unsigned char *)L.s->tc_rec;
-    A.walk_rec = walk_rec;
-    A.pref = L.pref;
-    A.idx = L.s->idx;
     A.d_count = L.s->d_count;
-    A.partial = L.partial;
-    A.per_pair = L.per_pair;
-    A.counter = L.counter;
+    A.out = L.rec;
     A.status = ctx->d_status;
-    for (int k = 0; k < L.plan.nev; ++k) {
-        A.wnode[k] = L.plan.wnode[k];
-        A.gamma[k] = L.plan.gamma[k];
-    }
     if (smem + 1024 > ctx->smem_optin) return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "tc kernel: shared memory");
     if (qcs_set_smem(ctx, (const void *)tc_pair_kernel, smem) != QCS_OK) return QCS_ERR_CUDA;
-    // one block per SM (its shared memory and its 2 x 256 tensor-memory columns take the
-    // SM), fewer when there are fewer tiles than teams
-    const int64_t ntiles = A.W * (int64_t)A.nchunks;
-    int64_t blocks = (int64_t)ctx->num_sms;
-    if (blocks > (ntiles + teams - 1) / teams) blocks = (ntiles + teams - 1) / teams;
-    if (blocks < 1) blocks = 1;
-    if (cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long), st) != cudaSuccess)
+    if (cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long) * qcs_tc_counters(L.W, L.wblock, L.nchunks), st) !=
+        cudaSuccess)
         return qcs_fail(ctx, QCS_ERR_CUDA, "tc tile counter reset");
-    qcs_log(3, "tc_pair_kernel: %lld blocks x %d teams, %zu bytes of shared memory, %d tensor-memory slots",
-            (long long)blocks, teams, smem, A.tslots);
+    qcs_pf_launch F;
+    F.n = n;
+    F.ne = L.ne;
+    F.s = L.s;
+    F.plan = &L.plan;
+    F.config = L.config;
+    F.rec = L.rec;
+    F.sum = L.sum;
+    F.span = L.span;
+    F.nchunks = L.nchunks;
+    const int want = qcs_decode_config(L.config).subs;
     qcs_prof_begin(ctx, st);
-    tc_pair_kernel<<<(unsigned)blocks, kTeamThreads * teams, smem, st>>>(A);
+    unsigned long long *counter = L.counter;
+    for (int64_t w0 = 0; w0 < L.W; w0 += L.wblock) {
+        A.W = F.W = L.W - w0 < L.wblock ? L.W - w0 : L.wblock;
+        A.walk_rec = walk_rec + (size_t)w0 * kWalkRecBytes;
+        F.pref = L.pref + w0;
+        F.per_pair = L.per_pair ? L.per_pair + w0 * L.P : nullptr;
+        for (int c = 0; c < L.nchunks; ++c) {
+            A.p0 = F.p0 = (int64_t)c * L.span;
+            int64_t here = L.P - A.p0 < A.span ? L.P - A.p0 : A.span;  // list positions, at most
+            if (here < 1) here = 1;  // an empty set still sums to zero
+            // the tile: a walker's record is loaded once per tile, but every team should
+            // have several tiles
+            A.subs = want > 0 ? want : kSubPerTile;
+            if (want <= 0)
+                while (A.subs > 1 && A.W * ((here + kSnapsPerSub * A.subs - 1) / (kSnapsPerSub * A.subs)) <
+                                         (int64_t)8 * ctx->num_sms * teams)
+                    A.subs >>= 1;
+            A.ntile = (int)((here + kSnapsPerSub * A.subs - 1) / (kSnapsPerSub * A.subs));
+            // one block per SM (its shared memory and its 2 x 256 tensor-memory columns take
+            // the SM), fewer when there are fewer tiles than teams
+            const int64_t ntiles = A.W * (int64_t)A.ntile;
+            int64_t blocks = (int64_t)ctx->num_sms;
+            if (blocks > (ntiles + teams - 1) / teams) blocks = (ntiles + teams - 1) / teams;
+            A.counter = counter++;
+            qcs_log(3, "tc_pair_kernel: %lld blocks x %d teams, %zu bytes of shared memory, %d tensor-memory slots",
+                    (long long)blocks, teams, smem, A.tslots);
+            tc_pair_kernel<<<(unsigned)blocks, kTeamThreads * teams, smem, st>>>(A);
+            qcs_status r = qcs_check_launch(ctx, "tc_pair_kernel");
+            if (r != QCS_OK) return r;
+            F.partial = L.partial + w0 * L.nchunks + c;
+            r = qcs_launch_pfaffians(ctx, F, st);
+            if (r != QCS_OK) return r;
+        }
+    }
     qcs_prof_end(ctx, st);
-    return qcs_check_launch(ctx, "tc_pair_kernel");
+    return QCS_OK;
 }

@@ -112,3 +112,78 @@ def test_rank2_entry_update(bits_g, bits_v):
             continue  # beyond the bound 4 2^mb 2^59 that pivoting gives for |g| <= sqrt 2
         for acc, ex in ((re, ere), (im, eim)):
             assert abs(Fraction(value(acc, 3)) - Fraction(ex, 1 << 59)) <= 6
+
+
+# ---- balanced slices of the tensor-core congruence (csrc/qcs_ozaki.cuh)
+
+BIAS = 0x80808080808080
+
+
+def row_exp(row):
+    return max(((int(np.float64(abs(x)).view(np.int64)) + (1 << 46)) >> 52) - 1022 for x in row if x != 0.0)
+
+
+def fixed(x, e):
+    v = Fraction(float(x)) * Fraction(2) ** (55 - e)
+    u = int(abs(v) + Fraction(1, 2))
+    return -u if v < 0 else u
+
+
+def digits(u):
+    b = u + BIAS
+    assert 0 <= b < 1 << 56
+    return [((b >> (8 * (7 - i))) & 0xFF) - 128 for i in range(1, 8)]
+
+
+def combine(acc):
+    """The level sums through the magic FP32 addition, modulo 2^64."""
+    magics = [12582912.0] * 6 + [12582944.0]
+    x = [int(np.float32(np.float32(a) + np.float32(m)).view(np.uint32)) for a, m in zip(acc, magics)]
+    magic = 0x4B400000
+    off = magic * 0x0000040404040404 + (magic >> 6)
+    z = 4 * x[5] + (x[6] >> 6) + (x[4] << 10) + (x[3] << 18) + (x[2] << 26)
+    z += ((x[0] * 1024 + x[1] * 4) & 0xFFFFFFFF) << 32
+    return s64(z - off)
+
+
+def sliced_dot(a, b):
+    ea, eb = row_exp(a), row_exp(b)
+    da, db = [digits(fixed(x, ea)) for x in a], [digits(fixed(x, eb)) for x in b]
+    acc = []
+    for L in range(2, 9):
+        t = sum(da[k][i - 1] * db[k][L - i - 1] for i in range(1, 8) if 1 <= L - i <= 7 for k in range(len(a)))
+        assert abs(t) < 1 << 22  # what the FP32 accumulators and the magic addition hold exactly
+        acc.append(t)
+    z = combine(acc)
+    assert z == sum(acc[L - 2] << (8 * (7 - L) + 2) for L in range(2, 8)) + ((acc[6] + 32) >> 6)
+    return Fraction(z) * Fraction(2) ** (ea + eb - 56), ea, eb
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0**-30, 1.0 - 2.0**-53, 3.0])
+def test_balanced_slices_reach_an_fp64_product(scale):
+    """Digits reproduce the rounded entry, level sums stay below 2^22, and the dot product's
+    error is within 2^-50 of the row scales: K = 32 entries with 2^-56 rounding each side
+    (2 * 32 * 2^-56) and the dropped levels (at most 6 * 32 * 128^2 2^{-72+16} = 2^-34.4 2^{-16}
+    per scale product, halved by the digits' signs)."""
+    rng = np.random.default_rng(3)
+    for t in range(60):
+        a, b = rng.uniform(-1, 1, 32) * scale, rng.uniform(-1, 1, 32)
+        if t % 3 == 0:
+            a[rng.integers(32)] = scale  # an entry at the top of the scale
+        if t % 4 == 0:
+            b = np.where(np.arange(32) == t % 32, -1.0, 0.0)
+        e = row_exp(a)
+        for x in a:
+            u = fixed(x, e)
+            assert sum(d << (8 * (7 - i)) for i, d in enumerate(digits(u), 1)) == u
+        got, ea, eb = sliced_dot(a, b)
+        exact = sum(Fraction(float(x)) * Fraction(float(y)) for x, y in zip(a, b))
+        assert abs(got - exact) <= Fraction(2) ** (ea + eb - 47)
+
+
+def test_largest_digits_accumulate_exactly():
+    a = np.full(32, 1.0 - 2.0**-7 - 2.0**-20)
+    for b in (a, -a):
+        got, ea, eb = sliced_dot(a, b)
+        exact = sum(Fraction(float(x)) * Fraction(float(y)) for x, y in zip(a, b))
+        assert abs(got - exact) <= Fraction(2) ** (ea + eb - 47)
