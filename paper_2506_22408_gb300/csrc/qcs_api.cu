@@ -412,7 +412,6 @@ struct OverlapWork {
     cd *sum;                   // ... and their Pfaffian sums
     int64_t wblock;
     int span;
-    int *mode;                 // FP64 ALU path: per-walker form of the occupied rows (walker prep)
     int nchunks, nparts;
     int config, chunk;         // resolved kernel configuration, ALU snapshots per warp in a tile
     bool split, tc;
@@ -501,11 +500,10 @@ qcs_status overlap_common(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t 
     size_t b_part = align16(sizeof(cd) * (size_t)W * wk->nparts);
     size_t b_slab = split ? align16(qcs_split_walker_bytes(n, W)) : 0;
     size_t b_rec = tc ? align16(qcs_tc_walker_bytes(W)) : 0;
-    size_t b_mode = (split || tc) ? 0 : align16(sizeof(int) * (size_t)(W > 0 ? W : 1));
     const size_t batch = tc ? (size_t)wk->wblock * wk->span : 0;
     size_t b_pair = tc ? align16(batch * qcs_pf_rec_bytes(n, ne)) : 0, b_sum = align16(batch * sizeof(cd));
     size_t b_cnt = tc ? align16(sizeof(unsigned long long) * (size_t)qcs_tc_counters(W > 0 ? W : 1, wk->wblock, wk->nchunks)) : 0;
-    const size_t b_all = 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec + b_mode;
+    const size_t b_all = 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec;
     void *base = nullptr;
     qcs_status ws = qcs_workspace(ctx, b_all + b_cnt + b_sum + b_pair, &base, st);
     if (ws != QCS_OK) return ws;
@@ -519,11 +517,8 @@ qcs_status overlap_common(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t 
     wk->Mhi = split ? (float *)(pb + 16 + b_ut + b_pref + b_part) : nullptr;
     wk->Mlo = split ? (float *)(pb + 16 + b_ut + b_pref + b_part + b_slab) : nullptr;
     wk->walk_rec = tc ? (unsigned char *)(pb + 16 + b_ut + b_pref + b_part + 2 * b_slab) : nullptr;
-    // the reduced form of the occupied rows serves the FP64 ALU pair kernel; the tensor
-    // paths keep the orthonormal echelon form
-    wk->mode = (split || tc) ? nullptr : (int *)(pb + 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec);
     return qcs_launch_walker_prep(ctx, n, ne, W, (const cd *)d_walkers, wk->Ut, wk->pref, st, nullptr, nullptr,
-                                  true, wk->mode);
+                                  true);
 }
 
 }  // namespace
@@ -553,7 +548,6 @@ extern "C" qcs_status qcs_overlap(qcs_ctx *ctx, const qcs_snapshots *s, int ne, 
     L.nchunks = wk.nchunks;
     L.Ut = wk.Ut;
     L.pref = wk.pref;
-    L.mode = wk.mode;
     L.s = s;
     L.partial = wk.partial;
     L.per_pair = (cd *)d_per_pair;
@@ -595,7 +589,7 @@ extern "C" qcs_status qcs_overlap_batched(qcs_ctx *ctx, int nsys, const qcs_syst
     if (opts) o = *opts;
     if (o.precision != QCS_FP64) return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "batched calls are FP64");
     qcs_pair_launch Ls[QCS_MAX_SYSTEMS];
-    size_t off[QCS_MAX_SYSTEMS][4];
+    size_t off[QCS_MAX_SYSTEMS][3];
     size_t total = 16;  // the tile counter first
     const int wpb = qcs_pair_warps_per_block();
     for (int i = 0; i < nsys; ++i) {
@@ -637,8 +631,6 @@ extern "C" qcs_status qcs_overlap_batched(qcs_ctx *ctx, int nsys, const qcs_syst
         total += align16(sizeof(cd) * (size_t)y.W);
         off[i][2] = total;
         total += align16(sizeof(cd) * (size_t)y.W * L.nchunks * wpb);
-        off[i][3] = total;
-        total += align16(sizeof(int) * (size_t)(y.W > 0 ? y.W : 1));
     }
     void *base = nullptr;
     qcs_status r = qcs_workspace(ctx, total, &base, st);
@@ -648,10 +640,8 @@ extern "C" qcs_status qcs_overlap_batched(qcs_ctx *ctx, int nsys, const qcs_syst
         Ls[i].Ut = (cd *)(pb + off[i][0]);
         Ls[i].pref = (cd *)(pb + off[i][1]);
         Ls[i].partial = (cd *)(pb + off[i][2]);
-        int *mode = (int *)(pb + off[i][3]);
-        Ls[i].mode = mode;
         r = qcs_launch_walker_prep(ctx, Ls[i].n, Ls[i].ne, Ls[i].W, (const cd *)systems[i].d_walkers,
-                                   (cd *)Ls[i].Ut, (cd *)Ls[i].pref, st, nullptr, nullptr, true, mode);
+                                   (cd *)Ls[i].Ut, (cd *)Ls[i].pref, st, nullptr, nullptr, true);
         if (r != QCS_OK) return r;
     }
     r = qcs_launch_pairs_batched(ctx, nsys, Ls, (unsigned long long *)pb, st);
@@ -715,8 +705,7 @@ extern "C" qcs_status qcs_overlap_grad(qcs_ctx *ctx, const qcs_snapshots *s, int
     cd *Wrot = (cd *)(pb + b_ut + b_pref + b_u + b_r + b_part);
     // echelon-form walker rows (the congruence skips their zeros); U is the rotated unitary,
     // R the QR's triangular factor and Wrot the occupied columns' rotation for the epilogue
-    qcs_status r = qcs_launch_walker_prep(ctx, n, ne, W, (const cd *)d_walkers, Ut, pref, st, U, R, true, nullptr,
-                                          Wrot);
+    qcs_status r = qcs_launch_walker_prep(ctx, n, ne, W, (const cd *)d_walkers, Ut, pref, st, U, R, true, Wrot);
     if (r != QCS_OK) return r;
     r = qcs_hform_prepare_snapshots(ctx, const_cast<qcs_snapshots *>(s), st);
     if (r != QCS_OK) return r;

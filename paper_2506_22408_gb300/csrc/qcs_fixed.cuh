@@ -4,10 +4,11 @@
 // 64-bit integer multiply-add (IMAD.WIDE) per 4.1 (register-only probes).  A matrix whose
 // entries share one power-of-two scale needs no exponent per entry, so the eliminations
 // hold every entry as a 64-bit integer X worth X 2^-f, f common to the matrix.  A product
-// of two of them takes three IMAD.WIDE on their 31-bit limbs,
-//     X = h 2^31 + l,  |l| <= 2^30:   X Y = hh 2^62 + (h l' + l h') 2^31 + l l',
-// the last term (below 2^-60 of the factors' scale, either sign) dropped: 12 to 13 clocks
-// against 76.  The largest entry of a matrix is kept at 54 to 60 bits, so an update rounds
+// of two of them takes three IMAD.WIDE on two limbs,
+//     X = h 2^S + l,  |l| <= 2^{S-1}:   X Y = hh 2^2S + (h l' + l h') 2^S + l l',
+// the last term dropped: 12 to 13 clocks against 76.  With S = 30 and entries of 58 to 60
+// bits it is below 2^-58 of the factors' scale, of either sign; longer sums of entries of 57
+// bits take S = 29 (2^-60), as S = 31 lost three bits of the congruence against FP64.  The largest entry of a matrix is kept at 54 to 60 bits, so an update rounds
 // at 2^-54 to 2^-60 of the matrix's largest entry where FP64 rounds at 2^-53 of each
 // operand: the elimination with pivoting is as accurate as that matrix norm allows either
 // way, and the errors against 64-bit references are those of the FP64 code it replaced or
@@ -29,12 +30,12 @@
 typedef longlong2 fx2;  // complex fixed point, worth (x + i y) 2^-f
 
 // Bits of the largest entry: after a (re)normalisation; before an update at most (limbs of
-// 31 bits) and at least.  |g| <= sqrt 2 2^eu and |v| <= sqrt 2 2^mb bound an update by
+// 32 bits) and at least.  |g| <= sqrt 2 2^eu and |v| <= sqrt 2 2^mb bound an update by
 // 4 2^{mb+eu}: its result is scaled down by q bits when mb + eu exceeds kFxRoom, so that
 // it stays below 2^62.4; the scale of the factors themselves is kept, which matters when
 // a pivot is small (scaling the matrix down before the update would cost eu bits of g v).
 constexpr int kFxTop = 58;
-constexpr int kFxMax = 61;
+constexpr int kFxMax = 60;
 constexpr int kFxLow = 54;
 constexpr int kFxRoom = 60;
 
@@ -83,12 +84,13 @@ inline void fx_make_plan(const qcs_node_plan &p, FxPlan &q) {
     }
 }
 
-struct fxl {  // a fixed-point number as limbs h 2^31 + l
+struct fxl {  // a fixed-point number as limbs h 2^S + l
     int h, l;
 };
+template <int S = 30>
 __device__ __forceinline__ fxl fx_split(long long X) {
-    const unsigned long long y = (unsigned long long)X + (1ull << 30);
-    return fxl{(int)__funnelshift_l((unsigned)y, (unsigned)(y >> 32), 1), (int)((unsigned)X << 1) >> 1};
+    const unsigned long long y = (unsigned long long)X + (1ull << (S - 1));
+    return fxl{(int)__funnelshift_l((unsigned)y, (unsigned)(y >> 32), 32 - S), (int)((unsigned)X << (32 - S)) >> (32 - S)};
 }
 __device__ __forceinline__ fxl fx_neg(fxl a) { return fxl{-a.h, -a.l}; }
 
@@ -105,7 +107,7 @@ __device__ __forceinline__ long long mad_wide(int a, int b, long long s) {
     return r;
 }
 
-struct fxacc {  // hh 2^62 + cr 2^31
+struct fxacc {  // hh 2^2S + cr 2^S
     long long hh, cr;
 };
 // The sum starts at half a unit of its fx_value: a mean over many pairs must not collect the
@@ -113,14 +115,20 @@ struct fxacc {  // hh 2^62 + cr 2^31
 __device__ __forceinline__ fxacc fx_mul(fxl a, fxl b, long long half) {
     return fxacc{mul_wide(a.h, b.h), mad_wide(a.l, b.h, mad_wide(a.h, b.l, half))};
 }
-__device__ __forceinline__ long long fx_half(int up) { return 1ll << (30 - up); }
+template <int S = 30>
+__device__ __forceinline__ long long fx_half(int dn) {
+    return 1ll << (dn - S - 1);
+}
 __device__ __forceinline__ void fx_mac(fxacc &s, fxl a, fxl b) {
     s.hh = mad_wide(a.h, b.h, s.hh);
     s.cr = mad_wide(a.h, b.l, s.cr);
     s.cr = mad_wide(a.l, b.h, s.cr);
 }
-// (hh 2^62 + cr 2^31) 2^{-62 + up}, 0 <= up < 31
-__device__ __forceinline__ long long fx_value(const fxacc &s, int up) { return (s.hh << up) + (s.cr >> (31 - up)); }
+// (hh 2^2S + cr 2^S) 2^-dn, S < dn <= 2S
+template <int S = 30>
+__device__ __forceinline__ long long fx_value(const fxacc &s, int dn) {
+    return (s.hh << (2 * S - dn)) + (s.cr >> (dn - S));
+}
 
 __device__ __forceinline__ int4 fx_pack(fxl re, fxl im) { return make_int4(re.h, re.l, im.h, im.l); }
 
@@ -184,14 +192,14 @@ static __device__ __noinline__ double fx_f64(long long X, int E) {
     return ok ? v : qcs_oz::fixed_to_f64_exact(X, E);
 }
 
-// 1 / (q.x + i q.y) 2^119 as packed limbs, for max(|q.x|, |q.y|) in [2^60, 2^61): conj(q) / |q|^2,
-// the reciprocal R = 2^118 / (|q|^2 2^-62) by one third-order step from the FP32 seed R0
+// 2^118 / (q.x + i q.y) as packed limbs, for max(|q.x|, |q.y|) in [2^59, 2^60): conj(q) / |q|^2,
+// the reciprocal R = 2^118 / (|q|^2 2^-60) by one third-order step from the FP32 seed R0
 // (relative error e < 2^-22: R = R0 (1 + e + e^2), e^3 < 2^-66) in integers.
 __device__ __forceinline__ int4 fx_inverse(fx2 q) {
     const fxl a = fx_split(q.x), b = fx_split(q.y);
     fxacc s = fx_mul(a, a, 0);
     fx_mac(s, b, b);
-    const long long D = s.hh + (s.cr >> 31);  // |q|^2 2^-62 in [2^58, 2^61]
+    const long long D = s.hh + (s.cr >> 30);  // |q|^2 2^-60 in [2^58, 2^61)
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((float)(int)(D >> 31)));
     const int R0 = (int)(y * 18014398509481984.0f);  // 2^54 y in [2^24, 2^27]
@@ -202,17 +210,17 @@ __device__ __forceinline__ int4 fx_inverse(fx2 q) {
     const long long R = ((long long)R0 << 33) + (mul_wide(R0, eh) >> 20) +
                         (long long)(__umulhi((unsigned)R0, (unsigned)e) >> 20) + (mul_wide(R0, e2) >> 41);
     const fxl r = fx_split(R);
-    const fxacc u = fx_mul(a, r, fx_half(1)), v = fx_mul(b, r, fx_half(1));
-    return fx_pack(fx_split(fx_value(u, 1)), fx_neg(fx_split(fx_value(v, 1))));
+    const fxacc u = fx_mul(a, r, fx_half(60)), v = fx_mul(b, r, fx_half(60));
+    return fx_pack(fx_split(fx_value(u, 60)), fx_neg(fx_split(fx_value(v, 60))));
 }
 
-// z I 2^-60 for I = 2^119 / q as limbs: 2^59 z / q, as packed limbs.
+// z I 2^-59 for I = 2^118 / q as limbs: 2^59 z / q, as packed limbs.
 __device__ __forceinline__ int4 fx_times_inverse(fx2 z, fxl ir, fxl ii) {
     const fxl a = fx_split(z.x), b = fx_split(z.y);
-    fxacc re = fx_mul(a, ir, fx_half(2)), im = fx_mul(a, ii, fx_half(2));
+    fxacc re = fx_mul(a, ir, fx_half(59)), im = fx_mul(a, ii, fx_half(59));
     fx_mac(re, fx_neg(b), ii);
     fx_mac(im, b, ir);
-    return fx_pack(fx_split(fx_value(re, 2)), fx_split(fx_value(im, 2)));
+    return fx_pack(fx_split(fx_value(re, 59)), fx_split(fx_value(im, 59)));
 }
 
 // A complex number (x + i y) 2^e, the larger part of 60 bits (61 at most) unless it is zero.
@@ -227,10 +235,10 @@ __device__ __forceinline__ fxp fx_norm(fx2 a, int e) {
 }
 __device__ __forceinline__ fxp fx_prod(fxp a, fxp b) {
     const fxl ar = fx_split(a.x), ai = fx_split(a.y), br = fx_split(b.x), bi = fx_split(b.y);
-    fxacc re = fx_mul(ar, br, fx_half(0)), im = fx_mul(ar, bi, fx_half(0));
+    fxacc re = fx_mul(ar, br, fx_half(60)), im = fx_mul(ar, bi, fx_half(60));
     fx_mac(re, fx_neg(ai), bi);
     fx_mac(im, ai, br);
-    return fx_norm(make_longlong2(fx_value(re, 0), fx_value(im, 0)), a.e + b.e + 62);
+    return fx_norm(make_longlong2(fx_value(re, 60), fx_value(im, 60)), a.e + b.e + 60);
 }
 __device__ __forceinline__ fxp fx_shfl_xor(const fxp &a, int o) {
     return fxp{__shfl_xor_sync(QCS_FULL, a.x, o), __shfl_xor_sync(QCS_FULL, a.y, o), __shfl_xor_sync(QCS_FULL, a.e, o)};
@@ -250,8 +258,8 @@ __device__ __forceinline__ unsigned fx_rank2(int t0, int nb, int T, int rv, fx2 
                                              const FxGauss *__restrict__ GV, int ldv, int eu, int q,
                                              const uint16_t *__restrict__ tab) {
     const int Tr = tri_count(rv), total = nb * Tr;
-    const int up = 3 + eu - q;
-    const long long half = fx_half(up), qhalf = (1ll << q) >> 1;
+    const int dn = 59 - eu + q;
+    const long long half = fx_half(dn), qhalf = (1ll << q) >> 1;
     unsigned top = 0u;
     int u = t0;
 #pragma unroll 1
@@ -285,8 +293,8 @@ __device__ __forceinline__ unsigned fx_rank2(int t0, int nb, int T, int rv, fx2 
             x.x = (x.x + qhalf) >> q;
             x.y = (x.y + qhalf) >> q;
         }
-        x.x += fx_value(re, up);
-        x.y += fx_value(im, up);
+        x.x += fx_value(re, dn);
+        x.y += fx_value(im, dn);
         top |= fx_top(x);
         Ns[u] = x;
         u += NT;
@@ -561,8 +569,8 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
                 wk.pe[rec] = fc;
             }
             if (r == 2) break;  // no empty modes: the last pivot closes the Pfaffian
-            const int sn = zero ? 0 : 61 - fx_bits(piv);
-            int4 inv = fx_inverse(zero ? make_longlong2(1ll << 60, 0ll) : make_longlong2(piv.x << sn, piv.y << sn));
+            const int sn = zero ? 0 : 60 - fx_bits(piv);
+            int4 inv = fx_inverse(zero ? make_longlong2(1ll << 59, 0ll) : make_longlong2(piv.x << sn, piv.y << sn));
             if (zero) inv = make_int4(0, 0, 0, 0);  // a zero row: g = 0, and the product is zero
             if (live) {
                 // g_i = A_{i,k} / A_{p,k} scaled by 2^{59-eu}, v_i = A_{i,p}, over the other r - 2
@@ -618,11 +626,11 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
             const fx2 y = fx_shift(Nv[t == 0 ? 5 : t == 1 ? 4 : 2], sh);
             x = fx_neg_if(x, t == 1);
             const fxl xr = fx_split(x.x), xi = fx_split(x.y), yr = fx_split(y.x), yi = fx_split(y.y);
-            fxacc re = fx_mul(xr, yr, fx_half(5)), im = fx_mul(xr, yi, fx_half(5));
+            fxacc re = fx_mul(xr, yr, fx_half(57)), im = fx_mul(xr, yi, fx_half(57));
             fx_mac(re, fx_neg(xi), yi);
             fx_mac(im, xi, yr);
             // |re|, |im| <= 2 2^{116} each: kept to 2^{-58} of that
-            const long long qx = fx_value(re, 5), qy = fx_value(im, 5);
+            const long long qx = fx_value(re, 57), qy = fx_value(im, 57);
             const long long q1 = __shfl_down_sync(QCS_FULL, qx, 1), q2 = __shfl_down_sync(QCS_FULL, qx, 2);
             const long long p1 = __shfl_down_sync(QCS_FULL, qy, 1), p2 = __shfl_down_sync(QCS_FULL, qy, 2);
             if (live && sl == 0) {

@@ -2,27 +2,24 @@
 //
 // For a pair (walker w, snapshot p) the estimator of Sec. "Classical shadows
 // and the evaluation of overlaps" needs the coefficients of
-// pf(A(z)), A(z) = C_0^(s) + z B^(s)  (Eqs. a_mat, b_mat).  The kernel forms:
+// pf(A(z)), A(z) = C_0^(s) + z B^(s)  (Eqs. a_mat, b_mat).  The kernel forms, all in fixed
+// point on the integer pipe (qcs_fixed.cuh, qcs_fxcong.cuh: the FP64 pipe, one 32-lane FMA
+// per 76 clocks and scheduler, bound it before):
 //
 //  1. T = Ut Qt^T (n x 2n complex): Ut holds the walker's orbitals (rows of
 //     U^T, occupied rows / sqrt2), Qt the snapshot's complexified sign-folded
 //     rows.  Row j of T is the selected row of W^* M_phi Q'^T for an occupied
 //     mode j; for an empty mode the two selected real rows are (Re T_j, -Im T_j).
 //     The walker prep leaves the orbitals in echelon form, so T skips the exact
-//     zeros of Ut; at n = 16 each lane holds one snapshot row in registers and
-//     takes three real products per complex multiply-add (build_T_reg).
+//     zeros of Ut.  Signed permutations gather T from Ut.
 //  2. B^(s)_ab = sum_k X_a,2k X_b,2k+1 - X_a,2k+1 X_b,2k  (X = selected rows),
-//     i.e. X J X^T with J the canonical skew form (C_b was folded into Qt).
-//     Computed as three classes (complex x complex, complex x real, real x real)
-//     so that every FP64 instruction runs with all 32 lanes busy.
+//     i.e. X J X^T with J the canonical skew form (C_b was folded into Qt).  Above 16
+//     modes K = Ut [H1 | G2] takes the place of T and B^(s) follows from K by n-term sums.
 //  3. pf(B + w_k D) at the node plan's evaluation points w_k (a Gauss rule on the
 //     unit circle by default, roots of unity on request), D = C_0^(s): the node
 //     matrices differ only in their empty x empty block, so the occupied block is
 //     eliminated once (pivots inside that block) and each node's 2d x 2d complement
-//     is eliminated by Parlett-Reid with partial pivoting, the nodes in lockstep;
-//     up to 16 modes in 64-bit fixed point on the integer pipe (qcs_fixed.cuh: the
-//     n = 12, 201 x 3001 per-pair case went from 29.5 to 23.5 ms), above in FP64 by
-//     two warps (qcs_group.cuh).
+//     is eliminated by Parlett-Reid with partial pivoting, the nodes in lockstep.
 //  4. S_p = sum_k gamma_k pf_k, where gamma_k folds the node plan's weights, the
 //     inverse-channel weights C(2n,2x)/C(n,x) and the palindromic symmetry
 //     c_{n-x} = c_x of parity +1 snapshots (parity -1 snapshots are exactly zero
@@ -33,29 +30,21 @@
 // snapshot of the tile in turn and writes one partial sum per warp slot, reduced
 // in a fixed order afterwards, so the result does not depend on scheduling.
 #include "qcs_internal.h"
-#include "qcs_fixed.cuh"
-#include "qcs_group.cuh"
+#include "qcs_fxcong.cuh"
 
 namespace {
 
 
 struct PairArgs {
-    int n, ne, m, d, nev, NB, all, chunk, nchunks;
-    int reg;          // n = 16: snapshot rows in registers, T by three real products (build_T_reg)
-    int grp;          // n > 16: two warps share a pair (64-thread groups, qcs_group.cuh)
-    int t3;           // n < 16: T by three real products from staged rows and their sums
-    int vm;           // entries per Gauss-vector buffer (the full matrix or NB node complements)
-    int off_kh, off_ph, off_scr, gz;  // group path: pivot history, scratch, S0 offset (entries) in Ns
-    int off_pvg;      // group path: the node products' records
-    int off_qs;       // re + im of the staged snapshot rows (warp and group paths)
+    int n, ne, m, NB, all, chunk, nchunks;
+    int grp;          // n > 16: two warps share a pair
     int64_t W, P;
-    int warp_bytes;   // shared bytes per warp
+    int team_bytes;   // shared bytes per team (one warp, or two)
     int tab_bytes;    // shared bytes of the pair table (per block)
     int ut_bytes;     // shared bytes of the walker rows Ut (per block)
-    int off_T, off_B, off_U, off_V, off_pf, off_inv, off_int, off_act, off_pv;  // byte offsets in a warp region
+    int off_T, off_U, off_pv, off_scr, npv;  // byte offsets in a team's region (staged rows, then B^(s), at 0)
     const cd *Ut;
     const cd *pref;
-    const int *wmode;  // per walker: occupied rows in reduced form (register path), or null
     const cd *Qt;
     const cd *Qh;        // rows [H1^T; G2^T] of the dense snapshots (null: T and B from Qt)
     const uint8_t *gth;  // gather codes of signed-permutation snapshots (or null)
@@ -64,32 +53,36 @@ struct PairArgs {
     cd *partial;
     cd *per_pair;
     unsigned *status;
-    cd wnode[QCS_MAX_NODES];
-    cd gamma[QCS_MAX_NODES];
-    FxPlan plan;  // the same in fixed point
+    FxPlan plan;
 };
 
-// One tile of system A: walker w = tile / nchunks, the tile's snapshots spread
-// over the block's warps; each warp writes one partial sum.  Every thread of the
-// block calls this (it contains block barriers around the shared walker rows).
-// GRP: the launch holds a system on the two-warp group path (n > 16); without one
-// the group code is left out of the kernel and its registers.
-template <bool GRP>
-__device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned char *wbase, size_t wstride, cd *Uts,
+// What a team's warps exchange.
+struct PairScratch {
+    unsigned red[4];
+    cd part;
+    int8_t rs[2 * QCS_MAX_N];  // row scales of the pair's snapshot
+};
+
+// One tile of system A: walker w = tile / nchunks, the tile's snapshots spread over the
+// block's teams of NW warps; each team writes one partial sum, in its first warp's slot (zero
+// in the second's).  Every thread of the block calls this (it contains block barriers
+// around the shared walker rows).
+template <int NW>
+__device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned char *base, int4 *Us,
                          const uint16_t *tab, int warp, int wpb, int lane) {
     const int n = A.n, n2 = 2 * n;
-    cd *Rg = reinterpret_cast<cd *>(wbase);
-    cd *Qs = Rg;  // staged snapshot rows (shared-memory path only)
-    cd *Ts = reinterpret_cast<cd *>(wbase + A.off_T);
-    fx2 *Xs = reinterpret_cast<fx2 *>(wbase);  // B^(s) in fixed point, once T is consumed
-    double *Uss = reinterpret_cast<double *>(Uts + n * ld_ut(n));  // re + im of Ut
-    cd *Bs = reinterpret_cast<cd *>(wbase + A.off_B);
-    const FxWarp tm = {lane, lane, 0, 0, nullptr};
-    const int npv = pv_records(A.vm, A.NB);
-    fx2 *pv = reinterpret_cast<fx2 *>(wbase + A.off_pv);
-    const FxWork wk = {reinterpret_cast<FxGauss *>(wbase + A.off_U), pv,
-                       reinterpret_cast<int *>(pv + npv + A.ne / 2), npv};
-    const int span = A.chunk * wpb;  // snapshots per tile; warp w takes every wpb-th
+    const int team = warp / NW, wid = warp % NW, teams = wpb / NW;
+    unsigned char *tb = base + (size_t)team * A.team_bytes;
+    int4 *Qs = reinterpret_cast<int4 *>(tb);            // half of the snapshot's rows
+    fx2 *Xs = reinterpret_cast<fx2 *>(tb);              // B^(s), once T is formed
+    int4 *Ts = reinterpret_cast<int4 *>(tb + A.off_T);
+    fx2 *Ns = reinterpret_cast<fx2 *>(tb + A.off_T);    // node matrices, once B^(s) is formed
+    fx2 *pv = reinterpret_cast<fx2 *>(tb + A.off_pv);
+    PairScratch *scr = reinterpret_cast<PairScratch *>(tb + A.off_scr);
+    const FxWork wk = {reinterpret_cast<FxGauss *>(tb + A.off_U), pv, reinterpret_cast<int *>(pv + A.npv + A.ne / 2),
+                       A.npv};
+    const FxTeam<NW> tm = {32 * wid + lane, lane, wid, 1 + team, scr->red};
+    const int span = A.chunk * wpb;  // snapshots per tile; team g takes every teams-th
     // chunk-major tile order: consecutive tiles share one snapshot chunk and run over
     // the walkers (whose rows all fit in L2), so each snapshot is fetched from HBM once
     const int ch = (int)(tile / A.W);
@@ -99,152 +92,82 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
     // the tile from the queue and the parity +1 count address this system's buffers
     // (block-uniform: every thread leaves before the first barrier)
     if (!QCS_IN_BOUNDS(tile >= 0 && ch < A.nchunks && L >= 0 && L <= A.P, A.status)) return;
-    __syncthreads();  // previous tile's readers of Uts are done
+    __syncthreads();  // previous tile's readers of Us are done
+    int fU = 0;
     if (p0 < L) {
         const cd *Utw = A.Ut + w * n * n;
-        const int lu = ld_ut(n);
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            const cd u = Utw[e];
-            Uts[(e / n) * lu + (e % n)] = u;
-            Uss[(e / n) * lu + (e % n)] = u.x + u.y;
-        }
+        fU = fx_fraction(fx_max_key(Utw, n * n, lane), 57);
+        fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, threadIdx.x, blockDim.x);
     }
     __syncthreads();
     cd acc = cmk(0.0, 0.0);
-    const bool redw = A.wmode != nullptr && A.wmode[w] != 0;
-    if (GRP && A.grp) {
-        // two warps per pair: group g = warps 2g, 2g+1 with the two warp regions as its
-        // workspace; group g takes every (wpb/2)-th snapshot of the tile
-        const int g = warp >> 1, t = ((warp & 1) << 5) + lane, bar = 1 + g, ng = wpb >> 1;
-        unsigned char *gb = wbase - (size_t)(warp & 1) * wstride;
-        cd *gQs = reinterpret_cast<cd *>(gb);
-        cd *gTs = reinterpret_cast<cd *>(gb + A.off_T);
-        double *gqs = reinterpret_cast<double *>(gb + A.off_qs);  // re + im of the staged rows
-        cd *gNs = reinterpret_cast<cd *>(gb);
-        cd *gSc = gNs + A.gz;
-        cd *gBs = reinterpret_cast<cd *>(gb + A.off_B);
-        cd *gUv = reinterpret_cast<cd *>(gb + A.off_U);
-        cd *gVv = reinterpret_cast<cd *>(gb + A.off_V);
-        cd *gpf = reinterpret_cast<cd *>(gb + A.off_pf);
-        cd *ginvh = reinterpret_cast<cd *>(gb + A.off_inv);
-        uint8_t *gacth = gb + A.off_act;
-        uint8_t *gkh = gb + A.off_kh;
-        uint8_t *gph = gb + A.off_ph;
-        SharedScratch *gscr = reinterpret_cast<SharedScratch *>(gb + A.off_scr);
-        cd *gpv = reinterpret_cast<cd *>(gb + A.off_pvg);
-        const int m = A.m, ne = A.ne, d2 = A.m - A.ne, Tn = tri_count(d2);
-        if (p0 < L) {
-            const cd prefw = A.pref[w];
-            for (int64_t pq = p0 + g; pq < p1; pq += ng) {
-                const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
-                if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // group-uniform
-                const uint8_t *gq = A.gth ? A.gth + q * n2 : nullptr;
-                group_sync(bar);
-                const bool gat = gq && gq[0] != 0xFF;
-                if (gat) {
-                    build_T_gather(n, Uts, gq, gTs, t, kGroup);
-                } else {
-                    // T (or K = Ut [H1 | G2] from the rows Qh) by column halves: half of the
-                    // snapshot's rows staged at a time
-                    const cd *Qr = (A.Qh ? A.Qh : A.Qt) + q * n2 * n;
-                    for (int h = 0; h < 2; ++h) {
-                        load_Qt_rows_sums(n, Qr + (int64_t)h * n * n, gQs, gqs, t, kGroup);
-                        group_sync(bar);
-                        build_T_half3(n, ne, redw, Uts, Uss, gQs, gqs, gTs, h * n, t, kGroup);
-                        group_sync(bar);
-                    }
-                }
-                group_sync(bar);
-                if (!gat && A.Qh) {
-                    // B from K: re + im of K1 and re - im of K2 into the staging region (free now)
-                    double *gks = reinterpret_cast<double *>(gQs);
-                    for (int e = t; e < n * n2; e += kGroup) {
-                        const int j = e / n2, c = e - j * n2;
-                        const cd k = gTs[j * ld_t(n) + c];
-                        gks[e] = c < n ? k.x + k.y : k.x - k.y;
-                    }
-                    group_sync(bar);
-                    build_B_from_K(n, ne, redw, Uts, Uss, gTs, gks, gBs, tab, t, kGroup);
-                } else {
-                    build_B(n, ne, gTs, gBs, tab, t, kGroup);
-                }
-                group_sync(bar);
-                cd S = cmk(0.0, 0.0);
-                if (shared_factor(m, ne, gBs, gNs, gUv, gVv, ginvh, gacth, gkh, gph, gscr, tab, t, bar)) {
-                    const cd pf0 = gscr->pf0;
-                    for (int e = t; e < Tn; e += kGroup) {
-                        int a, b;
-                        pair_of(tab, e, a, b);
-                        gSc[e] = gNs[tri_index(ne + a, ne + b)];
-                    }
-                    group_sync(bar);
-                    for (int k0 = 0; k0 < A.nev; k0 += A.NB) {
-                        const int nb = A.nev - k0 < A.NB ? A.nev - k0 : A.NB;
-                        group_node_pfaffians(d2, 0, A.wnode + k0, A.gamma + k0, nb, gSc, gNs, gUv, gVv, gpf, gacth,
-                                             gacth + A.vm, gpv, tab, t, bar);
-                        if (t == 0)
-                            for (int v = 0; v < nb; ++v) S = cadd(S, gpf[v]);  // gpf[v] carries gamma
-                        group_sync(bar);
-                    }
-                    S = cmul(S, pf0);
-                } else {  // the rare full eliminations: one node matrix per round
-                    for (int k0 = 0; k0 < A.nev; ++k0) {
-                        group_node_pfaffians(m, ne, A.wnode + k0, A.gamma + k0, 1, gBs, gNs, gUv, gVv, gpf, gacth,
-                                             gacth + A.vm, gpv, tab, t, bar);
-                        if (t == 0) S = cadd(S, gpf[0]);
-                        group_sync(bar);
-                    }
-                }
-                if (t == 0) {
-                    if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
-                    acc = cadd(acc, S);
-                    if (A.per_pair) A.per_pair[w * A.P + q] = cmul(prefw, S);
-                }
-            }
-        }
-        // one partial per warp slot: the group's sum in its first warp's slot, zero in the second
-        if (lane == 0) A.partial[(w * A.nchunks + ch) * wpb + warp] = (warp & 1) ? cmk(0.0, 0.0) : acc;
-        return;
-    }
     if (p0 < L) {
-        const cd prefw = A.pref[w];
-        for (int64_t pq = p0 + warp; pq < p1; pq += wpb) {
+        for (int64_t pq = p0 + team; pq < p1; pq += teams) {
             const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
-            if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // warp-uniform
+            if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // team-uniform
             const uint8_t *gq = A.gth ? A.gth + q * n2 : nullptr;
-            const bool gat = gq && gq[0] != 0xFF;
-            const cd *Qr = A.Qt + q * n2 * n;
-            __syncwarp();
+            const bool gat = gq && gq[0] != 0xFF, fromK = !gat && A.Qh;
+            cd S = cmk(__longlong_as_double(0x7ff8000000000000ll), 0.0);
+            bool finite = true;
+            int fT = fU, par = 0;
+            tm.sync();  // the previous pair is done with the team's region
             if (gat) {
-                build_T_gather(n, Uts, gq, Ts, lane);  // signed permutation: no products
-            } else if (A.reg) {
-                build_T_reg<16>(A.ne, Uts, Uss, Qr, Ts, lane, redw);
-            } else if (A.t3) {
-                // staged rows and their re + im sums; T by three real products per
-                // complex multiply-add, skipping the zeros of the echelon or reduced form
-                double *qs = reinterpret_cast<double *>(wbase + A.off_qs);
-                load_Qt_rows_sums(n, Qr, Qs, qs, lane, 32);
-                load_Qt_rows_sums(n, Qr + n * n, Qs + n * ld_qt(n), qs + n * n, lane, 32);
-                __syncwarp();
-                build_T_half3(n, A.ne, redw, Uts, Uss, Qs, qs, Ts, 0, lane, 32);
-                build_T_half3(n, A.ne, redw, Uts, Uss, Qs + n * ld_qt(n), qs + n * n, Ts, n, lane, 32);
-            } else {  // n > 16 configured to one warp per pair: no room for the sums
-                load_Qt(n, Qr, Qs, lane);
-                __syncwarp();
-                build_T_echelon(n, A.ne, Uts, Qs, Ts, lane);  // walker rows in echelon form
+                fx_gather_T(n, Us, gq, Ts, tm.t, tm.NT);  // signed permutation: no products
+            } else {
+                // T (or K) by column halves: half of the snapshot's rows staged at a time
+                const cd *Qr = (A.Qh ? A.Qh : A.Qt) + q * n2 * n;
+                const unsigned key = fromK ? fx_max_key(Qr, n2 * n, lane) : fx_balance_rows(n, Qr, scr->rs, lane);
+                finite = key < 0x7ff00000u;
+                const int fQ = fx_fraction(key, 57);
+                unsigned top = 0u;
+                tm.sync();
+                for (int h = 0; h < 2 && finite; ++h) {
+                    fx_stage_rows(n, n * n, Qr + (int64_t)h * n * n, fQ, fromK ? nullptr : scr->rs + h * n, Qs, tm.t,
+                                  tm.NT);
+                    tm.sync();
+                    top |= fx_build_T(n, A.ne, Us, Qs, reinterpret_cast<fx2 *>(Ts), h * n, tm.t, tm.NT);
+                    tm.sync();
+                }
+                if (finite) {
+                    top = tm.or_put(top, par);
+                    tm.sync();
+                    const int b = fx_top_bits(tm.or_get(top, par));
+                    par ^= 1;
+                    fT = fU + fQ - 58 + 56 - b;
+                    fx_T_limbs(n, Ts, b, tm.t, tm.NT);
+                }
             }
-            __syncwarp();
-            build_B(A.n, A.ne, Ts, Bs, tab, lane);
-            __syncwarp();
-            const cd S = fx_pair_sum(tm, A.m, A.ne, A.NB, A.plan, wk, Bs, Xs, tab);
-            if (lane == 0) {
+            tm.sync();
+            if (finite) {
+                bool shared = true, ok;
+#pragma unroll 1
+                do {  // rarely a second time: B^(s) again, every node matrix in full
+                    unsigned top = fromK ? fx_build_B_from_K(n, A.ne, Us, Ts, Xs, tab, tm.t, tm.NT)
+                                         : fx_build_B(n, A.ne, Ts, Xs, tab, tm.t, tm.NT);
+                    top = tm.or_put(top, par);
+                    tm.sync();
+                    const int mb = fx_top_bits(tm.or_get(top, par));
+                    par ^= 1;
+                    tm.sync();  // the words of the reduction are free again
+                    S = fx_pair_eliminate(tm, A.m, A.ne, shared, A.NB, A.plan, wk, Xs, Ns,
+                                          fromK ? fT + fU - 58 : 2 * fT - 58, mb, tab, ok);
+                    shared = false;
+                    tm.sync();
+                } while (!ok);
+            }
+            if (NW > 1) {  // the other warp's nodes
+                if (wid == 1 && lane == 0) scr->part = finite ? S : cmk(0.0, 0.0);
+                tm.sync();
+                if (wid == 0 && lane == 0) S = cadd(S, scr->part);
+            }
+            if (tm.t == 0) {
                 if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
                 acc = cadd(acc, S);
-                if (A.per_pair) A.per_pair[w * A.P + q] = cmul(prefw, S);
+                if (A.per_pair) A.per_pair[w * A.P + q] = cmul(A.pref[w], S);
             }
         }
     }
-    if (lane == 0) A.partial[(w * A.nchunks + ch) * wpb + warp] = acc;
+    if (lane == 0) A.partial[(w * A.nchunks + ch) * wpb + warp] = wid == 0 ? acc : cmk(0.0, 0.0);
 }
 
 // One or several systems (different n, ne, walkers, snapshots) in one persistent
@@ -254,29 +177,31 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
 // fill the tail.
 struct BatchArgs {
     int nsys;
-    int tab_bytes, ut_bytes, warp_bytes;  // maxima over the systems
+    int tab_bytes, ut_bytes, work_bytes;  // maxima over the systems
     int max_m;
     int64_t tile_end[QCS_MAX_SYSTEMS];    // cumulative tile counts in queue order
     unsigned long long *counter;
     PairArgs sys[QCS_MAX_SYSTEMS];         // in queue order
 };
 
-template <bool GRP>
-__global__ void __launch_bounds__(128, GRP ? 2 : 3) pair_overlap_kernel(const __grid_constant__ BatchArgs B) {
+// NWS: bit 0 set when a system of the launch runs one warp per pair, bit 1 when one runs two;
+// a kind that does not occur is left out of the kernel (its instructions and registers).
+template <int NWS>
+__global__ void __launch_bounds__(128, 4) pair_overlap_kernel(const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long next_tile;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
-    // the pair table, the walker rows and the warps' workspaces fit the launch's shared memory
+    // the pair table, the walker rows and the teams' workspaces fit the launch's shared memory
     if (!QCS_IN_BOUNDS(tri_count(B.max_m) * (int)sizeof(uint16_t) <= B.tab_bytes &&
-                           (size_t)B.tab_bytes + B.ut_bytes + (size_t)wpb * B.warp_bytes <= dyn_smem_bytes(),
+                           (size_t)B.tab_bytes + B.ut_bytes + B.work_bytes <= dyn_smem_bytes(),
                        B.sys[0].status))
         return;
     uint16_t *tab = reinterpret_cast<uint16_t *>(smem_raw);
     build_pair_table(tab, tri_count(B.max_m));
-    cd *Uts = reinterpret_cast<cd *>(smem_raw + B.tab_bytes);
-    unsigned char *wbase = smem_raw + B.tab_bytes + B.ut_bytes + (size_t)warp * B.warp_bytes;
+    int4 *Us = reinterpret_cast<int4 *>(smem_raw + B.tab_bytes);
+    unsigned char *base = smem_raw + B.tab_bytes + B.ut_bytes;
     const int64_t total = B.tile_end[B.nsys - 1];
     for (;;) {
         __syncthreads();  // every thread has read the previous tile index
@@ -289,7 +214,8 @@ __global__ void __launch_bounds__(128, GRP ? 2 : 3) pair_overlap_kernel(const __
         const int64_t local = t - (s > 0 ? B.tile_end[s - 1] : 0);
         const PairArgs &A = B.sys[s];
         const int64_t L = A.all ? A.P : (int64_t)(*A.d_count);
-        run_tile<GRP>(A, local, L, wbase, B.warp_bytes, Uts, tab, warp, wpb, lane);
+        if ((NWS & 2) && (!(NWS & 1) || A.grp)) run_tile<2>(A, local, L, base, Us, tab, warp, wpb, lane);
+        else run_tile<1>(A, local, L, base, Us, tab, warp, wpb, lane);
     }
 }
 
@@ -311,74 +237,23 @@ __global__ void reduce_kernel(int64_t W, int64_t P, int nparts, const cd *__rest
 
 namespace {
 
-// Per-warp shared layout for nb node matrices; returns bytes per warp.  The first
-// region holds the staged snapshot rows and T (T alone on the register path), then
-// B^(s) in fixed point, whose occupied block is eliminated there; the second B^(s) in
-// FP64, then the node matrices (NB complements of 2d x 2d, or a full matrix).
-size_t pair_group_layout(PairArgs &A, int NB);
-
-size_t pair_warp_layout(PairArgs &A, int NB) {
-    if (A.grp) return align16((pair_group_layout(A, NB) + 1) / 2);  // a group spans two warp regions
-    const int n = A.n, m = A.m, T = tri_count(m), d2 = m - A.ne;
-    const size_t qbytes = A.reg ? 0 : (size_t)2 * n * ld_qt(n) * sizeof(cd);
-    size_t R = qbytes + (size_t)n * ld_t(n) * sizeof(cd);
-    A.off_qs = (int)align16(R);  // staged rows' re + im sums (shared-memory path)
-    if (A.t3) R = (size_t)A.off_qs + (size_t)2 * n * n * sizeof(double);
-    if ((size_t)T * sizeof(cd) > R) R = (size_t)T * sizeof(cd);
-    A.vm = m > NB * d2 ? m : NB * d2;
-    A.off_T = (int)qbytes;
-    size_t o = align16(R);
-    A.off_B = (int)o;  // B^(s), then the node matrices
-    o = align16(o + (size_t)(T > NB * tri_count(d2) ? T : NB * tri_count(d2)) * sizeof(cd));
+// Shared workspace of one team for nb node matrices per round; returns its bytes.  The first
+// region holds half of the snapshot's rows, then B^(s); the second T (or K), then the node
+// matrices: NB complements of 2d x 2d, or one full matrix.
+size_t pair_team_layout(PairArgs &A, int NB) {
+    const int n = A.n, m = A.m, T = tri_count(m), d2 = m - A.ne, Tn = tri_count(d2);
+    const int vm = m > NB * d2 ? m : NB * d2;
+    const auto most = [](int a, int b) { return a > b ? a : b; };
+    size_t o = (size_t)most(n * (n + 1), T) * sizeof(int4);
+    A.off_T = (int)o;
+    o += (size_t)most(most(n * ld_t(n), T), NB * Tn) * sizeof(int4);
     A.off_U = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_V = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pv = (int)o;  // records of the node products, then of the occupied pivots
-    o = align16(o + pv_bytes(A.vm, NB, A.ne));
-    return o;
-}
-
-// Workspace of one 64-thread group (two warp regions) on the group path: half of the
-// snapshot rows and T, aliased by the node matrices (a full copy of B for the shared
-// elimination, NB complements, S0 after them), then B, the Gauss vectors and the
-// step history of qcs_group.cuh; returns bytes per group.
-size_t pair_group_layout(PairArgs &A, int NB) {
-    const int n = A.n, m = A.m, ne = A.ne, T = tri_count(m), d2 = m - ne, Tn = tri_count(d2), S = m / 2;
-    const size_t qbytes = (size_t)n * ld_qt(n) * sizeof(cd);
-    A.off_T = (int)align16(qbytes);
-    A.off_qs = (int)align16((size_t)A.off_T + (size_t)n * ld_t(n) * sizeof(cd));
-    size_t R = (size_t)A.off_qs + (size_t)n * n * sizeof(double);
-    A.gz = T > NB * Tn ? T : NB * Tn;
-    if ((size_t)(A.gz + Tn) * sizeof(cd) > R) R = (size_t)(A.gz + Tn) * sizeof(cd);
-    A.vm = m > NB * d2 ? m : NB * d2;
-    size_t o = align16(R);
-    A.off_B = (int)o;
-    o = align16(o + (size_t)T * sizeof(cd));
-    A.off_U = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_V = (int)o;
-    o = align16(o + (size_t)A.vm * sizeof(cd));
-    A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(cd));
-    const int hs = S > NB * (d2 / 2) ? S : NB * (d2 / 2);  // history steps
-    A.off_inv = (int)o;
-    o = align16(o + (size_t)hs * sizeof(cd));
-    A.off_int = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(int));
-    size_t ha = (size_t)(S + 1) * m;  // active lists: full matrix, one node
-    if ((size_t)NB * (d2 / 2 + 1) * d2 > ha) ha = (size_t)NB * (d2 / 2 + 1) * d2;
-    A.off_act = (int)o;
-    o = align16(o + ha);
-    A.off_kh = (int)o;
-    o = align16(o + (size_t)hs);
-    A.off_ph = (int)o;
-    o = align16(o + (size_t)hs);
+    o += (size_t)vm * sizeof(FxGauss);
+    A.off_pv = (int)o;
+    A.npv = pv_records(vm, NB);
+    o = align16(o + pv_bytes(vm, NB, A.ne));
     A.off_scr = (int)o;
-    o = align16(o + sizeof(SharedScratch));
-    A.off_pvg = (int)o;  // records of the node products: NB (d2/2 + 1) or, for a full round, m/2 + 1
-    o = align16(o + (size_t)(NB * (d2 / 2 + 1) > S + 1 ? NB * (d2 / 2 + 1) : S + 1) * sizeof(cd));
-    return o;
+    return align16(o + sizeof(PairScratch));
 }
 
 }  // namespace
@@ -395,60 +270,51 @@ void setup_pair_args(qcs_ctx *ctx, const qcs_pair_launch &L, PairArgs &A) {
     A.n = L.n;
     A.ne = L.ne;
     A.m = 2 * L.n - L.ne;
-    A.d = L.n - L.ne;
-    A.nev = L.plan.nev;
     A.all = L.plan.all;
     A.chunk = L.chunk;
     A.nchunks = L.nchunks;
     A.W = L.W;
     A.P = L.P;
     const qcs_config cfg = qcs_decode_config(L.config);
-    A.reg = L.n == 16;
     A.grp = qcs_pair_forms_K(L.n, L.config);  // n > 16: two warps per pair unless one is configured
-    A.t3 = L.n < 16;
-    const int n = A.n, m = A.m, T = tri_count(m);
-    const int wpb = qcs_pair_warps_per_block();
+    const int n = A.n, m = A.m, T = tri_count(m), nev = L.plan.nev;
+    const int teams = qcs_pair_warps_per_block() / (A.grp ? 2 : 1);
     A.tab_bytes = (int)align16((size_t)T * sizeof(uint16_t));
-    A.ut_bytes = (int)align16((size_t)n * ld_ut(n) * (sizeof(cd) + sizeof(double)));  // rows and re + im
-    // Node matrices per round: the requested count, or by default the largest
-    // count (balanced rounds, at most kMaxNB) for which three blocks (register
-    // path) or two blocks fit on an SM.
+    A.ut_bytes = (int)align16((size_t)n * (n + 1) * sizeof(int4));
+    const auto block = [&](int nb) { return (size_t)A.tab_bytes + A.ut_bytes + teams * pair_team_layout(A, nb) + 1024; };
+    // Node matrices per round: the requested count, or by default the largest balanced one
+    // (at most kMaxNB) that costs no resident block: more nodes share a round's pivot work,
+    // but warps in flight hide the eliminations' latencies.
     int NB = 1;
-    const int nbmax = A.grp ? kMaxNBG : kMaxNB;
+    const auto resident = [&](int nb) {
+        const int b = (int)((ctx->smem_optin + 1024) / block(nb));
+        return b < 4 ? b : 4;
+    };
     if (cfg.nb > 0) {
-        NB = cfg.nb < A.nev ? cfg.nb : A.nev;
-        if (NB > nbmax) NB = nbmax;
-        while (NB > 1 && (size_t)A.tab_bytes + A.ut_bytes + (size_t)wpb * pair_warp_layout(A, NB) > ctx->smem_optin)
-            --NB;
+        NB = cfg.nb < nev ? cfg.nb : nev;
+        if (NB > kMaxNB) NB = kMaxNB;
+        while (NB > 1 && block(NB) > ctx->smem_optin) --NB;
     } else {
-        const size_t sm_budget = ctx->smem_optin;
-        for (int rounds = 1; rounds <= A.nev; ++rounds) {
-            int nb = (A.nev + rounds - 1) / rounds;
-            if (nb > nbmax) continue;
-            size_t blk = (size_t)A.tab_bytes + A.ut_bytes + (size_t)wpb * pair_warp_layout(A, nb) + 1024;
-            if ((A.reg ? 3 : 2) * blk <= sm_budget + 1024) {
+        for (int rounds = 1; rounds <= nev; ++rounds) {
+            const int nb = (nev + rounds - 1) / rounds;
+            if (nb <= kMaxNB && resident(nb) >= 1 && resident(nb) >= resident(1)) {
                 NB = nb;
                 break;
             }
         }
     }
     A.NB = NB;
-    A.warp_bytes = (int)pair_warp_layout(A, NB);
+    A.team_bytes = (int)pair_team_layout(A, NB);
     A.Ut = L.Ut;
     A.pref = L.pref;
-    A.wmode = L.mode;
     A.Qt = L.s->Qt;
-    A.Qh = A.grp ? L.s->Qh : nullptr;  // the group path forms K and B from K; the warp path T
+    A.Qh = A.grp ? L.s->Qh : nullptr;  // two warps form K and B from K; one T
     A.gth = L.s->gth;
     A.idx = L.s->idx;
     A.d_count = L.s->d_count;
     A.partial = L.partial;
     A.per_pair = L.per_pair;
     A.status = ctx->d_status;
-    for (int k = 0; k < L.plan.nev; ++k) {
-        A.wnode[k] = L.plan.wnode[k];
-        A.gamma[k] = L.plan.gamma[k];
-    }
     fx_make_plan(L.plan, A.plan);
 }
 
@@ -488,17 +354,19 @@ qcs_status qcs_launch_pairs_batched(qcs_ctx *ctx, int nsys, const qcs_pair_launc
         B.tile_end[q] = acc;
         if (B.sys[q].tab_bytes > B.tab_bytes) B.tab_bytes = B.sys[q].tab_bytes;
         if (B.sys[q].ut_bytes > B.ut_bytes) B.ut_bytes = B.sys[q].ut_bytes;
-        if (B.sys[q].warp_bytes > B.warp_bytes) B.warp_bytes = B.sys[q].warp_bytes;
+        const int work = B.sys[q].team_bytes * (qcs_pair_warps_per_block() / (B.sys[q].grp ? 2 : 1));
+        if (work > B.work_bytes) B.work_bytes = work;
         if (B.sys[q].m > B.max_m) B.max_m = B.sys[q].m;
     }
     if (acc == 0) return QCS_OK;
     const int wpb = qcs_pair_warps_per_block();
-    size_t smem = (size_t)B.tab_bytes + B.ut_bytes + (size_t)wpb * B.warp_bytes;
+    size_t smem = (size_t)B.tab_bytes + B.ut_bytes + B.work_bytes;
     if (smem + 64 > ctx->smem_optin)  // + the kernel's static tile index
         return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "batched kernel: shared memory too large");
-    bool grp = false;
-    for (int q = 0; q < nsys; ++q) grp |= B.sys[q].grp != 0;
-    const void *kfn = grp ? (const void *)pair_overlap_kernel<true> : (const void *)pair_overlap_kernel<false>;
+    int kinds = 0;
+    for (int q = 0; q < nsys; ++q) kinds |= B.sys[q].grp ? 2 : 1;
+    void (*const kern)(BatchArgs) = kinds == 1 ? pair_overlap_kernel<1> : kinds == 2 ? pair_overlap_kernel<2> : pair_overlap_kernel<3>;
+    const void *kfn = (const void *)kern;
     if (qcs_set_smem(ctx, kfn, smem) != QCS_OK) return QCS_ERR_CUDA;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, wpb * 32, smem) !=
@@ -510,8 +378,7 @@ qcs_status qcs_launch_pairs_batched(qcs_ctx *ctx, int nsys, const qcs_pair_launc
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return qcs_fail(ctx, QCS_ERR_CUDA, "batched counter reset");
     qcs_prof_begin(ctx, st);
-    if (grp) pair_overlap_kernel<true><<<(unsigned)blocks, wpb * 32, smem, st>>>(B);
-    else pair_overlap_kernel<false><<<(unsigned)blocks, wpb * 32, smem, st>>>(B);
+    kern<<<(unsigned)blocks, wpb * 32, smem, st>>>(B);
     qcs_prof_end(ctx, st);
     return qcs_check_launch(ctx, "pair_overlap_kernel");
 }

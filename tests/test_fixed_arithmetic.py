@@ -1,9 +1,9 @@
 """CPU model of the eliminations' fixed-point arithmetic (csrc/qcs_fixed.cuh).
 
-An entry is a 64-bit integer X = h 2^31 + l with |l| <= 2^30; a product keeps
-hh 2^62 + (h l' + l h') 2^31 and drops l l'; the complex pivot reciprocal is one third-order
+An entry is a 64-bit integer X = h 2^30 + l with |l| <= 2^29; a product keeps
+hh 2^60 + (h l' + l h') 2^30 and drops l l'; the complex pivot reciprocal is one third-order
 step from a single-precision seed.  The bounds below are derived from the limb sizes:
-the dropped term is at most 2^60 of a product of 2^121 (|X| < 2^60.5), and the reciprocal
+the dropped term is at most 2^58 of a product of 2^119 (|X| < 2^60), and the reciprocal
 keeps at least 57 bits with at most four truncations of one unit each plus a seed error
 e <= 2^-22, e^3 <= 2^-66.
 """
@@ -27,9 +27,9 @@ def s32(x):
 
 
 def split(X):
-    h = s32((X + (1 << 30)) >> 31)
-    l = s32(X - (h << 31))
-    assert X == (h << 31) + l and abs(l) <= 1 << 30
+    h = s32((X + (1 << 29)) >> 30)
+    l = s32(X - (h << 30))
+    assert X == (h << 30) + l and abs(l) <= 1 << 29
     return h, l
 
 
@@ -39,19 +39,19 @@ def mac(acc, a, b):
     assert abs(acc[0]) < 1 << 63 and abs(acc[1]) < 1 << 63  # what the 64-bit accumulators hold
 
 
-def value(acc, up):
-    v = (acc[0] << up) + (acc[1] >> (31 - up))
+def value(acc, dn):
+    v = (acc[0] << (60 - dn)) + (acc[1] >> (dn - 30))
     assert abs(v) < 1 << 63
     return v
 
 
 def inverse(qx, qy):
-    """2^119 / (qx + i qy), as the device function."""
+    """2^118 / (qx + i qy), as the device function."""
     a, b = split(qx), split(qy)
     s = [0, 0]
     mac(s, a, a)
     mac(s, b, b)
-    D = s[0] + (s[1] >> 31)
+    D = s[0] + (s[1] >> 30)
     R0 = int(np.float32(np.float32(1) / np.float32(D >> 31)) * np.float32(2.0**54))
     e = s64(-(D * R0))
     eh = e >> 32
@@ -61,19 +61,19 @@ def inverse(qx, qy):
     u, v = [0, 0], [0, 0]
     mac(u, a, r)
     mac(v, b, r)
-    return value(u, 1), -value(v, 1)
+    return value(u, 60), -value(v, 60)
 
 
 def pivots(count, rng):
     for _ in range(count):
-        q = [rng.randrange(-(1 << 61) + 1, 1 << 61), rng.randrange(-(1 << 61) + 1, 1 << 61)]
+        q = [rng.randrange(-(1 << 60) + 1, 1 << 60), rng.randrange(-(1 << 60) + 1, 1 << 60)]
         k = rng.randrange(2)
-        q[k] = rng.choice([1, -1]) * rng.randrange(1 << 60, 1 << 61)
+        q[k] = rng.choice([1, -1]) * rng.randrange(1 << 59, 1 << 60)
         if rng.random() < 0.3:
             q[1 - k] >>= rng.randrange(62)
         yield q
-    for x in (1 << 60, (1 << 61) - 1):
-        for y in (0, 1, -1, 1 << 59, (1 << 61) - 1, -(1 << 61) + 1):
+    for x in (1 << 59, (1 << 60) - 1):
+        for y in (0, 1, -1, 1 << 58, (1 << 60) - 1, -(1 << 60) + 1):
             yield [x, y]
             yield [y, -x]
 
@@ -83,13 +83,13 @@ def test_pivot_reciprocal():
     for qx, qy in pivots(20000, random.Random(1)):
         ix, iy = inverse(qx, qy)
         n = qx * qx + qy * qy
-        ex, ey = Fraction(qx << 119, n), Fraction(-qy << 119, n)
+        ex, ey = Fraction(qx << 118, n), Fraction(-qy << 118, n)
         err = float(max(abs(ix - ex), abs(iy - ey))) / float(max(abs(ex), abs(ey)))
         worst = max(worst, err)
     assert worst <= 2.0**-54
 
 
-@pytest.mark.parametrize("bits_g,bits_v", [(59.5, 58), (59.5, 61), (40, 58), (59.5, 20)])
+@pytest.mark.parametrize("bits_g,bits_v", [(59.5, 58), (59.5, 60), (40, 58), (59.5, 20)])
 def test_rank2_entry_update(bits_g, bits_v):
     """A + g_i v_j - v_i g_j with g scaled by 2^59: the dropped limb products and the two
     shifts cost at most 6 units of the result's last place."""
@@ -111,7 +111,7 @@ def test_rank2_entry_update(bits_g, bits_v):
         if max(abs(ere), abs(eim)) >= 1 << 121:
             continue  # beyond the bound 4 2^mb 2^59 that pivoting gives for |g| <= sqrt 2
         for acc, ex in ((re, ere), (im, eim)):
-            assert abs(Fraction(value(acc, 3)) - Fraction(ex, 1 << 59)) <= 6
+            assert abs(Fraction(value(acc, 59)) - Fraction(ex, 1 << 59)) <= 6
 
 
 # ---- balanced slices of the tensor-core congruence (csrc/qcs_ozaki.cuh)
