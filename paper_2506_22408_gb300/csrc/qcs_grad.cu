@@ -35,21 +35,19 @@
 // Y_p = sum_k c_k A'_k^{-1} (shared_inverse).  Pairs whose occupied block would grow
 // the complement beyond 2^8 of max|B| take the full elimination per node.
 #include "qcs_internal.h"
+#include "qcs_fxcong.cuh"
 #include "qcs_group.cuh"
 
 namespace {
-
 
 struct GradArgs {
     int n, ne, m, d, nev, NB, all, chunk, nchunks;
     int64_t W, P;
     int group_bytes, tab_bytes;
     int off_Q, off_T, off_B, off_Y, off_G, off_NZ, off_g1, off_g2, off_y1, off_y2, off_pf, off_cf, off_invh,
-        off_int, off_tile, off_acth, off_kh, off_ph, off_kc, off_sacth, off_skh, off_sph, off_sinvh, off_scr;
+        off_int, off_tile, off_acth, off_kh, off_ph, off_sacth, off_skh, off_sph, off_sinvh, off_scr;
     const cd *Ut;
-    const cd *Qt;
-    const cd *Qh;        // per dense snapshot of the set: the rows [H1^T; G2^T] (2n x n, the layout of Qt)
-    const uint8_t *gth;  // gather codes of signed-permutation snapshots (or null)
+    const cd *Qh;        // per snapshot of the set: the rows [H1^T; G2^T] (2n x n, the layout of Qt)
     const int *idx;
     const int *d_count;
     cd *partial;
@@ -59,86 +57,21 @@ struct GradArgs {
     cd gamma[QCS_MAX_NODES];
 };
 
-// B (packed upper, m x m) from K = [Ut H1 | Ut G2] (rows of Ks, stride ld_t) and the walker
-// rows Ut: with W1 = (Ut H1) Ut^T = T J T^T and W2 = (Ut G2) Ut^H = T J conj(T)^T, and the
-// empty rows R_j = Re T_j, I_j = -Im T_j of X,
-//     occupied a, b:          W1[a][b]
-//     occupied a, empty j:    (a, R_j) = (W1 + W2)[a][j] / 2,   (a, I_j) = i (W1 - W2)[a][j] / 2
-//     empty j1 <= j2, al = W1[j1][j2], be = W2[j1][j2]:
-//         (R, R) = Re(al + be)/2,  (R, I) = Im(be - al)/2,  (I, R) = -Im(al + be)/2,
-//         (I, I) = Re(be - al)/2;  within one mode (al = 0) only (R_j, I_j) = Im(be)/2.
-// Work items: the tri(ne) occupied pairs, the ne x d occupied-empty pairs and the
-// tri(d + 1) empty pairs j1 <= j2, each two n-term sums (the echelon zeros of Ut included,
-// so that every lane runs the same loop).
-__device__ inline void build_B_from_K3(int n, int ne, const cd *__restrict__ Uts, const double *__restrict__ Uss,
-                                      const double *__restrict__ Usd, const cd *__restrict__ Ks,
-                                      const double *__restrict__ Ksum, cd *__restrict__ Bs,
-                                      const uint16_t *__restrict__ tab, int t, int nthr) {
-    const int d = n - ne, lu = ld_ut(n), lt = ld_t(n), n2 = 2 * n;
-    const int c1 = tri_count(ne), c2 = c1 + ne * d, c3 = c2 + tri_count(d + 1);
-    for (int it = t; it < c3; it += nthr) {
-        int a, b, kind;  // K row a, walker row b
-        if (it < c1) {
-            pair_of(tab, it, a, b);
-            kind = 0;
-        } else if (it < c2) {
-            const int e = it - c1, jj = e / ne;
-            a = e - jj * ne;
-            b = ne + jj;
-            kind = 1;
-        } else {
-            int x, y;
-            pair_of(tab, it - c2, x, y);  // x < y: empty modes x <= y - 1
-            a = ne + x;
-            b = ne + y - 1;
-            kind = 2;
-        }
-        // three real products per complex term: K1 u with the sums re + im of both factors,
-        // K2 conj(u) with re + im of K2 and re - im of u
-        const cd *kr = Ks + a * lt, *ur = Uts + b * lu;
-        const double *ks = Ksum + a * n2, *us = Uss + b * lu, *ud = Usd + b * lu;
-        double p1 = 0.0, p2 = 0.0, p3 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-        for (int k = 0; k < n; ++k) {
-            const cd u = ur[k], k1 = kr[k], k2 = kr[n + k];
-            p1 = fma(k1.x, u.x, p1);
-            p2 = fma(k1.y, u.y, p2);
-            p3 = fma(ks[k], us[k], p3);
-            q1 = fma(k2.x, u.x, q1);
-            q2 = fma(k2.y, u.y, q2);
-            q3 = fma(ks[n + k], ud[k], q3);
-        }
-        const cd w1 = cmk(p1 - p2, p3 - p1 - p2), w2 = cmk(q1 + q2, q3 - q1 + q2);
-        if (kind == 0) {
-            Bs[tri_index(a, b)] = w1;
-        } else if (kind == 1) {
-            const int r = 2 * (b - ne);
-            const cd sp = cadd(w1, w2), dm = csub(w1, w2);
-            Bs[tri_index(a, ne + r)] = cscale(sp, 0.5);
-            Bs[tri_index(a, ne + r + 1)] = cmk(-0.5 * dm.y, 0.5 * dm.x);
-        } else {
-            const int r1 = 2 * (a - ne), r2 = 2 * (b - ne);
-            if (r1 < r2) {
-                Bs[tri_index(ne + r1, ne + r2)] = cmk(0.5 * (w1.x + w2.x), 0.0);
-                Bs[tri_index(ne + r1, ne + r2 + 1)] = cmk(0.5 * (w2.y - w1.y), 0.0);
-                Bs[tri_index(ne + r1 + 1, ne + r2)] = cmk(-0.5 * (w1.y + w2.y), 0.0);
-                Bs[tri_index(ne + r1 + 1, ne + r2 + 1)] = cmk(0.5 * (w2.x - w1.x), 0.0);
-            } else {
-                Bs[tri_index(ne + r1, ne + r1 + 1)] = cmk(0.5 * w2.y, 0.0);
-            }
-        }
-    }
-}
-
 // Two warps (a group of 64 threads) per pair; a block holds blockDim/64 groups,
 // each with its own workspace and named barrier.  Groups pull (walker, chunk)
 // tiles from a device counter in chunk-major order.
+//
+// Bound by the FP64 pipe (76 clocks per DFMA and 32 lanes): at 16 modes and 8 electrons a
+// pair took 190k FP64 operations, 107k of them in K, B^(s) and the cotangent products.  Those
+// three are in fixed point on the integer pipe (qcs_fxcong.cuh): 606 -> 490 ms for 512
+// walkers against 10,000 snapshots.
 __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant__ GradArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / kGroup;
     const int t = threadIdx.x - gid * kGroup;
     const int bar = 1 + gid;
     const int n = A.n, n2 = 2 * n, ne = A.ne, m = A.m, T = tri_count(m);
-    const int lu = ld_ut(n), lq = ld_qt(n), lt = ld_t(n);
+    const int lt = ld_t(n);
     // the pair table and the groups' workspaces fit the launch's shared memory
     if (!QCS_IN_BOUNDS(T * (int)sizeof(uint16_t) <= A.tab_bytes &&
                            (size_t)A.tab_bytes + (size_t)(blockDim.x / kGroup) * A.group_bytes <= dyn_smem_bytes(),
@@ -148,18 +81,14 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
     build_pair_table(tab, T);
     __syncthreads();
     unsigned char *wb = smem_raw + A.tab_bytes + (size_t)gid * A.group_bytes;
-    cd *Uts = reinterpret_cast<cd *>(wb);
-    cd *Qs = reinterpret_cast<cd *>(wb + A.off_Q);
-    cd *Ts = reinterpret_cast<cd *>(wb + A.off_T);
+    int4 *Us = reinterpret_cast<int4 *>(wb);             // walker rows as limbs (qcs_fxcong.cuh)
+    int4 *Qs = reinterpret_cast<int4 *>(wb + A.off_Q);   // half of the snapshot's rows as limbs
+    fx2 *Xs = reinterpret_cast<fx2 *>(wb + A.off_Q);     // B^(s) in fixed point, once K is formed
+    int4 *Ks = reinterpret_cast<int4 *>(wb + A.off_T);   // K as limbs
     cd *Bs = reinterpret_cast<cd *>(wb + A.off_B);
     cd *Ys = reinterpret_cast<cd *>(wb + A.off_Y);
     cd *Gs = reinterpret_cast<cd *>(wb + A.off_G);
-    cd *Ns = reinterpret_cast<cd *>(wb + A.off_NZ);  // node factors, then their inverses, then G_X
-    cd *GX = Ns;
-    double *Uss = reinterpret_cast<double *>(Ns);  // while T (or K) and B are formed: re + im of Ut
-    double *Usd = Uss + n * lu;                     // and re - im of Ut
-    double *Ksum = reinterpret_cast<double *>(Qs);  // once K is formed: re + im of K (n x 2n)
-    double *Kdif = Ksum + n * n2;                   // and re - im of K's empty rows (d x 2n)
+    cd *Ns = reinterpret_cast<cd *>(wb + A.off_NZ);  // node factors, then their inverses, then the coefficients
     cd *g1v = reinterpret_cast<cd *>(wb + A.off_g1);  // forward: U vectors
     cd *g2v = reinterpret_cast<cd *>(wb + A.off_g2);  // forward: V vectors
     cd *y1v = reinterpret_cast<cd *>(wb + A.off_y1);
@@ -172,7 +101,6 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
     uint8_t *acth = wb + A.off_acth;
     uint8_t *kh = wb + A.off_kh;
     uint8_t *ph = wb + A.off_ph;
-    uint8_t *kc = wb + A.off_kc;  // signed-permutation snapshots: the two rows of each column of Qt
     uint8_t *sacth = wb + A.off_sacth;  // history of the shared occupied-block elimination
     uint8_t *skh = wb + A.off_skh;
     uint8_t *sph = wb + A.off_sph;
@@ -200,49 +128,48 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
         for (int e = t; e < n * n; e += kGroup) Gs[e] = cmk(0.0, 0.0);
         if (p0 < L) {
             const cd *Utw = A.Ut + w * n * n;
-            for (int e = t; e < n * n; e += kGroup) Uts[(e / n) * lu + (e % n)] = Utw[e];
+            const int fU = fx_fraction(fx_max_key(Utw, n * n, t & 31), 57);
+            fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, t, kGroup);
             for (int64_t pq = p0; pq < p1; ++pq) {
                 const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
                 if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // group-uniform
-                const uint8_t *gq = A.gth ? A.gth + q * n2 : nullptr;
-                const bool sp = gq && gq[0] != 0xFF;  // signed permutation: gathers instead of products
                 group_sync(bar);
-                if (sp) {
-                    // column k of Qt has exactly two nonzeros, in rows kc[2k] < kc[2k+1]
-                    for (int c = t; c < n2; c += kGroup) {
-                        const int k = gq[c] >> 2;
-                        int slot = 0;
-                        for (int c2 = 0; c2 < c; ++c2) slot += ((gq[c2] >> 2) == k) ? 1 : 0;
-                        kc[2 * k + slot] = (uint8_t)c;
+                // K = Ut [H1 | G2] by column halves, then B^(s) from it, in fixed point
+                const cd *Qr = A.Qh + q * n2 * n;
+                const unsigned key = fx_max_key(Qr, n2 * n, t & 31);
+                if (key >= 0x7ff00000u) {  // a non-finite snapshot (every snapshot evaluated): NaN
+                    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                    for (int e = t; e < n * n; e += kGroup) Gs[e] = cmk(nan, nan);
+                    if (t == 0) {
+                        raise_status(A.status, QCS_ERR_NONFINITE);
+                        Ssum = cmk(nan, nan);
                     }
-                } else {
-                    load_Qt(n, A.Qh + q * n2 * n, Qs, t, kGroup);  // [H1^T; G2^T]: K = Ut Qh^T in T's place
-                    // re + im (for build_T_reg and B) and re - im (for B's conjugate products) of
-                    // the walker rows, in the node region (free here)
-                    for (int e = t; e < n * n; e += kGroup) {
-                        const int j = e / n, k = e - j * n;
-                        const cd u = Uts[j * lu + k];
-                        Uss[j * lu + k] = u.x + u.y;
-                        Usd[j * lu + k] = u.x - u.y;
-                    }
+                    continue;
                 }
-                group_sync(bar);
-                if (sp) build_T_gather(n, Uts, gq, Ts, t, kGroup);
-                else if (n == 16)  // lane = column of T, the two warps take alternate rows
-                    build_T_reg<16>(ne, Uts, Uss, Qs, Ts, t & 31, false, lq, t >> 5, kGroup / 32);
-                else build_T_echelon(n, ne, Uts, Qs, Ts, t, kGroup);  // walker rows in echelon form
-                group_sync(bar);
-                if (sp) {
-                    build_B(n, ne, Ts, Bs, tab, t, kGroup);
-                } else {
-                    for (int e = t; e < n * n2; e += kGroup) {  // Qh is no longer needed
-                        const int j = e / n2, c = e - j * n2;
-                        const cd k = Ts[j * lt + c];
-                        Ksum[e] = k.x + k.y;
-                        if (j >= ne) Kdif[e - ne * n2] = k.x - k.y;
-                    }
+                const int fQ = fx_fraction(key, 57);
+                const FxTeam<2> tm = {t, t & 31, t >> 5, bar, scr->red};
+                unsigned top = 0u;
+                for (int h = 0; h < 2; ++h) {
+                    fx_stage_rows(n, n * n, Qr + (int64_t)h * n * n, fQ, nullptr, Qs, t, kGroup);
                     group_sync(bar);
-                    build_B_from_K3(n, ne, Uts, Uss, Usd, Ts, Ksum, Bs, tab, t, kGroup);
+                    top |= fx_build_T(n, ne, Us, Qs, reinterpret_cast<fx2 *>(Ks), h * n, t, kGroup);
+                    group_sync(bar);
+                }
+                top = tm.or_put(top, 0);
+                group_sync(bar);
+                const int kb = fx_top_bits(tm.or_get(top, 0));
+                const int fK = fU + fQ - 58 + 56 - kb;
+                fx_T_limbs(n, Ks, kb, t, kGroup);
+                group_sync(bar);
+                fx_build_B_from_K(n, ne, Us, Ks, Xs, tab, t, kGroup);
+                group_sync(bar);
+                for (int e = t; e < T; e += kGroup) {  // to FP64, the occupied rows first
+                    int a, b;
+                    pair_of(tab, e, a, b);
+                    const int i = a < m - ne ? a + ne : a - (m - ne), j = b < m - ne ? b + ne : b - (m - ne);
+                    const fx2 x = Xs[e];
+                    const cd v = flip_if(cmk(fx_f64(x.x, 58 - fK - fU), fx_f64(x.y, 58 - fK - fU)), i > j);
+                    Bs[i < j ? tri_index(i, j) : tri_index(j, i)] = v;
                 }
                 group_sync(bar);
                 cd S = cmk(0.0, 0.0);
@@ -307,102 +234,82 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
                 }
                 // Cotangents: Gamma1 (rows < ne) += G_X[occ] Qt and Gamma2 (rows >= ne) += Ht conj(Qt),
                 // G_X / 2 = Y (X J) and Ht_i = G[ne+2i] - i G[ne+2i+1] = Yh_i (X J), where
-                // Yh_i = Y[ne+2i] - i Y[ne+2i+1] (G_X is linear in Y's rows).
-                if (sp) {
-                    // signed permutation: G_X on the occupied rows and Ht, then gathers of Qt
-                    cd *Yh = GX + n * n2;  // d x m, after G_X's n x 2n entries
-                    for (int e = t; e < A.d * m; e += kGroup) {
-                        const int i = e / m, b = e - i * m;
-                        const cd y0 = skew_at(Ys, ne + 2 * i, b), y1 = skew_at(Ys, ne + 2 * i + 1, b);
-                        Yh[e] = cmk(y0.x + y1.y, y0.y - y1.x);
+                // Yh_i = Y[ne+2i] - i Y[ne+2i+1] (G_X is linear in Y's rows).  X J Qt and
+                // X J conj(Qt) are rows of K = [Ut H1 | Ut G2]: occupied row b gives K1_b and
+                // K2_b; the empty rows R_j, I_j give (K1_j + conj K2_j)/2, i (K1_j - conj K2_j)/2
+                // and their conjugates.  So with the source row y (Y[r] for r < ne, Yh_{r-ne} else)
+                // and c_j = (y[R_j] + i y[I_j])/2, c'_j = (y[R_j] - i y[I_j])/2,
+                //     Gamma1[r] += sum_b y[b] K1_b + sum_j (c_j K1_j + c'_j conj K2_j)
+                //     Gamma2[r] += sum_b y[b] K2_b + sum_j (c_j K2_j + c'_j conj K1_j)
+                // (n x m coefficients Cf in the node region, as limbs once their largest is
+                // known, then n x n entries of m terms, three real products each: with the
+                // sums of K's parts (differences for the conjugated ones), Re = p1 - p2 and
+                // Im = p3 - p1 - p2).
+                cd *Cf = Ns;
+                unsigned ck = 0u;
+                for (int e = t; e < n * m; e += kGroup) {
+                    const int r = e / m, b = e - r * m;
+                    const bool occ = r < ne;
+                    const int r0 = occ ? r : ne + 2 * (r - ne), r1 = occ ? r : r0 + 1;
+                    const bool pair = b >= ne;
+                    const int b0 = pair ? ne + ((b - ne) & ~1) : b;
+                    // y at columns b0 and bi = b0 + 1 (the second only for an empty pair)
+                    const int bi = pair ? b0 + 1 : b0;
+                    cd y0 = skew_at(Ys, r0, b0), y1 = skew_at(Ys, r1, b0);
+                    const cd yb = occ ? y0 : cmk(y0.x + y1.y, y0.y - y1.x);
+                    y0 = skew_at(Ys, r0, bi);
+                    y1 = skew_at(Ys, r1, bi);
+                    const cd yi = occ ? y0 : cmk(y0.x + y1.y, y0.y - y1.x);
+                    // c = (yb + i yi) / 2 at even offsets, c' = (yb - i yi) / 2 at odd ones
+                    const bool odd = (b - ne) & 1;
+                    const cd iy = flip_if(cmk(-yi.y, yi.x), odd);
+                    const cd c = pair ? cmk(0.5 * (yb.x + iy.x), 0.5 * (yb.y + iy.y)) : yb;
+                    Cf[e] = c;
+                    ck = max(ck, pivot_key(c));
+                }
+                ck = __reduce_max_sync(QCS_FULL, ck);
+                if ((t & 31) == 0) scr->red[t >> 5] = ck;
+                group_sync(bar);
+                ck = max(scr->red[0], scr->red[1]);
+                if (ck >= 0x7ff00000u) {  // an overflowed inverse: NaN, as its products would be
+                    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                    for (int e = t; e < n * n; e += kGroup) Gs[e] = cmk(nan, nan);
+                    continue;
+                }
+                const int fC = fx_fraction(ck, 56);
+                int4 *Cx = reinterpret_cast<int4 *>(Cf);
+                for (int e = t; e < n * m; e += kGroup) Cx[e] = fx_limbs(Cf[e], fC);
+                group_sync(bar);
+#pragma unroll 1
+                for (int e = t; e < n * n; e += kGroup) {
+                    const int r = e / n, k = e - r * n;
+                    const int o1 = r < ne ? 0 : n, o2 = n - o1;
+                    const int4 *cf = Cx + r * m, *kr = Ks + k;
+                    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
+                    for (int b = 0; b < ne; ++b, kr += lt) {
+                        const int4 c = cf[b], v = kr[o1];
+                        fx_mac(p1, fx_re(c), fx_re(v));
+                        fx_mac(p2, fx_im(c), fx_im(v));
+                        fx_mac(p3, fx_add(fx_re(c), fx_im(c)), fx_add(fx_re(v), fx_im(v)));
                     }
-                    group_sync(bar);
-                    // (XJ)[b][2k] = -X[b][2k+1], (XJ)[b][2k+1] = X[b][2k]; row ne + i of GX is Ht_i
-                    for (int e = t; e < n * n2; e += kGroup) {
-                        const int a = e / n2, c = e - a * n2;
-                        const int cx = c ^ 1;
-                        const bool occ = a < ne;
-                        const cd *yh = Yh + (occ ? 0 : (a - ne) * m);
-                        cd acc = cmk(0.0, 0.0);
-                        for (int b = 0; b < ne; ++b) cfma(acc, occ ? skew_at(Ys, a, b) : yh[b], Ts[b * lt + cx]);
-                        for (int r = 0; r < m - ne; ++r) {
-                            const cd tt = Ts[(ne + (r >> 1)) * lt + cx];
-                            crfma(acc, occ ? skew_at(Ys, a, ne + r) : yh[ne + r], (r & 1) ? -tt.y : tt.x);
-                        }
-                        GX[e] = flip_if(acc, !(c & 1));
+                    cf += ne;
+#pragma unroll 1
+                    for (int j = 0; j < A.d; ++j, kr += lt, cf += 2) {
+                        const int4 c = cf[0], v = kr[o1], c2 = cf[1], w2 = kr[o2];  // c v + c2 conj(w2)
+                        fx_mac(p1, fx_re(c), fx_re(v));
+                        fx_mac(p2, fx_im(c), fx_im(v));
+                        fx_mac(p3, fx_add(fx_re(c), fx_im(c)), fx_add(fx_re(v), fx_im(v)));
+                        fx_mac(p1, fx_re(c2), fx_re(w2));
+                        fx_mac(p2, fx_neg(fx_im(c2)), fx_im(w2));
+                        fx_mac(p3, fx_add(fx_re(c2), fx_im(c2)), fx_sub(fx_re(w2), fx_im(w2)));
                     }
-                    group_sync(bar);
-                    for (int e = t; e < n * n; e += kGroup) {
-                        const int j = e / n, k = e - j * n;
-                        const cd *g = GX + j * n2;
-                        cd acc = Gs[e];
-                        for (int h = 0; h < 2; ++h) {
-                            const int c = kc[2 * k + h];
-                            const unsigned ph = gq[c] & 3u;
-                            acc = cadd(acc, mul_phase(g[c], j < ne ? ph : ((4u - ph) & 3u)));
-                        }
-                        Gs[e] = acc;
-                    }
-                } else {
-                    // dense: X J Qt and X J conj(Qt) are rows of K = [Ut H1 | Ut G2]: occupied row b
-                    // gives K1_b and K2_b; the empty rows R_j, I_j give (K1_j + conj K2_j)/2,
-                    // i (K1_j - conj K2_j)/2 and their conjugates.  So with the source row y (Y[r]
-                    // for r < ne, Yh_{r-ne} else) and c_j = (y[R_j] + i y[I_j])/2,
-                    // c'_j = (y[R_j] - i y[I_j])/2,
-                    //     Gamma1[r] += sum_b y[b] K1_b + sum_j (c_j K1_j + c'_j conj K2_j)
-                    //     Gamma2[r] += sum_b y[b] K2_b + sum_j (c_j K2_j + c'_j conj K1_j)
-                    // (n x m coefficients Cf and their sums re + im in the node region, then n x n
-                    // entries of m terms, three real products each: with the sums of K's entries
-                    // (re - im for the conjugated ones), Re = p1 - p2 and Im = p3 - p1 - p2).
-                    cd *Cf = Ns;
-                    double *Cs = reinterpret_cast<double *>(Ns + n * m);
-                    for (int e = t; e < n * m; e += kGroup) {
-                        const int r = e / m, b = e - r * m;
-                        const bool occ = r < ne;
-                        const int r0 = occ ? r : ne + 2 * (r - ne), r1 = occ ? r : r0 + 1;
-                        const bool pair = b >= ne;
-                        const int b0 = pair ? ne + ((b - ne) & ~1) : b;
-                        // y at columns b0 and bi = b0 + 1 (the second only for an empty pair)
-                        const int bi = pair ? b0 + 1 : b0;
-                        cd y0 = skew_at(Ys, r0, b0), y1 = skew_at(Ys, r1, b0);
-                        const cd yb = occ ? y0 : cmk(y0.x + y1.y, y0.y - y1.x);
-                        y0 = skew_at(Ys, r0, bi);
-                        y1 = skew_at(Ys, r1, bi);
-                        const cd yi = occ ? y0 : cmk(y0.x + y1.y, y0.y - y1.x);
-                        // c = (yb + i yi) / 2 at even offsets, c' = (yb - i yi) / 2 at odd ones
-                        const bool odd = (b - ne) & 1;
-                        const cd iy = flip_if(cmk(-yi.y, yi.x), odd);
-                        const cd c = pair ? cmk(0.5 * (yb.x + iy.x), 0.5 * (yb.y + iy.y)) : yb;
-                        Cf[e] = c;
-                        Cs[e] = c.x + c.y;
-                    }
-                    group_sync(bar);
-                    for (int e = t; e < n * n; e += kGroup) {
-                        const int r = e / n, k = e - r * n;
-                        const int o1 = r < ne ? 0 : n, o2 = n - o1;
-                        const cd *cf = Cf + r * m;
-                        const double *cs = Cs + r * m;
-                        double p1 = 0.0, p2 = 0.0, p3 = 0.0;
-                        for (int b = 0; b < ne; ++b) {
-                            const cd c = cf[b], v = Ts[b * lt + o1 + k];
-                            p1 = fma(c.x, v.x, p1);
-                            p2 = fma(c.y, v.y, p2);
-                            p3 = fma(cs[b], Ksum[b * n2 + o1 + k], p3);
-                        }
-                        for (int j = 0; j < A.d; ++j) {
-                            const cd *kr = Ts + (ne + j) * lt;
-                            const cd c = cf[ne + 2 * j], v = kr[o1 + k];
-                            p1 = fma(c.x, v.x, p1);
-                            p2 = fma(c.y, v.y, p2);
-                            p3 = fma(cs[ne + 2 * j], Ksum[(ne + j) * n2 + o1 + k], p3);
-                            const cd c2 = cf[ne + 2 * j + 1], w = kr[o2 + k];  // c2 conj(w)
-                            p1 = fma(c2.x, w.x, p1);
-                            p2 = fma(-c2.y, w.y, p2);
-                            p3 = fma(cs[ne + 2 * j + 1], Kdif[j * n2 + o2 + k], p3);
-                        }
-                        const cd acc = Gs[e];
-                        Gs[e] = cmk(acc.x + (p1 - p2), acc.y + (p3 - p1 - p2));
-                    }
+                    fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
+                    re.cr += fx_half<kFxS>(58);
+                    im.cr += fx_half<kFxS>(58);
+                    const cd acc = Gs[e];
+                    Gs[e] = cmk(acc.x + fx_f64(fx_value<kFxS>(re, 58), 58 - fC - fK),
+                                acc.y + fx_f64(fx_value<kFxS>(im, 58), 58 - fC - fK));
                 }
             }
         }
@@ -572,9 +479,9 @@ __global__ void force_bias_kernel(int n, int ne, int64_t W, int nchol, const cd 
 
 size_t grad_group_layout(GradArgs &A) {
     const int n = A.n, m = A.m, T = tri_count(m), NB = A.NB, S = m / 2;
-    size_t o = align16((size_t)n * ld_ut(n) * sizeof(cd));
+    size_t o = align16((size_t)n * (n + 1) * sizeof(int4));
     A.off_Q = (int)o;
-    o = align16(o + (size_t)2 * n * ld_qt(n) * sizeof(cd));
+    o = align16(o + (size_t)(n * (n + 1) > T ? n * (n + 1) : T) * sizeof(int4));
     A.off_T = (int)o;
     o = align16(o + (size_t)n * ld_t(n) * sizeof(cd));
     A.off_B = (int)o;
@@ -585,7 +492,7 @@ size_t grad_group_layout(GradArgs &A) {
     o = align16(o + (size_t)n * n * sizeof(cd));
     A.off_NZ = (int)o;
     size_t nz = (size_t)NB * T;
-    if ((size_t)m * 2 * n > nz) nz = (size_t)m * 2 * n;
+    if ((size_t)m * n > nz) nz = (size_t)m * n;
     o = align16(o + nz * sizeof(cd));
     A.off_g1 = (int)o;
     o = align16(o + (size_t)NB * m * sizeof(cd));
@@ -611,8 +518,6 @@ size_t grad_group_layout(GradArgs &A) {
     o = align16(o + (size_t)NB * S);
     A.off_ph = (int)o;
     o = align16(o + (size_t)NB * S);
-    A.off_kc = (int)o;
-    o = align16(o + (size_t)2 * n);
     A.off_sacth = (int)o;
     o = align16(o + (size_t)(A.ne / 2 + 1) * m);
     A.off_skh = (int)o;
@@ -643,9 +548,7 @@ qcs_status qcs_launch_grad(qcs_ctx *ctx, const qcs_grad_launch &L, cudaStream_t 
     A.P = L.P;
     A.tab_bytes = (int)align16((size_t)tri_count(A.m) * sizeof(uint16_t));
     A.Ut = L.Ut;
-    A.Qt = L.s->Qt;
     A.Qh = L.s->Qh;
-    A.gth = L.s->gth;
     A.idx = L.s->idx;
     A.d_count = L.s->d_count;
     A.partial = L.partial;

@@ -331,6 +331,7 @@ __device__ inline void node_inverse(int m, int nb, cd *__restrict__ Ns, cd *__re
 // constant -1/a of each step scaled by c = sum_k c_k.
 
 struct SharedScratch {  // per-group scalars exchanged between the two warps
+    unsigned red[4];
     unsigned key[2];
     int flag, ak, ap, pad_;
     cd pf0;

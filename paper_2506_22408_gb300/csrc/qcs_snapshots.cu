@@ -168,7 +168,7 @@ __global__ void snapshot_compact_kernel(int64_t P, const int8_t *__restrict__ pa
     if (tid == 0) *count = base;
 }
 
-// Per dense snapshot (gather code 0xFF, or no codes): Qh = [H1^T; G2^T] (2n x n, Qt's
+// Per snapshot: Qh = [H1^T; G2^T] (2n x n, Qt's
 // layout) with H1 = Qt^T J Qt and G2 = Qt^T J conj(Qt) (n x n; J pairs the Majorana
 // indices 2a, 2a + 1 with J[2a][2a+1] = 1).  The FP64 ALU overlap kernel and the gradient
 // form K = Ut Qh^T = [Ut H1 | Ut G2] in place of T = Ut Qt^T, from which
@@ -176,14 +176,12 @@ __global__ void snapshot_compact_kernel(int64_t P, const int8_t *__restrict__ pa
 //     T_j J Qt = (Ut H1)[j],              T_j J conj(Qt) = (Ut G2)[j]
 // give B^(s) and the gradient's cotangents over n-term sums instead of 2n-term ones.
 // One block per snapshot (grid-stride), the snapshot's rows staged in shared memory.
-__global__ void hform_kernel(int n, int64_t P, const cd *__restrict__ Qt, const uint8_t *__restrict__ gth,
-                             cd *__restrict__ Qh, unsigned *status) {
+__global__ void hform_kernel(int n, int64_t P, const cd *__restrict__ Qt, cd *__restrict__ Qh, unsigned *status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cd *Qs = reinterpret_cast<cd *>(smem_raw);  // 2n x n
     const int n2 = 2 * n;
     if (!QCS_IN_BOUNDS((size_t)n2 * n * sizeof(cd) <= dyn_smem_bytes(), status)) return;
     for (int64_t q = blockIdx.x; q < P; q += gridDim.x) {
-        if (gth && gth[q * n2] != 0xFF) continue;  // signed permutation: its kernels gather instead
         __syncthreads();
         for (int e = threadIdx.x; e < n2 * n; e += blockDim.x) Qs[e] = Qt[q * n2 * n + e];
         __syncthreads();
@@ -241,6 +239,6 @@ qcs_status qcs_hform_prepare_snapshots(qcs_ctx *ctx, qcs_snapshots *s, cudaStrea
     if (qcs_set_smem(ctx, (const void *)hform_kernel, smem) != QCS_OK) return QCS_ERR_CUDA;
     int64_t blocks = (int64_t)ctx->num_sms * 8;
     if (blocks > s->P) blocks = s->P;
-    hform_kernel<<<(unsigned)blocks, 256, smem, st>>>(n, s->P, s->Qt, s->gth, s->Qh, ctx->d_status);
+    hform_kernel<<<(unsigned)blocks, 256, smem, st>>>(n, s->P, s->Qt, s->Qh, ctx->d_status);
     return qcs_check_launch(ctx, "hform_kernel");
 }
