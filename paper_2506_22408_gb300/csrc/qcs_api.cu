@@ -765,7 +765,7 @@ static double grad_B_from_T_flops(int n, int ne) {
     return 8.0 * 2.0 * n * tri_count(ne) + 4.0 * 2.0 * n * ne * 2 * d + 2.0 * 2.0 * n * tri_count(2 * d);
 }
 
-// B from K in the two-warp overlap kernel above 16 modes (build_B_from_K of qcs_pair.cuh):
+// B from K in the two-warp overlap kernel above 16 modes (fx_build_B_from_K):
 // each sum runs over the non-zero columns of its walker row with three real products per
 // term (6 flop) and three additions per sum: occupied pairs W1 alone over the reduced row's
 // 1 + d columns; completion row ne + j carries ne + j + 1 items of W1 and W2 over n - j

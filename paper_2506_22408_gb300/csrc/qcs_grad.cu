@@ -21,31 +21,24 @@
 // (qcs_walker.cu): U_occ = U_qr W, and R above is W^H R_qr, so the epilogue
 // takes adj(R_qr) det(conj W) W and det(conj W) det(R_qr).
 //
-// A'_k^{-1} is recomputed per pair and node, never stored in global memory: the
-// Parlett-Reid elimination (as in the overlap kernel, original index order)
-// leaves its Gauss vectors in place, and a backward recursion over the
-// elimination steps assembles the inverse from the 2x2 pivot blocks:
-//     (A^{-1})_{rest,k} = -Z g1,  (A^{-1})_{rest,p} = -Z g2,
-//     (A^{-1})_{k,p} = -1/a + g1^T Z g2,  g1 = v/a, g2 = -u/a,
-// where Z is the inverse of the step's Schur complement and (u, v, a) the
-// step's pivot columns and pivot.  The node matrices share their occupied block, so
-// its steps are taken once per pair (shared_factor); each node then factors and
-// inverts only its 2d x 2d complement, and since every backward step is affine in Z,
-// one backward pass over the shared steps, started from sum_k c_k Z_k, gives
-// Y_p = sum_k c_k A'_k^{-1} (shared_inverse).  Pairs whose occupied block would grow
-// the complement beyond 2^8 of max|B| take the full elimination per node.
+// A'_k^{-1} is recomputed per pair and node, never stored in global memory, by sweeps in
+// 64-bit fixed point (qcs_fxsweep.cuh): the occupied block, which the node matrices share,
+// once per pair; then each node's complement as a whole; then Y_p = sum_k c_k A'_k^{-1} from
+// the blocks, which is affine in the complements' inverses (grad_sweeps).  Pairs that the
+// sweeps refuse (vanishing pivots, singular node matrices) take an FP64 factorisation and
+// backward recursion per node (grad_full_nodes).
 #include "qcs_internal.h"
 #include "qcs_fxcong.cuh"
+#include "qcs_fxsweep.cuh"
 #include "qcs_group.cuh"
 
 namespace {
 
 struct GradArgs {
-    int n, ne, m, d, nev, NB, all, chunk, nchunks;
+    int n, ne, m, d, nev, NB, nz, nv, all, chunk, nchunks;
     int64_t W, P;
     int group_bytes, tab_bytes;
-    int off_Q, off_T, off_B, off_Y, off_G, off_NZ, off_g1, off_g2, off_y1, off_y2, off_pf, off_cf, off_invh,
-        off_int, off_tile, off_acth, off_kh, off_ph, off_sacth, off_skh, off_sph, off_sinvh, off_scr;
+    int off_Q, off_T, off_NZ, off_g, off_pv, off_pe, off_se, off_perm, off_cf, off_invh, off_hist, off_scr;
     const cd *Ut;
     const cd *Qh;        // per snapshot of the set: the rows [H1^T; G2^T] (2n x n, the layout of Qt)
     const int *idx;
@@ -53,19 +46,268 @@ struct GradArgs {
     cd *partial;
     unsigned long long *counter;  // tile counter: groups pull tiles dynamically
     unsigned *status;
+    FxPlan plan;
     cd wnode[QCS_MAX_NODES];
     cd gamma[QCS_MAX_NODES];
 };
+
+struct GradShared {  // per-group scalars exchanged between the two warps
+    unsigned red[4];
+    int bad[kMaxNBG], pos;
+    long long slot;
+    cd pf;
+};
+
+// Y = (1/2) sum_k gamma_k pf_k A'_k^{-1} in FP64, every node matrix factored and inverted in
+// full, for pairs that the fixed-point sweeps refuse (small pivots, singular matrices).
+// Bs: B^(s), the occupied rows first.  Returns S_p on thread 0.
+static __device__ __noinline__ cd grad_full_nodes(const GradArgs &A, const cd *Bs, cd *Ys, cd *Ns, unsigned char *wb,
+                                                  const uint16_t *tab, int t, int bar) {
+    const int m = A.m, T = tri_count(m);
+    cd *vec = reinterpret_cast<cd *>(wb + A.off_g), *invh = reinterpret_cast<cd *>(wb + A.off_invh);
+    uint8_t *acth = wb + A.off_hist, *kh = acth + (m / 2 + 1) * m, *ph = kh + m / 2;
+    GradShared *scr = reinterpret_cast<GradShared *>(wb + A.off_scr);
+    cd S = cmk(0.0, 0.0);
+    for (int e = t; e < T; e += kGroup) Ys[e] = cmk(0.0, 0.0);
+    group_sync(bar);
+    for (int k = 0; k < A.nev; ++k) {
+        node_factor(m, A.ne, A.wnode + k, 1, Bs, Ns, vec, vec + m, &scr->pf, invh, &scr->pos, acth, kh, ph, tab, t, bar,
+                    A.status);
+        node_inverse(m, 1, Ns, vec, vec + m, vec + 2 * m, vec + 3 * m, invh, acth, kh, ph, t, bar);
+        const cd c = cmul(A.gamma[k], scr->pf), h = cscale(c, 0.5);
+        S = cadd(S, c);
+        for (int e = t; e < T; e += kGroup) {
+            cd y = Ys[e];
+            cfma(y, h, Ns[e]);
+            Ys[e] = y;
+        }
+        group_sync(bar);
+    }
+    return S;
+}
+
+// The same by fixed-point sweeps (qcs_fxsweep.cuh), from B^(s) in X (empties first, worth
+// X 2^-f, at most mb bits; overwritten).  The node matrices differ only in their empty x
+// empty block, so with the occupied block P swept once (all of it but for pairs of small
+// pivots, which stay with the empty modes' rows),
+//     [[C, E], [-E^T, Pi]],   C the Schur complement, E = B_eo P^-1, Pi = P^-1,
+// and Z_k = (C + w_k D)^-1 by one sweep of a whole matrix per node,
+//     A'_k^{-1} = [[Z_k, -Z_k E], [-E^T Z_k, Pi + E^T Z_k E]],
+// which is affine in Z_k: one assembly from Zc = sum_k c_k Z_k, c_k = gamma_k pf_k / 2.
+// Returns false (uniform over the group) when a sweep is refused or C exceeds 2^8 times B;
+// S = S_p on every thread.
+static __device__ __noinline__ bool grad_sweeps(const GradArgs &A, fx2 *X, cd *Ys, fx2 *Ns, unsigned char *wb, int f,
+                                                int mb, cd &S, const uint16_t *tab, int t, int bar) {
+    const int m = A.m, ne = A.ne, d2 = m - ne;
+    GradShared *scr = reinterpret_cast<GradShared *>(wb + A.off_scr);
+    const FxTeam<2> tm = {t, t & 31, t >> 5, bar, scr->red};
+    FxGauss *GV = reinterpret_cast<FxGauss *>(wb + A.off_g);
+    fx2 *pv = reinterpret_cast<fx2 *>(wb + A.off_pv);
+    int *pe = reinterpret_cast<int *>(wb + A.off_pe), *seo = reinterpret_cast<int *>(wb + A.off_se);
+    uint8_t *permo = wb + A.off_perm, *at = permo + m + A.nv;  // at: position of each index, per node
+    int8_t *dl = reinterpret_cast<int8_t *>(at + A.nv);
+    cd *cf = reinterpret_cast<cd *>(wb + A.off_cf);
+    const FxSweepWork wo = {GV, pv, pe, scr->bad, seo, dl, permo};
+    const FxSweepWork wn = {GV, pv + ne / 2, pe + ne / 2, scr->bad, seo + m, dl, permo + m};
+    const int bound = mb - f + 8;
+    const FxSwept o = fx_sweep(tm, m, d2, true, 1, X, f, mb, wo, tab);
+    if (o.mb < 0) return false;
+    f = o.f;
+    // rows and columns of C: md positions; of Pi: no
+    const int md = d2 + o.left, no = ne - o.left, npo = no / 2, Tn = tri_count(md);
+    // selected row at position x
+    auto sel = [&](int x) { return x < d2 ? ne + x : permo[x] - d2; };
+    auto put = [&](int x, int y, cd v) {  // A^-1 at positions (x, y), to selected rows
+        const int a = sel(x), b = sel(y);
+        Ys[a < b ? tri_index(a, b) : tri_index(b, a)] = flip_if(v, a > b);
+    };
+    // scales of C (room for w_k, of modulus one) and E
+    int sb = -0x10000, eb = -0x10000;
+    for (int e = t; e < Tn; e += kGroup) {
+        int a, b;
+        pair_of(tab, e, a, b);
+        sb = max(sb, fx_bits(X[e]) - seo[a] - seo[b]);
+        put(a, b, cmk(0.0, 0.0));
+    }
+    for (int e = t; e < md * no; e += kGroup) {
+        const int c = e / md, i = e - c * md;
+        eb = max(eb, fx_bits(X[tri_index(i, md + c)]) - seo[i]);
+    }
+    sb = __reduce_max_sync(QCS_FULL, sb);
+    eb = __reduce_max_sync(QCS_FULL, eb);
+    group_sync(bar);
+    if (tm.lane == 0) {
+        scr->red[tm.wid] = (unsigned)sb;
+        scr->red[2 + tm.wid] = (unsigned)eb;
+    }
+    group_sync(bar);
+    sb = max((int)scr->red[0], (int)scr->red[1]);
+    eb = max((int)scr->red[2], (int)scr->red[3]);
+    if (md > 0 && sb - f > bound) return false;
+    int fn = f + kFxTop - sb;
+    fn = fn < kFxTop ? fn : kFxTop;
+    int NB = A.NB;
+    if (md > d2) {
+        if (NB * Tn > A.nz) NB = A.nz / Tn;
+        if (NB * md > A.nv) NB = A.nv / md;
+    }
+    cd csum = cmk(0.0, 0.0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < A.nev; k0 += NB) {
+        const int nb = A.nev - k0 < NB ? A.nev - k0 : NB;
+        FxSwept z = {0, 0, 0};
+        if (md > 0) {
+#pragma unroll 1
+            for (int e = t; e < Tn; e += kGroup) {
+                int a, b;
+                pair_of(tab, e, a, b);
+                const fx2 x = fx_shift(X[e], fn - f - seo[a] - seo[b]);
+                const bool dd = (a & 1) == 0 && b == a + 1 && b < d2;
+                for (int w = 0; w < nb; ++w) {
+                    fx2 y = x;
+                    if (dd) {
+                        const fx2 d = fx_shift(A.plan.w[k0 + w], fn - kFxTop);
+                        y = make_longlong2(x.x + d.x, x.y + d.y);
+                    }
+                    Ns[w * Tn + e] = y;
+                }
+            }
+            z = fx_sweep(tm, md, 0, false, nb, Ns, fn, kFxTop + 1, wn, tab);
+            if (z.mb < 0) return false;
+        }
+        int v;
+        bool lead;
+        const cd c = fx_sweep_product(tm, nb, md / 2, wn, npo, pv, pe, A.plan.g + k0, A.plan.ge + k0, v, lead);
+        if (lead) cf[v] = cscale(c, 0.5);
+        for (int e = t; e < nb * md; e += kGroup) {
+            const int w = e / md;
+            at[w * md + wn.perm[e]] = (uint8_t)(e - w * md);
+        }
+        group_sync(bar);
+        for (int w = 0; w < nb; ++w) csum = cadd(csum, cf[w]);
+#pragma unroll 1
+        for (int e = t; e < Tn; e += kGroup) {
+            int a, b;
+            pair_of(tab, e, a, b);
+            cd y = cmk(0.0, 0.0);
+#pragma unroll 1
+            for (int w = 0; w < nb; ++w) {
+                const int i = at[w * md + a], j = at[w * md + b];
+                const fx2 x = fx_neg_if(Ns[w * Tn + (i < j ? tri_index(i, j) : tri_index(j, i))], i > j);
+                const int E = -z.f - wn.se[w * md + i] - wn.se[w * md + j];
+                cfma(y, cf[w], cmk(fx_f64(x.x, E), fx_f64(x.y, E)));
+            }
+            put(a, b, k0 == 0 ? y : cadd(y, skew_at(Ys, sel(a), sel(b))));
+        }
+        group_sync(bar);
+    }
+    S = cscale(csum, 2.0);
+    if (no == 0) return true;
+    // F = Zc E (worth F 2^{-fF - se_c} in column c)
+    unsigned kz = 0u;
+    for (int e = t; e < Tn; e += kGroup) {
+        int a, b;
+        pair_of(tab, e, a, b);
+        kz = max(kz, pivot_key(skew_at(Ys, sel(a), sel(b))));
+    }
+    kz = __reduce_max_sync(QCS_FULL, kz);
+    if (tm.lane == 0) scr->red[tm.wid] = kz;
+    group_sync(bar);
+    kz = max(scr->red[0], scr->red[1]);
+    if (kz >= 0x7ff00000u) return false;
+    const int fz = fx_fraction(kz, 56), fE = f + 56 - eb;
+    const int dn = 51 + (md > 1 ? 32 - __clz(md - 1) : 0);  // md products of 2^113 stay below 2^63
+    int4 *Zl = reinterpret_cast<int4 *>(Ns), *El = Zl + Tn, *Fl = El + md * no;
+    for (int e = t; e < Tn; e += kGroup) {
+        int a, b;
+        pair_of(tab, e, a, b);
+        Zl[e] = fx_limbs(skew_at(Ys, sel(a), sel(b)), fz);
+    }
+    for (int e = t; e < md * no; e += kGroup) {
+        const int c = e / md, i = e - c * md;
+        const fx2 x = fx_shift(X[tri_index(i, md + c)], 56 - eb - seo[i]);
+        El[e] = fx_pack(fx_split<kFxS>(x.x), fx_split<kFxS>(x.y));
+    }
+    group_sync(bar);
+    unsigned top = 0u;
+#pragma unroll 1
+    for (int e = t; e < md * no; e += kGroup) {
+        const int c = e / md, i = e - c * md;
+        const int4 *er = El + c * md, *zr = Zl + tri_count(i);
+        fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
+        for (int j = 0; j < md; ++j) {
+            if (j == i) {  // below: -Z_ij = Z_ji; from here on Z_ij
+                p1 = fx_accsub(fxacc{0, 0}, p1);
+                p2 = fx_accsub(fxacc{0, 0}, p2);
+                p3 = fx_accsub(fxacc{0, 0}, p3);
+                continue;
+            }
+            const int4 z = j < i ? zr[j] : Zl[tri_count(j) + i], x = er[j];
+            fx_mac(p1, fx_re(z), fx_re(x));
+            fx_mac(p2, fx_im(z), fx_im(x));
+            fx_mac(p3, fx_add(fx_re(z), fx_im(z)), fx_add(fx_re(x), fx_im(x)));
+        }
+        fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
+        re.cr += fx_half<kFxS>(dn);
+        im.cr += fx_half<kFxS>(dn);
+        const fx2 F = make_longlong2(fx_value<kFxS>(re, dn), fx_value<kFxS>(im, dn));
+        top |= fx_top(F);
+        X[tri_index(i, md + c)] = F;
+    }
+    top = tm.or_put(top, 1);
+    group_sync(bar);
+    const int fb = fx_top_bits(tm.or_get(top, 1)), fF = fz + fE - dn;
+#pragma unroll 1
+    for (int e = t; e < md * no; e += kGroup) {
+        const int c = e / md, i = e - c * md;
+        const fx2 F = X[tri_index(i, md + c)], x = fx_shift(F, 56 - fb);
+        Fl[e] = fx_pack(fx_split<kFxS>(x.x), fx_split<kFxS>(x.y));
+        const int E = -fF - seo[md + c];
+        put(i, md + c, cmk(-fx_f64(F.x, E), -fx_f64(F.y, E)));
+    }
+    group_sync(bar);
+    const int fP = fE + fF + 56 - fb - dn;
+#pragma unroll 1
+    for (int e = t; e < tri_count(no); e += kGroup) {
+        int c, c2;
+        pair_of(tab, e, c, c2);
+        fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
+        for (int i = 0; i < md; ++i) {
+            const int4 z = El[c * md + i], x = Fl[c2 * md + i];
+            fx_mac(p1, fx_re(z), fx_re(x));
+            fx_mac(p2, fx_im(z), fx_im(x));
+            fx_mac(p3, fx_add(fx_re(z), fx_im(z)), fx_add(fx_re(x), fx_im(x)));
+        }
+        fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
+        re.cr += fx_half<kFxS>(dn);
+        im.cr += fx_half<kFxS>(dn);
+        const int sc = seo[md + c] + seo[md + c2];
+        const fx2 pi = X[tri_index(md + c, md + c2)];
+        cd y = cmul(csum, cmk(fx_f64(pi.x, -f - sc), fx_f64(pi.y, -f - sc)));
+        y.x += fx_f64(fx_value<kFxS>(re, dn), -fP - sc);
+        y.y += fx_f64(fx_value<kFxS>(im, dn), -fP - sc);
+        put(md + c, md + c2, y);
+    }
+    group_sync(bar);
+    return true;
+}
 
 // Two warps (a group of 64 threads) per pair; a block holds blockDim/64 groups,
 // each with its own workspace and named barrier.  Groups pull (walker, chunk)
 // tiles from a device counter in chunk-major order.
 //
-// Bound by the FP64 pipe (76 clocks per DFMA and 32 lanes): at 16 modes and 8 electrons a
-// pair took 190k FP64 operations, 107k of them in K, B^(s) and the cotangent products.  Those
-// three are in fixed point on the integer pipe (qcs_fxcong.cuh): 606 -> 490 ms for 512
-// walkers against 10,000 snapshots.
-__global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant__ GradArgs A) {
+// In FP64 a pair at 16 modes and 8 electrons took 190k operations on a pipe that issues 32
+// lanes per 76 clocks: 606 ms for 512 walkers against 10,000 snapshots.  K, B^(s) and the
+// cotangent products as two-limb integers: 490 ms.  The inverses by fixed-point sweeps:
+// 343 ms, now 33k instructions a pair at an issue rate of 45 %, bound by latency (dependent
+// multiply-adds, pivot searches and the barriers of each sweep step).  Of that, K and B take
+// a seventh, the occupied sweeps a sixth, the nodes a third, the assembly of Y a fifth and
+// the cotangents a sixth.  Four blocks of two groups per SM (128 registers, 28 KB a group:
+// Y in the walker rows' place, which are staged anew for each pair, and the cotangents
+// accumulated in global memory) against three: 1.03x, 1.08x at 10 modes.
+__global__ void __launch_bounds__(128, 4) grad_pair_kernel(const __grid_constant__ GradArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / kGroup;
     const int t = threadIdx.x - gid * kGroup;
@@ -85,35 +327,17 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
     int4 *Qs = reinterpret_cast<int4 *>(wb + A.off_Q);   // half of the snapshot's rows as limbs
     fx2 *Xs = reinterpret_cast<fx2 *>(wb + A.off_Q);     // B^(s) in fixed point, once K is formed
     int4 *Ks = reinterpret_cast<int4 *>(wb + A.off_T);   // K as limbs
-    cd *Bs = reinterpret_cast<cd *>(wb + A.off_B);
-    cd *Ys = reinterpret_cast<cd *>(wb + A.off_Y);
-    cd *Gs = reinterpret_cast<cd *>(wb + A.off_G);
-    cd *Ns = reinterpret_cast<cd *>(wb + A.off_NZ);  // node factors, then their inverses, then the coefficients
-    cd *g1v = reinterpret_cast<cd *>(wb + A.off_g1);  // forward: U vectors
-    cd *g2v = reinterpret_cast<cd *>(wb + A.off_g2);  // forward: V vectors
-    cd *y1v = reinterpret_cast<cd *>(wb + A.off_y1);
-    cd *y2v = reinterpret_cast<cd *>(wb + A.off_y2);
-    cd *pf = reinterpret_cast<cd *>(wb + A.off_pf);
-    cd *cf = reinterpret_cast<cd *>(wb + A.off_cf);
-    cd *invh = reinterpret_cast<cd *>(wb + A.off_invh);
-    int *pos = reinterpret_cast<int *>(wb + A.off_int);
-    long long *slot = reinterpret_cast<long long *>(wb + A.off_tile);
-    uint8_t *acth = wb + A.off_acth;
-    uint8_t *kh = wb + A.off_kh;
-    uint8_t *ph = wb + A.off_ph;
-    uint8_t *sacth = wb + A.off_sacth;  // history of the shared occupied-block elimination
-    uint8_t *skh = wb + A.off_skh;
-    uint8_t *sph = wb + A.off_sph;
-    cd *sinvh = reinterpret_cast<cd *>(wb + A.off_sinvh);
-    SharedScratch *scr = reinterpret_cast<SharedScratch *>(wb + A.off_scr);
+    cd *Ys = reinterpret_cast<cd *>(wb);  // in the walker rows' place, once B^(s) is formed
+    cd *Ns = reinterpret_cast<cd *>(wb + A.off_NZ);  // node matrices, then their inverses, then the coefficients
+    GradShared *scr = reinterpret_cast<GradShared *>(wb + A.off_scr);
 
     const int64_t L = A.all ? A.P : (int64_t)(*A.d_count);
     const int64_t ntiles = A.W * A.nchunks;
     const size_t rec = 1 + (size_t)n * n;
     for (;;) {
-        if (t == 0) *slot = (long long)atomicAdd(A.counter, 1ull);
+        if (t == 0) scr->slot = (long long)atomicAdd(A.counter, 1ull);
         group_sync(bar);
-        const int64_t tile = (int64_t)*slot;  // rewritten only after the barriers below
+        const int64_t tile = (int64_t)scr->slot;  // rewritten only after the barriers below
         if (tile >= ntiles) break;
         const int ch = (int)(tile / A.W);  // chunk-major: a snapshot chunk is fetched once
         const int64_t w = tile - (int64_t)ch * A.W;
@@ -123,13 +347,12 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
             group_sync(bar);  // every thread has read the slot before it is rewritten
             continue;
         }
-        cd *out = A.partial + (w * A.nchunks + ch) * rec;
+        cd *out = A.partial + (w * A.nchunks + ch) * rec, *Gs = out + 1;  // entry e: thread e mod 64
         cd Ssum = cmk(0.0, 0.0);
         for (int e = t; e < n * n; e += kGroup) Gs[e] = cmk(0.0, 0.0);
         if (p0 < L) {
             const cd *Utw = A.Ut + w * n * n;
             const int fU = fx_fraction(fx_max_key(Utw, n * n, t & 31), 57);
-            fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, t, kGroup);
             for (int64_t pq = p0; pq < p1; ++pq) {
                 const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
                 if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // group-uniform
@@ -149,6 +372,7 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
                 const int fQ = fx_fraction(key, 57);
                 const FxTeam<2> tm = {t, t & 31, t >> 5, bar, scr->red};
                 unsigned top = 0u;
+                fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, t, kGroup);
                 for (int h = 0; h < 2; ++h) {
                     fx_stage_rows(n, n * n, Qr + (int64_t)h * n * n, fQ, nullptr, Qs, t, kGroup);
                     group_sync(bar);
@@ -161,72 +385,28 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
                 const int fK = fU + fQ - 58 + 56 - kb;
                 fx_T_limbs(n, Ks, kb, t, kGroup);
                 group_sync(bar);
-                fx_build_B_from_K(n, ne, Us, Ks, Xs, tab, t, kGroup);
+                top = tm.or_put(fx_build_B_from_K(n, ne, Us, Ks, Xs, tab, t, kGroup), 1);
                 group_sync(bar);
-                for (int e = t; e < T; e += kGroup) {  // to FP64, the occupied rows first
-                    int a, b;
-                    pair_of(tab, e, a, b);
-                    const int i = a < m - ne ? a + ne : a - (m - ne), j = b < m - ne ? b + ne : b - (m - ne);
-                    const fx2 x = Xs[e];
-                    const cd v = flip_if(cmk(fx_f64(x.x, 58 - fK - fU), fx_f64(x.y, 58 - fK - fU)), i > j);
-                    Bs[i < j ? tri_index(i, j) : tri_index(j, i)] = v;
-                }
-                group_sync(bar);
-                cd S = cmk(0.0, 0.0);
-                // Y = (1/2) sum_k gamma_k pf_k A_k^{-1}: block form when the occupied block
-                // eliminates stably (shared_factor), else every node matrix in full
-                if (shared_factor(m, ne, Bs, Ys, g1v, g2v, sinvh, sacth, skh, sph, scr, tab, t, bar)) {
-                    const int md = m - ne, Tn = tri_count(md);
-                    const cd pf0 = scr->pf0;
-                    for (int e = t; e < Tn; e += kGroup) {  // S0 to Bs; Zc accumulates in its place
+                const int fB = fK + fU - 58;
+                cd S;
+                if (!grad_sweeps(A, Xs, Ys, reinterpret_cast<fx2 *>(Ns), wb, fB, fx_top_bits(tm.or_get(top, 1)), S, tab,
+                                 t, bar)) {
+                    group_sync(bar);
+                    fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, t, kGroup);
+                    group_sync(bar);
+                    fx2 *Bx = reinterpret_cast<fx2 *>(Ns);
+                    cd *Bs = reinterpret_cast<cd *>(Xs);
+                    fx_build_B_from_K(n, ne, Us, Ks, Bx, tab, t, kGroup);
+                    group_sync(bar);
+                    for (int e = t; e < T; e += kGroup) {  // to FP64, the occupied rows first
                         int a, b;
                         pair_of(tab, e, a, b);
-                        cd *y = Ys + tri_index(ne + a, ne + b);
-                        Bs[e] = *y;
-                        *y = cmk(0.0, 0.0);
+                        const int i = a < m - ne ? a + ne : a - (m - ne), j = b < m - ne ? b + ne : b - (m - ne);
+                        const cd v = flip_if(cmk(fx_f64(Bx[e].x, -fB), fx_f64(Bx[e].y, -fB)), i > j);
+                        Bs[i < j ? tri_index(i, j) : tri_index(j, i)] = v;
                     }
                     group_sync(bar);
-                    cd csum = cmk(0.0, 0.0);
-                    for (int k0 = 0; k0 < A.nev; k0 += A.NB) {
-                        const int nb = A.nev - k0 < A.NB ? A.nev - k0 : A.NB;
-                        node_factor(md, 0, A.wnode + k0, nb, Bs, Ns, g1v, g2v, pf, invh, pos, acth, kh, ph, tab, t,
-                                    bar, A.status);
-                        node_inverse(md, nb, Ns, g1v, g2v, y1v, y2v, invh, acth, kh, ph, t, bar);
-                        if (t < nb) cf[t] = cscale(cmul(A.gamma[k0 + t], cmul(pf0, pf[t])), 0.5);
-                        if (t == 0)
-                            for (int v = 0; v < nb; ++v) cfma(S, A.gamma[k0 + v], cmul(pf0, pf[v]));
-                        group_sync(bar);
-                        for (int v = 0; v < nb; ++v) csum = cadd(csum, cf[v]);
-                        for (int e = t; e < Tn; e += kGroup) {
-                            int a, b;
-                            pair_of(tab, e, a, b);
-                            cd *yp = Ys + tri_index(ne + a, ne + b);
-                            cd y = *yp;
-                            for (int v = 0; v < nb; ++v) cfma(y, cf[v], Ns[v * Tn + e]);
-                            *yp = y;
-                        }
-                        group_sync(bar);
-                    }
-                    shared_inverse(m, ne, Ys, g1v, g2v, y1v, y2v, sinvh, sacth, skh, sph, csum, scr, t, bar);
-                } else {
-                    for (int e = t; e < T; e += kGroup) Ys[e] = cmk(0.0, 0.0);
-                    group_sync(bar);
-                    for (int k0 = 0; k0 < A.nev; k0 += A.NB) {
-                        const int nb = A.nev - k0 < A.NB ? A.nev - k0 : A.NB;
-                        node_factor(m, ne, A.wnode + k0, nb, Bs, Ns, g1v, g2v, pf, invh, pos, acth, kh, ph, tab, t,
-                                    bar, A.status);
-                        node_inverse(m, nb, Ns, g1v, g2v, y1v, y2v, invh, acth, kh, ph, t, bar);
-                        if (t < nb) cf[t] = cscale(cmul(A.gamma[k0 + t], pf[t]), 0.5);
-                        if (t == 0)
-                            for (int v = 0; v < nb; ++v) cfma(S, A.gamma[k0 + v], pf[v]);
-                        group_sync(bar);
-                        for (int e = t; e < T; e += kGroup) {
-                            cd y = Ys[e];
-                            for (int v = 0; v < nb; ++v) cfma(y, cf[v], Ns[v * T + e]);
-                            Ys[e] = y;
-                        }
-                        group_sync(bar);
-                    }
+                    S = grad_full_nodes(A, Bs, Ys, Ns, wb, tab, t, bar);
                 }
                 if (t == 0) {
                     if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
@@ -314,7 +494,6 @@ __global__ void __launch_bounds__(128, 2) grad_pair_kernel(const __grid_constant
             }
         }
         group_sync(bar);
-        for (int e = t; e < n * n; e += kGroup) out[1 + e] = Gs[e];
         if (t == 0) out[0] = Ssum;
     }
 }
@@ -479,55 +658,44 @@ __global__ void force_bias_kernel(int n, int ne, int64_t W, int nchol, const cd 
 
 size_t grad_group_layout(GradArgs &A) {
     const int n = A.n, m = A.m, T = tri_count(m), NB = A.NB, S = m / 2;
-    size_t o = align16((size_t)n * (n + 1) * sizeof(int4));
+    const size_t rows = (size_t)(n * (n + 1) > T ? n * (n + 1) : T) * sizeof(int4);
+    size_t o = align16(rows);  // the walker's rows, then Y
     A.off_Q = (int)o;
-    o = align16(o + (size_t)(n * (n + 1) > T ? n * (n + 1) : T) * sizeof(int4));
+    o = align16(o + rows);
     A.off_T = (int)o;
     o = align16(o + (size_t)n * ld_t(n) * sizeof(cd));
-    A.off_B = (int)o;
-    o = align16(o + (size_t)T * sizeof(cd));
-    A.off_Y = (int)o;
-    o = align16(o + (size_t)T * sizeof(cd));
-    A.off_G = (int)o;
-    o = align16(o + (size_t)n * n * sizeof(cd));
     A.off_NZ = (int)o;
-    size_t nz = (size_t)NB * T;
-    if ((size_t)m * n > nz) nz = (size_t)m * n;
+    // node matrices and their entries per round, one occupied pair left to them; also B in
+    // full, the assembly's limbs for any number of such pairs, the coefficients
+    const int md = m - A.ne, mx = md + (A.ne > 0 ? 2 : 0), nv = NB * mx > m ? NB * mx : m;
+    int nz = NB * tri_count(mx);
+    if (T > nz) nz = T;
+    for (int left = 0; left <= A.ne; left += 2) {
+        const int need = tri_count(md + left) + 2 * (md + left) * (A.ne - left);
+        if (need > nz) nz = need;
+    }
+    if (m * n > nz) nz = m * n;
+    A.nz = nz;
+    A.nv = nv;
     o = align16(o + nz * sizeof(cd));
-    A.off_g1 = (int)o;
-    o = align16(o + (size_t)NB * m * sizeof(cd));
-    A.off_g2 = (int)o;
-    o = align16(o + (size_t)NB * m * sizeof(cd));
-    A.off_y1 = (int)o;
-    o = align16(o + (size_t)NB * m * sizeof(cd));
-    A.off_y2 = (int)o;
-    o = align16(o + (size_t)NB * m * sizeof(cd));
-    A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(cd));
+    A.off_g = (int)o;  // Gauss vectors; the four vectors of grad_full_nodes
+    o = align16(o + (size_t)(nv > 2 * m ? nv : 2 * m) * sizeof(FxGauss));
+    A.off_pv = (int)o;
+    o = align16(o + (size_t)(A.ne / 2 + nv / 2) * sizeof(fx2));
+    A.off_pe = (int)o;
+    o = align16(o + (size_t)(A.ne / 2 + nv / 2) * sizeof(int));
+    A.off_se = (int)o;
+    o = align16(o + (size_t)(m + nv) * sizeof(int));
+    A.off_perm = (int)o;
+    o = align16(o + (size_t)m + 3 * nv);
     A.off_cf = (int)o;
     o = align16(o + (size_t)kMaxNBG * sizeof(cd));
     A.off_invh = (int)o;
-    o = align16(o + (size_t)NB * S * sizeof(cd));
-    A.off_int = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(int));
-    A.off_tile = (int)o;
-    o = align16(o + sizeof(long long));
-    A.off_acth = (int)o;
-    o = align16(o + (size_t)NB * (S + 1) * m);
-    A.off_kh = (int)o;
-    o = align16(o + (size_t)NB * S);
-    A.off_ph = (int)o;
-    o = align16(o + (size_t)NB * S);
-    A.off_sacth = (int)o;
-    o = align16(o + (size_t)(A.ne / 2 + 1) * m);
-    A.off_skh = (int)o;
-    o = align16(o + (size_t)A.ne / 2);
-    A.off_sph = (int)o;
-    o = align16(o + (size_t)A.ne / 2);
-    A.off_sinvh = (int)o;
-    o = align16(o + (size_t)(A.ne / 2) * sizeof(cd));
+    o = align16(o + (size_t)S * sizeof(cd));
+    A.off_hist = (int)o;
+    o = align16(o + (size_t)(S + 1) * m + 2 * S);
     A.off_scr = (int)o;
-    o = align16(o + sizeof(SharedScratch));
+    o = align16(o + sizeof(GradShared));
     return o;
 }
 
@@ -554,12 +722,13 @@ qcs_status qcs_launch_grad(qcs_ctx *ctx, const qcs_grad_launch &L, cudaStream_t 
     A.partial = L.partial;
     A.counter = L.counter;
     A.status = ctx->d_status;
+    fx_make_plan(L.plan, A.plan);
     for (int k = 0; k < L.plan.nev; ++k) {
         A.wnode[k] = L.plan.wnode[k];
         A.gamma[k] = L.plan.gamma[k];
     }
     // Node matrices per round (NB) and groups per block: the most resident groups
-    // (at most 4 per SM, i.e. two warps per SM sub-partition), then the largest NB.
+    // (at most 8 per SM, i.e. four warps per SM sub-partition), then the largest NB.
     int best_nb = 0, best_g = 1, best_score = -1;
     const int nbmax = L.plan.nev < kMaxNBG ? L.plan.nev : kMaxNBG;
     for (int nb = nbmax; nb >= 1; --nb) {
@@ -569,9 +738,9 @@ qcs_status qcs_launch_grad(qcs_ctx *ctx, const qcs_grad_launch &L, cudaStream_t 
             const size_t sm = (size_t)A.tab_bytes + (size_t)g * gb;
             if (sm > ctx->smem_optin) continue;
             int per_sm = (int)(ctx->smem_per_sm / (sm + 1024));
-            if (per_sm > 2) per_sm = 2;
+            if (per_sm > 4) per_sm = 4;
             int groups = per_sm * g;
-            if (groups > 4) groups = 4;
+            if (groups > 8) groups = 8;
             const int score = groups * 16 + nb;
             if (per_sm >= 1 && score > best_score) {
                 best_score = score;
