@@ -30,10 +30,14 @@
 // the pair costs O(m^2 n + m^2 d + nodes d^3).  The second-order term's sum_gamma X'_g J X'_g^T is
 // K Lambda_p K^T with Lambda_p = sum_gamma ell_gamma G_p ell_gamma^T formed once per
 // snapshot (energy_lambda_kernel).
+#include "qcs_fxcong.cuh"
 #include "qcs_group.cuh"
 #include "qcs_internal.h"
 
 namespace {
+
+constexpr int kMaxNBE = 8;  // node matrices per round, at most
+constexpr int kNan = 1 << 20;  // exponent of products of entries that are not finite
 
 struct EnergyArgs {
     int n, ne, m, d, nev, NB, nop, nchol, has_h, all, chunk, nchunks;
@@ -45,8 +49,10 @@ struct EnergyArgs {
     const cd *Qt;
     const int *idx;
     const int *d_count;
-    const cd *Kop;  // W x nop x m x 2n: K ell_o (o < nchol: Cholesky vectors; o = nchol: h)
-    const cd *K2;   // W x m x 2n: sum_gamma K ell_gamma^2
+    // W x (nop + 1) x m x 2n, as limbs: K ell_o (o < nchol: Cholesky vectors; o = nchol: h),
+    // then sum_gamma K ell_gamma^2; Kf: their fraction bits
+    const int4 *Kop;
+    const int *Kf;
     const cd *Kg;   // W x m x 2n: K, the walker's selected rows
     const cd *Lam;  // per parity +1 snapshot (list order): Lambda_p, packed upper 2n x 2n
     cd *partial;    // W x nchunks x 3: (sum o_p, sum first-derivative term, sum second-derivative term)
@@ -65,6 +71,35 @@ __device__ __forceinline__ cd group_sum(cd v, cd *red, int t, int bar) {
     const cd s = cadd(red[0], red[1]);
     group_sync(bar);
     return s;
+}
+
+// Fraction bits that bring the largest of count entries to 56 bits (a group maximum); an
+// entry that is not finite gives a value below -968.
+__device__ __forceinline__ int group_fraction(const cd *x, int count, unsigned *red, int t, int bar) {
+    unsigned k = 0u;
+    for (int e = t; e < count; e += kGroup) k = max(k, pivot_key(x[e]));
+    k = __reduce_max_sync(QCS_FULL, k);
+    if ((t & 31) == 0) red[t >> 5] = k;
+    group_sync(bar);
+    k = max(red[0], red[1]);
+    group_sync(bar);
+    return fx_fraction(k, 56);
+}
+
+// sum_e Z_e G_e over this thread's entries, as limbs (fractions fz and fg), in FP64.
+__device__ __forceinline__ cd limb_dot(const int4 *Z, const int4 *G, int count, int E, int t) {
+    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
+    for (int e = t; e < count; e += kGroup) {
+        const int4 z = Z[e], g = G[e];
+        fx_mac(p1, fx_re(z), fx_re(g));
+        fx_mac(p2, fx_im(z), fx_im(g));
+        fx_mac(p3, fx_add(fx_re(z), fx_im(z)), fx_add(fx_re(g), fx_im(g)));
+    }
+    fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
+    re.cr += fx_half<kFxS>(58);
+    im.cr += fx_half<kFxS>(58);
+    return cmk(fx_f64(fx_value<kFxS>(re, 58), E), fx_f64(fx_value<kFxS>(im, 58), E));
 }
 
 // Sacc = sum_gamma X'_g J X'_g^T = K Lambda_p K^T (packed upper, m x m), with Lambda_p
@@ -132,68 +167,98 @@ __device__ inline void build_Mt(int n, int ne, int m, const cd *__restrict__ Qs,
 }
 
 // A' = N - N^T with N = X' J X^T = Ks Mt^T (Ks: the operator's rows K ell staged in shared
-// memory, Mt from build_Mt), plus 2 Sacc on the A'' pass:
+// memory, Mt from build_Mt, both as limbs), plus 2 Sacc on the A'' pass:
 //     A'_ab = sum_mu Ks[a][mu] Mt[b][mu] - Ks[b][mu] Mt[a][mu],
 // in three uniform loops over the pairs a < b: both occupied, occupied x empty, both
 // empty.  The rows of Mt for empty modes are real, so products with them take two real
-// multiply-adds instead of four.
-__device__ inline void build_Ap(int n, int ne, int m, const cd *__restrict__ Ks, int lx, const cd *__restrict__ Mt,
-                                cd *__restrict__ Ap, const cd *__restrict__ Sacc, bool last,
-                                const uint16_t *__restrict__ tab, int t) {
+// products instead of three.  E: the products' exponent, 58 - fraction bits.
+__device__ inline void build_Ap(int n, int ne, int m, const int4 *__restrict__ Ks, int lx,
+                                const int4 *__restrict__ Mt, int E, cd *__restrict__ Ap, const cd *__restrict__ Sacc,
+                                bool last, const uint16_t *__restrict__ tab, int t) {
     const int n2 = 2 * n, d2 = m - ne, c1 = tri_count(ne), c2 = ne * d2, c3 = tri_count(d2);
-    auto finish = [&](int a, int b, cd v) {
+    auto finish = [&](int a, int b, fxacc re, fxacc im) {
+        re.cr += fx_half<kFxS>(58);
+        im.cr += fx_half<kFxS>(58);
+        cd v = cmk(fx_f64(fx_value<kFxS>(re, 58), E), fx_f64(fx_value<kFxS>(im, 58), E));
+        if (E == kNan) v = cmk(nan(""), nan(""));
         const int e = tri_index(a, b);
         if (last) v = cadd(v, cscale(Sacc[e], 2.0));
         Ap[e] = v;
     };
+#pragma unroll 1
     for (int u = t; u < c1; u += kGroup) {  // occupied x occupied: complex rows of Mt
         int a, b;
         pair_of(tab, u, a, b);
-        const cd *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
-        cd v = cmk(0.0, 0.0);
+        const int4 *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
+        fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
         for (int mu = 0; mu < n2; ++mu) {
-            cfma(v, ka[mu], mb[mu]);
-            cfms(v, kb[mu], ma[mu]);
+            const int4 x = ka[mu], y = mb[mu], k = kb[mu], z = ma[mu];
+            const int4 w = make_int4(-k.x, -k.y, -k.z, -k.w);
+            fx_mac(p1, fx_re(x), fx_re(y));
+            fx_mac(p2, fx_im(x), fx_im(y));
+            fx_mac(p3, fx_add(fx_re(x), fx_im(x)), fx_add(fx_re(y), fx_im(y)));
+            fx_mac(p1, fx_re(w), fx_re(z));
+            fx_mac(p2, fx_im(w), fx_im(z));
+            fx_mac(p3, fx_add(fx_re(w), fx_im(w)), fx_add(fx_re(z), fx_im(z)));
         }
-        finish(a, b, v);
+        finish(a, b, fx_accsub(p1, p2), fx_accsub(fx_accsub(p3, p1), p2));
     }
+#pragma unroll 1
     for (int u = t; u < c2; u += kGroup) {  // occupied a x empty b = ne + r
         const int a = u / d2, r = u - a * d2, b = ne + r;
-        const cd *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
-        cd v = cmk(0.0, 0.0);
+        const int4 *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
+        fxacc re = {0, 0}, im = {0, 0}, p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+#pragma unroll 1
         for (int mu = 0; mu < n2; ++mu) {
-            crfma(v, ka[mu], mb[mu].x);
-            cfms(v, kb[mu], ma[mu]);
+            const int4 x = ka[mu], w = kb[mu], z = ma[mu];
+            const fxl y = fx_re(mb[mu]);
+            fx_mac(re, fx_re(x), y);
+            fx_mac(im, fx_im(x), y);
+            fx_mac(p1, fx_re(w), fx_re(z));
+            fx_mac(p2, fx_im(w), fx_im(z));
+            fx_mac(p3, fx_add(fx_re(w), fx_im(w)), fx_add(fx_re(z), fx_im(z)));
         }
-        finish(a, b, v);
+        finish(a, b, fx_accsub(re, fx_accsub(p1, p2)), fx_accsub(im, fx_accsub(fx_accsub(p3, p1), p2)));
     }
+#pragma unroll 1
     for (int u = t; u < c3; u += kGroup) {  // empty x empty: real rows of Mt
         int ra, rb;
         pair_of(tab, u, ra, rb);
         const int a = ne + ra, b = ne + rb;
-        const cd *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
-        cd v = cmk(0.0, 0.0);
+        const int4 *ka = Ks + a * lx, *kb = Ks + b * lx, *ma = Mt + a * lx, *mb = Mt + b * lx;
+        fxacc re = {0, 0}, im = {0, 0};
+#pragma unroll 1
         for (int mu = 0; mu < n2; ++mu) {
-            crfma(v, ka[mu], mb[mu].x);
-            crfma(v, kb[mu], -ma[mu].x);
+            const int4 x = ka[mu], w = kb[mu];
+            const fxl y = fx_re(mb[mu]), z = fx_neg(fx_re(ma[mu]));
+            fx_mac(re, fx_re(x), y);
+            fx_mac(im, fx_im(x), y);
+            fx_mac(re, fx_re(w), z);
+            fx_mac(im, fx_im(w), z);
         }
-        finish(a, b, v);
+        finish(a, b, re, im);
     }
 }
 
 // Per pair, before the first operator: Mt into the X' region (free between the node
 // rounds and the operator loop), then into the snapshot-row and T regions, which are
 // contiguous and no longer needed for this pair.
-__device__ inline void stage_Mt(int n, int ne, int m, const cd *__restrict__ Qs, int lq, const cd *__restrict__ Ts,
-                                int lt, cd *__restrict__ X1, int lx, cd *__restrict__ Mt, int t, int bar) {
+// As limbs; returns their fraction bits.
+__device__ inline int stage_Mt(int n, int ne, int m, const cd *__restrict__ Qs, int lq, const cd *__restrict__ Ts,
+                               int lt, cd *__restrict__ X1, int lx, int4 *__restrict__ Mt, unsigned *red, int t,
+                               int bar) {
+    for (int a = t; a < m; a += kGroup) X1[a * lx + lx - 1] = cmk(0.0, 0.0);  // the rows' padding
     build_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, t);
     group_sync(bar);
-    for (int e = t; e < m * lx; e += kGroup) Mt[e] = X1[e];
+    const int f = group_fraction(X1, m * lx, red, t, bar);
+    for (int e = t; e < m * lx; e += kGroup) Mt[e] = fx_limbs(X1[e], f);
     group_sync(bar);
+    return f;
 }
 
 // The operator's rows K ell (global memory, m x 2n) into the X' region, row stride lx.
-__device__ inline void stage_Ko(int n, int m, const cd *__restrict__ Ko, cd *__restrict__ Ks, int lx, int t,
+__device__ inline void stage_Ko(int n, int m, const int4 *__restrict__ Ko, int4 *__restrict__ Ks, int lx, int t,
                                 int bar) {
     const int n2 = 2 * n;
     for (int e = t; e < m * n2; e += kGroup) {
@@ -203,6 +268,12 @@ __device__ inline void stage_Ko(int n, int m, const cd *__restrict__ Ko, cd *__r
     group_sync(bar);
 }
 
+// Per operator and pair the kernel forms A', W, G, H and the nodes' tr((Z G)^2): 110k FP64
+// multiply-adds at 16 modes, 8 electrons and 3 nodes, on a pipe that issues 32 of them per 76
+// clocks (555 ms for 64 walkers, 1000 snapshots of either parity and 64 vectors).  A' (47k)
+// and the traces (39k) run on the integer pipe as 56-bit numbers of two limbs, one scale per
+// matrix: 339 ms, the FP64 products W, G, V and H a third of it.  The operators' rows K ell
+// come from energy_prep_kernel as limbs already, since every pair of a walker stages them.
 __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_constant__ EnergyArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / kGroup;
@@ -239,7 +310,8 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
     uint8_t *kh = wb + A.off_kh;
     uint8_t *ph = wb + A.off_ph;
     cd *X1 = reinterpret_cast<cd *>(wb + A.off_X1);     // K ell (or K ell^2) rows, m x (2n+1)
-    cd *Mt = Qs;  // from the operator loop on: Mt (m x (2n+1)) over the snapshot-row and T regions
+    int4 *Kx = reinterpret_cast<int4 *>(X1);
+    int4 *Mt = reinterpret_cast<int4 *>(Qs);  // from the operator loop on: Mt (m x (2n+1)) over the snapshot-row and T regions
     cd *Ap = reinterpret_cast<cd *>(wb + A.off_Ap);     // A' (packed upper skew)
     cd *Sacc = reinterpret_cast<cd *>(wb + A.off_Sacc); // sum_gamma X'_g J X'_g^T (packed)
     cd *red = reinterpret_cast<cd *>(wb + A.off_red);   // 2 entries
@@ -264,8 +336,8 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
         cd So = cmk(0.0, 0.0), S1 = cmk(0.0, 0.0), S2 = cmk(0.0, 0.0);
         if (p0 < L) {
             const cd *Utw = A.Ut + w * n * n;
-            const cd *Kw = A.Kop + (size_t)w * A.nop * m * n2;
-            const cd *K2w = A.K2 + (size_t)w * m * n2;
+            const int4 *Kw = A.Kop + (size_t)w * (A.nop + 1) * m * n2;
+            const int *Kfw = A.Kf + w * (A.nop + 1);
             const cd *Kgw = A.Kg + (size_t)w * m * n2;
             for (int64_t pq = p0; pq < p1; ++pq) {
                 const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
@@ -278,6 +350,7 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                 group_sync(bar);
                 build_B(n, ne, Ts, Bs, tab, t, kGroup);
                 group_sync(bar);
+                int fm = 0;  // fraction bits of Mt
                 cd Sop = cmk(0.0, 0.0), S1p = cmk(0.0, 0.0), S2p = cmk(0.0, 0.0);
                 if (shared_factor(m, ne, Bs, Ns, g1v, g2v, invh, acth, kh, ph, scr, tab, t, bar)) {
                     // Block form: A_k^{-1} = F0 + F Z_k F^T with F0 = [[P^-1, 0], [0, 0]],
@@ -324,18 +397,25 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                         if (t == 0)
                             for (int v = 0; v < nb; ++v) cfma(Sop, A.gamma[k0 + v], cmul(pf0, pf[v]));
                         group_sync(bar);
-                        if (k0 == 0) stage_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, Mt, t, bar);
+                        // the nodes' inverses as limbs, one scale each
+                        int4 *Zl = reinterpret_cast<int4 *>(Ns);
+                        for (int v = 0; v < nb; ++v) {
+                            const int f = group_fraction(Ns + v * Tn, Tn, scr->red, t, bar);
+                            for (int e = t; e < Tn; e += kGroup) Zl[v * Tn + e] = fx_limbs(Ns[v * Tn + e], f);
+                            if (t == 0) pos[v] = f;
+                        }
+                        if (k0 == 0) fm = stage_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, Mt, scr->red, t, bar);
                         for (int o = 0; o <= A.nop; ++o) {
                             const bool is_h = A.has_h && o == A.nchol;
                             const bool last = o == A.nop;
                             const bool second = !is_h && !last;  // a Cholesky vector: second derivative
-                            const cd *Ko = last ? K2w : Kw + (size_t)o * m * n2;
+                            const int fk = Kfw[o];
                             if (last) build_Sacc(n, m, Kgw, A.Lam + pq * tri_count(n2), X1, lx, Sacc, tab, t, bar);
-                            stage_Ko(n, m, Ko, X1, lx, t, bar);
-                            build_Ap(n, ne, m, X1, lx, Mt, Ap, Sacc, last, tab, t);
+                            stage_Ko(n, m, Kw + (size_t)o * m * n2, Kx, lx, t, bar);
+                            build_Ap(n, ne, m, Kx, lx, Mt, fk < -968 || fm < -968 ? kNan : 58 - fk - fm, Ap, Sacc, last, tab, t);
                             group_sync(bar);
                             // X' is consumed: its region holds W, G, V, H
-                            cd *Wm = X1, *Gp = X1 + m * d2, *Vm = Gp + Tn, *Hp = Vm + ne * d2;
+                            cd *Wm = X1, *Gp = X1 + m * d2, *Vm = Gp + Tn + 1, *Hp = Vm + ne * d2;
                             for (int e = t; e < m * d2; e += kGroup) {
                                 const int a = e / d2, j = e - a * d2;
                                 cd s = (a == ne + j) ? cmk(0.0, 0.0) : skew_get(Ap, a, ne + j);
@@ -391,22 +471,31 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                                 }
                                 c0 = group_sum(c0, red, t, bar);
                             }
-                            // tr((Z G)^2) by three real products per complex multiply-add: re + im
-                            // of G and of each node's Z staged in A''s region (A' is consumed)
-                            const bool sums = second && (A.NB + 1) * Tn <= 2 * T;
-                            double *gsm = reinterpret_cast<double *>(Ap), *zsm = gsm + Tn;
-                            if (sums) {
-                                for (int e = t; e < Tn; e += kGroup) gsm[e] = Gp[e].x + Gp[e].y;
-                                for (int e = t; e < nb * Tn; e += kGroup) zsm[e] = Ns[e].x + Ns[e].y;
-                                group_sync(bar);
+                            // G and H as limbs in place, a zero behind G for the diagonals
+                            int4 *Gl = reinterpret_cast<int4 *>(Gp), *Hl = reinterpret_cast<int4 *>(Hp);
+                            if (!second) group_sync(bar);  // G complete
+                            const int fg = group_fraction(Gp, Tn, scr->red, t, bar);
+                            const int fh = second ? group_fraction(Hp, Tn, scr->red, t, bar) : 0;
+                            for (int e = t; e < Tn; e += kGroup) {
+                                Gl[e] = fx_limbs(Gp[e], fg);
+                                if (second) Hl[e] = fx_limbs(Hp[e], fh);
                             }
+                            if (t == 0) Gl[Tn] = make_int4(0, 0, 0, 0);
+                            // an overflowed inverse or operator: the sums are not finite either
+                            bool wild = fg < -968 || fh < -968;
+                            for (int v = 0; v < nb; ++v) wild = wild || pos[v] < -968;
+                            if (wild) {
+                                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                                if (t < nb) acc[t] = acc[A.NB + t] = cmk(nan, nan);
+                                group_sync(bar);
+                                continue;
+                            }
+                            group_sync(bar);
                             for (int v = 0; v < nb; ++v) {
-                                const cd *Zv = Ns + v * Tn;  // Z_v, packed upper
-                                cd zg = cmk(0.0, 0.0), zh = cmk(0.0, 0.0);
-                                for (int e = t; e < Tn; e += kGroup) {
-                                    cfma(zg, Zv[e], Gp[e]);
-                                    if (second) cfma(zh, Zv[e], Hp[e]);
-                                }
+                                const int4 *Zv = Zl + v * Tn;  // Z_v, packed upper
+                                const int fz = pos[v];
+                                const cd zg = limb_dot(Zv, Gl, Tn, 58 - fz - fg, t);
+                                const cd zh = second ? limb_dot(Zv, Hl, Tn, 58 - fz - fh, t) : cmk(0.0, 0.0);
                                 const cd t1 = cadd(tP, cscale(group_sum(zg, red, t, bar), -2.0));
                                 if (last) {
                                     if (t == 0) acc[A.NB + v] = cadd(acc[A.NB + v], t1);
@@ -425,41 +514,36 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                                         ++a;
                                     }
                                     const int b = a + r;
-                                    cd pab = cmk(0.0, 0.0), pba = cmk(0.0, 0.0);
-                                    if (sums) {
-                                        const double *zs = zsm + v * Tn;
-                                        double p1 = 0.0, p2 = 0.0, p3 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-                                        for (int c = 0; c < d2; ++c) {
-                                            // Z(a,c) G(c,b) and Z(b,c) G(c,a) from the packed upper
-                                            // triangles; c = a or c = b adds nothing (a zero diagonal),
-                                            // taken by selects so that no lane branches
-                                            const bool skip = c == a || c == b;
-                                            const int iz = skip ? 0 : (a < c ? tri_index(a, c) : tri_index(c, a));
-                                            const int ig = skip ? 0 : (c < b ? tri_index(c, b) : tri_index(b, c));
-                                            const int jz = skip ? 0 : (b < c ? tri_index(b, c) : tri_index(c, b));
-                                            const int jg = skip ? 0 : (c < a ? tri_index(c, a) : tri_index(a, c));
-                                            const bool s1 = (a > c) != (c > b), s2 = (b > c) != (c > a);
-                                            const cd zero = cmk(0.0, 0.0);
-                                            const cd z1 = skip ? zero : flip_if(Zv[iz], s1);
-                                            const cd z2 = skip ? zero : flip_if(Zv[jz], s2);
-                                            const double w1 = skip ? 0.0 : __longlong_as_double(__double_as_longlong(zs[iz]) ^ (s1 ? (long long)0x8000000000000000ull : 0ll));
-                                            const double w2 = skip ? 0.0 : __longlong_as_double(__double_as_longlong(zs[jz]) ^ (s2 ? (long long)0x8000000000000000ull : 0ll));
-                                            const cd g1 = Gp[ig], g2 = Gp[jg];
-                                            p1 = fma(z1.x, g1.x, p1);
-                                            p2 = fma(z1.y, g1.y, p2);
-                                            p3 = fma(w1, gsm[ig], p3);
-                                            q1 = fma(z2.x, g2.x, q1);
-                                            q2 = fma(z2.y, g2.y, q2);
-                                            q3 = fma(w2, gsm[jg], q3);
-                                        }
-                                        pab = cmk(p1 - p2, p3 - p1 - p2);
-                                        pba = cmk(q1 - q2, q3 - q1 - q2);
-                                    } else {
-                                        for (int c = 0; c < d2; ++c) {  // zero diagonals: c = a, b add nothing
-                                            cfma(pab, skew_get0(Zv, a, c), skew_get0(Gp, c, b));
-                                            cfma(pba, skew_get0(Zv, b, c), skew_get0(Gp, c, a));
-                                        }
+                                    // (Z G)_ab = sum_c Z(a,c) G(c,b) and (Z G)_ba from the packed upper
+                                    // triangles: both products of an index c have the same sign,
+                                    // plus between a and b and minus outside; c = a and c = b read
+                                    // G's zero
+                                    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+                                    fxacc q1 = {0, 0}, q2 = {0, 0}, q3 = {0, 0};
+#pragma unroll 1
+                                    for (int c = 0; c < d2; ++c) {
+                                        const bool skip = c == a || c == b, la = c < a, lb = c < b;
+                                        const int ca = la ? tri_count(a) + c : tri_count(c) + a;  // {a, c}
+                                        const int cb = lb ? tri_count(b) + c : tri_count(c) + b;  // {b, c}
+                                        const int s = la == lb ? -1 : 0;
+                                        int4 z1 = Zv[ca], z2 = Zv[cb];
+                                        const int4 g1 = Gl[skip ? Tn : cb], g2 = Gl[skip ? Tn : ca];
+                                        z1 = make_int4((z1.x ^ s) - s, (z1.y ^ s) - s, (z1.z ^ s) - s, (z1.w ^ s) - s);
+                                        z2 = make_int4((z2.x ^ s) - s, (z2.y ^ s) - s, (z2.z ^ s) - s, (z2.w ^ s) - s);
+                                        fx_mac(p1, fx_re(z1), fx_re(g1));
+                                        fx_mac(p2, fx_im(z1), fx_im(g1));
+                                        fx_mac(p3, fx_add(fx_re(z1), fx_im(z1)), fx_add(fx_re(g1), fx_im(g1)));
+                                        fx_mac(q1, fx_re(z2), fx_re(g2));
+                                        fx_mac(q2, fx_im(z2), fx_im(g2));
+                                        fx_mac(q3, fx_add(fx_re(z2), fx_im(z2)), fx_add(fx_re(g2), fx_im(g2)));
                                     }
+                                    const int E = 58 - fz - fg;
+                                    auto whole = [&](fxacc s) {
+                                        s.cr += fx_half<kFxS>(58);
+                                        return fx_f64(fx_value<kFxS>(s, 58), E);
+                                    };
+                                    const cd pab = cmk(whole(fx_accsub(p1, p2)), whole(fx_accsub(fx_accsub(p3, p1), p2)));
+                                    const cd pba = cmk(whole(fx_accsub(q1, q2)), whole(fx_accsub(fx_accsub(q3, q1), q2)));
                                     const cd pr = cmul(pab, pba);
                                     t2 = (a == b) ? cadd(t2, pr) : cadd(t2, cscale(pr, 2.0));
                                 }
@@ -488,16 +572,16 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                         if (t == 0)
                             for (int v = 0; v < nb; ++v) cfma(Sop, A.gamma[k0 + v], pf[v]);
                         group_sync(bar);
-                        if (k0 == 0) stage_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, Mt, t, bar);
+                        if (k0 == 0) fm = stage_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, Mt, scr->red, t, bar);
                         // operators: Cholesky vectors (second derivative), then h (first derivative);
                         // the last pass (o = nop) forms A'' = X'' J X^T + X J X''^T + 2 Sacc
                         for (int o = 0; o <= A.nop; ++o) {
                             const bool is_h = A.has_h && o == A.nchol;
                             const bool last = o == A.nop;
-                            const cd *Ko = last ? K2w : Kw + (size_t)o * m * n2;
+                            const int fk = Kfw[o];
                             if (last) build_Sacc(n, m, Kgw, A.Lam + pq * tri_count(n2), X1, lx, Sacc, tab, t, bar);
-                            stage_Ko(n, m, Ko, X1, lx, t, bar);
-                            build_Ap(n, ne, m, X1, lx, Mt, Ap, Sacc, last, tab, t);
+                            stage_Ko(n, m, Kw + (size_t)o * m * n2, Kx, lx, t, bar);
+                            build_Ap(n, ne, m, Kx, lx, Mt, fk < -968 || fm < -968 ? kNan : 58 - fk - fm, Ap, Sacc, last, tab, t);
                             group_sync(bar);
                             for (int v = 0; v < nb; ++v) {
                                 const cd *Zv = Ns + v * T;  // A_v^-1
@@ -563,14 +647,31 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
     }
 }
 
+// count entries of x (shared memory, each written by the thread that reads it here) as limbs
+// with one scale, and its fraction bits; a barrier on both sides of the maximum.
+__device__ __forceinline__ void store_limbs(const cd *x, int count, int4 *__restrict__ out, int *__restrict__ f,
+                                            unsigned *keys) {
+    unsigned k = 0u;
+    for (int e = threadIdx.x; e < count; e += blockDim.x) k = max(k, pivot_key(x[e]));
+    k = __reduce_max_sync(QCS_FULL, k);
+    if ((threadIdx.x & 31) == 0) keys[threadIdx.x >> 5] = k;
+    __syncthreads();
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) k = max(k, keys[i]);
+    const int fr = fx_fraction(k, 56);
+    for (int e = threadIdx.x; e < count; e += blockDim.x) out[e] = fx_limbs(x[e], fr);
+    if (threadIdx.x == 0) *f = fr;
+    __syncthreads();
+}
+
 // Per walker: K (m x 2n) from the rotated rows Ut, and for each operator o the
 // Majorana form ell_o of its one-body matrix, [Lhat, g_mu] = sum_a ell_{mu a} g_a:
 //   ell[2r][2q] = ell[2r+1][2q+1] = (L_qr - L_rq)/2,
 //   ell[2r][2q+1] = -i (L_rq + L_qr)/2,  ell[2r+1][2q] = i (L_rq + L_qr)/2;
-// Kop[w][o] = K ell_o and K2[w] = sum_gamma K ell_gamma^2.  One block per walker.
+// Kop[w][o] = K ell_o and Kop[w][nop] = sum_gamma K ell_gamma^2, as limbs.  One block per walker.
 __global__ void energy_prep_kernel(int n, int ne, int64_t W, int nchol, int has_h, const cd *__restrict__ Ut,
-                                   const cd *__restrict__ Lg, const cd *__restrict__ h, cd *__restrict__ Kop,
-                                   cd *__restrict__ K2, cd *__restrict__ Kg) {
+                                   const cd *__restrict__ Lg, const cd *__restrict__ h, int4 *__restrict__ Kop,
+                                   int *__restrict__ Kf, cd *__restrict__ Kg) {
+    __shared__ unsigned keys[32];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n2 = 2 * n, m = 2 * n - ne, nop = nchol + has_h;
     cd *K = reinterpret_cast<cd *>(smem_raw);   // m x 2n
@@ -604,15 +705,13 @@ __global__ void energy_prep_kernel(int n, int ne, int64_t W, int nchol, int has_
                 ell[e] = v;
             }
             __syncthreads();
-            cd *Ko = Kop + ((size_t)w * nop + o) * m * n2;
             for (int e = threadIdx.x; e < m * n2; e += blockDim.x) {
                 const int a = e / n2, c = e - a * n2;
                 cd s = cmk(0.0, 0.0);
                 for (int k = 0; k < n2; ++k) cfma(s, K[a * n2 + k], ell[k * n2 + c]);
                 K1[e] = s;
-                Ko[e] = s;
             }
-            __syncthreads();
+            store_limbs(K1, m * n2, Kop + ((size_t)w * (nop + 1) + o) * m * n2, Kf + w * (nop + 1) + o, keys);
             if (o < nchol)
                 for (int e = threadIdx.x; e < m * n2; e += blockDim.x) {
                     const int a = e / n2, c = e - a * n2;
@@ -622,8 +721,7 @@ __global__ void energy_prep_kernel(int n, int ne, int64_t W, int nchol, int has_
                 }
             __syncthreads();
         }
-        for (int e = threadIdx.x; e < m * n2; e += blockDim.x) K2[(size_t)w * m * n2 + e] = Ka[e];
-        __syncthreads();
+        store_limbs(Ka, m * n2, Kop + ((size_t)w * (nop + 1) + nop) * m * n2, Kf + w * (nop + 1) + nop, keys);
     }
 }
 
@@ -756,7 +854,7 @@ size_t energy_group_layout(EnergyArgs &A) {
     size_t r = (size_t)m * (2 * n + 1);
     if ((size_t)n * ld_ut(n) > r) r = (size_t)n * ld_ut(n);
     if ((size_t)4 * NB * m > r) r = (size_t)4 * NB * m;
-    if ((size_t)d2 * (m + A.ne) + 2 * (size_t)Tn > r) r = (size_t)d2 * (m + A.ne) + 2 * (size_t)Tn;
+    if ((size_t)d2 * (m + A.ne) + 2 * (size_t)Tn + 1 > r) r = (size_t)d2 * (m + A.ne) + 2 * (size_t)Tn + 1;
     A.off_X1 = (int)o;
     A.off_g1 = (int)o;
     A.off_g2 = (int)(o + (size_t)NB * m * sizeof(cd));
@@ -764,13 +862,13 @@ size_t energy_group_layout(EnergyArgs &A) {
     A.off_y2 = (int)(o + (size_t)3 * NB * m * sizeof(cd));
     o = align16(o + r * sizeof(cd));
     A.off_pf = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(cd));
+    o = align16(o + (size_t)kMaxNBE * sizeof(cd));
     A.off_cf = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(cd));
+    o = align16(o + (size_t)kMaxNBE * sizeof(cd));
     A.off_invh = (int)o;
     o = align16(o + (size_t)NB * S * sizeof(cd));
     A.off_int = (int)o;
-    o = align16(o + (size_t)kMaxNBG * sizeof(int));
+    o = align16(o + (size_t)kMaxNBE * sizeof(int));
     A.off_tile = (int)o;
     o = align16(o + sizeof(long long));
     A.off_acth = (int)o;
@@ -790,7 +888,7 @@ size_t energy_group_layout(EnergyArgs &A) {
     A.off_red = (int)o;
     o = align16(o + (size_t)2 * sizeof(cd));
     A.off_acc = (int)o;
-    o = align16(o + (size_t)2 * kMaxNBG * sizeof(cd));
+    o = align16(o + (size_t)2 * kMaxNBE * sizeof(cd));
     A.off_scr = (int)o;
     o = align16(o + sizeof(SharedScratch));
     return o;
@@ -833,23 +931,23 @@ extern "C" qcs_status qcs_local_energy(qcs_ctx *ctx, const qcs_snapshots *s, int
     if (nchunks < 1) nchunks = 1;
     const size_t b_ut = align16(sizeof(cd) * (size_t)W * n * n);
     const size_t b_pref = align16(sizeof(cd) * (size_t)W);
-    const size_t b_kop = align16(sizeof(cd) * (size_t)W * (nop > 0 ? nop : 1) * m * n2);
-    const size_t b_k2 = align16(sizeof(cd) * (size_t)W * m * n2);
+    const size_t b_kop = align16(sizeof(int4) * (size_t)W * (nop + 1) * m * n2);
+    const size_t b_kf = align16(sizeof(int) * (size_t)W * (nop + 1));
     const size_t b_kg = align16(sizeof(cd) * (size_t)W * m * n2);
     const size_t b_lam = align16(sizeof(cd) * (size_t)(s->P > 0 ? s->P : 1) * tri_count(n2));
     const size_t b_part = align16(sizeof(cd) * (size_t)W * nchunks * 3);
     void *base = nullptr;
-    qcs_status ws = qcs_workspace(ctx, 16 + b_ut + b_pref + b_kop + b_k2 + b_part + b_kg + b_lam, &base, st);
+    qcs_status ws = qcs_workspace(ctx, 16 + b_ut + b_pref + b_kop + b_kf + b_part + b_kg + b_lam, &base, st);
     if (ws != QCS_OK) return ws;
     char *pb = (char *)base;
     unsigned long long *counter = (unsigned long long *)pb;
     cd *Ut = (cd *)(pb + 16);
     cd *pref = (cd *)(pb + 16 + b_ut);
-    cd *Kop = (cd *)(pb + 16 + b_ut + b_pref);
-    cd *K2 = (cd *)(pb + 16 + b_ut + b_pref + b_kop);
-    cd *part = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_k2);
-    cd *Kg = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_k2 + b_part);
-    cd *Lam = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_k2 + b_part + b_kg);
+    int4 *Kop = (int4 *)(pb + 16 + b_ut + b_pref);
+    int *Kf = (int *)(pb + 16 + b_ut + b_pref + b_kop);
+    cd *part = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_kf);
+    cd *Kg = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_kf + b_part);
+    cd *Lam = (cd *)(pb + 16 + b_ut + b_pref + b_kop + b_kf + b_part + b_kg);
     qcs_status r = qcs_launch_walker_prep(ctx, n, ne, W, (const cd *)d_walkers, Ut, pref, st);
     if (r != QCS_OK) return r;
     {
@@ -857,7 +955,7 @@ extern "C" qcs_status qcs_local_energy(qcs_ctx *ctx, const qcs_snapshots *s, int
         if (qcs_set_smem(ctx, (const void *)energy_prep_kernel, sm) != QCS_OK) return QCS_ERR_CUDA;
         int64_t blocks = W < (int64_t)ctx->num_sms * 4 ? W : (int64_t)ctx->num_sms * 4;
         energy_prep_kernel<<<(unsigned)blocks, 256, sm, st>>>(n, ne, W, nchol, has_h, Ut, (const cd *)d_L,
-                                                               (const cd *)d_h, Kop, K2, Kg);
+                                                               (const cd *)d_h, Kop, Kf, Kg);
         r = qcs_check_launch(ctx, "energy_prep_kernel");
         if (r != QCS_OK) return r;
     }
@@ -891,7 +989,7 @@ extern "C" qcs_status qcs_local_energy(qcs_ctx *ctx, const qcs_snapshots *s, int
     A.idx = s->idx;
     A.d_count = s->d_count;
     A.Kop = Kop;
-    A.K2 = K2;
+    A.Kf = Kf;
     A.Kg = Kg;
     A.Lam = Lam;
     A.partial = part;
@@ -901,21 +999,26 @@ extern "C" qcs_status qcs_local_energy(qcs_ctx *ctx, const qcs_snapshots *s, int
         A.wnode[k] = plan.wnode[k];
         A.gamma[k] = plan.gamma[k];
     }
-    // node matrices per round: all when they fit, else fewer (rounds then repeat the
-    // per-operator work); one or two groups per block
-    int NB = plan.nev < kMaxNBG ? plan.nev : kMaxNBG, gpb = 2;
-    for (;;) {
-        A.NB = NB;
-        A.group_bytes = (int)energy_group_layout(A);
-        if ((size_t)A.tab_bytes + (size_t)gpb * A.group_bytes <= ctx->smem_optin) break;
-        if (gpb == 2) gpb = 1;
-        else if (NB > 1) {
-            --NB;
-            gpb = 2;
-        } else {
-            return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "local-energy kernel: shared memory too large");
+    // Node matrices per round: the rounds repeat the per-operator work (A', W, G, H), so the
+    // most groups per SM and round count; two groups share a block where they fit.
+    int NB = 0, gpb = 0, best = 0;
+    for (int nb = plan.nev < kMaxNBE ? plan.nev : kMaxNBE; nb >= 1; --nb)
+        for (int g = 2; g >= 1; --g) {
+            A.NB = nb;
+            const size_t need = (size_t)A.tab_bytes + (size_t)g * energy_group_layout(A);
+            if (need > ctx->smem_optin) continue;
+            int blocks = (int)(ctx->smem_per_sm / (need + 1024));
+            blocks = blocks > 2 ? 2 : blocks < 1 ? 1 : blocks;
+            const int score = 5040 * blocks * g / ((plan.nev + nb - 1) / nb);
+            if (score > best) {
+                best = score;
+                NB = nb;
+                gpb = g;
+            }
         }
-    }
+    if (NB == 0) return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "local-energy kernel: shared memory too large");
+    A.NB = NB;
+    A.group_bytes = (int)energy_group_layout(A);
     const size_t smem = (size_t)A.tab_bytes + (size_t)gpb * A.group_bytes;
     if (qcs_set_smem(ctx, (const void *)energy_pair_kernel, smem) != QCS_OK) return QCS_ERR_CUDA;
     int per_sm = 0;
@@ -966,13 +1069,9 @@ extern "C" double qcs_local_energy_flops_per_pair(int n, int ne, int nchol, int 
     const double vh = 8.0 * ne * d2 * (ne - 1) + 8.0 * Tn * ne       // V = P^-1 W_o, H = -W_o^T V
                       + 8.0 * (ne * (ne + 1) / 2.0) * 2.0 * (ne - 1);  // tr((P^-1 A'_oo)^2)
     const double t1 = 8.0 * Tn;                                       // tr(Z_k G) per node
-    // tr(Z_k H), tr((Z_k G)^2): three real products per complex multiply-add where the
-    // sums of G and of the round's Z_k fit in A''s region (NB as the launcher takes it when
-    // the workspace fits), else four
-    const int nbr = plan.nev < kMaxNBG ? plan.nev : kMaxNBG;
-    const bool sums = (nbr + 1) * Tn <= 2 * T;
+    // tr(Z_k H), tr((Z_k G)^2) by three real products per complex multiply-add
     const double items = d2 * (d2 + 1) / 2;
-    const double t2 = 8.0 * Tn + (sums ? items * 2.0 * (6.0 * (d2 - 1) + 3.0) : items * 2.0 * 8.0 * (d2 - 1));
+    const double t2 = 8.0 * Tn + items * 2.0 * (6.0 * (d2 - 1) + 3.0);
     const double npass = nchol + has_h + 1.0;                         // operators and the A'' pass
     f += mt + npass * (aprime + wg + nev * t1);
     f += nchol * (vh + nev * t2);

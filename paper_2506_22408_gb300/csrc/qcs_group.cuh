@@ -55,7 +55,7 @@ __device__ inline void node_factor(int m, int ne, const cd *__restrict__ wnode, 
         if (t < 32) {
             // pivot: largest |A_{k,i}| over the active row of k = cur[0].  Warp 0 alone:
             // nb segments of seg lanes, a shuffle reduction inside each segment.
-            const int seg = nb <= 1 ? 32 : nb <= 2 ? 16 : 8;
+            const int seg = nb <= 1 ? 32 : nb <= 2 ? 16 : nb <= 4 ? 8 : 4;
             const int v = lane / seg, sl = lane - v * seg;
             unsigned long long bk = 0ull;
             if (v < nb) {
@@ -297,7 +297,7 @@ __device__ inline void node_inverse(int m, int nb, cd *__restrict__ Ns, cd *__re
         group_sync(bar);
         // corner g1^T Z g2 per node (warp 0: segmented shuffle sums), then the new entries
         if (t < 32) {
-            const int seg = nb <= 1 ? 32 : nb <= 2 ? 16 : 8;
+            const int seg = nb <= 1 ? 32 : nb <= 2 ? 16 : nb <= 4 ? 8 : 4;
             const int v = lane / seg, sl = lane - v * seg;
             cd corner = cmk(0.0, 0.0);
             if (v < nb)
