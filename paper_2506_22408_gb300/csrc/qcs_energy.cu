@@ -86,20 +86,43 @@ __device__ __forceinline__ int group_fraction(const cd *x, int count, unsigned *
     return fx_fraction(k, 56);
 }
 
+// A sum of complex products of limbs by three real products each, in units of 2^58 (value) or
+// as FP64 times 2^E (f64); negate() changes the sign of what has been summed.
+struct limb_sum {
+    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+    __device__ __forceinline__ void mac(int4 x, int4 y) {
+        fx_mac(p1, fx_re(x), fx_re(y));
+        fx_mac(p2, fx_im(x), fx_im(y));
+        fx_mac(p3, fx_add(fx_re(x), fx_im(x)), fx_add(fx_re(y), fx_im(y)));
+    }
+    __device__ __forceinline__ void scaled(int4 x, fxl r) {  // + x r, r real
+        fx_mac(p1, fx_re(x), r);
+        fx_mac(p3, fx_add(fx_re(x), fx_im(x)), r);
+    }
+    __device__ __forceinline__ void negate() {
+        const fxacc z = {0, 0};
+        p1 = fx_accsub(z, p1);
+        p2 = fx_accsub(z, p2);
+        p3 = fx_accsub(z, p3);
+    }
+    __device__ __forceinline__ fx2 value() const {
+        fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
+        re.cr += fx_half<kFxS>(58);
+        im.cr += fx_half<kFxS>(58);
+        return make_longlong2(fx_value<kFxS>(re, 58), fx_value<kFxS>(im, 58));
+    }
+    __device__ __forceinline__ cd f64(int E) const {
+        const fx2 v = value();
+        return cmk(fx_f64(v.x, E), fx_f64(v.y, E));
+    }
+};
+
 // sum_e Z_e G_e over this thread's entries, as limbs (fractions fz and fg), in FP64.
 __device__ __forceinline__ cd limb_dot(const int4 *Z, const int4 *G, int count, int E, int t) {
-    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
+    limb_sum s;
 #pragma unroll 1
-    for (int e = t; e < count; e += kGroup) {
-        const int4 z = Z[e], g = G[e];
-        fx_mac(p1, fx_re(z), fx_re(g));
-        fx_mac(p2, fx_im(z), fx_im(g));
-        fx_mac(p3, fx_add(fx_re(z), fx_im(z)), fx_add(fx_re(g), fx_im(g)));
-    }
-    fxacc re = fx_accsub(p1, p2), im = fx_accsub(fx_accsub(p3, p1), p2);
-    re.cr += fx_half<kFxS>(58);
-    im.cr += fx_half<kFxS>(58);
-    return cmk(fx_f64(fx_value<kFxS>(re, 58), E), fx_f64(fx_value<kFxS>(im, 58), E));
+    for (int e = t; e < count; e += kGroup) s.mac(Z[e], G[e]);
+    return s.f64(E);
 }
 
 // Sacc = sum_gamma X'_g J X'_g^T = K Lambda_p K^T (packed upper, m x m), with Lambda_p
@@ -268,12 +291,15 @@ __device__ inline void stage_Ko(int n, int m, const int4 *__restrict__ Ko, int4 
     group_sync(bar);
 }
 
-// Per operator and pair the kernel forms A', W, G, H and the nodes' tr((Z G)^2): 110k FP64
+// Per operator and pair the kernel forms A', W, G, V, H and the nodes' tr((Z G)^2): 110k FP64
 // multiply-adds at 16 modes, 8 electrons and 3 nodes, on a pipe that issues 32 of them per 76
-// clocks (555 ms for 64 walkers, 1000 snapshots of either parity and 64 vectors).  A' (47k)
-// and the traces (39k) run on the integer pipe as 56-bit numbers of two limbs, one scale per
-// matrix: 339 ms, the FP64 products W, G, V and H a third of it.  The operators' rows K ell
-// come from energy_prep_kernel as limbs already, since every pair of a walker stages them.
+// clocks (556 ms for 64 walkers, 1000 snapshots of either parity and 64 vectors).  They run
+// on the integer pipe as 56-bit numbers of two limbs, one scale per matrix, each result kept as
+// integers and rescaled by its largest entry: A' and the traces 339 ms, the others as well
+// 301 ms.  Errors against 64-bit-mantissa references are FP64's (1e-14 of e1).  Two blocks of
+// two groups per SM (54 KB of operands a group, 236 registers): bound by the latency of the
+// multiply-add chains at two warps per SM sub-partition.  The operators' rows K ell come from
+// energy_prep_kernel as limbs already, since every pair of a walker stages them.
 __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_constant__ EnergyArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / kGroup;
@@ -384,6 +410,15 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                         Es[e] = s;
                     }
                     group_sync(bar);
+                    // P^-1 and E as limbs in place; one = 1 at E's scale
+                    int4 *Pl = reinterpret_cast<int4 *>(Pinv), *El = reinterpret_cast<int4 *>(Es);
+                    const int fp = group_fraction(Pinv, To, scr->red, t, bar);
+                    int fe = group_fraction(Es, ne * d2, scr->red, t, bar);
+                    const bool wild0 = fp < -968 || fe < -968;
+                    fe = fe < 55 ? fe : 55;
+                    const fxl one = fx_split<kFxS>(fe >= 0 ? 1ll << fe : 0ll);
+                    for (int e = t; e < To; e += kGroup) Pl[e] = fx_limbs(Pinv[e], fp);
+                    for (int e = t; e < ne * d2; e += kGroup) El[e] = fx_limbs(Es[e], fe);
                     for (int k0 = 0; k0 < A.nev; k0 += A.NB) {
                         const int nb = A.nev - k0 < A.NB ? A.nev - k0 : A.NB;
                         node_factor(d2, 0, A.wnode + k0, nb, Sc, Ns, g1v, g2v, pf, invh, pos, acth, kh, ph, tab, t,
@@ -414,46 +449,117 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                             stage_Ko(n, m, Kw + (size_t)o * m * n2, Kx, lx, t, bar);
                             build_Ap(n, ne, m, Kx, lx, Mt, fk < -968 || fm < -968 ? kNan : 58 - fk - fm, Ap, Sacc, last, tab, t);
                             group_sync(bar);
-                            // X' is consumed: its region holds W, G, V, H
-                            cd *Wm = X1, *Gp = X1 + m * d2, *Vm = Gp + Tn + 1, *Hp = Vm + ne * d2;
+                            // X' is consumed: its region holds W, G, V, H, each of them integers,
+                            // then limbs once its largest entry is known
+                            const int fa = group_fraction(Ap, T, scr->red, t, bar);
+                            int4 *Al = reinterpret_cast<int4 *>(Ap);
+                            for (int e = t; e < T; e += kGroup) Al[e] = fx_limbs(Ap[e], fa);
+                            int4 *Wl = Kx, *Gl = Wl + m * d2, *Vl = Gl + Tn + 1, *Hl = Vl + ne * d2;
+                            auto put_top = [&](unsigned top, int slot) {
+                                top = __reduce_or_sync(QCS_FULL, top);
+                                if ((t & 31) == 0) scr->red[2 * slot + (t >> 5)] = top;
+                            };
+                            auto get_bits = [&](int slot) {
+                                return fx_top_bits(scr->red[2 * slot] | scr->red[2 * slot + 1]);
+                            };
+                            auto limbs = [&](int4 *x, int count, int bits) {
+                                for (int e = t; e < count; e += kGroup) {
+                                    const fx2 v = fx_shift(reinterpret_cast<fx2 *>(x)[e], 56 - bits);
+                                    x[e] = fx_pack(fx_split<kFxS>(v.x), fx_split<kFxS>(v.y));
+                                }
+                            };
+                            group_sync(bar);
+                            unsigned top = 0u;
+#pragma unroll 1
                             for (int e = t; e < m * d2; e += kGroup) {
                                 const int a = e / d2, j = e - a * d2;
-                                cd s = (a == ne + j) ? cmk(0.0, 0.0) : skew_get(Ap, a, ne + j);
-                                for (int l = 0; l < ne; ++l)
-                                    if (l != a) cfms(s, skew_get(Ap, a, l), Es[l * d2 + j]);
-                                Wm[e] = s;
+                                limb_sum s;
+#pragma unroll 1
+                                for (int l = 0; l < ne; ++l) {  // -A'_al E_lj: A'_la E_lj below a
+                                    if (l == a) {
+                                        s.negate();
+                                        continue;
+                                    }
+                                    s.mac(Al[l < a ? tri_count(a) + l : tri_count(l) + a], El[l * d2 + j]);
+                                }
+                                if (a < ne) s.negate();
+                                if (a != ne + j) {  // + A'_{a,ne+j}
+                                    const bool lo = a < ne + j;
+                                    s.scaled(Al[lo ? tri_index(a, ne + j) : tri_index(ne + j, a)], lo ? one : fx_neg(one));
+                                }
+                                const fx2 v = s.value();
+                                top |= fx_top(v);
+                                reinterpret_cast<fx2 *>(Wl)[e] = v;
                             }
+                            put_top(top, 0);
                             group_sync(bar);
+                            int wb = get_bits(0);
+                            const int fw = fa + fe - 58 + 56 - wb;
+                            limbs(Wl, m * d2, wb);
+                            group_sync(bar);
+                            top = 0u;
+#pragma unroll 1
                             for (int e = t; e < Tn; e += kGroup) {
                                 int i, j;
                                 pair_of(tab, e, i, j);
-                                cd s = Wm[(ne + i) * d2 + j];
-                                for (int l = 0; l < ne; ++l) cfms(s, Es[l * d2 + i], Wm[l * d2 + j]);
-                                Gp[e] = s;
+                                limb_sum s;
+#pragma unroll 1
+                                for (int l = 0; l < ne; ++l) s.mac(El[l * d2 + i], Wl[l * d2 + j]);
+                                s.negate();
+                                s.scaled(Wl[(ne + i) * d2 + j], one);
+                                const fx2 v = s.value();
+                                top |= fx_top(v);
+                                reinterpret_cast<fx2 *>(Gl)[e] = v;
                             }
-                            if (second)
+                            put_top(top, 1);
+                            if (second) {
+                                top = 0u;
+#pragma unroll 1
                                 for (int e = t; e < ne * d2; e += kGroup) {
                                     const int i = e / d2, j = e - i * d2;
-                                    cd s = cmk(0.0, 0.0);
-                                    for (int l = 0; l < ne; ++l)
-                                        if (l != i) cfma(s, skew_get(Pinv, i, l), Wm[l * d2 + j]);
-                                    Vm[e] = s;
+                                    limb_sum s;
+#pragma unroll 1
+                                    for (int l = 0; l < ne; ++l) {  // P^-1_il W_lj: -P^-1_li below i
+                                        if (l == i) {
+                                            s.negate();
+                                            continue;
+                                        }
+                                        s.mac(Pl[l < i ? tri_count(i) + l : tri_count(l) + i], Wl[l * d2 + j]);
+                                    }
+                                    const fx2 v = s.value();
+                                    top |= fx_top(v);
+                                    reinterpret_cast<fx2 *>(Vl)[e] = v;
                                 }
+                                put_top(top, 0);
+                            }
                             // tr(P^-1 A'_oo) = -2 sum_{a<b} P^-1_ab A'_ab
-                            cd tP = cmk(0.0, 0.0);
-                            for (int e = t; e < To; e += kGroup) cfma(tP, Pinv[e], Ap[e]);
+                            cd tP = limb_dot(Pl, Al, To, 58 - fp - fa, t);
                             group_sync(bar);
-                            tP = cscale(group_sum(tP, red, t, bar), -2.0);
+                            const int gb = get_bits(1), fg = fw + fe - 58 + 56 - gb;
+                            limbs(Gl, Tn, gb);
                             cd c0 = cmk(0.0, 0.0);
+                            int fh = 0;
                             if (second) {
+                                const int vb = get_bits(0), fv = fw + fp - 58 + 56 - vb;
+                                limbs(Vl, ne * d2, vb);
+                                group_sync(bar);
+                                top = 0u;
+#pragma unroll 1
                                 for (int e = t; e < Tn; e += kGroup) {
                                     int i, j;
                                     pair_of(tab, e, i, j);
-                                    cd s = cmk(0.0, 0.0);
-                                    for (int l = 0; l < ne; ++l) cfms(s, Wm[l * d2 + i], Vm[l * d2 + j]);
-                                    Hp[e] = s;
+                                    limb_sum s;
+#pragma unroll 1
+                                    for (int l = 0; l < ne; ++l) s.mac(Wl[l * d2 + i], Vl[l * d2 + j]);
+                                    s.negate();
+                                    const fx2 v = s.value();
+                                    top |= fx_top(v);
+                                    reinterpret_cast<fx2 *>(Hl)[e] = v;
                                 }
-                                // tr((P^-1 A'_oo)^2): one unordered pair {a, b} of occupied indices per item
+                                put_top(top, 1);
+                                // tr((P^-1 A'_oo)^2): one unordered pair {a, b} of occupied indices per
+                                // item; both products of an index c have the same sign (as below)
+#pragma unroll 1
                                 for (int e = t; e < ne * (ne + 1) / 2; e += kGroup) {
                                     int a = 0, r = e;
                                     while (r >= ne - a) {
@@ -461,28 +567,35 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                                         ++a;
                                     }
                                     const int b = a + r;
-                                    cd pab = cmk(0.0, 0.0), pba = cmk(0.0, 0.0);
+                                    limb_sum p, q;
+#pragma unroll 1
                                     for (int c = 0; c < ne; ++c) {
-                                        if (c != a && c != b) cfma(pab, skew_get(Pinv, a, c), skew_get(Ap, c, b));
-                                        if (c != b && c != a) cfma(pba, skew_get(Pinv, b, c), skew_get(Ap, c, a));
+                                        if (c == a || c == b) {
+                                            if (a != b) {
+                                                p.negate();
+                                                q.negate();
+                                            }
+                                            continue;
+                                        }
+                                        const int ca = c < a ? tri_count(a) + c : tri_count(c) + a;
+                                        const int cb = c < b ? tri_count(b) + c : tri_count(c) + b;
+                                        p.mac(Pl[ca], Al[cb]);
+                                        q.mac(Pl[cb], Al[ca]);
                                     }
-                                    const cd pr = cmul(pab, pba);
+                                    const cd pr = cmul(p.f64(58 - fp - fa), q.f64(58 - fp - fa));
                                     c0 = (a == b) ? cadd(c0, pr) : cadd(c0, cscale(pr, 2.0));
                                 }
+                                group_sync(bar);
+                                const int hb = get_bits(1);
+                                fh = fw + fv - 58 + 56 - hb;
+                                limbs(Hl, Tn, hb);
                                 c0 = group_sum(c0, red, t, bar);
                             }
-                            // G and H as limbs in place, a zero behind G for the diagonals
-                            int4 *Gl = reinterpret_cast<int4 *>(Gp), *Hl = reinterpret_cast<int4 *>(Hp);
-                            if (!second) group_sync(bar);  // G complete
-                            const int fg = group_fraction(Gp, Tn, scr->red, t, bar);
-                            const int fh = second ? group_fraction(Hp, Tn, scr->red, t, bar) : 0;
-                            for (int e = t; e < Tn; e += kGroup) {
-                                Gl[e] = fx_limbs(Gp[e], fg);
-                                if (second) Hl[e] = fx_limbs(Hp[e], fh);
-                            }
+                            tP = cscale(group_sum(tP, red, t, bar), -2.0);
+                            // a zero behind G for the diagonals
                             if (t == 0) Gl[Tn] = make_int4(0, 0, 0, 0);
                             // an overflowed inverse or operator: the sums are not finite either
-                            bool wild = fg < -968 || fh < -968;
+                            bool wild = wild0 || fa < -968;
                             for (int v = 0; v < nb; ++v) wild = wild || pos[v] < -968;
                             if (wild) {
                                 const double nan = __longlong_as_double(0x7ff8000000000000ll);
@@ -518,8 +631,7 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                                     // triangles: both products of an index c have the same sign,
                                     // plus between a and b and minus outside; c = a and c = b read
                                     // G's zero
-                                    fxacc p1 = {0, 0}, p2 = {0, 0}, p3 = {0, 0};
-                                    fxacc q1 = {0, 0}, q2 = {0, 0}, q3 = {0, 0};
+                                    limb_sum p, q;
 #pragma unroll 1
                                     for (int c = 0; c < d2; ++c) {
                                         const bool skip = c == a || c == b, la = c < a, lb = c < b;
@@ -530,20 +642,10 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
                                         const int4 g1 = Gl[skip ? Tn : cb], g2 = Gl[skip ? Tn : ca];
                                         z1 = make_int4((z1.x ^ s) - s, (z1.y ^ s) - s, (z1.z ^ s) - s, (z1.w ^ s) - s);
                                         z2 = make_int4((z2.x ^ s) - s, (z2.y ^ s) - s, (z2.z ^ s) - s, (z2.w ^ s) - s);
-                                        fx_mac(p1, fx_re(z1), fx_re(g1));
-                                        fx_mac(p2, fx_im(z1), fx_im(g1));
-                                        fx_mac(p3, fx_add(fx_re(z1), fx_im(z1)), fx_add(fx_re(g1), fx_im(g1)));
-                                        fx_mac(q1, fx_re(z2), fx_re(g2));
-                                        fx_mac(q2, fx_im(z2), fx_im(g2));
-                                        fx_mac(q3, fx_add(fx_re(z2), fx_im(z2)), fx_add(fx_re(g2), fx_im(g2)));
+                                        p.mac(z1, g1);
+                                        q.mac(z2, g2);
                                     }
-                                    const int E = 58 - fz - fg;
-                                    auto whole = [&](fxacc s) {
-                                        s.cr += fx_half<kFxS>(58);
-                                        return fx_f64(fx_value<kFxS>(s, 58), E);
-                                    };
-                                    const cd pab = cmk(whole(fx_accsub(p1, p2)), whole(fx_accsub(fx_accsub(p3, p1), p2)));
-                                    const cd pba = cmk(whole(fx_accsub(q1, q2)), whole(fx_accsub(fx_accsub(q3, q1), q2)));
+                                    const cd pab = p.f64(58 - fz - fg), pba = q.f64(58 - fz - fg);
                                     const cd pr = cmul(pab, pba);
                                     t2 = (a == b) ? cadd(t2, pr) : cadd(t2, cscale(pr, 2.0));
                                 }
