@@ -152,15 +152,19 @@ CSRC = os.path.join(ROOT, "paper_2506_22408_gb300", "csrc")
 # Source files each timed kernel is compiled from; the committed DRAM figure of a
 # kernel is used only while all of them are unchanged.
 KERNEL_SOURCES = {
-    "tc_pair_kernel": ["qcs_tcpair.cu", "qcs_ozaki.cuh", "qcs_tc.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
-    "pair_overlap_kernel": ["qcs_overlap.cu", "qcs_group.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
-    "split_pair_kernel": ["qcs_split.cu", "qcs_pair.cuh", "qcs_tc.cuh", "qcs_common.cuh"],
-    "grad_pair_kernel": ["qcs_grad.cu", "qcs_group.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "tc_pair_kernel": ["qcs_tcpair.cu", "qcs_pfaff.cu", "qcs_fixed.cuh", "qcs_ozaki.cuh", "qcs_tc.cuh", "qcs_pair.cuh",
+                       "qcs_common.cuh"],
+    "pair_overlap_kernel": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "split_pair_kernel": ["qcs_split.cu", "qcs_fixed.cuh", "qcs_pair.cuh", "qcs_tc.cuh", "qcs_common.cuh"],
+    "grad_pair_kernel": ["qcs_grad.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_fxsweep.cuh", "qcs_group.cuh",
+                         "qcs_pair.cuh", "qcs_common.cuh"],
     "rdm_syrk_kernel": ["qcs_rdm.cu"],
-    "energy_pair_kernel": ["qcs_energy.cu", "qcs_group.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "rdm_tc_moment_kernel": ["qcs_rdm.cu", "qcs_ozaki.cuh", "qcs_tc.cuh"],
+    "energy_pair_kernel": ["qcs_energy.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_group.cuh", "qcs_pair.cuh",
+                           "qcs_common.cuh"],
     # the FP64 ALU pair kernel in its batched launch over the five systems of the batching
     # workload (a record of its own: another workload)
-    "pair_overlap_kernel_batched": ["qcs_overlap.cu", "qcs_group.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "pair_overlap_kernel_batched": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
 }
 
 # workload name of the batched launch's traffic record
@@ -667,9 +671,9 @@ def run_rdm(args, ctx, dev, flush, barrier, ws, steps=3):
             "config": {"workload": f"shadow RDM n={n} {P} snapshots (Haar Q, uniform b, seed 0)"},
             "particle_number": float(out["npart"].item()),
             "roofline": {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": ach / FP64_PEAK_TFLOPS, "kernel": "rdm_syrk_kernel", "kernel_ms": avg,
+                         "frac": ach / FP64_PEAK_TFLOPS, "kernel": "rdm_tc_moment_kernel", "kernel_ms": avg,
                          "flops_per_launch": fl,
-                         "traffic": traffic_for("rdm_syrk_kernel", f"shadow RDM n={n} {P} snapshots")}}
+                         "traffic": traffic_for("rdm_tc_moment_kernel", f"shadow RDM n={n} {P} snapshots")}}
 
 
 def run_vce(args, ctx, dev, flush, barrier, ws, steps=3):

@@ -270,9 +270,10 @@ qcs_status qcs_overlap(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t W, 
  * slices exact in BF16, the 28 slice products of the leading levels accumulate exactly
  * in FP32, and the levels are combined exactly in 64-bit fixed point, so each entry of P
  * carries an error of about 2^-53 times the row scales, like an FP64 product; the
- * Pfaffians stay on the FP64 pipe.  The snapshot set then holds 57,856 bytes per four
+ * Pfaffians run in 64-bit fixed point.  The snapshot set then holds 57,856 bytes per four
  * parity +1 snapshots of slice records (formed by qcs_build_snapshots at n = 16,
- * otherwise on first use), and the context workspace 14,464 bytes per walker. */
+ * otherwise on first use), and the context workspace 14,464 bytes per walker and at most
+ * 512 MB of pair records, worked off in batches. */
 
 /* ---------------------------------------------------- local energy terms */
 
@@ -315,12 +316,12 @@ double qcs_local_energy_flops_per_pair(int n, int ne, int nchol, int has_h, int 
  *   d_gam2  : 2n x 2n doubles or NULL: <g~_mu g~_nu> = i gam2[mu][nu] (mu != nu), 0 on the diagonal
  *   d_gam4  : C(2n,4) doubles or NULL: <g~_mu g~_nu g~_rho g~_sigma> (real) for
  *             mu < nu < rho < sigma in lexicographic order, formed from the second
- *             moments of the covariance entries (a rank-P update, FP64)
+ *             moments of the covariance entries (a rank-P update at FP64 accuracy)
  *   d_rdm1  : n x n complex or NULL: <a~_p^dagger a~_q>, a~_p = (g~_2p + i g~_2p+1)/2
  *             (Eqs. 1rdm_off_diagonal, 1rdm_diagonal)
  *   d_npart : 1 double or NULL: the particle number, trace of the 1-RDM
  * Outputs are device buffers owned by the caller.  The call uses context workspace
- * (P n (2n-1) doubles for the covariance entries, plus the moment partials).
+ * (P n (2n-1) 8-byte covariance entries, their slices, and the moment partials).
  * Errors: QCS_ERR_ARG (empty set, set on another device, d_gam4 with n < 2), QCS_ERR_CUDA. */
 qcs_status qcs_shadow_rdm(qcs_ctx *ctx, const qcs_snapshots *s, const double *d_R, double *d_gam2, double *d_gam4,
                           double *d_rdm1, double *d_npart, void *stream);
@@ -399,7 +400,7 @@ qcs_status qcs_overlap_batched(qcs_ctx *ctx, int nsys, const qcs_system *systems
  * need no special case.  Context workspace: per walker its rows, QR factors and
  * per-chunk records, and per snapshot of the set 32 n^2 bytes (the rows
  * [H1^T; G2^T], H1 = Qt^T J Qt and G2 = Qt^T J conj(Qt), through which B and the
- * cotangents of a dense snapshot are formed). */
+ * cotangents are formed). */
 qcs_status qcs_overlap_grad(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t W, const double *d_walkers,
                             double *d_overlap, double *d_grad, const qcs_opts *opts, void *stream);
 
@@ -495,11 +496,11 @@ qcs_status qcs_fp64_fma_rate(qcs_ctx *ctx, double *tflops, void *stream);
  * orbitals are first rotated to echelon form (a reflection of the occupied
  * columns changes det R by its sign, one of the complement changes nothing),
  * which makes ne(ne-1)/2 + d(d-1)/2 entries of U exact zeros that T skips.
- * The occupied orbitals are further taken in reduced form [I; X]
- * (an invertible change of basis, det folded into det R), leaving one non-zero
- * among the first ne entries of each occupied row; walkers whose X would exceed
- * 16 in magnitude (about 3 % of random walkers) keep the echelon form and do
- * ne(ne-1)/2 more products than counted.
+ * The count further assumes the occupied orbitals in reduced form [I; X]
+ * (an invertible change of basis, det folded into det R), which leaves one non-zero
+ * among the first ne entries of each occupied row: the FP64 arithmetic the path
+ * needs.  The kernels do that work in 64-bit fixed point, on the echelon form, whose
+ * rows of norm one keep the accuracy under one scale.
  * The node matrices differ only in their empty x empty block, so the occupied
  * block is eliminated once per pair and each node then costs a 2d x 2d
  * Pfaffian; the count is that of this path (pairs whose occupied block would

@@ -866,7 +866,8 @@ double qcs_pf_elim_flops(int m, int stop) {
 // Parts of the count: [0] congruence T, [1] covariance B, [2] Pfaffian eliminations.
 static void overlap_flops_parts(int n, int ne, int nev, bool overlap_kernel, double *part) {
     const int d = n - ne, m = 2 * n - ne;
-    // skipped entries of Ut: the reduced form of the occupied rows ([I; X], all but one of
+    // skipped entries of Ut (counted; the kernels run the echelon form in fixed point): the
+    // reduced form of the occupied rows ([I; X], all but one of
     // the columns k < ne zero) and the echelon form of the completion; three real products
     // per complex multiply-add (every T of the overlap kernel in its default
     // configuration; n > 16 configured to one warp per pair takes four)

@@ -99,7 +99,7 @@ struct FxSwept {
 // The occupied sweeps end early, left > 0, when a multiplier of the pivot's column would reach
 // 2^kFxMaxMult: an inverse assembled from the blocks loses twice those bits, which a sweep of
 // the whole matrix does not.  Limit 3 keeps the gradients' errors below those of the FP64
-// code (at 16 modes 2 % of the pairs, at 10 modes 14 % leave a pair of indices to the
+// code (at 10 to 16 modes one pair in six or seven leaves some indices to the
 // nodes); limit 4 was 2 % faster and doubled the largest errors.
 //
 // mb = -1 when a pivot is below 2^-14 of its matrix or a row exceeds it by more than
