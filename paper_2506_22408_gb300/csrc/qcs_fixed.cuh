@@ -8,8 +8,8 @@
 //     X = h 2^S + l,  |l| <= 2^{S-1}:   X Y = hh 2^2S + (h l' + l h') 2^S + l l',
 // the last term dropped: 12 to 13 clocks against 76.  With S = 30 and entries of 58 to 60
 // bits it is below 2^-58 of the factors' scale, of either sign; longer sums of entries of 57
-// bits take S = 29 (2^-60), as S = 31 lost three bits of the congruence against FP64.  The largest entry of a matrix is kept at 54 to 60 bits, so an update rounds
-// at 2^-54 to 2^-60 of the matrix's largest entry where FP64 rounds at 2^-53 of each
+// bits take S = 29 (2^-60), as S = 31 lost three bits of the congruence against FP64.  The
+// largest entry of a matrix is kept at 54 to 60 bits, so an update rounds at 2^-54 to 2^-60 of the matrix's largest entry where FP64 rounds at 2^-53 of each
 // operand: the elimination with pivoting is as accurate as that matrix norm allows either
 // way, and the errors against 64-bit references are those of the FP64 code it replaced or
 // smaller.

@@ -2,7 +2,8 @@
 // of 64 threads with its own named barrier) share one walker-snapshot pair: the
 // forward Parlett-Reid elimination of a round of node matrices that keeps its step
 // history, and the backward recursion that assembles each node matrix's inverse in
-// place over its factors (used by the adjoint and the local-energy kernels).
+// place over its factors (used by the local-energy kernel, by the adjoint for the pairs that
+// its fixed-point sweeps refuse, and by the split kernel above 16 modes).
 #pragma once
 #include "qcs_pair.cuh"
 
@@ -321,7 +322,7 @@ __device__ inline void node_inverse(int m, int nb, cd *__restrict__ Ns, cd *__re
 }
 
 // ---------------------------------------------------------------------------
-// Block form for the adjoint: the node matrices A_k = B + w_k D differ only in their
+// Block form for the local energy: the node matrices A_k = B + w_k D differ only in their
 // empty x empty block, so with the occupied block eliminated once (Schur complement
 // S0 on the empty indices) A_k = [[P, Boe], [-Boe^T, S0 + w_k D + ...]] and
 //     A_k^{-1} = F(Z_k),  Z_k = (S0 + w_k D)^{-1},
