@@ -515,8 +515,11 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
                 P += d2;
                 K += d2;
                 neg = false;
+                // Every warp has scanned the block before any entry of it is written, here or by
+                // the Gauss vectors below: x and -x differ by one in fx_mag32, so a warp that
+                // scanned rewritten entries could see another tie and take another pivot.
+                tm.sync();
                 if (K != r - 1) {
-                    tm.sync();  // every warp has scanned the block
                     fx_swap_last(tm, X, r, K);
                     neg = true;
                     tm.sync();
