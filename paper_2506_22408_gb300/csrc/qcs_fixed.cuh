@@ -168,11 +168,12 @@ __device__ __forceinline__ long long fx_shift1(long long X, int s) {
 }
 __device__ __forceinline__ fx2 fx_shift(fx2 a, int s) { return make_longlong2(fx_shift1(a.x, s), fx_shift1(a.y, s)); }
 
-// The same without a branch.
+// The same without a branch, |X| < 2^62.
 __device__ __forceinline__ long long fx_shift_any(long long X, int s) {
-    const int r = s < 0 ? (s > -63 ? -s : 63) : 0;
+    const int r = s < 0 ? (s > -62 ? -s : 62) : 0;
     const long long y = X << (s > 0 ? s : 0);
-    return (y + ((1ll << r) >> 1)) >> r;
+    const long long v = (y + ((1ll << r) >> 1)) >> r;
+    return s < -62 ? 0ll : v;
 }
 
 // x 2^f rounded to an integer, from the bit pattern (|x| 2^f < 2^62; no FP64 instruction).

@@ -80,7 +80,7 @@ __device__ __forceinline__ long long fixed_of(double x, int e) {
     if (hx == 0) return 0ll;  // zeros (and subnormals, far below any row scale here)
     const long long m = (b & ((1ll << 52) - 1)) | (1ll << 52);  // |x| = m 2^{hx-1075}
     const int sh = hx - 1075 + 55 - e;                             // |u| = m 2^sh, sh <= 2
-    const int r = sh < 0 ? (sh > -63 ? -sh : 63) : 0;
+    const int r = sh < 0 ? (sh > -62 ? -sh : 62) : 0;              // m < 2^53: zero from 55 on
     const long long u = ((m << (sh > 0 ? (sh < 2 ? sh : 2) : 0)) + ((1ll << r) >> 1)) >> r;
     return b < 0 ? -u : u;
 }

@@ -1,0 +1,60 @@
+"""The conversions and shifts of the fixed-point code (csrc/qcs_ozaki.cuh, csrc/qcs_fixed.cuh) on
+the CPU, over every exponent: the nearest integer, ties away from zero for the sliced entries
+and upward for the shifts; entries far below the scale, and zeros, give zero."""
+from __future__ import annotations
+
+import ctypes
+import random
+from fractions import Fraction
+from math import floor
+
+import pytest
+
+import warp_emulation
+
+SOURCE = """
+extern "C" long long host_fixed_of(double x, int e) { return qcs_oz::fixed_of(x, e); }
+extern "C" long long host_fx_of1(double x, int f) { return fx_of1(x, f); }
+extern "C" long long host_shift1(long long X, int s) { return fx_shift1(X, s); }
+extern "C" long long host_shift_any(long long X, int s) { return fx_shift_any(X, s); }
+"""
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    lib = warp_emulation.compile_host(SOURCE, ["qcs_fixed.cuh"], str(tmp_path_factory.mktemp("emu")))
+    for f in ("host_fixed_of", "host_fx_of1", "host_shift1", "host_shift_any"):
+        getattr(lib, f).restype = ctypes.c_longlong
+        getattr(lib, f).argtypes = [ctypes.c_double if "of" in f else ctypes.c_longlong, ctypes.c_int]
+    return lib
+
+
+def mantissas(rng):
+    return [1.0, 1.5, 2.0 - 2.0**-52, 1.0 + 2.0**-52] + [1.0 + rng.random() for _ in range(4)]
+
+
+def test_conversions_round_to_nearest(host):
+    """fixed_of for |x| (1 + 2^-7) < 2^e, fx_of1 for |x| 2^f < 2^62: half away from zero."""
+    rng = random.Random(4)
+    for k in range(-1000, 1):
+        for m in mantissas(rng):
+            for x in (m * 2.0**k, -m * 2.0**k):
+                away = lambda v: (1 if v >= 0 else -1) * floor(abs(v) + Fraction(1, 2))
+                e = 2
+                assert host.host_fixed_of(x, e) == away(Fraction(x) * Fraction(2) ** (55 - e)), (x, e)
+                f = 60
+                assert host.host_fx_of1(x, f) == away(Fraction(x) * Fraction(2) ** f), (x, f)
+    for x in (0.0, -0.0):
+        assert host.host_fixed_of(x, 1) == 0 and host.host_fixed_of(x, 900) == 0 and host.host_fx_of1(x, 50) == 0
+
+
+def test_shifts_round_to_nearest(host):
+    """X 2^s for |X| < 2^62 and a result below 2^62: halves upward."""
+    rng = random.Random(5)
+    values = [0, 1, -1, 2, -2, 3, -3, (1 << 61) - 1, 1 << 61, -(1 << 61), (1 << 62) - 1, -(1 << 62) + 1]
+    values += [rng.choice([1, -1]) * rng.randrange(1 << b) for b in range(1, 63)]
+    for X in values:
+        for s in list(range(-140, 62 - abs(X).bit_length() + 1)) + [-100000, -1 << 30]:
+            exact = 0 if s < -200 else floor(Fraction(X) * Fraction(2) ** s + Fraction(1, 2))
+            assert host.host_shift_any(X, s) == exact, (X, s)
+            assert host.host_shift1(X, s) == exact, (X, s)
