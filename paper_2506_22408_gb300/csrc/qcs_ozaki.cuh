@@ -104,10 +104,13 @@ __device__ __forceinline__ long long combine_levels(const float (&acc)[kLevels])
     return (long long)(z - kOff);
 }
 
-// Number of significant bits of |z| (0 for z = 0).
-__device__ __forceinline__ int bitlen64(long long z) {
-    const unsigned long long u = z < 0 ? (unsigned long long)(-z) : (unsigned long long)z;
-    return 64 - __clzll((long long)u);
+// Exponent G with |z| 2^g (1 + 2^-7) < 2^G, from the upper word where it is not zero (at most
+// two bits above the least one), g + 33 below it; kNoRow for z = 0.  A maximum of these over
+// entries of different g is a scale of them all: an entry of a zero upper word counts too, as
+// its g may exceed the others'.
+__device__ __forceinline__ int scale_of_fixed(long long z, int g) {
+    const int zh = (int)(z >> 32), zm = zh < 0 ? -zh : zh;
+    return zm != 0 ? g + 64 - __clz(zm + (zm >> 6) + 1) : z != 0 ? g + 33 : kNoRow;
 }
 
 // z 2^E as an FP64 (round to nearest on the 11 dropped bits), assembled from the bits

@@ -275,9 +275,9 @@ __host__ __device__ __forceinline__ uint32_t mnmajor16(int row, int k) {
 
 // Slices of Z_i^T, read from tensor memory (lane k holds row k of Z_i, z_kb worth
 // z 2^{g_k + e_b - 56}): row b of Z_i^T gets the scale 2^{F_b}, F_b = e_b + G_b - 56 with
-// 2^{G_b} above max_k |z_kb| 2^{g_k} (1 + 2^-7) (a warp max-reduction on the upper words;
-// on the whole ones for a row that is zero there); the slices go MN-major into the A operand
-// rows row0 + b.  Returns F_b for b = lane (kNoRow for a zero row).
+// 2^{G_b} above max_k |z_kb| 2^{g_k} (1 + 2^-7) (scale_of_fixed and a warp max-reduction; a row
+// whose entries have no upper word keeps them whole, as g spans a few bits); the slices go MN-major into the A
+// operand rows row0 + b.  Returns F_b for b = lane (kNoRow for a zero row).
 __device__ __forceinline__ int slice_zt(uint32_t tlane, int gk, int eb_lane, unsigned char *Abase, int row0, int lane) {
     int Gl = kNoRow;
 #pragma unroll 1
@@ -287,9 +287,7 @@ __device__ __forceinline__ int slice_zt(uint32_t tlane, int gk, int eb_lane, uns
         uint64_t u[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const int zh = abs((int)(z[c] >> 32));
-            int G = __reduce_max_sync(QCS_FULL, zh != 0 ? gk + 64 - __clz(zh + (zh >> 6) + 1) : kNoRow);
-            if (G == kNoRow) G = __reduce_max_sync(QCS_FULL, z[c] != 0 ? gk + bitlen64(z[c]) + 1 : kNoRow);
+            const int G = __reduce_max_sync(QCS_FULL, scale_of_fixed(z[c], gk));
             if (8 * cb + c == lane) Gl = G;
             const long long v = G == kNoRow ? 0ll : fx_shift_any(z[c], 55 + gk - G);
             u[c] = (uint64_t)v + kDigitBias;

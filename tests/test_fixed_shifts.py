@@ -16,6 +16,7 @@ SOURCE = """
 extern "C" long long host_fixed_of(double x, int e) { return qcs_oz::fixed_of(x, e); }
 extern "C" long long host_fx_of1(double x, int f) { return fx_of1(x, f); }
 extern "C" long long host_shift1(long long X, int s) { return fx_shift1(X, s); }
+extern "C" long long host_scale(long long z, int g) { return qcs_oz::scale_of_fixed(z, g); }
 extern "C" long long host_shift_any(long long X, int s) { return fx_shift_any(X, s); }
 """
 
@@ -23,7 +24,7 @@ extern "C" long long host_shift_any(long long X, int s) { return fx_shift_any(X,
 @pytest.fixture(scope="module")
 def host(tmp_path_factory):
     lib = warp_emulation.compile_host(SOURCE, ["qcs_fixed.cuh"], str(tmp_path_factory.mktemp("emu")))
-    for f in ("host_fixed_of", "host_fx_of1", "host_shift1", "host_shift_any"):
+    for f in ("host_fixed_of", "host_fx_of1", "host_shift1", "host_scale", "host_shift_any"):
         getattr(lib, f).restype = ctypes.c_longlong
         getattr(lib, f).argtypes = [ctypes.c_double if "of" in f else ctypes.c_longlong, ctypes.c_int]
     return lib
@@ -58,3 +59,26 @@ def test_shifts_round_to_nearest(host):
             exact = 0 if s < -200 else floor(Fraction(X) * Fraction(2) ** s + Fraction(1, 2))
             assert host.host_shift_any(X, s) == exact, (X, s)
             assert host.host_shift1(X, s) == exact, (X, s)
+
+
+def test_scale_bounds_every_entry(host):
+    """2^G lies above every |z| 2^g (1 + 2^-7), whichever entry has the largest g, so that the
+    slices' integers z 2^{55 + g - G} fit 55 bits; and by at most three bits where the upper
+    word decides."""
+    rng = random.Random(6)
+    zs = [s * ((1 << b) + d) for b in range(61) for d in (-1, 0, 1) for s in (1, -1)] + [rng.randrange(-(1 << 62), 1 << 62)
+                                                                                        for _ in range(200)]
+    for z in zs:
+        for g in (-80, 0, 40):
+            G = host.host_scale(z, g)
+            if z == 0:
+                assert G == -100000
+                continue
+            assert abs(z) * 129 < 128 << (G - g), (z, g)
+            if abs(z) >> 33:
+                assert abs(z) << 3 >= 1 << (G - g), (z, g)
+    # an entry without an upper word whose exponent exceeds the others'
+    for za, ga, zb, gb in ((1 << 55, -80, 1 << 21, 0), (1 << 55, 0, 1 << 26, 40)):
+        G = max(host.host_scale(za, ga), host.host_scale(zb, gb))
+        for z, g in ((za, ga), (zb, gb)):
+            assert abs(z) * Fraction(2) ** (55 + g - G) < 1 << 55
