@@ -54,8 +54,11 @@
  *   cudaMalloc, synchronously, or with the caller's allocator set by
  *   qcs_set_allocator) when a call needs more than it holds.  Call each entry
  *   point once with the largest sizes before capturing it in a CUDA graph so
- *   that no allocation happens during capture.  Calls on the same context must
- *   not overlap in time on different streams.
+ *   that no allocation happens during capture.  Where a call works in batches
+ *   (tensor-core overlaps, RDMs) and the allocator refuses the largest, it takes
+ *   half of it and so on; the context remembers the refusal until
+ *   qcs_set_allocator is called, so a repeated call asks for nothing.  Calls on
+ *   the same context must not overlap in time on different streams.
  */
 #ifndef QCS_H
 #define QCS_H
@@ -273,7 +276,8 @@ qcs_status qcs_overlap(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t W, 
  * Pfaffians run in 64-bit fixed point.  The snapshot set then holds 57,856 bytes per four
  * parity +1 snapshots of slice records (formed by qcs_build_snapshots at n = 16,
  * otherwise on first use), and the context workspace 14,464 bytes per walker and at most
- * 512 MB of pair records, worked off in batches. */
+ * 512 MB of pair records, worked off in batches (smaller ones, down to 32 snapshots of one
+ * walker, when the allocator refuses the workspace). */
 
 /* ---------------------------------------------------- local energy terms */
 
@@ -321,7 +325,8 @@ double qcs_local_energy_flops_per_pair(int n, int ne, int nchol, int has_h, int 
  *             (Eqs. 1rdm_off_diagonal, 1rdm_diagonal)
  *   d_npart : 1 double or NULL: the particle number, trace of the 1-RDM
  * Outputs are device buffers owned by the caller.  The call uses context workspace
- * (P n (2n-1) 8-byte covariance entries, their slices, and the moment partials).
+ * (P n (2n-1) 8-byte covariance entries, the slices of at most 65536 snapshots, fewer when the
+ * allocator refuses them, and the moment partials).
  * Errors: QCS_ERR_ARG (empty set, set on another device, d_gam4 with n < 2), QCS_ERR_CUDA. */
 qcs_status qcs_shadow_rdm(qcs_ctx *ctx, const qcs_snapshots *s, const double *d_R, double *d_gam2, double *d_gam4,
                           double *d_rdm1, double *d_npart, void *stream);

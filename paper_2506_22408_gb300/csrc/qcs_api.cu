@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -73,7 +74,10 @@ qcs_status qcs_dev_alloc(const qcs_allocator &a, void **p, size_t bytes, cudaStr
         *p = a.alloc(bytes, (void *)st, a.user);
         return *p ? QCS_OK : QCS_ERR_CUDA;
     }
-    return cudaMalloc(p, bytes) == cudaSuccess ? QCS_OK : QCS_ERR_CUDA;
+    if (cudaMalloc(p, bytes) == cudaSuccess) return QCS_OK;
+    cudaGetLastError();  // a refusal is this call's answer, not the next launch's error
+    *p = nullptr;
+    return QCS_ERR_CUDA;
 }
 
 void qcs_dev_free(const qcs_allocator &a, void *p, size_t bytes) {
@@ -100,6 +104,22 @@ qcs_status qcs_workspace(qcs_ctx *ctx, size_t bytes, void **out, cudaStream_t st
     return QCS_OK;
 }
 
+// The workspace of a call that works in batches: bytes(batch) for the largest batch among
+// most, most / 2, ... (at least `least`) that the allocator gives.  A refused size is not asked
+// for again until the allocator is set (so that a repeated call allocates nothing, also under
+// capture), but for the smallest batch.
+qcs_status qcs_workspace_batched(qcs_ctx *ctx, int64_t most, int64_t least,
+                                 const std::function<size_t(int64_t)> &bytes, void **out, cudaStream_t st) {
+    for (int64_t batch = most;; batch = batch / 2 > least ? batch / 2 : least) {
+        const size_t need = align16(bytes(batch));
+        if (batch > least && need > ctx->work_bytes && need >= ctx->work_refused) continue;
+        const qcs_status r = qcs_workspace(ctx, need, out, st);
+        if (r == QCS_OK || batch <= least) return r;
+        ctx->work_refused = need;
+        qcs_log(2, "  workspace of %zu bytes refused: smaller batches", need);
+    }
+}
+
 extern "C" qcs_status qcs_set_allocator(qcs_ctx *ctx, qcs_alloc_fn alloc_fn, qcs_free_fn free_fn, void *user) {
     if (!ctx) return QCS_ERR_ARG;
     if ((alloc_fn == nullptr) != (free_fn == nullptr))
@@ -111,6 +131,7 @@ extern "C" qcs_status qcs_set_allocator(qcs_ctx *ctx, qcs_alloc_fn alloc_fn, qcs
         ctx->work = nullptr;
         ctx->work_bytes = 0;
     }
+    ctx->work_refused = SIZE_MAX;
     ctx->alloc.alloc = alloc_fn;
     ctx->alloc.free = free_fn;
     ctx->alloc.user = user;
@@ -401,7 +422,7 @@ extern "C" int qcs_snapshots_modes(const qcs_snapshots *s) { return s ? s->n : -
 namespace {
 
 const int kChunk = 4;  // snapshots per warp in an overlap tile
-const size_t kBatchBytes = (size_t)512 << 20;  // pair records of one tensor-core batch
+const int64_t kBatchBytes = (int64_t)512 << 20;  // pair records of one tensor-core batch, at most
 
 struct OverlapWork {
     cd *Ut, *pref, *partial;
@@ -476,37 +497,42 @@ qcs_status overlap_common(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t 
     wk->chunk = cfg.chunk > 0 ? cfg.chunk : kChunk;
     // partial sums: FP64 ALU path one per (walker, tile, warp); split path one per
     // (walker, tile of snapshots); tensor-core path one per (walker, batch)
-    wk->wblock = W > 0 ? W : 1;
-    int span = split ? qcs_split_snaps_per_tile(n, cfg.subs) : wk->chunk * qcs_pair_warps_per_block();
-    if (tc) {
-        // a batch's pair records take at most kBatchBytes: all walkers and as many list
-        // positions as fit, walkers in blocks when 32 positions of all of them do not
-        const int64_t fit = (int64_t)(kBatchBytes / (size_t)qcs_pf_rec_bytes(n, ne));
-        if (wk->wblock > fit / 32) wk->wblock = fit / 32;
-        const int64_t all = (s->P + 31) / 32 * 32;
-        int64_t sp = fit / wk->wblock / 32 * 32;
-        if (sp > all) sp = all > 0 ? all : 32;
-        span = (int)sp;
-    }
-    wk->span = span;
-    wk->nchunks = (int)((s->P + span - 1) / span);
-    if (wk->nchunks < 1) wk->nchunks = 1;
-    wk->nparts = (split || tc) ? wk->nchunks : wk->nchunks * qcs_pair_warps_per_block();
+    const size_t b_ut = align16(sizeof(cd) * (size_t)W * n * n);
+    const size_t b_pref = align16(sizeof(cd) * (size_t)W);
+    const size_t b_slab = split ? align16(qcs_split_walker_bytes(n, W)) : 0;
+    const size_t b_rec = tc ? align16(qcs_tc_walker_bytes(W)) : 0;
+    size_t b_part = 0, b_sum = 0, b_cnt = 0, b_all = 0;
+    const int64_t pair_bytes = qcs_pf_rec_bytes(n, ne);
+    auto layout = [&](int64_t batch_bytes) {
+        wk->wblock = W > 0 ? W : 1;
+        wk->span = split ? qcs_split_snaps_per_tile(n, cfg.subs) : wk->chunk * qcs_pair_warps_per_block();
+        if (tc) {
+            // a batch's pair records take at most batch_bytes: all walkers and as many list
+            // positions as fit, walkers in blocks when 32 positions of all of them do not
+            const int64_t fit = batch_bytes / pair_bytes;
+            if (wk->wblock > fit / 32) wk->wblock = fit / 32;
+            const int64_t all = (s->P + 31) / 32 * 32;
+            int64_t sp = fit / wk->wblock / 32 * 32;
+            if (sp > all) sp = all > 0 ? all : 32;
+            wk->span = (int)sp;
+        }
+        wk->nchunks = (int)((s->P + wk->span - 1) / wk->span);
+        if (wk->nchunks < 1) wk->nchunks = 1;
+        wk->nparts = (split || tc) ? wk->nchunks : wk->nchunks * qcs_pair_warps_per_block();
+        const size_t batch = tc ? (size_t)wk->wblock * wk->span : 0;
+        b_part = align16(sizeof(cd) * (size_t)W * wk->nparts);
+        b_sum = align16(batch * sizeof(cd));
+        b_cnt = tc ? align16(sizeof(unsigned long long) * (size_t)qcs_tc_counters(W > 0 ? W : 1, wk->wblock, wk->nchunks)) : 0;
+        b_all = 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec;
+        return b_all + b_cnt + b_sum + (tc ? align16(batch * (size_t)pair_bytes) : 0);
+    };
+    void *base = nullptr;
+    const int64_t most = tc ? kBatchBytes : 1;
+    qcs_status ws = qcs_workspace_batched(ctx, most, tc ? 32 * pair_bytes : most, layout, &base, st);
+    if (ws != QCS_OK) return ws;
     qcs_log(2, "  n=%d ne=%d W=%lld P=%lld nodes=%d path=%s config=0x%x tiles of %d snapshots", n, ne, (long long)W,
             (long long)s->P, plan->nev, split ? "split-tf32x3" : (tc ? "fp64-tensor-core" : "fp64-alu"),
-            (unsigned)wk->config, span);
-    size_t b_ut = align16(sizeof(cd) * (size_t)W * n * n);
-    size_t b_pref = align16(sizeof(cd) * (size_t)W);
-    size_t b_part = align16(sizeof(cd) * (size_t)W * wk->nparts);
-    size_t b_slab = split ? align16(qcs_split_walker_bytes(n, W)) : 0;
-    size_t b_rec = tc ? align16(qcs_tc_walker_bytes(W)) : 0;
-    const size_t batch = tc ? (size_t)wk->wblock * wk->span : 0;
-    size_t b_pair = tc ? align16(batch * qcs_pf_rec_bytes(n, ne)) : 0, b_sum = align16(batch * sizeof(cd));
-    size_t b_cnt = tc ? align16(sizeof(unsigned long long) * (size_t)qcs_tc_counters(W > 0 ? W : 1, wk->wblock, wk->nchunks)) : 0;
-    const size_t b_all = 16 + b_ut + b_pref + b_part + 2 * b_slab + b_rec;
-    void *base = nullptr;
-    qcs_status ws = qcs_workspace(ctx, b_all + b_cnt + b_sum + b_pair, &base, st);
-    if (ws != QCS_OK) return ws;
+            (unsigned)wk->config, wk->span);
     char *pb = (char *)base;
     wk->counter = (unsigned long long *)(tc ? pb + b_all : pb);
     wk->sum = (cd *)(pb + b_all + b_cnt);

@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <functional>
 #include <map>
 #include <string>
 #include <tuple>
@@ -31,6 +32,7 @@ struct qcs_ctx {
     unsigned *h_status = nullptr;  // pinned host mirror
     void *work = nullptr;          // device workspace
     size_t work_bytes = 0;
+    size_t work_refused = SIZE_MAX;  // smallest workspace the allocator has refused
     qcs_allocator alloc;           // where the workspace and snapshot buffers come from
     std::string last_error;
     std::map<std::tuple<int, int, int, unsigned>, int> tuned;  // (n, ne, nodes, flags) -> config
@@ -94,6 +96,8 @@ struct QcsRange {
 };
 qcs_status qcs_set_smem(qcs_ctx *ctx, const void *func, size_t bytes);
 qcs_status qcs_workspace(qcs_ctx *ctx, size_t bytes, void **out, cudaStream_t st = nullptr);
+qcs_status qcs_workspace_batched(qcs_ctx *ctx, int64_t most, int64_t least,
+                                 const std::function<size_t(int64_t)> &bytes, void **out, cudaStream_t st);
 
 // Launchers implemented in the kernel translation units
 qcs_status qcs_launch_snapshot_build(qcs_ctx *ctx, qcs_snapshots *s, const double *d_Q, const uint8_t *d_b,

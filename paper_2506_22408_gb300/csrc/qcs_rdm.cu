@@ -28,7 +28,7 @@ constexpr int kTile = 32;     // S2 tile edge (small tiles: less work in the low
 constexpr int kTThreads = 64; // threads per S2 tile: 8 x 8, each 4 x 4 entries
 constexpr int kKStep = 16;    // snapshots staged per step
 constexpr int kColRows = 256; // rows per column-sum partial (at least)
-constexpr int64_t kMBatch = 65536;  // snapshots whose slices are held at once (0.47 GB at n = 16)
+constexpr int64_t kMBatch = 65536;  // snapshots whose slices are held at once, at most (0.47 GB at n = 16)
 
 // Upper-triangle pair index of (mu, nu), mu < nu < N2, in row-major order.
 __host__ __device__ __forceinline__ int pair_rank(int mu, int nu, int N2) {
@@ -593,22 +593,26 @@ extern "C" qcs_status qcs_shadow_rdm(qcs_ctx *ctx, const qcs_snapshots *s, const
     int ntc = 0;
     for (int ti = 0; 2 * ti < ncol; ++ti) ntc += ncol - 2 * ti;
     constexpr int64_t kSum = (int64_t)kMStagesPerSum * kMK;
-    const int64_t batch = P < kMBatch ? (P + kSum - 1) / kSum * kSum : kMBatch;
+    const size_t b_gu = align16(sizeof(double) * (size_t)P * npair);
+    const size_t b_part = align16(sizeof(double) * (size_t)nrow * npair);
     int nks = 1;
-    if (d_gam4) {
-        nks = ctx->num_sms / ntc;
-        const int64_t maxks = batch / kSum;
-        if (nks > maxks) nks = (int)maxks;
-        if (nks < 1) nks = 1;
-    }
-    const int64_t krange = ((P + nks - 1) / nks + kKStep - 1) / kKStep * kKStep;
-    size_t b_gu = align16(sizeof(double) * (size_t)P * npair);
-    size_t b_part = align16(sizeof(double) * (size_t)nrow * npair);
-    size_t b_s2 = d_gam4 ? align16(sizeof(double) * (size_t)nks * npair * npair) : 0;
-    size_t b_rec = d_gam4 ? (size_t)ncol * (size_t)(batch / kMK) * kMRec : 0;
+    int64_t batch = 0;
+    size_t b_s2 = 0;
+    auto layout = [&](int64_t sums) {
+        batch = sums * kSum;
+        if (d_gam4) {
+            nks = ctx->num_sms / ntc;
+            if (nks > sums) nks = (int)sums;
+            if (nks < 1) nks = 1;
+        }
+        b_s2 = d_gam4 ? align16(sizeof(double) * (size_t)nks * npair * npair) : 0;
+        return 16 + b_gu + b_part + b_s2 + (d_gam4 ? (size_t)ncol * (size_t)(batch / kMK) * kMRec : 0);
+    };
     void *base = nullptr;
-    qcs_status ws = qcs_workspace(ctx, 16 + b_gu + b_part + b_s2 + b_rec, &base, st);
+    const int64_t most = P < kMBatch ? (P + kSum - 1) / kSum : kMBatch / kSum;
+    qcs_status ws = qcs_workspace_batched(ctx, most, d_gam4 ? 1 : most, layout, &base, st);
     if (ws != QCS_OK) return ws;
+    const int64_t krange = ((P + nks - 1) / nks + kKStep - 1) / kKStep * kKStep;
     unsigned *d_max = (unsigned *)base;
     double *Gu = (double *)((char *)base + 16);
     double *part = (double *)((char *)base + 16 + b_gu);
