@@ -11,12 +11,23 @@
 // one scale loses nothing (the reduced form [I; X], with entries up to 16, would cost the
 // others four bits).
 //
-// Ranges: with entries below 2^57 (walker and snapshot rows) or 2^56 (T, K) and at most 48
-// terms, the final sums stay below 2^63; partial ones may wrap, which two's complement undoes.
+// T is held in 56 bits as two limbs of 28: the dropped products of the lower limbs are below
+// 2^54, a quarter of what limbs of 29 drop, and B keeps 56 bits instead of 54 (n = 6, ne = 4:
+// pair errors of 4 10^-16 rms instead of 1.1 10^-15; the same instructions).
+//
+// Ranges, for rows of any values: a sum's hh and cr are formed modulo 2^64, so partial sums and
+// the three products' own sums may wrap, but the final hh, cr and value must stay below 2^63.
+// Per real product |h h'| and |h l'| + |l h'| are at most
+//     T (57 bits times 57, S = 29):  2^56, 2^57    2n products: 2^61.6, 2^62.6 (n = 24)
+//     B from T (56 times 56, S = 28): 2^56, 2^56   4n products: 2^62.6, 2^62.6, value 2^62.6
+//     B from K (56 times 57, S = 29): 2^55, 2^55 + 2^56   4n products: 2^61.6, and for cr
+//         2^62.7: a walker row has norm one, so its parts sum to at most sqrt(2n) of it, 28 of
+//         48 times the scale 2^-2 that its largest part has at least (n = 24).
 #pragma once
 #include "qcs_fixed.cuh"
 
-constexpr int kFxS = 29;  // the limbs of this file: X = h 2^29 + l
+constexpr int kFxS = 29;   // the limbs of this file: X = h 2^29 + l
+constexpr int kFxST = 28;  // ... of T, both factors of B: 56 bits in two equal limbs
 
 __device__ __forceinline__ fxl fx_re(int4 q) { return fxl{q.x, q.y}; }
 __device__ __forceinline__ fxl fx_im(int4 q) { return fxl{q.z, q.w}; }
@@ -112,7 +123,8 @@ __device__ inline unsigned fx_build_T(int n, int ne, const int4 *__restrict__ U,
 }
 
 // T of a signed-permutation snapshot: row c of Qt has one nonzero entry, the phase
-// code & 3 at column code >> 2, so T[j][c] = Ut[j][k_c] ph_c is a gather of limbs.
+// code & 3 at column code >> 2, so T[j][c] = Ut[j][k_c] ph_c is a gather, of 56 bits (worth
+// V 2^{1-fU}).
 __device__ inline void fx_gather_T(int n, const int4 *__restrict__ U, const uint8_t *__restrict__ code,
                                    int4 *__restrict__ T, int t, int nthr) {
     const int n2 = 2 * n, lt = ld_t(n);
@@ -120,14 +132,16 @@ __device__ inline void fx_gather_T(int n, const int4 *__restrict__ U, const uint
         const int j = e / n2, c = e - j * n2;
         const unsigned q = code[c], ph = q & 3u;
         const int4 u = U[j * (n + 1) + (int)(q >> 2)];
-        fxl re = (ph & 1u) ? fx_im(u) : fx_re(u), im = (ph & 1u) ? fx_re(u) : fx_im(u);
-        if (ph == 1u || ph == 2u) re = fx_neg(re);
-        if (ph >= 2u) im = fx_neg(im);
-        T[j * lt + c] = fx_pack(re, im);
+        const fxl a = (ph & 1u) ? fx_im(u) : fx_re(u), b = (ph & 1u) ? fx_re(u) : fx_im(u);
+        long long re = (((long long)a.h << kFxS) + a.l + 1) >> 1, im = (((long long)b.h << kFxS) + b.l + 1) >> 1;
+        if (ph == 1u || ph == 2u) re = -re;
+        if (ph >= 2u) im = -im;
+        T[j * lt + c] = fx_pack(fx_split<kFxST>(re), fx_split<kFxST>(im));
     }
 }
 
 // n x 2n integers of T in place as limbs, the largest (b bits) shifted to 56 bits.
+template <int S>
 __device__ __forceinline__ void fx_T_limbs(int n, void *T, int b, int t, int nthr) {
     const int n2 = 2 * n, lt = ld_t(n);
     fx2 *v = reinterpret_cast<fx2 *>(T);
@@ -136,14 +150,14 @@ __device__ __forceinline__ void fx_T_limbs(int n, void *T, int b, int t, int nth
     for (int e = t; e < n * n2; e += nthr) {
         const int j = e / n2, i = j * lt + e - j * n2;
         const fx2 x = fx_shift(v[i], 56 - b);
-        q[i] = fx_pack(fx_split<kFxS>(x.x), fx_split<kFxS>(x.y));
+        q[i] = fx_pack(fx_split<S>(x.x), fx_split<S>(x.y));
     }
 }
 
 // Real part (odd = false) or imaginary part of a limb entry.
 __device__ __forceinline__ fxl fx_part(int4 q, bool odd) { return odd ? fx_im(q) : fx_re(q); }
 
-// B^(s) (packed, the empty modes' rows first, worth X 2^{58-2f} for T worth 2^-f) from T: row c
+// B^(s) (packed, the empty modes' rows first, worth X 2^{56-2f} for T worth 2^-f) from T: row c
 // of an empty mode j = ne + c/2 is Re T_j (c even) or -Im T_j (c odd), the occupied row x is
 // T_x; B_ab = sum_k X_a,2k X_b,2k+1 - X_a,2k+1 X_b,2k.  One loop per block (real x real, real x
 // complex, complex x complex).  Returns this thread's OR of the upper words.
@@ -157,13 +171,13 @@ __device__ inline unsigned fx_build_B(int n, int ne, const int4 *__restrict__ T,
         pair_of(tab, e, a, b);
         const bool oa = a & 1, ob = b & 1;
         const int4 *ra = T + (ne + (a >> 1)) * lt, *rb = T + (ne + (b >> 1)) * lt;
-        fxacc s = {0, fx_half<kFxS>(58)};
+        fxacc s = {0, fx_half<kFxST>(56)};
 #pragma unroll 1
         for (int k = 0; k < n; ++k) {
             fx_mac(s, fx_part(ra[2 * k], oa), fx_part(rb[2 * k + 1], ob));
             fx_mac(s, fx_neg(fx_part(ra[2 * k + 1], oa)), fx_part(rb[2 * k], ob));
         }
-        const long long v = fx_value<kFxS>(s, 58);
+        const long long v = fx_value<kFxST>(s, 56);
         const fx2 x = make_longlong2(oa != ob ? -v : v, 0ll);
         top |= fx_top(x);
         B[e] = x;
@@ -173,7 +187,7 @@ __device__ inline unsigned fx_build_B(int n, int ne, const int4 *__restrict__ T,
         const int x = e / d2, c = e - x * d2;
         const bool odd = c & 1;
         const int4 *rc = T + (ne + (c >> 1)) * lt, *rx = T + x * lt;
-        fxacc re = {0, fx_half<kFxS>(58)}, im = {0, fx_half<kFxS>(58)};
+        fxacc re = {0, fx_half<kFxST>(56)}, im = {0, fx_half<kFxST>(56)};
 #pragma unroll 1
         for (int k = 0; k < n; ++k) {
             const fxl c0 = fx_part(rc[2 * k], odd), c1 = fx_neg(fx_part(rc[2 * k + 1], odd));
@@ -183,7 +197,7 @@ __device__ inline unsigned fx_build_B(int n, int ne, const int4 *__restrict__ T,
             fx_mac(re, c1, fx_re(x0));
             fx_mac(im, c1, fx_im(x0));
         }
-        const fx2 v = fx_neg_if(make_longlong2(fx_value<kFxS>(re, 58), fx_value<kFxS>(im, 58)), odd);
+        const fx2 v = fx_neg_if(make_longlong2(fx_value<kFxST>(re, 56), fx_value<kFxST>(im, 56)), odd);
         top |= fx_top(v);
         B[tri_index(c, d2 + x)] = v;
     }
@@ -192,7 +206,7 @@ __device__ inline unsigned fx_build_B(int n, int ne, const int4 *__restrict__ T,
         int a, b;
         pair_of(tab, e, a, b);
         const int4 *ra = T + a * lt, *rb = T + b * lt;
-        fxacc re = {0, fx_half<kFxS>(58)}, im = {0, fx_half<kFxS>(58)};
+        fxacc re = {0, fx_half<kFxST>(56)}, im = {0, fx_half<kFxST>(56)};
 #pragma unroll 1
         for (int k = 0; k < n; ++k) {
             const int4 a0 = ra[2 * k], a1 = ra[2 * k + 1], b0 = rb[2 * k], b1 = rb[2 * k + 1];
@@ -205,7 +219,7 @@ __device__ inline unsigned fx_build_B(int n, int ne, const int4 *__restrict__ T,
             fx_mac(re, fx_im(a1), fx_im(b0));
             fx_mac(im, fx_neg(fx_im(a1)), fx_re(b0));
         }
-        const fx2 v = make_longlong2(fx_value<kFxS>(re, 58), fx_value<kFxS>(im, 58));
+        const fx2 v = make_longlong2(fx_value<kFxST>(re, 56), fx_value<kFxST>(im, 56));
         top |= fx_top(v);
         B[tri_index(d2 + a, d2 + b)] = v;
     }

@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(128, 4) grad_pair_kernel(const __grid_constant
                 group_sync(bar);
                 const int kb = fx_top_bits(tm.or_get(top, 0));
                 const int fK = fU + fQ - 58 + 56 - kb;
-                fx_T_limbs(n, Ks, kb, t, kGroup);
+                fx_T_limbs<kFxS>(n, Ks, kb, t, kGroup);
                 group_sync(bar);
                 top = tm.or_put(fx_build_B_from_K(n, ne, Us, Ks, Xs, tab, t, kGroup), 1);
                 group_sync(bar);

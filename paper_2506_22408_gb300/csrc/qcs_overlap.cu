@@ -113,6 +113,7 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
             tm.sync();  // the previous pair is done with the team's region
             if (gat) {
                 fx_gather_T(n, Us, gq, Ts, tm.t, tm.NT);  // signed permutation: no products
+                fT = fU - 1;
             } else {
                 // T (or K) by column halves: half of the snapshot's rows staged at a time
                 const cd *Qr = (A.Qh ? A.Qh : A.Qt) + q * n2 * n;
@@ -134,7 +135,8 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
                     const int b = fx_top_bits(tm.or_get(top, par));
                     par ^= 1;
                     fT = fU + fQ - 58 + 56 - b;
-                    fx_T_limbs(n, Ts, b, tm.t, tm.NT);
+                    if (fromK) fx_T_limbs<kFxS>(n, Ts, b, tm.t, tm.NT);
+                    else fx_T_limbs<kFxST>(n, Ts, b, tm.t, tm.NT);
                 }
             }
             tm.sync();
@@ -150,7 +152,7 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
                     par ^= 1;
                     tm.sync();  // the words of the reduction are free again
                     S = fx_pair_eliminate(tm, A.m, A.ne, shared, A.NB, A.plan, wk, Xs, Ns,
-                                          fromK ? fT + fU - 58 : 2 * fT - 58, mb, tab, ok);
+                                          fromK ? fT + fU - 58 : 2 * fT - 56, mb, tab, ok);
                     shared = false;
                     tm.sync();
                 } while (!ok);

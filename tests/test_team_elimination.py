@@ -6,6 +6,7 @@ just below it, whose truncated magnitude then ties with the pivot's."""
 from __future__ import annotations
 
 import ctypes
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -159,3 +160,32 @@ def test_schedules_agree(host, NW, d2, ne, shared, kind):
     assert all(x == results[0] for x in results) and results[0][0] >= 0
     if results[0][0] == 1:
         assert abs(results[0][1] - ref) <= 1e-10 * scale
+
+
+def exact_pf4(X, w, f):
+    """Exact pf of the 4 x 4 matrix X 2^-f + w D (D pairs (0, 1) and (2, 3))."""
+    z = [(Fraction(int(x), 1 << f), Fraction(int(y), 1 << f)) for x, y in X]  # 01, 02, 12, 03, 13, 23
+    wd = (Fraction(w.real), Fraction(w.imag))
+    add = lambda a, b: (a[0] + b[0], a[1] + b[1])
+    mul = lambda a, b: (a[0] * b[0] - a[1] * b[1], a[0] * b[1] + a[1] * b[0])
+    p, q, r = mul(add(z[0], wd), add(z[5], wd)), mul(z[1], z[4]), mul(z[3], z[2])
+    return p[0] - q[0] + r[0], p[1] - q[1] + r[1]
+
+
+@pytest.mark.parametrize("bits", [52, 54, 57])
+def test_a_complement_of_four_keeps_its_bits(host, bits):
+    """Without an occupied index or an update, whatever bits B arrives with: entries below two
+    in modulus are held to 2^-57 (half a unit lost in the closing shift, w to 2^-59), which a
+    product of two turns into at most 4 * 2 * 2^-58 for its part, its dropped limb product and
+    rounding into as much again; three products: 6 2^-55.  The value's own rounding to FP64 and
+    the product with gamma (normalised to 60 bits) add 2^-53 + 2^-56 of its modulus."""
+    rng = np.random.default_rng(bits)
+    for _ in range(40):
+        X = rng.integers(-(1 << bits), 1 << bits, (6, 2))
+        X[rng.integers(6)] = ((1 << bits) - 1, 0)
+        w = np.exp(2j * np.pi * rng.random())
+        r, S = host(1, 4, 0, True, 1, [(w, 1.0 + 0j)], X, bits, bits, 0)
+        ex = exact_pf4(X, w, bits)
+        assert r == 1
+        tol = Fraction(6, 1 << 55) + Fraction(abs(S)) * Fraction(9, 1 << 56)
+        assert max(abs(Fraction(S.real) - ex[0]), abs(Fraction(S.imag) - ex[1])) <= tol
