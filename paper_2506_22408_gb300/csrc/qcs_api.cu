@@ -357,7 +357,7 @@ extern "C" qcs_status qcs_build_snapshots(qcs_ctx *ctx, int n, int64_t P, const 
     qcs_status ae = qcs_dev_alloc(s->alloc, (void **)&s->Qt, sizeof(cd) * (size_t)Pa * 2 * n * n, cs);
     if (ae == QCS_OK) ae = qcs_dev_alloc(s->alloc, (void **)&s->parity, (size_t)Pa, cs);
     if (ae == QCS_OK) ae = qcs_dev_alloc(s->alloc, (void **)&s->idx, sizeof(int) * (size_t)Pa, cs);
-    if (ae == QCS_OK) ae = qcs_dev_alloc(s->alloc, (void **)&s->d_count, 2 * sizeof(int), cs);
+    if (ae == QCS_OK) ae = qcs_dev_alloc(s->alloc, (void **)&s->d_count, 3 * sizeof(int), cs);
     if (ae == QCS_OK) ae = qcs_dev_alloc(s->alloc, (void **)&s->gth, (size_t)Pa * 2 * n, cs);
     if (ae != QCS_OK) {
         qcs_snapshots_free(s);
@@ -396,7 +396,7 @@ extern "C" qcs_status qcs_snapshots_free(qcs_snapshots *s) {
     qcs_dev_free(s->alloc, s->Qt, sizeof(cd) * Pa * 2 * n * n);
     qcs_dev_free(s->alloc, s->parity, Pa);
     qcs_dev_free(s->alloc, s->idx, sizeof(int) * Pa);
-    qcs_dev_free(s->alloc, s->d_count, 2 * sizeof(int));
+    qcs_dev_free(s->alloc, s->d_count, 3 * sizeof(int));
     qcs_dev_free(s->alloc, s->gth, Pa * 2 * n);
     qcs_dev_free(s->alloc, s->split_hi, s->split_bytes);
     qcs_dev_free(s->alloc, s->split_lo, s->split_bytes);
@@ -616,7 +616,7 @@ extern "C" qcs_status qcs_overlap_batched(qcs_ctx *ctx, int nsys, const qcs_syst
     if (o.precision != QCS_FP64) return qcs_fail(ctx, QCS_ERR_UNSUPPORTED, "batched calls are FP64");
     qcs_pair_launch Ls[QCS_MAX_SYSTEMS];
     size_t off[QCS_MAX_SYSTEMS][3];
-    size_t total = 16;  // the tile counter first
+    size_t total = 16;  // the tile counters first
     const int wpb = qcs_pair_warps_per_block();
     for (int i = 0; i < nsys; ++i) {
         const qcs_system &y = systems[i];

@@ -421,10 +421,19 @@ __device__ __forceinline__ void fx_swap_last(const Team &tm, fx2 *__restrict__ N
 // Both kinds of job run the same step code: one copy keeps the loop in the instruction
 // caches (two inlined copies cost the 20-warp kernel 20 % of its issue slots in
 // instruction misses).
-template <class Team>
+//
+// With kGuard, *lost is set (and ok cleared) when a node's pivot is below 2^-kFxGuard of its
+// matrix, or its closing Pfaffian below 2^-(kFxGuard + 6): B is held to 2^-57 of its largest
+// entry, so little would be left of such a pair; an occupied pivot that small sends the pair to the
+// full elimination.  The records of the product are looked at, not each step's pivot, which took
+// 3 % of the steps' time.  Walkers at 10^-2 to 10^-6 from a basis determinant against signed
+// permutations (5 and 6 modes) keep 6 10^-11 of a pair's magnitude at worst, 3 10^-10 with
+// kFxGuard = 12; a tenth to a half of their pairs is handed over, none of a random walker's.
+constexpr int kFxGuard = 10;
+template <bool kGuard = false, class Team>
 __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool shared, int NB, const FxPlan &plan,
                                        const FxWork &wk, fx2 *X, fx2 *Ns, int f, int mb,
-                                       const uint16_t *__restrict__ tab, bool &ok) {
+                                       const uint16_t *__restrict__ tab, bool &ok, bool *lost = nullptr) {
     const int d2 = m - ne, nev = plan.nev;
     const int bound = mb - f + 8;
     const int mm = shared ? d2 : m, npo = shared ? ne / 2 : 0, NBr = shared ? NB : 1;
@@ -446,6 +455,8 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
         const int S0 = mm == 0 ? 0 : (mm >= 4 ? mm / 2 - 1 : 1);  // a node's pivots and closing Pfaffian
         fx2 *N0 = occ ? X : Ns;  // the job's matrices, stride T
         int fc = f, mbc = mb;
+        // pivots below 2^least are refused (w_k has modulus one)
+        const int least = (occ || mb > f ? mb - f : 0) - kFxGuard;
         if (!occ && mm > 0) {
             // scale: room for S and for w_k (of modulus one).  A complement of four has no update
             // whose renormalisation would give entries of few bits their place: always scaled.
@@ -537,7 +548,7 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
                 for (int a = tm.lane; a < r - 1; a += 32) rt |= fx_top(row[a]);
                 const int rb = fx_top_bits(__reduce_or_sync(QCS_FULL, rt)), pb = fx_bits(row[P]);
                 if (rb >= pb) eu = rb - pb + 1;  // |g| 2^-eu < sqrt 2
-                if (eu > kFxMaxOcc) {
+                if (eu > kFxMaxOcc || (kGuard && pb - fc <= least)) {
                     ok = false;
                     return total;
                 }
@@ -654,6 +665,7 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
         tm.sync();
         // gamma[v] times the records of node v and the npo common ones: each lane of the segment
         // multiplies every seg-th of them, then a shuffle tree over the segment
+        bool tiny = false;
         fxp z = {1ll << 59, 0, -59};
         const int nrec = S0 + npo + 1, w = nrec < seg ? nrec : seg;  // lanes that hold a factor
 #pragma unroll 1
@@ -666,6 +678,7 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
                 const fx2 *x = !mul || node ? wk.pv + vr * S0 + (mul ? i : 0) : po ? pvo + (i - S0) : plan.g + k0 + vr;
                 const int e = !mul ? 0 : node ? -wk.pe[vr * S0 + i] : po ? -peo[i - S0] : plan.ge[k0 + vr];
                 if (mul) y = fx_norm(*x, e);
+                if (kGuard) tiny |= mul && po && ((y.x | y.y) == 0ll || y.e + 60 <= (i == S0 - 1 ? least - 6 : least));
                 i += seg;
             } else {
                 o >>= 1;
@@ -674,6 +687,15 @@ __device__ inline cd fx_pair_eliminate(const Team &tm, int m, int ne, bool share
                 mul = w > o;  // lanes without a factor hold one
             }
             if (mul) z = fx_prod(z, y);
+        }
+        if (kGuard) {
+            const unsigned t = tm.or_put(tiny, s & 1);
+            tm.sync();
+            if (tm.or_get(t, s & 1)) {
+                ok = false;
+                *lost = true;
+                return total;
+            }
         }
         // sum over the warp's nodes on the segments' first lanes
         cd S = cmk(0.0, 0.0);

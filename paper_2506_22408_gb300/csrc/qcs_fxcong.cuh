@@ -45,6 +45,25 @@ __device__ __forceinline__ unsigned fx_max_key(const cd *__restrict__ src, int c
     }
     return __reduce_max_sync(QCS_FULL, k);
 }
+// Whether more than one in 32, and four, of the parts that are not zero, of count complex FP64
+// numbers, lie below 2^-kFxSpan of the largest (key: its upper word), over a warp: one in a
+// hundred of a random walker's do, a quarter of one's at 10^-2 from a basis determinant.
+constexpr int kFxSpan = 8;
+__device__ __forceinline__ bool fx_wide(const cd *__restrict__ src, int count, unsigned key, int lane) {
+    const int lim = (int)(key >> 20) - kFxSpan;
+    unsigned small = 0u, all = 0u;
+    for (int e = lane; e < count; e += 32) {
+        const cd x = src[e];
+        const double parts[2] = {x.x, x.y};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned nz = (__double_as_longlong(parts[h]) << 1) != 0ll;
+            all += nz;
+            small += nz & (unsigned)((int)(((unsigned)__double2hiint(parts[h]) >> 20) & 0x7ff) < lim);
+        }
+    }
+    return 32u * __reduce_add_sync(QCS_FULL, small) > __reduce_add_sync(QCS_FULL, all) + 128u;
+}
 // Fraction bits with |x| 2^f < 2^bits for entries whose largest upper word is key.
 __device__ __forceinline__ int fx_fraction(unsigned key, int bits) { return bits + 1022 - (int)(key >> 20); }
 

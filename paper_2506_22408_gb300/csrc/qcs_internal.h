@@ -52,7 +52,8 @@ struct qcs_snapshots {
     cd *Qt = nullptr;         // P x 2n x n complexified sign-folded rows
     int8_t *parity = nullptr; // P: +1 / -1 (0: singular or non-finite Q)
     int *idx = nullptr;       // P: indices with parity +1, ascending (first *d_count valid)
-    int *d_count = nullptr;   // 2: number of parity +1 snapshots, number of signed permutations
+    int *d_count = nullptr;   // 3: number of parity +1 snapshots, of signed permutations, and of dense
+                              // snapshots with many zeros or small entries
     uint8_t *gth = nullptr;   // P x 2n gather codes of signed-permutation snapshots (row c of Qt:
                               // (k << 2) | phase, phase 0..3 = 1, i, -1, -i); first code 0xFF: dense
     void *split_hi = nullptr; // P x 4 KB TF32 operand slabs (split precision), built on first use
@@ -179,7 +180,7 @@ struct qcs_pair_launch {
     cd *per_pair;    // W x P or null
     qcs_node_plan plan;
     int config;      // qcs_config encoding; 0 = heuristic
-    unsigned long long *counter;  // device tile counters (reset by the launcher)
+    unsigned long long *counter;  // device tile counters, two at least (reset by the launcher)
     // tensor-core path: batches of wblock walkers x span list positions through pair records
     unsigned char *rec = nullptr;  // wblock x span records of qcs_pf_rec_bytes
     cd *sum = nullptr;             // wblock x span

@@ -31,6 +31,7 @@
 // in a fixed order afterwards, so the result does not depend on scheduling.
 #include "qcs_internal.h"
 #include "qcs_fxcong.cuh"
+#include "qcs_pairfp64.cuh"
 
 namespace {
 
@@ -63,16 +64,13 @@ struct PairScratch {
     int8_t rs[2 * QCS_MAX_N];  // row scales of the pair's snapshot
 };
 
-// One tile of system A: walker w = tile / nchunks, the tile's snapshots spread over the
-// block's teams of NW warps; each team writes one partial sum, in its first warp's slot (zero
-// in the second's).  Every thread of the block calls this (it contains block barriers
-// around the shared walker rows).
-template <int NW>
-__device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned char *base, int4 *Us,
-                         const uint16_t *tab, int warp, int wpb, int lane) {
+// The sum over the pairs of walker w with the snapshots p0, p0 + teams, ... below p1 of the list, on
+// the team's first thread.  Guarded pairs whose pivots show lost bits are evaluated in FP64.
+template <int NW, bool kGuarded>
+__device__ __forceinline__ cd tile_pairs(const PairArgs &A, int64_t w, int64_t p0, int64_t p1, int teams, int fU,
+                                         unsigned char *tb, const int4 *Us, const uint16_t *tab, int bar, int wid,
+                                         int lane) {
     const int n = A.n, n2 = 2 * n;
-    const int team = warp / NW, wid = warp % NW, teams = wpb / NW;
-    unsigned char *tb = base + (size_t)team * A.team_bytes;
     int4 *Qs = reinterpret_cast<int4 *>(tb);            // half of the snapshot's rows
     fx2 *Xs = reinterpret_cast<fx2 *>(tb);              // B^(s), once T is formed
     int4 *Ts = reinterpret_cast<int4 *>(tb + A.off_T);
@@ -81,7 +79,100 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
     PairScratch *scr = reinterpret_cast<PairScratch *>(tb + A.off_scr);
     const FxWork wk = {reinterpret_cast<FxGauss *>(tb + A.off_U), pv, reinterpret_cast<int *>(pv + A.npv + A.ne / 2),
                        A.npv};
-    const FxTeam<NW> tm = {32 * wid + lane, lane, wid, 1 + team, scr->red};
+    const FxTeam<NW> tm = {32 * wid + lane, lane, wid, bar, scr->red};
+    cd acc = cmk(0.0, 0.0);
+    for (int64_t pq = p0; pq < p1; pq += teams) {
+        const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
+        if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // team-uniform
+        const uint8_t *gq = A.gth ? A.gth + q * n2 : nullptr;
+        const bool gat = gq && gq[0] != 0xFF, fromK = !gat && A.Qh;
+        cd S = cmk(__longlong_as_double(0x7ff8000000000000ll), 0.0);
+        bool finite = true;
+        int fT = fU, par = 0;
+        tm.sync();  // the previous pair is done with the team's region
+        if (gat) {
+            fx_gather_T(n, Us, gq, Ts, tm.t, tm.NT);  // signed permutation: no products
+            fT = fU - 1;
+        } else {
+            // T (or K) by column halves: half of the snapshot's rows staged at a time
+            const cd *Qr = (A.Qh ? A.Qh : A.Qt) + q * n2 * n;
+            const unsigned key = fromK ? fx_max_key(Qr, n2 * n, lane) : fx_balance_rows(n, Qr, scr->rs, lane);
+            finite = key < 0x7ff00000u;
+            const int fQ = fx_fraction(key, 57);
+            unsigned top = 0u;
+            tm.sync();
+            for (int h = 0; h < 2 && finite; ++h) {
+                fx_stage_rows(n, n * n, Qr + (int64_t)h * n * n, fQ, fromK ? nullptr : scr->rs + h * n, Qs, tm.t, tm.NT);
+                tm.sync();
+                top |= fx_build_T(n, A.ne, Us, Qs, reinterpret_cast<fx2 *>(Ts), h * n, tm.t, tm.NT);
+                tm.sync();
+            }
+            if (finite) {
+                top = tm.or_put(top, par);
+                tm.sync();
+                const int b = fx_top_bits(tm.or_get(top, par));
+                par ^= 1;
+                fT = fU + fQ - 58 + 56 - b;
+                if (fromK) fx_T_limbs<kFxS>(n, Ts, b, tm.t, tm.NT);
+                else fx_T_limbs<kFxST>(n, Ts, b, tm.t, tm.NT);
+            }
+        }
+        tm.sync();
+        if (finite) {
+            bool shared = true, ok, lost = false;
+#pragma unroll 1
+            do {  // rarely a second time: B^(s) again, every node matrix in full
+                unsigned top = fromK ? fx_build_B_from_K(n, A.ne, Us, Ts, Xs, tab, tm.t, tm.NT)
+                                     : fx_build_B(n, A.ne, Ts, Xs, tab, tm.t, tm.NT);
+                top = tm.or_put(top, par);
+                tm.sync();
+                const int mb = fx_top_bits(tm.or_get(top, par));
+                par ^= 1;
+                tm.sync();  // the words of the reduction are free again
+                S = fx_pair_eliminate<kGuarded>(tm, A.m, A.ne, shared, A.NB, A.plan, wk, Xs, Ns,
+                                                fromK ? fT + fU - 58 : 2 * fT - 56, mb, tab, ok, &lost);
+                shared = false;
+                tm.sync();
+            } while (!ok && !lost);
+            if (kGuarded && lost) {  // in FP64, the first warp's value alone
+                S = fp64_pair_sum(tm, n, A.ne, A.plan, A.Ut + w * n * n, A.Qt + q * n2 * n, gat ? gq : nullptr,
+                                  reinterpret_cast<cd *>(Xs), reinterpret_cast<cd *>(Ns),
+                                  reinterpret_cast<cd *>(wk.GV), tab);
+                if (wid != 0) S = cmk(0.0, 0.0);
+            }
+        }
+        if (NW > 1) {  // the other warp's nodes
+            if (wid == 1 && lane == 0) scr->part = finite ? S : cmk(0.0, 0.0);
+            tm.sync();
+            if (wid == 0 && lane == 0) S = cadd(S, scr->part);
+        }
+        if (tm.t == 0) {
+            if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
+            acc = cadd(acc, S);
+            if (A.per_pair) A.per_pair[w * A.P + q] = cmul(A.pref[w], S);
+        }
+    }
+    return acc;
+}
+// One tile of system A: walker w = tile / nchunks, the tile's snapshots spread over the
+// block's teams of NW warps; each team writes one partial sum, in its first warp's slot (zero
+// in the second's).  Every thread of the block calls this (it contains block barriers
+// around the shared walker rows).  Returns whether the tile was left to the other pass.
+//
+// Guarded are the tiles in which B^(s) can hold entries of very different sizes, of which one
+// scale loses the small ones: a walker that has such entries where the set has signed
+// permutations, which copy them (the exact zeros of a basis determinant stay exact), and all
+// tiles of a set with a dense snapshot that is sparse or graded itself; both counted when the
+// set is built.  Haar-random snapshots mix the entries.  The guarded tiles are a pass of their
+// own, a call after the loop over the others: with the guard and the FP64 call in the only loop,
+// 12 modes took 13.88 instead of 13.26 ms and 8 modes 152 instead of 138 us without a single
+// guarded pair; with the choice made for each pair 13.45 ms and 143 us, for each tile 13.35 ms
+// and 141 us.
+template <int NW, bool kGuarded>
+__device__ bool run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned char *base, int4 *Us,
+                         const uint16_t *tab, int warp, int wpb, int lane) {
+    const int n = A.n;
+    const int team = warp / NW, wid = warp % NW, teams = wpb / NW;
     const int span = A.chunk * wpb;  // snapshots per tile; team g takes every teams-th
     // chunk-major tile order: consecutive tiles share one snapshot chunk and run over
     // the walkers (whose rows all fit in L2), so each snapshot is fetched from HBM once
@@ -91,85 +182,26 @@ __device__ void run_tile(const PairArgs &A, int64_t tile, int64_t L, unsigned ch
     const int64_t p1 = p0 + span < L ? p0 + span : L;
     // the tile from the queue and the parity +1 count address this system's buffers
     // (block-uniform: every thread leaves before the first barrier)
-    if (!QCS_IN_BOUNDS(tile >= 0 && ch < A.nchunks && L >= 0 && L <= A.P, A.status)) return;
+    if (!QCS_IN_BOUNDS(tile >= 0 && ch < A.nchunks && L >= 0 && L <= A.P, A.status)) return false;
     __syncthreads();  // previous tile's readers of Us are done
     int fU = 0;
     if (p0 < L) {
         const cd *Utw = A.Ut + w * n * n;
-        fU = fx_fraction(fx_max_key(Utw, n * n, lane), 57);
+        const unsigned key = fx_max_key(Utw, n * n, lane);
+        fU = fx_fraction(key, 57);
+        const bool guard = A.d_count[2] > 0 || (A.d_count[1] > 0 && fx_wide(Utw, n * n, key, lane));
+        if (guard != kGuarded) return true;  // block-uniform
         fx_stage_rows(n, n * n, Utw, fU, nullptr, Us, threadIdx.x, blockDim.x);
+    } else if (kGuarded) {
+        return true;
     }
     __syncthreads();
     cd acc = cmk(0.0, 0.0);
-    if (p0 < L) {
-        for (int64_t pq = p0 + team; pq < p1; pq += teams) {
-            const int64_t q = A.all ? pq : (int64_t)A.idx[pq];
-            if (!QCS_IN_BOUNDS(q >= 0 && q < A.P, A.status)) continue;  // team-uniform
-            const uint8_t *gq = A.gth ? A.gth + q * n2 : nullptr;
-            const bool gat = gq && gq[0] != 0xFF, fromK = !gat && A.Qh;
-            cd S = cmk(__longlong_as_double(0x7ff8000000000000ll), 0.0);
-            bool finite = true;
-            int fT = fU, par = 0;
-            tm.sync();  // the previous pair is done with the team's region
-            if (gat) {
-                fx_gather_T(n, Us, gq, Ts, tm.t, tm.NT);  // signed permutation: no products
-                fT = fU - 1;
-            } else {
-                // T (or K) by column halves: half of the snapshot's rows staged at a time
-                const cd *Qr = (A.Qh ? A.Qh : A.Qt) + q * n2 * n;
-                const unsigned key = fromK ? fx_max_key(Qr, n2 * n, lane) : fx_balance_rows(n, Qr, scr->rs, lane);
-                finite = key < 0x7ff00000u;
-                const int fQ = fx_fraction(key, 57);
-                unsigned top = 0u;
-                tm.sync();
-                for (int h = 0; h < 2 && finite; ++h) {
-                    fx_stage_rows(n, n * n, Qr + (int64_t)h * n * n, fQ, fromK ? nullptr : scr->rs + h * n, Qs, tm.t,
-                                  tm.NT);
-                    tm.sync();
-                    top |= fx_build_T(n, A.ne, Us, Qs, reinterpret_cast<fx2 *>(Ts), h * n, tm.t, tm.NT);
-                    tm.sync();
-                }
-                if (finite) {
-                    top = tm.or_put(top, par);
-                    tm.sync();
-                    const int b = fx_top_bits(tm.or_get(top, par));
-                    par ^= 1;
-                    fT = fU + fQ - 58 + 56 - b;
-                    if (fromK) fx_T_limbs<kFxS>(n, Ts, b, tm.t, tm.NT);
-                    else fx_T_limbs<kFxST>(n, Ts, b, tm.t, tm.NT);
-                }
-            }
-            tm.sync();
-            if (finite) {
-                bool shared = true, ok;
-#pragma unroll 1
-                do {  // rarely a second time: B^(s) again, every node matrix in full
-                    unsigned top = fromK ? fx_build_B_from_K(n, A.ne, Us, Ts, Xs, tab, tm.t, tm.NT)
-                                         : fx_build_B(n, A.ne, Ts, Xs, tab, tm.t, tm.NT);
-                    top = tm.or_put(top, par);
-                    tm.sync();
-                    const int mb = fx_top_bits(tm.or_get(top, par));
-                    par ^= 1;
-                    tm.sync();  // the words of the reduction are free again
-                    S = fx_pair_eliminate(tm, A.m, A.ne, shared, A.NB, A.plan, wk, Xs, Ns,
-                                          fromK ? fT + fU - 58 : 2 * fT - 56, mb, tab, ok);
-                    shared = false;
-                    tm.sync();
-                } while (!ok);
-            }
-            if (NW > 1) {  // the other warp's nodes
-                if (wid == 1 && lane == 0) scr->part = finite ? S : cmk(0.0, 0.0);
-                tm.sync();
-                if (wid == 0 && lane == 0) S = cadd(S, scr->part);
-            }
-            if (tm.t == 0) {
-                if (!cfinite(S)) raise_status(A.status, QCS_ERR_NONFINITE);
-                acc = cadd(acc, S);
-                if (A.per_pair) A.per_pair[w * A.P + q] = cmul(A.pref[w], S);
-            }
-        }
-    }
+    if (p0 < L)
+        acc = tile_pairs<NW, kGuarded>(A, w, p0 + team, p1, teams, fU, base + (size_t)team * A.team_bytes, Us, tab,
+                                       1 + team, wid, lane);
     if (lane == 0) A.partial[(w * A.nchunks + ch) * wpb + warp] = wid == 0 ? acc : cmk(0.0, 0.0);
+    return false;
 }
 
 // One or several systems (different n, ne, walkers, snapshots) in one persistent
@@ -182,9 +214,42 @@ struct BatchArgs {
     int tab_bytes, ut_bytes, work_bytes;  // maxima over the systems
     int max_m;
     int64_t tile_end[QCS_MAX_SYSTEMS];    // cumulative tile counts in queue order
-    unsigned long long *counter;
+    unsigned long long *counter;          // tiles handed out in the first pass and in the second
     PairArgs sys[QCS_MAX_SYSTEMS];         // in queue order
 };
+
+// The guarded tiles, or the others; whether this block met tiles of the other kind.
+template <int NWS, bool kGuarded>
+__device__ __forceinline__ bool overlap_tiles(const BatchArgs &B, unsigned char *smem_raw, long long *next_tile) {
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int wpb = blockDim.x >> 5;
+    const uint16_t *tab = reinterpret_cast<uint16_t *>(smem_raw);
+    int4 *Us = reinterpret_cast<int4 *>(smem_raw + B.tab_bytes);
+    unsigned char *base = smem_raw + B.tab_bytes + B.ut_bytes;
+    const int64_t total = B.tile_end[B.nsys - 1];
+    bool other = false;
+    for (;;) {
+        __syncthreads();  // every thread has read the previous tile index
+        if (threadIdx.x == 0) *next_tile = (long long)atomicAdd(B.counter + (kGuarded ? 1 : 0), 1ull);
+        __syncthreads();
+        const int64_t t = *next_tile;
+        if (t >= total) break;
+        int s = 0;
+        while (t >= B.tile_end[s]) ++s;
+        const int64_t local = t - (s > 0 ? B.tile_end[s - 1] : 0);
+        const PairArgs &A = B.sys[s];
+        const int64_t L = A.all ? A.P : (int64_t)(*A.d_count);
+        if ((NWS & 2) && (!(NWS & 1) || A.grp))
+            other |= run_tile<2, kGuarded>(A, local, L, base, Us, tab, warp, wpb, lane);
+        else other |= run_tile<1, kGuarded>(A, local, L, base, Us, tab, warp, wpb, lane);
+    }
+    return other;
+}
+template <int NWS>
+static __device__ __noinline__ void guarded_tiles(const BatchArgs &B, unsigned char *smem_raw, long long *next_tile) {
+    overlap_tiles<NWS, true>(B, smem_raw, next_tile);
+}
 
 // NWS: bit 0 set when a system of the launch runs one warp per pair, bit 1 when one runs two;
 // a kind that does not occur is left out of the kernel (its instructions and registers).
@@ -192,33 +257,14 @@ template <int NWS>
 __global__ void __launch_bounds__(128, 4) pair_overlap_kernel(const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long next_tile;
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
     // the pair table, the walker rows and the teams' workspaces fit the launch's shared memory
     if (!QCS_IN_BOUNDS(tri_count(B.max_m) * (int)sizeof(uint16_t) <= B.tab_bytes &&
                            (size_t)B.tab_bytes + B.ut_bytes + B.work_bytes <= dyn_smem_bytes(),
                        B.sys[0].status))
         return;
-    uint16_t *tab = reinterpret_cast<uint16_t *>(smem_raw);
-    build_pair_table(tab, tri_count(B.max_m));
-    int4 *Us = reinterpret_cast<int4 *>(smem_raw + B.tab_bytes);
-    unsigned char *base = smem_raw + B.tab_bytes + B.ut_bytes;
-    const int64_t total = B.tile_end[B.nsys - 1];
-    for (;;) {
-        __syncthreads();  // every thread has read the previous tile index
-        if (threadIdx.x == 0) next_tile = (long long)atomicAdd(B.counter, 1ull);
-        __syncthreads();
-        const int64_t t = next_tile;
-        if (t >= total) break;
-        int s = 0;
-        while (t >= B.tile_end[s]) ++s;
-        const int64_t local = t - (s > 0 ? B.tile_end[s - 1] : 0);
-        const PairArgs &A = B.sys[s];
-        const int64_t L = A.all ? A.P : (int64_t)(*A.d_count);
-        if ((NWS & 2) && (!(NWS & 1) || A.grp)) run_tile<2>(A, local, L, base, Us, tab, warp, wpb, lane);
-        else run_tile<1>(A, local, L, base, Us, tab, warp, wpb, lane);
-    }
+    build_pair_table(reinterpret_cast<uint16_t *>(smem_raw), tri_count(B.max_m));
+    // a block that met guarded tiles takes part in the second pass, over all tiles
+    if (overlap_tiles<NWS, false>(B, smem_raw, &next_tile)) guarded_tiles<NWS>(B, smem_raw, &next_tile);
 }
 
 // One warp per walker: lanes sum strided partials, then a fixed-order tree.
@@ -377,7 +423,7 @@ qcs_status qcs_launch_pairs_batched(qcs_ctx *ctx, int nsys, const qcs_pair_launc
         per_sm = 1;
     int64_t blocks = (int64_t)ctx->num_sms * per_sm;
     if (blocks > acc) blocks = acc;
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st);
+    cudaError_t e = cudaMemsetAsync(counter, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return qcs_fail(ctx, QCS_ERR_CUDA, "batched counter reset");
     qcs_prof_begin(ctx, st);
     kern<<<(unsigned)blocks, wpb * 32, smem, st>>>(B);

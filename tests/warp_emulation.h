@@ -152,6 +152,13 @@ inline unsigned __reduce_or_sync(unsigned, unsigned v) {
     for (int i = 0; i < 32; ++i) r |= (unsigned)c[i];
     return r;
 }
+inline unsigned __reduce_add_sync(unsigned, unsigned v) {
+    uint64_t c[32];
+    emu::exchange(v, c);
+    unsigned r = 0;
+    for (int i = 0; i < 32; ++i) r += (unsigned)c[i];
+    return r;
+}
 template <class T>
 inline T __reduce_max_sync(unsigned, T v) {
     uint64_t c[32];
