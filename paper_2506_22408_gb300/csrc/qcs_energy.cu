@@ -73,9 +73,9 @@ __device__ __forceinline__ cd group_sum(cd v, cd *red, int t, int bar) {
     return s;
 }
 
-// Fraction bits that bring the largest of count entries to 56 bits (a group maximum); an
+// Fraction bits that bring the largest of count entries to `bits` bits (a group maximum); an
 // entry that is not finite gives a value below -968.
-__device__ __forceinline__ int group_fraction(const cd *x, int count, unsigned *red, int t, int bar) {
+__device__ __forceinline__ int group_fraction(const cd *x, int count, unsigned *red, int t, int bar, int bits = 56) {
     unsigned k = 0u;
     for (int e = t; e < count; e += kGroup) k = max(k, pivot_key(x[e]));
     k = __reduce_max_sync(QCS_FULL, k);
@@ -83,7 +83,7 @@ __device__ __forceinline__ int group_fraction(const cd *x, int count, unsigned *
     group_sync(bar);
     k = max(red[0], red[1]);
     group_sync(bar);
-    return fx_fraction(k, 56);
+    return fx_fraction(k, bits);
 }
 
 // A sum of complex products of limbs by three real products each, in units of 2^58 (value) or
@@ -274,7 +274,7 @@ __device__ inline int stage_Mt(int n, int ne, int m, const cd *__restrict__ Qs, 
     for (int a = t; a < m; a += kGroup) X1[a * lx + lx - 1] = cmk(0.0, 0.0);  // the rows' padding
     build_Mt(n, ne, m, Qs, lq, Ts, lt, X1, lx, t);
     group_sync(bar);
-    const int f = group_fraction(X1, m * lx, red, t, bar);
+    const int f = group_fraction(X1, m * lx, red, t, bar, fx_ap_bits(n));
     for (int e = t; e < m * lx; e += kGroup) Mt[e] = fx_limbs(X1[e], f);
     group_sync(bar);
     return f;
@@ -750,16 +750,17 @@ __global__ void __launch_bounds__(128, 2) energy_pair_kernel(const __grid_consta
 }
 
 // count entries of x (shared memory, each written by the thread that reads it here) as limbs
-// with one scale, and its fraction bits; a barrier on both sides of the maximum.
-__device__ __forceinline__ void store_limbs(const cd *x, int count, int4 *__restrict__ out, int *__restrict__ f,
-                                            unsigned *keys) {
+// with one scale, the largest of `bits` bits, and its fraction bits; a barrier on both sides of
+// the maximum.
+__device__ __forceinline__ void store_limbs(const cd *x, int count, int bits, int4 *__restrict__ out,
+                                            int *__restrict__ f, unsigned *keys) {
     unsigned k = 0u;
     for (int e = threadIdx.x; e < count; e += blockDim.x) k = max(k, pivot_key(x[e]));
     k = __reduce_max_sync(QCS_FULL, k);
     if ((threadIdx.x & 31) == 0) keys[threadIdx.x >> 5] = k;
     __syncthreads();
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) k = max(k, keys[i]);
-    const int fr = fx_fraction(k, 56);
+    const int fr = fx_fraction(k, bits);
     for (int e = threadIdx.x; e < count; e += blockDim.x) out[e] = fx_limbs(x[e], fr);
     if (threadIdx.x == 0) *f = fr;
     __syncthreads();
@@ -813,7 +814,7 @@ __global__ void energy_prep_kernel(int n, int ne, int64_t W, int nchol, int has_
                 for (int k = 0; k < n2; ++k) cfma(s, K[a * n2 + k], ell[k * n2 + c]);
                 K1[e] = s;
             }
-            store_limbs(K1, m * n2, Kop + ((size_t)w * (nop + 1) + o) * m * n2, Kf + w * (nop + 1) + o, keys);
+            store_limbs(K1, m * n2, fx_ap_bits(n), Kop + ((size_t)w * (nop + 1) + o) * m * n2, Kf + w * (nop + 1) + o, keys);
             if (o < nchol)
                 for (int e = threadIdx.x; e < m * n2; e += blockDim.x) {
                     const int a = e / n2, c = e - a * n2;
@@ -823,7 +824,7 @@ __global__ void energy_prep_kernel(int n, int ne, int64_t W, int nchol, int has_
                 }
             __syncthreads();
         }
-        store_limbs(Ka, m * n2, Kop + ((size_t)w * (nop + 1) + nop) * m * n2, Kf + w * (nop + 1) + nop, keys);
+        store_limbs(Ka, m * n2, fx_ap_bits(n), Kop + ((size_t)w * (nop + 1) + nop) * m * n2, Kf + w * (nop + 1) + nop, keys);
     }
 }
 

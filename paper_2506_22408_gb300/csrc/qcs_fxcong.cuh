@@ -29,6 +29,11 @@
 constexpr int kFxS = 29;   // the limbs of this file: X = h 2^29 + l
 constexpr int kFxST = 28;  // ... of T, both factors of B: 56 bits in two equal limbs
 
+// Bits of the local energy's Mt and K ell, of which A'_ab = sum over 2n columns of
+// K_a M_b - K_b M_a, four real products each: |h l'| + |l h'| are below 2^56 at 56 bits, a cr of
+// up to 8n 2^56 (2^63.6 at n = 24), so one bit less above 16 modes.
+__host__ __device__ constexpr int fx_ap_bits(int n) { return n <= 16 ? 56 : 55; }
+
 __device__ __forceinline__ fxl fx_re(int4 q) { return fxl{q.x, q.y}; }
 __device__ __forceinline__ fxl fx_im(int4 q) { return fxl{q.z, q.w}; }
 __device__ __forceinline__ fxl fx_add(fxl a, fxl b) { return fxl{a.h + b.h, a.l + b.l}; }
