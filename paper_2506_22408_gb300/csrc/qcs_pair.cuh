@@ -1,6 +1,6 @@
-// qcs_pair.cuh -- per-pair device building blocks shared by the overlap and
-// adjoint kernels: the packed-pair table, the congruence T = Ut Qt^T and the
-// selected covariance B^(s) of Eqs. (a_mat), (b_mat).
+// qcs_pair.cuh -- per-pair device building blocks: the packed-pair table, and in FP64 the
+// congruence T = Ut Qt^T (local energy) and the selected covariance B^(s) of Eqs. (a_mat),
+// (b_mat) (local energy, and the overlaps' pairs that leave fixed point).
 #pragma once
 #include "qcs_common.cuh"
 
@@ -35,110 +35,6 @@ __device__ inline void build_T(int n, const cd *__restrict__ Uts, const cd *__re
         for (int k = 0; k < n; ++k) cfma(s, ur[k], qr[k]);
         Ts[j * lt + c] = s;
     }
-}
-
-// T from walker rows in echelon form (see qcs_walker.cu): row j < ne of Ut is zero in
-// columns k < j, row ne + j' zero in columns [ne, ne + j'); those products are skipped.
-// With 2n = 32 every warp pass covers one row, so the loop bounds are warp-uniform.
-__device__ inline void build_T_echelon(int n, int ne, const cd *__restrict__ Uts, const cd *__restrict__ Qs,
-                                       cd *__restrict__ Ts, int lane, int nthr = 32) {
-    const int n2 = 2 * n, lu = ld_ut(n), lq = ld_qt(n), lt = ld_t(n);
-    for (int e = lane; e < n * n2; e += nthr) {
-        const int j = e / n2, c = e - j * n2;
-        const cd *ur = Uts + j * lu, *qr = Qs + c * lq;
-        cd s = cmk(0.0, 0.0);
-        if (j < ne) {
-            for (int k = j; k < n; ++k) cfma(s, ur[k], qr[k]);
-        } else {
-            for (int k = 0; k < ne; ++k) cfma(s, ur[k], qr[k]);
-            for (int k = j; k < n; ++k) cfma(s, ur[k], qr[k]);  // j = ne + j'
-        }
-        Ts[j * lt + c] = s;
-    }
-}
-
-// T from echelon-form walker rows for n = N (2N = 32 lanes): lane c holds row c of the
-// snapshot's Qt in registers and owns column c of T.  Each complex multiply-add takes
-// three real products (Gauss's 3-multiplication form): with s = re + im of both
-// factors, Re = sum ur qr - sum ui qi and Im = sum us qs - sum ur qr - sum ui qi, so
-// the sums us of the walker rows (Uss, per block) and qs of the snapshot row (here)
-// are formed once.  The skipped zeros follow build_T_echelon, or for a walker in
-// reduced form (occupied rows [I; X]: row j < ne has its one entry at column j
-// among the columns k < ne) that single entry and the columns k >= ne; the row loop
-// is warp-uniform and enters the unrolled k sequences by a switch, so the register
-// arrays are indexed by constants.
-#define QCS_T3M(K)                            \
-    case K: {                                 \
-        const cd u_ = ur[K];                  \
-        p1 = fma(u_.x, qr[K], p1);            \
-        p2 = fma(u_.y, qi[K], p2);            \
-        p3 = fma(us[K], qs[K], p3);           \
-    }
-#define QCS_T3M1(K)                           \
-    case K: {                                 \
-        const cd u_ = ur[K];                  \
-        p1 = fma(u_.x, qr[K], p1);            \
-        p2 = fma(u_.y, qi[K], p2);            \
-        p3 = fma(us[K], qs[K], p3);           \
-        break;                                \
-    }
-// Qg holds the snapshot's rows with stride ldq (global memory or staged); rows
-// j0, j0 + jstep, ... of T are formed, so that several warps can share one T.
-template <int N>
-__device__ inline void build_T_reg(int ne, const cd *__restrict__ Uts, const double *__restrict__ Uss,
-                                   const cd *__restrict__ Qg, cd *__restrict__ Ts, int lane, bool reduced,
-                                   int ldq = N, int j0 = 0, int jstep = 1) {
-    static_assert(N == 16, "one lane per column of T: 2N must be the warp width");
-    const int lu = ld_ut(N), lt = ld_t(N);
-    double qr[N], qi[N], qs[N];
-    const cd *qrow = Qg + lane * ldq;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        const cd q = qrow[k];
-        qr[k] = q.x;
-        qi[k] = q.y;
-        qs[k] = q.x + q.y;
-    }
-    for (int j = j0; j < N; j += jstep) {
-        const cd *ur = Uts + j * lu;
-        const double *us = Uss + j * lu;
-        double p1 = 0.0, p2 = 0.0, p3 = 0.0;
-        int kstart = j;
-        if (j < ne && reduced) {
-            switch (j) {  // the single entry among the columns k < ne
-                QCS_T3M1(0) QCS_T3M1(1) QCS_T3M1(2) QCS_T3M1(3) QCS_T3M1(4) QCS_T3M1(5) QCS_T3M1(6) QCS_T3M1(7)
-                QCS_T3M1(8) QCS_T3M1(9) QCS_T3M1(10) QCS_T3M1(11) QCS_T3M1(12) QCS_T3M1(13) QCS_T3M1(14)
-                QCS_T3M1(15)
-                default: break;
-            }
-            kstart = ne;
-        }
-        if (j >= ne) {
-            switch (ne - 1) {  // k = ne-1 down to 0
-                QCS_T3M(15) QCS_T3M(14) QCS_T3M(13) QCS_T3M(12) QCS_T3M(11) QCS_T3M(10) QCS_T3M(9) QCS_T3M(8)
-                QCS_T3M(7) QCS_T3M(6) QCS_T3M(5) QCS_T3M(4) QCS_T3M(3) QCS_T3M(2) QCS_T3M(1) QCS_T3M(0)
-                default: break;
-            }
-        }
-        switch (kstart) {  // k = kstart up to N-1
-            QCS_T3M(0) QCS_T3M(1) QCS_T3M(2) QCS_T3M(3) QCS_T3M(4) QCS_T3M(5) QCS_T3M(6) QCS_T3M(7)
-            QCS_T3M(8) QCS_T3M(9) QCS_T3M(10) QCS_T3M(11) QCS_T3M(12) QCS_T3M(13) QCS_T3M(14) QCS_T3M(15)
-            default: break;
-        }
-        Ts[j * lt + lane] = cmk(p1 - p2, p3 - p1 - p2);
-    }
-}
-#undef QCS_T3M
-#undef QCS_T3M1
-
-// x * ph for a phase code ph = 0..3 (1, i, -1, -i): a swap of the parts and sign
-// flips of the bit patterns, no floating-point arithmetic.
-__device__ __forceinline__ cd mul_phase(cd x, unsigned ph) {
-    cd r = (ph & 1u) ? cmk(x.y, x.x) : x;
-    const bool fre = ph == 1u || ph == 2u, fim = ph >= 2u;
-    if (fre) r.x = __longlong_as_double(__double_as_longlong(r.x) ^ (long long)0x8000000000000000ull);
-    if (fim) r.y = __longlong_as_double(__double_as_longlong(r.y) ^ (long long)0x8000000000000000ull);
-    return r;
 }
 
 // Stage a snapshot's rows Qt (2n x n, global) into padded shared rows.
