@@ -91,11 +91,12 @@ typedef enum {
 } qcs_status;
 
 typedef enum {
-    QCS_FP64 = 0,  /* every product and the Pfaffians in FP64 */
+    QCS_FP64 = 0,  /* at FP64 accuracy: in 64-bit fixed point with one scale per matrix, by
+                      error-free tensor-core products, and in FP64 where those would lose bits */
     QCS_TF32X3 = 1 /* qcs_overlap only, any n <= QCS_MAX_N: the congruence T = U^T Qt^T on
                       tensor cores (tcgen05 kind::tf32, hi/lo splits, hi*hi + hi*lo + lo*hi
-                      accumulated in FP32), B^(s) in FP32; Pfaffians, pivoting and node sums in
-                      FP64.  Rows and the contraction are padded to 32 for n <= 16 (tiles of 4
+                      accumulated in FP32), B^(s) in FP32; Pfaffians and node sums as in
+                      QCS_FP64.  Rows and the contraction are padded to 32 for n <= 16 (tiles of 4
                       walkers x 4 snapshots, a warp per pair) and to 64 x 48 for 16 < n <= 24
                       (2 x 2 tiles, two warps per pair).  The snapshot set gets TF32 operand
                       slabs (8 KB per snapshot for n <= 16, 24 KB above, from the context's
@@ -107,7 +108,7 @@ typedef enum {
                                  snapshot (disables the parity shortcuts described at qcs_overlap) */
 #define QCS_FLAG_DFT_NODES 2u /* roots of unity with the parity shortcuts, also when nodes = 0
                                  (then N = n-ne+1) */
-#define QCS_FLAG_FP64_ALU 4u  /* qcs_overlap, QCS_FP64: form the congruence on the FP64 ALU (the
+#define QCS_FLAG_FP64_ALU 4u  /* qcs_overlap, QCS_FP64: form the congruence on the ALU (the
                                  default for n != 16) instead of on tensor cores */
 #define QCS_FLAG_FP64_TC 8u   /* qcs_overlap, QCS_FP64: form the congruence on tensor cores at FP64
                                  accuracy (the default for n = 16) for any n <= 16; not with
@@ -234,8 +235,8 @@ qcs_status qcs_snapshots_parity(const qcs_snapshots *s, int8_t *d_parity, void *
 
 /* Number of snapshots of the set that are signed permutations (every row of Q_p
  * has one nonzero entry, exactly +-1: the ensemble of the paper's experiment).
- * For those the pair kernels form the congruence T = U^T Qt^T as a gather with
- * sign flips (no FP64 work), and the gradient's cotangent product likewise.
+ * For those the ALU pair kernel forms the congruence T = U^T Qt^T as a gather with
+ * sign flips; the gradient takes the dense rows [H1^T; G2^T] for every snapshot.
  * Waits for `stream` (the build must have been issued on it or before it).
  * Errors: QCS_ERR_ARG (null pointers), QCS_ERR_CUDA. */
 qcs_status qcs_snapshots_signed_perm_count(const qcs_snapshots *s, int64_t *count, void *stream);
@@ -272,8 +273,10 @@ qcs_status qcs_overlap(qcs_ctx *ctx, const qcs_snapshots *s, int ne, int64_t W, 
  * run on tensor cores by error-free slicing: each FP64 row is cut into seven 8-bit
  * slices exact in BF16, the 28 slice products of the leading levels accumulate exactly
  * in FP32, and the levels are combined exactly in 64-bit fixed point, so each entry of P
- * carries an error of about 2^-53 times the row scales, like an FP64 product; the
- * Pfaffians run in 64-bit fixed point.  The snapshot set then holds 57,856 bytes per four
+ * carries an error of about 2^-53 times the row scales; the Pfaffians run in 64-bit fixed
+ * point.  That is an FP64 product's error for orthogonal Q and rows of similar entries; a
+ * pair made of entries far below their rows' largest (a walker within 1e-6 of a basis
+ * determinant against a signed permutation) keeps its own precision on the ALU path only.  The snapshot set then holds 57,856 bytes per four
  * parity +1 snapshots of slice records (formed by qcs_build_snapshots at n = 16,
  * otherwise on first use), and the context workspace 14,464 bytes per walker and at most
  * 512 MB of pair records, worked off in batches (smaller ones, down to 32 snapshots of one

@@ -805,7 +805,7 @@ static double alu_B_from_K_flops(int n, int ne) {
            2.0 * n * n;
 }
 
-// B from K in the gradient (build_B_from_K3): two n-term complex sums per work item (tri(ne) occupied
+// B from K in the gradient: two n-term complex sums per work item (tri(ne) occupied
 // pairs, ne d occupied-empty pairs, tri(d + 1) empty pairs j1 <= j2) with three real
 // products per term and three additions per sum, then the halved sums and differences of
 // the occupied-empty (8 flop) and distinct empty pairs (8 flop) and one product per mode;

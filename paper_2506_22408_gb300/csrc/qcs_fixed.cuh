@@ -8,11 +8,14 @@
 //     X = h 2^S + l,  |l| <= 2^{S-1}:   X Y = hh 2^2S + (h l' + l h') 2^S + l l',
 // the last term dropped: 12 to 13 clocks against 76.  With S = 30 and entries of 58 to 60
 // bits it is below 2^-58 of the factors' scale, of either sign; longer sums of entries of 57
-// bits take S = 29 (2^-60), as S = 31 lost three bits of the congruence against FP64.  The
-// largest entry of a matrix is kept at 54 to 60 bits, so an update rounds at 2^-54 to 2^-60 of the matrix's largest entry where FP64 rounds at 2^-53 of each
-// operand: the elimination with pivoting is as accurate as that matrix norm allows either
-// way, and the errors against 64-bit references are those of the FP64 code it replaced or
-// smaller.
+// bits take S = 29 (2^-60), as S = 31 lost three bits of the congruence against FP64, and of 56
+// bits S = 28.  The largest entry of a matrix is kept at 54 to 60 bits, so an update rounds at
+// 2^-54 to 2^-60 of it, where FP64 rounds at 2^-53 of each operand: no worse for matrices whose
+// entries are of similar size (errors per pair against the oracle, n = 6 to 24, Haar and signed
+// permutations, random and near-diagonal walkers: 1.1 to 3.5 10^-15 of the pair scale rms,
+// 1.1 to 8.4 10^-15 in FP64, but for n = 8, ne = 4 near-diagonal, 6 10^-15 against 5 10^-14).  An
+// entry 2^-k below the largest keeps k bits fewer; where pairs are made of such entries the
+// callers leave fixed point (qcs_pairfp64.cuh).
 //
 // One rank-2 entry update (two complex products) is 24 IMAD.WIDE and about 35 one-clock
 // instructions, near 140 clocks per 32 entries, against 8 DFMA = 611 clocks.  With the
@@ -317,7 +320,7 @@ static __device__ __noinline__ void fx_renorm(const Team &tm, int nb, int T, int
     tm.sync();
 }
 
-// Records of fx_node_pfaffians' products per warp for NB node matrices per round (vm: the
+// Records of fx_pair_eliminate's products per warp for NB node matrices per round (vm: the
 // entries of the kernel's Gauss-vector buffers, the full matrix or NB complements); the
 // ne/2 signed pivots of the shared occupied elimination follow them.  A record is an entry
 // worth X 2^-f with its f: 16 + 4 bytes, the f after all the entries.

@@ -1,4 +1,4 @@
-// qcs_overlap.cu -- walker x snapshot shadow overlaps on the FP64 pipe.
+// qcs_overlap.cu -- walker x snapshot shadow overlaps without a tensor-core congruence.
 //
 // For a pair (walker w, snapshot p) the estimator of Sec. "Classical shadows
 // and the evaluation of overlaps" needs the coefficients of

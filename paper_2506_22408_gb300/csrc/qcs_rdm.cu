@@ -6,8 +6,8 @@
 // |S| = 4: pf(i X|_S) = -(X_01 X_23 - X_02 X_13 + X_03 X_12), so the estimates of all
 // products of four distinct Majoranas are fixed combinations of the second moments
 //     S2[(mu nu), (rho sigma)] = sum_p X_p,mu nu X_p,rho sigma
-// of the covariance entries: a symmetric rank-P update (K = P), the FP64 contraction
-// that dominates this path.  The 1-RDM follows Eqs. (1rdm_off_diagonal) and
+// of the covariance entries: a symmetric rank-P update (K = P), the contraction that
+// dominates this path.  The 1-RDM follows Eqs. (1rdm_off_diagonal) and
 // (1rdm_diagonal): a~_p = (g~_2p + i g~_2p+1)/2.
 //
 // Kernels: rdm_cov_kernel (warp per snapshot: X_p = (Q' R^T)^T J (Q' R^T) from the
@@ -38,7 +38,7 @@ __host__ __device__ __forceinline__ int pair_rank(int mu, int nu, int N2) {
 // X_p for every snapshot (warp per snapshot), FP64 packed upper triangle to Gu, and the
 // largest upper word of |X| over all of them to *d_max.
 //
-// Q' (and R) are held as fixed point (qcs_fixed.cuh: one scale per matrix, 31-bit limbs):
+// Q' (and R) are held as fixed point (qcs_fixed.cuh: one scale per matrix, limbs of 29 bits):
 // the products then run on the integer pipe, three IMAD.WIDE (12 clocks per 32 of them)
 // where the FP64 pipe takes 76, and are exact to 2^-57 of the matrix scale; the two limbs
 // of an entry are one 8-byte load.  A snapshot or rotation with a non-finite entry takes

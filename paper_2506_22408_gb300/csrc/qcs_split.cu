@@ -15,11 +15,12 @@
 // layout and staged into shared memory by bulk asynchronous copies that complete
 // on an mbarrier.  Each warp then reads its walker's 32 accumulator lanes, forms
 // the selected covariance B^(s) in FP32, and evaluates the Pfaffians of the node
-// matrices in FP64 exactly as the FP64 path does.
+// matrices as the FP64 paths do: in fixed point up to 16 modes (qcs_fixed.cuh), in FP64 by
+// the groups of qcs_group.cuh above.
 //
 // Accuracy: T carries the ~2^-21 relative error of the split TF32 products
 // accumulated in FP32, B^(s) an FP32 rounding of its 2n-term sums; the Pfaffian
-// elimination, its pivoting and the node sums stay FP64.
+// eliminations and the node sums add nothing of that size.
 #include "qcs_internal.h"
 #include "qcs_fixed.cuh"
 #include "qcs_group.cuh"

@@ -17,7 +17,7 @@
 // FP32 in tensor memory (one accumulator per level), and the levels are combined
 // exactly into 64-bit fixed point on the integer pipe.  The walker's slices are
 // formed once per walker, the snapshot's once per snapshot; Z is re-sliced per pair
-// between the two products.  The FP64 pipe is left with the Pfaffians alone.
+// between the two products.  The Pfaffians are a kernel of their own (qcs_pfaff.cu).
 //
 // Tiles: one walker and 4 subs consecutive parity +1 snapshots (subs sub-tiles of four,
 // 8 by default, tuned by qcs_autotune);
@@ -61,8 +61,8 @@ constexpr uint32_t kWaitIter = 1u << 26;                      // bounded mbarrie
 constexpr int kSnapSlab = kSnapsPerSub * kSliceBytes;         // one slice of 4 snapshots: 8 KB
 constexpr int kSnapRecBytes = kSlices * kSnapSlab + kSnapsPerSub * kRowsPer * 4;  // + row exponents
 constexpr int kWalkRecBytes = kSlices * kSliceBytes + kRowsPer * 4;
-constexpr int kOperandBytes = kSlices * kSnapSlab;           // operand region: later four warp workspaces
-constexpr int kPuBytes = (kRowsPer * (kRowsPer - 1) / 2) * 8; // upper triangle of P (32 x 32), FP64
+constexpr int kOperandBytes = kSlices * kSnapSlab;           // operand region: later P of four warps
+constexpr int kPuBytes = (kRowsPer * (kRowsPer - 1) / 2) * 8; // upper triangle of P (32 x 32), fixed point
 
 static_assert(kSnapRecBytes % 16 == 0 && kWalkRecBytes % 16 == 0, "bulk copies move multiples of 16 bytes");
 
@@ -322,12 +322,12 @@ __device__ __forceinline__ bool team_and(int team, bool v) {
 }
 
 // One block per SM holds up to kMaxTeams teams of four warps.  Each team has its own
-// operand records (and, in them, its warps' Pfaffian workspaces) and runs the tile loop
-// of the header on its own: a team is what a block of four warps would be, except that
-// the tensor memory of the SM (512 columns) is shared as two 256-column accumulators.
-// A team holds one from its first product of a sub-tile to the end of the readout of
-// P (a bounded spin on a lock word in shared memory), so three teams, twelve warps per
-// SM, keep the FP64 pipe fed while the tensor memory would only allow two blocks of four.
+// operand records (and, in their place, its warps' P) and runs the tile loop of the header
+// on its own: a team is what a block of four warps would be, except that the tensor memory
+// of the SM (512 columns) is shared as two 256-column accumulators.  A team holds one from
+// its first product of a sub-tile to the end of the readout of P (a bounded spin on a lock
+// word in shared memory), so three teams, twelve warps per SM, hide each other's copies,
+// MMAs and barriers where the tensor memory would only allow two blocks of four.
 __global__ void __launch_bounds__(kTeamThreads * kMaxTeams, 1) tc_pair_kernel(const __grid_constant__ TcArgs A) {
     extern __shared__ __align__(128) unsigned char smem_tc[];
     __shared__ uint32_t tmem_base;
