@@ -18,6 +18,23 @@ extern "C" long long host_fx_of1(double x, int f) { return fx_of1(x, f); }
 extern "C" long long host_shift1(long long X, int s) { return fx_shift1(X, s); }
 extern "C" long long host_scale(long long z, int g) { return qcs_oz::scale_of_fixed(z, g); }
 extern "C" long long host_shift_any(long long X, int s) { return fx_shift_any(X, s); }
+// a . b of two rows through the slices: z and its exponent
+extern "C" long long host_sliced_dot(int n, const double *a, const double *b, int *exponent) {
+    using namespace qcs_oz;
+    int e[2] = {kNoRow, kNoRow};
+    for (int k = 0; k < n; ++k) {
+        if (a[k] != 0.0) e[0] = std::max(e[0], row_exp_of(a[k]));
+        if (b[k] != 0.0) e[1] = std::max(e[1], row_exp_of(b[k]));
+    }
+    float acc[kLevels] = {};
+    for (int k = 0; k < n; ++k) {
+        const uint64_t u = (uint64_t)fixed_of(a[k], e[0]) + kDigitBias, v = (uint64_t)fixed_of(b[k], e[1]) + kDigitBias;
+        for (int i = 1; i <= kSlices; ++i)
+            for (int j = 1; i + j <= 8; ++j) acc[i + j - 2] += slice_f32(u, i) * slice_f32(v, j);  // exact in FP32
+    }
+    *exponent = e[0] + e[1] - 56;
+    return combine_levels(acc);
+}
 """
 
 
@@ -27,6 +44,7 @@ def host(tmp_path_factory):
     for f in ("host_fixed_of", "host_fx_of1", "host_shift1", "host_scale", "host_shift_any"):
         getattr(lib, f).restype = ctypes.c_longlong
         getattr(lib, f).argtypes = [ctypes.c_double if "of" in f else ctypes.c_longlong, ctypes.c_int]
+    lib.host_sliced_dot.restype = ctypes.c_longlong
     return lib
 
 
@@ -82,3 +100,26 @@ def test_scale_bounds_every_entry(host):
         G = max(host.host_scale(za, ga), host.host_scale(zb, gb))
         for z, g in ((za, ga), (zb, gb)):
             assert abs(z) * Fraction(2) ** (55 + g - G) < 1 << 55
+
+
+@pytest.mark.parametrize("kind", ["uniform", "tiny", "top", "zeros"])
+def test_sliced_dot(host, kind):
+    """Within 2^-47 of the row scales: the entries' rounding (2^-56 each, 64 of them: 2^-50) and the
+    dropped levels (level 9: 6 * 32 * 128^2 2^-70 = 2^-48.4, the others 2^-8 of it)."""
+    rng = random.Random(8)
+    for t in range(60):
+        a = [rng.uniform(-1, 1) for _ in range(32)]
+        b = [rng.uniform(-1, 1) * 2.0 ** rng.randrange(-4, 4) for _ in range(32)]
+        if kind == "tiny":  # entries far below the scale, which must not leave a unit behind
+            a = [x if k < 3 else x * 2.0 ** -rng.randrange(50, 200) for k, x in enumerate(a)]
+        if kind == "top":  # digits at their bounds
+            a = [rng.choice([1, -1]) * (1 - 2.0**-7 - 2.0**-20) for _ in a]
+            b = [rng.choice([1, -1]) * (1 - 2.0**-7 - 2.0**-20) for _ in b]
+        if kind == "zeros":
+            b = [x if k % 5 == t % 5 else 0.0 for k, x in enumerate(b)]
+        arr = ctypes.c_double * 32
+        e = ctypes.c_int()
+        z = host.host_sliced_dot(32, arr(*a), arr(*b), ctypes.byref(e))
+        exact = sum(Fraction(x) * Fraction(y) for x, y in zip(a, b))
+        scale = Fraction(2) ** (e.value + 56)
+        assert abs(z * Fraction(2) ** e.value - exact) <= scale / 2**47
