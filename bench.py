@@ -61,9 +61,12 @@ def measured_peaks() -> dict:
 
 
 def add_dfma_context(obj, rate):
-    """Beside every FP64 ("alu") roofline, the fraction of the measured FMA rate."""
+    """Beside every FP64 ("alu") roofline, the fraction of the measured FMA rate and what it says."""
     if isinstance(obj, dict):
         if obj.get("bound") == "alu" and isinstance(obj.get("achieved"), float):
+            obj["basis"] = ("counted FP64 work of the method over the FP64 peak: a comparison with an FP64 kernel at "
+                            "full rate, not the load of a pipe (most of the work runs as 64-bit integers or "
+                            "tensor-core slices)")
             obj["dfma_probe"] = {"tflops": rate, "frac": obj["achieved"] / rate,
                                  "source": "register-only FP64 FMA chains on this GPU in this run "
                                            "(qcs_fp64_fma_rate)"}
@@ -72,6 +75,17 @@ def add_dfma_context(obj, rate):
     elif isinstance(obj, list):
         for v in obj:
             add_dfma_context(v, rate)
+
+
+def headline_launches(wl) -> int:
+    """Kernels of one timed step: snapshot build (prepare, compaction, tensor-core records), walker
+    prep and slices, three per batch of pair records (records, Pfaffians, sums; 512 MB of records
+    of 16 (tri(m) + 1) bytes, walkers in blocks when 32 positions of all do not fit), reduction."""
+    m = 2 * wl.n - wl.ne
+    fit = (512 << 20) // (16 * (m * (m - 1) // 2 + 1))
+    block = min(wl.W, fit // 32)
+    span = min(fit // block // 32 * 32, -(-wl.P // 32) * 32)
+    return 3 + 2 + 3 * (-(-wl.W // block)) * (-(-wl.P // span)) + 1
 
 
 def max_over_ranks(t: float, ws: int) -> float:
@@ -154,7 +168,8 @@ CSRC = os.path.join(ROOT, "paper_2506_22408_gb300", "csrc")
 KERNEL_SOURCES = {
     "tc_pair_kernel": ["qcs_tcpair.cu", "qcs_pfaff.cu", "qcs_fixed.cuh", "qcs_ozaki.cuh", "qcs_tc.cuh", "qcs_pair.cuh",
                        "qcs_common.cuh"],
-    "pair_overlap_kernel": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "pair_overlap_kernel": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pairfp64.cuh", "qcs_pair.cuh",
+                            "qcs_common.cuh"],
     "split_pair_kernel": ["qcs_split.cu", "qcs_fixed.cuh", "qcs_pair.cuh", "qcs_tc.cuh", "qcs_common.cuh"],
     "grad_pair_kernel": ["qcs_grad.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_fxsweep.cuh", "qcs_group.cuh",
                          "qcs_pair.cuh", "qcs_common.cuh"],
@@ -164,7 +179,8 @@ KERNEL_SOURCES = {
                            "qcs_common.cuh"],
     # the FP64 ALU pair kernel in its batched launch over the five systems of the batching
     # workload (a record of its own: another workload)
-    "pair_overlap_kernel_batched": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pair.cuh", "qcs_common.cuh"],
+    "pair_overlap_kernel_batched": ["qcs_overlap.cu", "qcs_fixed.cuh", "qcs_fxcong.cuh", "qcs_pairfp64.cuh",
+                                    "qcs_pair.cuh", "qcs_common.cuh"],
 }
 
 # workload name of the batched launch's traffic record
@@ -666,6 +682,8 @@ def run_rdm(args, ctx, dev, flush, barrier, ws, steps=3):
     avg = kms / max(kl, 1)
     fl = qcs.shadow_rdm_flops(n, P)
     ach = fl / (avg * 1e-3) / 1e12
+    peaks = measured_peaks()
+    bf16 = peaks["bf16_tflops"]
     return {"metric": "snapshots/s, shadow estimates of the 1-RDM, particle number and all four-Majorana correlators",
             "value": ws * P * steps / t, "unit": "snapshots/s", "steps": steps, "ms_per_step": 1e3 * t / steps,
             "config": {"workload": f"shadow RDM n={n} {P} snapshots (Haar Q, uniform b, seed 0)"},
@@ -673,6 +691,9 @@ def run_rdm(args, ctx, dev, flush, barrier, ws, steps=3):
             "roofline": {"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": ach / FP64_PEAK_TFLOPS, "kernel": "rdm_tc_moment_kernel", "kernel_ms": avg,
                          "flops_per_launch": fl,
+                         "tensor": {"achieved": 28 * ach, "peak": bf16, "unit": "TFLOP/s", "frac": 28 * ach / bf16,
+                                    "source": "28 BF16 slice products per FP64 product; bf16_tflops "
+                                              f"({peaks['source']})"},
                          "traffic": traffic_for("rdm_tc_moment_kernel", f"shadow RDM n={n} {P} snapshots")}}
 
 
@@ -1094,9 +1115,7 @@ def main():
             "rdm": rdm,
             "vce": vce,
             "local_energy": energy,
-            # per step: snapshot build (prepare, compaction, tensor-core records) and the
-            # overlap (walker prep, walker slices, pair kernel, reduction)
-            "gpu_launches": args.steps * 7}
+            "gpu_launches": args.steps * headline_launches(wl)}
     if rank == 0 and not args.no_cpu_baseline:
         def gpu_sample(Wc, Pc):
             s2 = qcs.Snapshots(ctx, Qd[:Pc].contiguous(), bd[:Pc].contiguous())
